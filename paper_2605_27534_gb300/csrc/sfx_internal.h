@@ -201,6 +201,7 @@ struct sfx_ctx {
   sfx::F32Scratch f32;
   sfx::AdjScratch adj;
   float* chi32 = nullptr;            // SFX_F32 redistancing: chi0, two iterates
+  void* rd_list = nullptr;           // redistancing: active blocks and their flags
   double* vofH = nullptr;            // VoF: indicator H, face fluxes Q
   double* vofQ = nullptr;
   double* acdi = nullptr;            // ACDI: phi*, r, psi, unit normals
