@@ -94,10 +94,11 @@ typedef struct {
   int nu1, nu2;       /* red-black Gauss-Seidel sweeps before / after the
                          coarse-grid correction */
   int mg_levels;      /* levels in the V-cycle (1 = smoother only; 0 = auto:
-                         SFX_F64 every level; SFX_F32 relaxation alone when
-                         max(Df, DF) dt/h^2 <= 1, else a V-cycle on the
-                         Newton correction over the levels whose h <= 3 eps,
-                         at least two) */
+                         relaxation of a Newton correction alone when
+                         max(Df, DF) dt/h^2 <= 1; else SFX_F64 Picard
+                         iteration over every level, SFX_F32 a V-cycle on
+                         the Newton correction over the levels whose
+                         h <= 3 eps, at least two) */
   int vcycles;        /* V-cycles per field per Picard iteration (>= 1) */
   int check_every;    /* Picard iterations between residual checks (>= 1) */
   int coarse_sweeps;  /* Gauss-Seidel sweeps on the coarsest level */
@@ -198,7 +199,12 @@ sfx_status sfx_vof_advect(sfx_ctx* ctx, const void* ux, const void* uy, const vo
    (0 for q <= 1e-3, the unit vector for q >= 2e-3), and n = 0 where
    |grad phi| < 1e-30.  f and F
    (state layout of the context) are updated in place; phi is double, the
-   velocities are in the context precision.  SFX_F32 contexts solve the
+   velocities are in the context precision.  SFX_F64 contexts with
+   opts->mg_levels = 0 and max(Df, DF) dt/h^2 <= 1 solve the coupled system
+   by Newton defect correction instead (FP64 state and residuals, the
+   correction relaxed by nu1 + nu2 FP32 red-black sweeps with a 2x2 block
+   solve per cell) and fall back to Picard iteration where it does not
+   converge; stats then count its iterations.  SFX_F32 contexts solve the
    same system by coupled Newton defect correction (SFX_TUNE_F32_SOLVER):
    each iteration evaluates both residuals in pair arithmetic and relaxes
    the correction by nu1 + nu2 FP32 red-black sweeps with a 2x2 block solve

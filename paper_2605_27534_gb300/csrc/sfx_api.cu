@@ -151,6 +151,9 @@ void sfx_ctx_destroy(sfx_ctx* c) {
   for (void* p : c->allocations) cudaFree(p);
   if (c->h_norms) cudaFreeHost(c->h_norms);
   if (c->h_sums) cudaFreeHost(c->h_sums);
+  for (cudaEvent_t e : c->n64.ev)
+    if (e) cudaEventDestroy(e);
+  if (c->n64.report) cudaFreeHost(c->n64.report);
   if (c->adj.h_out) cudaFreeHost(c->adj.h_out);
   if (c->adj.h_nrm) cudaFreeHost(c->adj.h_nrm);
   if (c->adj.relax) cudaGraphExecDestroy(c->adj.relax);

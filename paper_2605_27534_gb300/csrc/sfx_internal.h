@@ -164,6 +164,17 @@ struct AdjScratch {
   int relax_sweeps = 0;           // S of the captured graph
 };
 
+// Work arrays of the FP64 coupled Newton solve, allocated on first use.
+struct N64Scratch {
+  bool ready = false;
+  __half2* H[3] = {};             // (B_f, B_F) per face in half precision
+  float2* e2 = nullptr;           // corrections (e_f, e_F), colour-packed
+  float4* rc = nullptr;           // r_f, r_F, u, v, colour-packed
+  void* ctl = nullptr;            // norms and convergence flags (device)
+  unsigned int* report = nullptr; // two iterations' norms and verdicts (pinned host)
+  cudaEvent_t ev[2] = {nullptr, nullptr};
+};
+
 struct Prof {
   bool on = false;
   long long launches[K_COUNT] = {};
@@ -200,6 +211,7 @@ struct sfx_ctx {
   sfx::Prof prof;
   sfx::F32Scratch f32;
   sfx::AdjScratch adj;
+  sfx::N64Scratch n64;
   float* chi32 = nullptr;            // SFX_F32 redistancing: chi0, two iterates
   void* rd_list = nullptr;           // redistancing: active blocks and their flags
   double* vofH = nullptr;            // VoF: indicator H, face fluxes Q
@@ -254,9 +266,18 @@ sfx_status mg_solve(sfx_ctx* c, double D, const double* Bx, const double* By, co
 sfx_status surfactant_step(sfx_ctx* c, const sfx_params* p, const void* phi, const void* ux,
                            const void* uy, const void* uz, double* f, double* F, double dt,
                            const sfx_solve_opts* o, sfx_step_stats* st, cudaStream_t s);
-// sfx_solver.cu: drift faces of both problems from a double phi
+// sfx_newton64.cu: drift faces of both problems from a double phi
 sfx_status drift_faces64(sfx_ctx* c, const double* phi, double Df, double DF, double eps,
                          double* const* Bf, double* const* BF, cudaStream_t s);
+// sfx_newton64.cu: the coupled Newton solve of a step in FP64 contexts (drift
+// faces and coefficients first; the first iterate is (f, F), or (f*, F*) with
+// from_star).  It ends with *conv false when it should be left to the Picard
+// solver.
+bool newton64_eligible(const sfx_ctx* c, const sfx_params* p, double dt, const sfx_solve_opts* o);
+sfx_status newton64_prepare(sfx_ctx* c, const sfx_params* p, const double* phi, cudaStream_t s);
+sfx_status newton64_solve(sfx_ctx* c, const sfx_params* p, double* f, double* F, double dt,
+                          bool from_star, const sfx_solve_opts* o, int* iters, double* rel,
+                          bool* conv, cudaStream_t s);
 // sfx_acdi.cu
 sfx_status acdi_step(sfx_ctx* c, const void* ux, const void* uy, const void* uz, double dt,
                      double zeta, double eps, int clip, double* phi, cudaStream_t s);

@@ -308,13 +308,12 @@ struct Kin {
 
 // f problem: lambda_f = 1/dt + r_d + r_a F/(phi+eta),
 //            b_f = f_star/dt + r_a F/(phi+eta) Gamma_inf phi(1-phi)/eps
-template <typename P>
-__global__ void k_setup_f(size_t n, Kin q, const P* __restrict__ phi, const double* __restrict__ F,
+__global__ void k_setup_f(size_t n, Kin q, const double* __restrict__ phi, const double* __restrict__ F,
                           const double* __restrict__ fstar, double* __restrict__ lam,
                           double* __restrict__ b) {
   for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
        c += (size_t)gridDim.x * blockDim.x) {
-    double p = (double)phi[c];
+    double p = phi[c];
     double Fs = F[c] / (p + q.eta);
     lam[c] = q.inv_dt + q.kd + q.ka * Fs;
     b[c] = fstar[c] * q.inv_dt + q.ka * Fs * (q.ginf * p * (1.0 - p) / q.eps);
@@ -322,13 +321,12 @@ __global__ void k_setup_f(size_t n, Kin q, const P* __restrict__ phi, const doub
 }
 
 // F problem: lambda_F = 1/dt + r_a (f_inf - f)/(phi+eta), b_F = F_star/dt + r_d f
-template <typename P>
-__global__ void k_setup_F(size_t n, Kin q, const P* __restrict__ phi, const double* __restrict__ f,
+__global__ void k_setup_F(size_t n, Kin q, const double* __restrict__ phi, const double* __restrict__ f,
                           const double* __restrict__ Fstar, double* __restrict__ lam,
                           double* __restrict__ b) {
   for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
        c += (size_t)gridDim.x * blockDim.x) {
-    double p = (double)phi[c];
+    double p = phi[c];
     double finf = q.ginf * p * (1.0 - p) / q.eps;
     lam[c] = q.inv_dt + q.ka * (finf - f[c]) / (p + q.eta);
     b[c] = Fstar[c] * q.inv_dt + q.kd * f[c];
@@ -337,8 +335,7 @@ __global__ void k_setup_F(size_t n, Kin q, const P* __restrict__ phi, const doub
 
 // Both nonlinear residuals of App. C at the current (f, F):
 // norms[0..3] = |r_f|, |b_f|, |r_F|, |b_F| (infinity norms).
-template <typename P>
-__global__ void k_coupled_resid(Level L, Kin q, Op opf, Op opF, const P* __restrict__ phi,
+__global__ void k_coupled_resid(Level L, Kin q, Op opf, Op opF, const double* __restrict__ phi,
                                 const double* __restrict__ f, const double* __restrict__ F,
                                 const double* __restrict__ fstar,
                                 const double* __restrict__ Fstar, unsigned long long* norms,
@@ -348,7 +345,7 @@ __global__ void k_coupled_resid(Level L, Kin q, Op opf, Op opF, const P* __restr
   for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
        c += (size_t)gridDim.x * blockDim.x) {
     int i = (int)(c % L.nx), j = (int)((c / L.nx) % L.ny), k = (int)(c / ((size_t)L.nx * L.ny));
-    double p = (double)phi[c];
+    double p = phi[c];
     double pe = p + q.eta, finf = q.ginf * p * (1.0 - p) / q.eps;
     double iv = 1.0 / cell_volume(L, i);
     double sd, sn;
@@ -373,27 +370,6 @@ __global__ void k_coupled_resid(Level L, Kin q, Op opf, Op opF, const P* __restr
   for (int s = 0; s < 4; ++s) {
     double v = warp_max(m[s]);
     if ((threadIdx.x & 31) == 0) atomic_max_nonneg(&norms[s], v);
-  }
-}
-
-// Face drifts of both problems in direction d (App. C):
-//   B_f = -Df 2(0.5 - phi)/eps n,  B_F = -DF (1 - phi)/eps n,
-// face value = mean of the two adjacent cell values; walls 0.
-template <typename P>
-__global__ void k_drift_faces(Level L, int d, const P* __restrict__ phi, double Df, double DF,
-                              double eps, double* __restrict__ Bf, double* __restrict__ BF) {
-  size_t n = L.nface(d);
-  int fx = L.nx + (d == 0), fy = L.ny + (d == 1);
-  for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n;
-       q += (size_t)gridDim.x * blockDim.x) {
-    int i = (int)(q % fx), j = (int)((q / fx) % fy), k = (int)(q / ((size_t)fx * fy));
-    int pos = d == 0 ? i : (d == 1 ? j : k);
-    if (pos == 0 || pos == L.extent(d)) { Bf[q] = 0.0; BF[q] = 0.0; continue; }
-    int li = i - (d == 0), lj = j - (d == 1), lk = k - (d == 2);
-    double pL = (double)phi[cidx(L, li, lj, lk)], pR = (double)phi[cidx(L, i, j, k)];
-    double nL = normal_comp(L, phi, li, lj, lk, d, eps), nR = normal_comp(L, phi, i, j, k, d, eps);
-    Bf[q] = 0.5 * ((-Df * 2.0 * (0.5 - pL) / eps) * nL + (-Df * 2.0 * (0.5 - pR) / eps) * nR);
-    BF[q] = 0.5 * ((-DF * (1.0 - pL) / eps) * nL + (-DF * (1.0 - pR) / eps) * nR);
   }
 }
 
@@ -519,36 +495,23 @@ sfx_status clear_norms(sfx_ctx* c, cudaStream_t s) {
 
 double rel(double r, double b) { return r / (b > 1e-300 ? b : 1e-300); }
 
-template <typename P>
-sfx_status step_impl(sfx_ctx* c, const sfx_params* p, const P* phi, const void* ux,
-                     const void* uy, const void* uz, double* f, double* F, double dt,
-                     const sfx_solve_opts* o, sfx_step_stats* stats, cudaStream_t s) {
+// App. C by Picard iteration from the (f, F) given: each iteration the f
+// problem with the latest F, then the F problem with the new f, each by
+// multigrid V-cycles, until both nonlinear residuals pass.  The drift faces
+// of the finest level are in place; (f*, F*) are in the context.
+sfx_status picard(sfx_ctx* c, const sfx_params* p, const double* phi, double* f, double* F,
+                  double dt, const sfx_solve_opts* o, int* iters, int* cyc, double* res,
+                  bool* converged, cudaStream_t s) {
   const Level& L = c->lev[0].lv;
   const size_t n = L.ncell();
   const int nlev = levels_to_use(c, o);
   const int nd = L.ndim();
-  // drift faces of both problems at every level (phi is fixed over the step)
-  for (int d = 0; d < nd; ++d)
-    SFX_KERNEL(c, K_SETUP, k_drift_faces<P>, blocks_for(L.nface(d), 256), 256, s, 
-        L, d, phi, p->Df, p->DF, p->eps, c->lev[0].B[0][d], c->lev[0].B[1][d]);
   for (int l = 1; l < nlev; ++l)
     for (int fld = 0; fld < 2; ++fld)
       for (int d = 0; d < nd; ++d)
         SFX_KERNEL(c, K_SETUP, k_restrict_faces, blocks_for(c->lev[l].lv.nface(d), 256), 256, s, 
             c->lev[l - 1].lv, c->lev[l].lv, d, c->lev[l - 1].B[fld][d], c->lev[l].B[fld][d]);
   SFX_LAUNCH_CHECK();
-  // a3: explicit advection, then start the implicit solve from (f*, F*)
-  if (ux) {
-    sfx_status st = advect(c, ux, uy, uz, dt, f, p->bc_f, c->fstar, s);
-    if (st != SFX_OK) return st;
-    st = advect(c, ux, uy, uz, dt, F, p->bc_F, c->Fstar, s);
-    if (st != SFX_OK) return st;
-    SFX_CUDA(cudaMemcpyAsync(f, c->fstar, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    SFX_CUDA(cudaMemcpyAsync(F, c->Fstar, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
-  } else {
-    SFX_CUDA(cudaMemcpyAsync(c->fstar, f, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    SFX_CUDA(cudaMemcpyAsync(c->Fstar, F, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
-  }
   Kin q{p->ka, p->kd, p->gamma_inf, p->eps, p->eta, 1.0 / dt};
   Hier Hf{}, HF{};
   Hf.nlev = HF.nlev = nlev;
@@ -569,7 +532,7 @@ sfx_status step_impl(sfx_ctx* c, const sfx_params* p, const P* phi, const void* 
   double nrm[4] = {0, 0, 0, 0};
   const int nb = blocks_for(n, 256);
   for (it = 1; it <= o->max_cycles; ++it) {
-    SFX_KERNEL(c, K_SETUP, k_setup_f<P>, nb, 256, s, n, q, phi, F, c->fstar, lam0, b0);
+    SFX_KERNEL(c, K_SETUP, k_setup_f, nb, 256, s, n, q, phi, F, c->fstar, lam0, b0);
     SFX_LAUNCH_CHECK();
     sfx_status st = restrict_lambda(c, nlev, s);
     if (st != SFX_OK) return st;
@@ -578,7 +541,7 @@ sfx_status step_impl(sfx_ctx* c, const sfx_params* p, const P* phi, const void* 
       if (st != SFX_OK) return st;
       ++cycles;
     }
-    SFX_KERNEL(c, K_SETUP, k_setup_F<P>, nb, 256, s, n, q, phi, f, c->Fstar, lam0, b0);
+    SFX_KERNEL(c, K_SETUP, k_setup_F, nb, 256, s, n, q, phi, f, c->Fstar, lam0, b0);
     SFX_LAUNCH_CHECK();
     st = restrict_lambda(c, nlev, s);
     if (st != SFX_OK) return st;
@@ -590,28 +553,75 @@ sfx_status step_impl(sfx_ctx* c, const sfx_params* p, const P* phi, const void* 
     if (it % o->check_every == 0 || it == o->max_cycles) {
       st = clear_norms(c, s);
       if (st != SFX_OK) return st;
-      SFX_KERNEL(c, K_RESIDUAL, k_coupled_resid<P>, blocks_for(n, 256), 256, s, L, q, op_at(Hf, 0), op_at(HF, 0), phi,
+      SFX_KERNEL(c, K_RESIDUAL, k_coupled_resid, blocks_for(n, 256), 256, s, L, q, op_at(Hf, 0), op_at(HF, 0), phi,
                                                             f, F, c->fstar, c->Fstar, c->d_norms,
                                                             c->d_flag);
       SFX_LAUNCH_CHECK();
       bool bad = false;
       st = read_norms(c, s, nrm, &bad);
       if (st != SFX_OK) return st;
-      if (bad) {
-        if (stats) stats->converged = 0;
-        return SFX_ERR_NONFINITE;
-      }
+      if (bad) return SFX_ERR_NONFINITE;
       if (rel(nrm[0], nrm[1]) <= o->tol && rel(nrm[2], nrm[3]) <= o->tol) {
         conv = true;
         break;
       }
     }
   }
+  *iters = std::min(it, o->max_cycles);
+  *cyc = cycles;
+  res[0] = rel(nrm[0], nrm[1]);
+  res[1] = rel(nrm[2], nrm[3]);
+  *converged = conv;
+  return SFX_OK;
+}
+
+sfx_status step_impl(sfx_ctx* c, const sfx_params* p, const double* phi, const void* ux,
+                     const void* uy, const void* uz, double* f, double* F, double dt,
+                     const sfx_solve_opts* o, sfx_step_stats* stats, cudaStream_t s) {
+  const Level& L = c->lev[0].lv;
+  const size_t n = L.ncell();
+  // drift faces of both problems (phi is fixed over the step)
+  const bool newton = newton64_eligible(c, p, dt, o);
+  sfx_status ds = newton ? newton64_prepare(c, p, phi, s)
+                         : drift_faces64(c, phi, p->Df, p->DF, p->eps, c->lev[0].B[0],
+                                         c->lev[0].B[1], s);
+  if (ds != SFX_OK) return ds;
+  // a3: explicit advection, then start the implicit solve from (f*, F*)
+  if (ux) {
+    sfx_status st = advect(c, ux, uy, uz, dt, f, p->bc_f, c->fstar, s);
+    if (st != SFX_OK) return st;
+    st = advect(c, ux, uy, uz, dt, F, p->bc_F, c->Fstar, s);
+    if (st != SFX_OK) return st;
+  } else {
+    SFX_CUDA(cudaMemcpyAsync(c->fstar, f, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    SFX_CUDA(cudaMemcpyAsync(c->Fstar, F, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
+  }
+  int it = 0, cycles = 0;
+  bool conv = false;
+  double res[2] = {0, 0};
+  if (newton) {
+    // the coupled Newton solve; where it does not converge the Picard
+    // solver below starts again from (f*, F*)
+    sfx_status st = newton64_solve(c, p, f, F, dt, ux != nullptr, o, &it, res, &conv, s);
+    if (st != SFX_OK) return st;
+    cycles = 2 * it * std::max(1, o->nu1 + o->nu2);
+  }
+  if (!conv) {
+    if (ux || newton) {
+      SFX_CUDA(cudaMemcpyAsync(f, c->fstar, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
+      SFX_CUDA(cudaMemcpyAsync(F, c->Fstar, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    }
+    sfx_status st = picard(c, p, phi, f, F, dt, o, &it, &cycles, res, &conv, s);
+    if (st != SFX_OK) {
+      if (st == SFX_ERR_NONFINITE && stats) stats->converged = 0;
+      return st;
+    }
+  }
   if (stats) {
-    stats->picard = std::min(it, o->max_cycles);
+    stats->picard = it;
     stats->vcycles = cycles;
-    stats->res_f = rel(nrm[0], nrm[1]);
-    stats->res_F = rel(nrm[2], nrm[3]);
+    stats->res_f = res[0];
+    stats->res_F = res[1];
     stats->converged = conv ? 1 : 0;
     const double* fl[2] = {f, F};
     double m[2];
@@ -625,22 +635,10 @@ sfx_status step_impl(sfx_ctx* c, const sfx_params* p, const P* phi, const void* 
 
 }  // namespace
 
-sfx_status drift_faces64(sfx_ctx* c, const double* phi, double Df, double DF, double eps,
-                         double* const* Bf, double* const* BF, cudaStream_t s) {
-  const Level& L = c->lev[0].lv;
-  for (int d = 0; d < L.ndim(); ++d)
-    SFX_KERNEL(c, K_SETUP, k_drift_faces<double>, blocks_for(L.nface(d), 256), 256, s, L, d, phi,
-               Df, DF, eps, Bf[d], BF[d]);
-  SFX_LAUNCH_CHECK();
-  return SFX_OK;
-}
-
 sfx_status surfactant_step(sfx_ctx* c, const sfx_params* p, const void* phi, const void* ux,
                            const void* uy, const void* uz, double* f, double* F, double dt,
                            const sfx_solve_opts* o, sfx_step_stats* st, cudaStream_t s) {
-  if (c->prec == SFX_F64)
-    return step_impl<double>(c, p, (const double*)phi, ux, uy, uz, f, F, dt, o, st, s);
-  return step_impl<float>(c, p, (const float*)phi, ux, uy, uz, f, F, dt, o, st, s);
+  return step_impl(c, p, (const double*)phi, ux, uy, uz, f, F, dt, o, st, s);
 }
 
 sfx_status mg_solve(sfx_ctx* c, double D, const double* Bx, const double* By, const double* Bz,
