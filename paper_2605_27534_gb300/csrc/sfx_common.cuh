@@ -50,6 +50,28 @@ __host__ __device__ inline double face_area(const Level& L, int d, int i) {
   return kPi * (double)(2 * i + 1) * h * h;
 }
 
+// float to double without the conversion instruction, which issues at the
+// rate of the FP64 pipe (1/59 of the integer words'): sign, exponent + 896,
+// mantissa << 29.  Zeros, denormals, infinities and NaN take the instruction.
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x), e = b & 0x7f800000u;
+  if (e == 0u || e == 0x7f800000u) return (b << 1) == 0u ? __hiloint2double((int)b, 0) : (double)x;
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)),
+                          (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
+// Row r = k ny + j of a row-walking kernel (64-bit division only past 2^32).
+__device__ __forceinline__ void row_jk(size_t r, int ny, int& j, int& k) {
+  if (r >> 32) {
+    k = (int)(r / (size_t)ny);
+    j = (int)(r - (size_t)k * ny);
+  } else {
+    k = (int)((unsigned)r / (unsigned)ny);
+    j = (int)((unsigned)r - (unsigned)k * (unsigned)ny);
+  }
+}
+
 // ---------------------------------------------------------------- reductions
 // Max of non-negative doubles via their bit patterns (order-independent,
 // hence deterministic).  NaN sets the flag instead.

@@ -588,9 +588,8 @@ sfx_status step_impl(sfx_ctx* c, const sfx_params* p, const double* phi, const v
   if (ds != SFX_OK) return ds;
   // a3: explicit advection, then start the implicit solve from (f*, F*)
   if (ux) {
-    sfx_status st = advect(c, ux, uy, uz, dt, f, p->bc_f, c->fstar, s);
-    if (st != SFX_OK) return st;
-    st = advect(c, ux, uy, uz, dt, F, p->bc_F, c->Fstar, s);
+    const sfx_status st = advect2(c, (const double*)ux, (const double*)uy, (const double*)uz, dt, f,
+                                  F, p->bc_f, p->bc_F, c->fstar, c->Fstar, s);
     if (st != SFX_OK) return st;
   } else {
     SFX_CUDA(cudaMemcpyAsync(c->fstar, f, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
