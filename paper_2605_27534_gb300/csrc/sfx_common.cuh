@@ -61,16 +61,32 @@ __device__ __forceinline__ double widen(float x) {
 }
 __device__ __forceinline__ double widen(double x) { return x; }
 
-// Row r = k ny + j of a row-walking kernel (64-bit division only past 2^32).
-__device__ __forceinline__ void row_jk(size_t r, int ny, int& j, int& k) {
-  if (r >> 32) {
-    k = (int)(r / (size_t)ny);
-    j = (int)(r - (size_t)k * ny);
-  } else {
-    k = (int)((unsigned)r / (unsigned)ny);
-    j = (int)((unsigned)r - (unsigned)k * (unsigned)ny);
+// Blocks of 32 x 4 x 4 cells (32 x 16 in 2D) with 512 threads for kernels
+// whose work sits in a band around the interface: a warp holds 8 x 2 x 2
+// cells (8 x 4), so that few warps straddle the band's edge.
+template <int ND>
+struct CellBlock {
+  static constexpr int bx = 32, by = ND == 3 ? 4 : 16, bz = ND == 3 ? 4 : 1, threads = 512;
+  static __device__ __forceinline__ int3 cell(int t) {
+    const int l = t & 31, w = t >> 5;
+    return ND == 3 ? make_int3((w & 3) * 8 + (l & 7), (w >> 2 & 1) * 2 + (l >> 3 & 1),
+                               (w >> 3) * 2 + (l >> 4))
+                   : make_int3((w & 3) * 8 + (l & 7), (w >> 2) * 4 + (l >> 3), 0);
   }
-}
+  static size_t count(const Level& L) {
+    return (((size_t)L.nx + bx - 1) / bx) * (((size_t)L.ny + by - 1) / by) *
+           (((size_t)L.nz + bz - 1) / bz);
+  }
+  // the cell of this thread in block b; false past the grid
+  static __device__ __forceinline__ bool at(const Level& L, unsigned b, int* x) {
+    const unsigned nbx = (L.nx + bx - 1) / bx, nby = (L.ny + by - 1) / by;
+    const int3 l = cell(threadIdx.x);
+    x[0] = (int)(b % nbx) * bx + l.x;
+    x[1] = (int)(b / nbx % nby) * by + l.y;
+    x[2] = (int)(b / nbx / nby) * bz + l.z;
+    return x[0] < L.nx && x[1] < L.ny && x[2] < L.nz;
+  }
+};
 
 // ---------------------------------------------------------------- reductions
 // Max of non-negative doubles via their bit patterns (order-independent,

@@ -323,24 +323,6 @@ sfx_status marangoni32(sfx_ctx* c, const sfx_params* p, const float2* f, const d
 sfx_status df_pack(const double* in, void* out, size_t n, cudaStream_t s);
 sfx_status df_unpack(const void* in, double* out, size_t n, cudaStream_t s);
 
-// Launch shape of the row-walking kernels: x chunks of up to 256 threads (a
-// multiple of 32), rows k ny + j in turn, one row per block up to 16 row
-// groups per SM and chunk of 256 threads.
-struct RowShape {
-  dim3 grid, block;
-};
-inline RowShape row_shape(const Level& L, int sms) {
-  RowShape g;
-  const int tx = L.nx >= 256 ? 256 : ((L.nx + 31) / 32) * 32;
-  const size_t xb = ((size_t)L.nx + tx - 1) / tx, rows = (size_t)L.ny * L.nz;
-  size_t want = (size_t)sms * 16 * (256 / tx) / xb;
-  if (want < 1) want = 1;
-  if (want > 65535) want = 65535;
-  g.block = dim3(tx);
-  g.grid = dim3((unsigned)xb, (unsigned)(rows < want ? rows : want));
-  return g;
-}
-
 inline int blocks_for(size_t n, int threads) {
   size_t b = (n + threads - 1) / threads;
   if (b > 152 * 64) b = 152 * 64;

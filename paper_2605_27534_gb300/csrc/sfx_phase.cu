@@ -88,18 +88,7 @@ __device__ __forceinline__ T redist_update(int nd, T s0, T x0, const T* z0m, con
 // cell from its definition, 1.87 ms with active blocks.
 constexpr int kBx = 32;
 template <int ND>
-struct RdBlk {
-  static constexpr int by = ND == 3 ? 4 : 16, bz = ND == 3 ? 4 : 1;
-  // the cell of a thread: a warp holds 8 x 2 x 2 cells (8 x 4 in 2D), so that
-  // few warps straddle the edge of the moving front (rows of 32 cells
-  // stepped 1.6 times as many warps)
-  static __device__ __forceinline__ int3 cell(int t) {
-    const int l = t & 31, w = t >> 5;
-    return ND == 3 ? make_int3((w & 3) * 8 + (l & 7), (w >> 2 & 1) * 2 + (l >> 3 & 1),
-                               (w >> 3) * 2 + (l >> 4))
-                   : make_int3((w & 3) * 8 + (l & 7), (w >> 2) * 4 + (l >> 3), 0);
-  }
-};
+using RdBlk = CellBlock<ND>;   // (rows of 32 cells per warp stepped 1.6 times as many warps)
 
 struct RdGrid {
   int nbx, nby, nbz;   // blocks per direction
