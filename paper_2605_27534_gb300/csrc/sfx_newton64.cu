@@ -204,13 +204,18 @@ __device__ __forceinline__ double flux64(const Newton64& q, double Doh, const do
   return fma(Doh, fma(-cnt, a, S), T) * q.invh;
 }
 
-// The exchange is bilinear, so the difference (df, dF) of two solutions
-// solves the linearised system at their mean, with u + r_d and v there.
-// Its columns are dominated by their diagonals by 1/dt - 2 max(0, -(u + r_d))
-// and 1/dt - 2 max(0, -v): where both stay above -1/(2 dt) there is one
-// solution.  Iterates outside that region (an advected F below zero where
-// phi is small, f above Gamma_inf delta) are left to the Picard solver, so
-// that a step does not change branch.
+// The system may have several solutions.  The exchange is bilinear, so the
+// difference (df, dF) of two solutions solves the linearised system at their
+// mean, with U = u + r_d and v there; its columns are dominated by their
+// diagonals by 1/dt - 2 max(0, -U) and 1/dt - 2 max(0, -v), so where both stay
+// above -1/(2 dt) there is one.  Pointwise the exchange leaves a quadratic in
+// F whose roots have opposite signs wherever f* and F* are not negative; the
+// physical one, F >= 0, is where its slope 1/dt + U + v is positive.  Newton
+// is kept to iterates with U > -0.45/dt (F not below zero where phi is
+// small), v > -0.98/dt (f above Gamma_inf delta in the tails of phi reaches
+// -0.9/dt in the transient of an adsorption run; at -1/dt the F problem loses
+// its diagonal) and a positive slope; any other is left to the Picard
+// solver, so that a step does not change branch.
 //
 // Both residuals at every cell, rc = (r_f, r_F, u, v) and the first red
 // half-sweep of the correction (e = M^-1 r from zero), the norms, and in
@@ -288,9 +293,10 @@ k_resid64(Newton64 q, const double* __restrict__ f, const double* __restrict__ F
     m[1] = fmaxf(m[1], fabsf(__fmaf_rn((float)fst, idt, __fmul_rn(u, (float)finf))));
     m[2] = fmaxf(m[2], fabsf(rF));
     m[3] = fmaxf(m[3], fabsf(__fmaf_rn((float)Fst, idt, __fmul_rn((float)q.kd, (float)fc))));
-    // outside the region of a unique solution (below): as a non-finite norm
-    if (!(fabsf(rf) <= 3.0e38f) || !(fabsf(rF) <= 3.0e38f) ||
-        fminf(__fadd_rn(u, (float)q.kd), v) < -0.45f * idt)
+    // off the branch (above): as a non-finite norm
+    const float U = __fadd_rn(u, (float)q.kd);
+    if (!(fabsf(rf) <= 3.0e38f) || !(fabsf(rF) <= 3.0e38f) || U < -0.45f * idt ||
+        v < -0.98f * idt || __fadd_rn(U, v) < -0.98f * idt)
       m[0] = m[2] = __int_as_float(0x7f800000);
   }
   resid_norms(m, ctl->nrm);
