@@ -213,8 +213,8 @@ struct sfx_ctx {
   sfx::AdjScratch adj;
   sfx::N64Scratch n64;
   float* chi32 = nullptr;            // SFX_F32 redistancing: chi0, two iterates
-  void* rd_list = nullptr;           // redistancing: active blocks and their flags
-  double* vofH = nullptr;            // VoF: indicator H, face fluxes Q
+  void* block_list = nullptr;        // redistancing and VoF: active blocks and their flags
+  unsigned char* vofH = nullptr;     // VoF: indicator H, minus-face fluxes Q by cell
   double* vofQ = nullptr;
   double* acdi = nullptr;            // ACDI: phi*, r, psi, unit normals
 };
@@ -257,6 +257,9 @@ sfx_status phase_field_from_chi(sfx_ctx* c, const double* chi, double* phi, doub
 // sfx_advect.cu
 sfx_status advect(sfx_ctx* c, const void* ux, const void* uy, const void* uz, double dt,
                   const double* xi, double bc_in, double* out, cudaStream_t s);
+// phi of an ACDI step
+sfx_status advect_phi(sfx_ctx* c, const void* ux, const void* uy, const void* uz, double dt,
+                      const double* xi, double bc_in, double* out, cudaStream_t s);
 // both transported fields of an SFX_F64 context at once
 sfx_status advect2(sfx_ctx* c, const double* ux, const double* uy, const double* uz, double dt,
                    const double* f, const double* F, double bc_f, double bc_F, double* fout,
@@ -288,6 +291,9 @@ sfx_status acdi_step(sfx_ctx* c, const void* ux, const void* uy, const void* uz,
 // sfx_capillary.cu
 sfx_status capillary(sfx_ctx* c, const sfx_params* p, const double* phi, const void* C,
                      const void* sigma, void* kappa, void* force, cudaStream_t s);
+// sfx_phase.cu: ctx->block_list for nb blocks of cells: a count, nb int2 and
+// two flags per block (allocated on first use; each pass fills it anew)
+sfx_status block_list(sfx_ctx* c, size_t nb);
 // sfx_vof.cu
 sfx_status vof_advect(sfx_ctx* c, const void* ux, const void* uy, const void* uz, double dt,
                       int order, double* C, cudaStream_t s);

@@ -433,11 +433,9 @@ static sfx_status redistance_blocks(sfx_ctx* c, const double* C, T* aux, T* a, T
   using B = RdBlk<ND>;
   const RdGrid R{(L.nx + kBx - 1) / kBx, (L.ny + B::by - 1) / B::by, (L.nz + B::bz - 1) / B::bz};
   const size_t nb = (size_t)R.nbx * R.nby * R.nbz;
-  if (!c->rd_list) {
-    SFX_CUDA(cudaMalloc((void**)&c->rd_list, (nb + 1) * sizeof(int2) + 2 * nb));
-    c->allocations.push_back(c->rd_list);
-  }
-  int2* list = (int2*)c->rd_list;
+  const sfx_status st = block_list(c, nb);
+  if (st != SFX_OK) return st;
+  int2* list = (int2*)c->block_list;
   unsigned char* f0 = (unsigned char*)(list + nb + 1);
   unsigned char* f1 = f0 + nb;
   // blocks of 512 threads in turn over the list, two to three per SM
@@ -460,6 +458,13 @@ static sfx_status redistance_blocks(sfx_ctx* c, const double* C, T* aux, T* a, T
   SFX_KERNEL(c, K_PHASE, (k_rd_finish<T, ND>), full, 512, s, L, R, (T)dtau, iters, eps, fi, C, a,
              chi, phi, delta);
   SFX_LAUNCH_CHECK();
+  return SFX_OK;
+}
+
+sfx_status block_list(sfx_ctx* c, size_t nb) {
+  if (c->block_list) return SFX_OK;
+  SFX_CUDA(cudaMalloc(&c->block_list, (nb + 1) * sizeof(int2) + 2 * nb));
+  c->allocations.push_back(c->block_list);
   return SFX_OK;
 }
 
