@@ -28,6 +28,11 @@
 // every cell in FP64 and six faces of a root and a quotient each, 0.42 ms with
 // a band of nine cells marked, 1.08 ms once the profile has spread over 96 % of
 // the box (cells 0.39, normals 0.14, update 0.51 ms).
+//
+// SFX_F64 contexts (BITS) keep every rounding of the definition: on a plateau
+// of phi its last bits set how far the normal of the forces is faded in, and
+// the curvature, double there, moved by up to 4e-8 of its scale with the
+// shorter forms.
 #include <algorithm>
 
 #include "sfx_internal.h"
@@ -91,8 +96,9 @@ __global__ void k_acdi_mark(Level L, const float* __restrict__ psi, float thr2,
   mark[c] = m2 < thr2 ? 0 : 1;
 }
 
-// r^(1/2) and psi of the cells that a marked cell's normal or faces read
-template <int ND>
+// r^(1/2) (BITS: r) and psi of the cells that a marked cell's normal or faces
+// read
+template <int ND, bool BITS>
 __global__ void k_acdi_cell(Level L, const unsigned char* __restrict__ mark,
                             const double* __restrict__ ps, double eps, double* __restrict__ g,
                             double* __restrict__ psi) {
@@ -108,13 +114,13 @@ __global__ void k_acdi_cell(Level L, const unsigned char* __restrict__ mark,
   if (!any) return;
   const double p = fmin(fmax(ps[c], 0.0), 1.0);
   const double rc = (p + kAcdiVeps) / (1.0 - p + kAcdiVeps);
-  g[c] = sqrt(rc);
+  g[c] = BITS ? rc : sqrt(rc);
   psi[c] = eps * log(rc);
 }
 
 // n = grad psi/|grad psi| of the marked cells (centred differences,
 // zero-gradient ghosts), 0 where psi is flat (above)
-template <int ND>
+template <int ND, bool BITS>
 __global__ void k_acdi_normal(Level L, const unsigned char* __restrict__ mark,
                               const double* __restrict__ psi, double* __restrict__ nv) {
   int x[3];
@@ -128,6 +134,16 @@ __global__ void k_acdi_normal(Level L, const unsigned char* __restrict__ mark,
   bool has[2 * ND];
   neighbours<ND>(L, x, c, o, has);
   double v[ND], m2 = 0.0;
+  if (BITS) {
+    const double inv2h = 0.5 / L.h;
+    for (int d = 0; d < ND; ++d) {
+      v[d] = (psi[o[2 * d + 1]] - psi[o[2 * d]]) * inv2h;
+      m2 += v[d] * v[d];
+    }
+    const double m = sqrt(m2);
+    for (int d = 0; d < ND; ++d) nv[(size_t)d * n + c] = m < kAcdiKappa ? 0.0 : v[d] / m;
+    return;
+  }
 #pragma unroll
   for (int d = 0; d < ND; ++d) {
     v[d] = psi[o[2 * d + 1]] - psi[o[2 * d]];
@@ -136,6 +152,44 @@ __global__ void k_acdi_normal(Level L, const unsigned char* __restrict__ mark,
   const double s = m2 < thr * thr ? 0.0 : rsqrt(m2);
 #pragma unroll
   for (int d = 0; d < ND; ++d) nv[(size_t)d * n + c] = v[d] * s;
+}
+
+// The BITS form of the update below: per face the flux
+// zeta [eps (phi*_R - phi*_L)/h - 1/4 w_f nbar_f], w_f = 4 s/(1 + s)^2.
+template <int ND, bool AXI>
+__global__ void k_acdi_update_bits(Level L, const unsigned char* __restrict__ mark,
+                                   const double* __restrict__ ps, const double* __restrict__ r,
+                                   const double* __restrict__ nv, double zeta, double eps,
+                                   double dt, int clip, double* __restrict__ phi) {
+  int x[3];
+  if (!CellBlock<ND>::at(L, blockIdx.x, x)) return;
+  const size_t c = cidx(L, x[0], x[1], x[2]), n = L.ncell();
+  size_t o[2 * ND];
+  bool has[2 * ND];
+  neighbours<ND>(L, x, c, o, has);
+  const double invh = 1.0 / L.h, pc = ps[c];
+  const int mc = mark[c];
+  double div = 0.0;
+  for (int q = 0; q < 2 * ND; ++q) {
+    if (!has[q]) continue;
+    const double s = q & 1 ? 1.0 : -1.0;
+    double w = 1.0;
+    if (AXI && q < 2) w = 2.0 * (double)(x[0] + q) / (double)(2 * x[0] + 1);
+    const int mo = mark[o[q]];
+    double af;
+    if (mc | mo) {
+      const double* nd = nv + (size_t)(q / 2) * n;
+      const double sq = sqrt(r[c] * r[o[q]]);
+      const double wt = 4.0 * sq / ((1.0 + sq) * (1.0 + sq));
+      const double nbar = 0.5 * ((mc ? nd[c] : 0.0) + (mo ? nd[o[q]] : 0.0));
+      af = zeta * (eps * s * (ps[o[q]] - pc) * invh - 0.25 * wt * nbar);
+    } else {
+      af = zeta * (eps * s * (ps[o[q]] - pc) * invh);
+    }
+    div += s * w * af;
+  }
+  const double v = pc + dt * div * invh;
+  phi[c] = clip ? fmin(fmax(v, 0.0), 1.0) : v;
 }
 
 // phi = phi* + dt/V sum_f (+-) A_f a_f; wall faces carry nothing and the
@@ -191,6 +245,26 @@ __global__ void k_acdi_update(Level L, const unsigned char* __restrict__ mark,
   phi[c] = clip ? fmin(fmax(v, 0.0), 1.0) : v;
 }
 
+template <int ND, bool AXI>
+void acdi_passes(sfx_ctx* c, const double* ps, double* g, double* psi, double* nv,
+                 const float* psi32, unsigned char* mark, float thr2, double zeta, double eps,
+                 double dt, int clip, double* phi, cudaStream_t s) {
+  const Level& L = c->lev[0].lv;
+  const int nb = (int)CellBlock<ND>::count(L), nt = CellBlock<ND>::threads;
+  SFX_KERNEL(c, K_PHASE, k_acdi_mark<ND>, nb, nt, s, L, psi32, thr2, mark);
+  if (c->prec == SFX_F64) {
+    SFX_KERNEL(c, K_PHASE, (k_acdi_cell<ND, true>), nb, nt, s, L, mark, ps, eps, g, psi);
+    SFX_KERNEL(c, K_PHASE, (k_acdi_normal<ND, true>), nb, nt, s, L, mark, psi, nv);
+    SFX_KERNEL(c, K_PHASE, (k_acdi_update_bits<ND, AXI>), nb, nt, s, L, mark, ps, g, nv, zeta, eps,
+               dt, clip, phi);
+  } else {
+    const double k1 = dt * zeta * eps / (L.h * L.h), k2 = 0.5 * dt * zeta / L.h;
+    SFX_KERNEL(c, K_PHASE, (k_acdi_cell<ND, false>), nb, nt, s, L, mark, ps, eps, g, psi);
+    SFX_KERNEL(c, K_PHASE, (k_acdi_normal<ND, false>), nb, nt, s, L, mark, psi, nv);
+    SFX_KERNEL(c, K_PHASE, (k_acdi_update<ND, AXI>), nb, nt, s, L, mark, ps, g, nv, k1, k2, clip, phi);
+  }
+}
+
 }  // namespace
 
 sfx_status acdi_step(sfx_ctx* c, const void* ux, const void* uy, const void* uz, double dt,
@@ -208,7 +282,7 @@ sfx_status acdi_step(sfx_ctx* c, const void* ux, const void* uy, const void* uz,
   float* psi32 = (float*)nv;              // read before the normals are written
   unsigned char* mark = (unsigned char*)(nv + (size_t)L.ndim() * n);
   if (ux) {
-    sfx_status st = advect(c, ux, uy, uz, dt, phi, 1.0, ps, s);
+    sfx_status st = advect_phi(c, ux, uy, uz, dt, phi, 1.0, ps, s);
     if (st != SFX_OK) return st;
   } else {
     SFX_CUDA(cudaMemcpyAsync(ps, phi, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
@@ -218,25 +292,9 @@ sfx_status acdi_step(sfx_ctx* c, const void* ux, const void* uy, const void* uz,
   // the float psi/(2h) is good to a few 1e-7 of its largest value 7 eps/h
   const double thr = std::max(0.0, 0.9 * kAcdiKappa - 1e-4 * eps / L.h);
   const float thr2 = (float)(thr * thr);
-  const int b3 = (int)CellBlock<3>::count(L), b2 = (int)CellBlock<2>::count(L), bt = 512;
-  const double k1 = dt * zeta * eps / (L.h * L.h), k2 = 0.5 * dt * zeta / L.h;
-  if (L.ndim() == 3) {
-    SFX_KERNEL(c, K_PHASE, k_acdi_mark<3>, b3, bt, s, L, psi32, thr2, mark);
-    SFX_KERNEL(c, K_PHASE, k_acdi_cell<3>, b3, bt, s, L, mark, ps, eps, g, psi);
-    SFX_KERNEL(c, K_PHASE, k_acdi_normal<3>, b3, bt, s, L, mark, psi, nv);
-    SFX_KERNEL(c, K_PHASE, (k_acdi_update<3, false>), b3, bt, s, L, mark, ps, g, nv, k1,
-               k2, clip, phi);
-  } else {
-    SFX_KERNEL(c, K_PHASE, k_acdi_mark<2>, b2, bt, s, L, psi32, thr2, mark);
-    SFX_KERNEL(c, K_PHASE, k_acdi_cell<2>, b2, bt, s, L, mark, ps, eps, g, psi);
-    SFX_KERNEL(c, K_PHASE, k_acdi_normal<2>, b2, bt, s, L, mark, psi, nv);
-    if (L.geom == SFX_AXISYM)
-      SFX_KERNEL(c, K_PHASE, (k_acdi_update<2, true>), b2, bt, s, L, mark, ps, g, nv, k1,
-                 k2, clip, phi);
-    else
-      SFX_KERNEL(c, K_PHASE, (k_acdi_update<2, false>), b2, bt, s, L, mark, ps, g, nv, k1,
-                 k2, clip, phi);
-  }
+  if (L.geom == SFX_CART3D) acdi_passes<3, false>(c, ps, g, psi, nv, psi32, mark, thr2, zeta, eps, dt, clip, phi, s);
+  else if (L.geom == SFX_AXISYM) acdi_passes<2, true>(c, ps, g, psi, nv, psi32, mark, thr2, zeta, eps, dt, clip, phi, s);
+  else acdi_passes<2, false>(c, ps, g, psi, nv, psi32, mark, thr2, zeta, eps, dt, clip, phi, s);
   SFX_LAUNCH_CHECK();
   return SFX_OK;
 }

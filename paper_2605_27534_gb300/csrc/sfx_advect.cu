@@ -22,6 +22,82 @@ struct Vel {
   const U* u[3];
 };
 
+// The step cell by cell, six face values each.  SFX_F64 contexts take phi of
+// an ACDI step through it: where phi is a plateau its last bits set how far
+// the normal is faded in, and with 1e3 of amplification the curvature (double
+// there) moves by 2e-9 when the fluxes are rounded in another order.
+// Everywhere else the tiles below give the same step several times faster.
+__device__ __forceinline__ double mc_limited(double xm, double x0, double xp) {
+  double dl = x0 - xm, dr = xp - x0;
+  if (dl * dr <= 0.0) return 0.0;
+  double dc = 0.5 * (xp - xm);
+  double m = fmin(fabs(dc), 2.0 * fmin(fabs(dl), fabs(dr)));
+  return dc > 0.0 ? m : -m;
+}
+
+// value of xi at cell idx shifted by s along d (the cell itself outside)
+__device__ __forceinline__ double nb(const Level& L, const double* __restrict__ xi,
+                                     const int* idx, size_t c, int d, int s) {
+  int p = idx[d] + s;
+  if (p < 0 || p >= L.extent(d)) return xi[c];
+  size_t stride = d == 0 ? 1 : (d == 1 ? (size_t)L.nx : (size_t)L.nx * L.ny);
+  return s > 0 ? xi[c + stride] : xi[c - stride];
+}
+
+// BCG face value on the face of direction d whose plus-side cell is f
+// (f[d] in 0..extent; f[d] = 0 or extent is a wall).
+template <typename U>
+__device__ double face_value(const Level& L, const Vel<U>& v, double dt,
+                             const double* __restrict__ xi, double bc_in, int d, const int* f,
+                             double u) {
+  int n = L.extent(d);
+  int uc[3] = {f[0], f[1], f[2]};
+  if (u > 0.0) {
+    if (f[d] == 0) return bc_in;
+    uc[d] -= 1;
+  } else if (f[d] == n) {
+    return bc_in;
+  }
+  size_t U_ = cidx(L, uc[0], uc[1], uc[2]);
+  double x0 = xi[U_];
+  double sgn = u > 0.0 ? 1.0 : -1.0;
+  double slope = mc_limited(nb(L, xi, uc, U_, d, -1), x0, nb(L, xi, uc, U_, d, +1));
+  double val = x0 + 0.5 * (sgn - u * dt / L.h) * slope;
+  for (int t = 0; t < L.ndim(); ++t) {
+    if (t == d) continue;
+    int ap[3] = {uc[0], uc[1], uc[2]};
+    ap[t] += 1;
+    double vbar = 0.5 * ((double)v.u[t][fidx(L, t, uc[0], uc[1], uc[2])] +
+                         (double)v.u[t][fidx(L, t, ap[0], ap[1], ap[2])]);
+    double dif = vbar > 0.0 ? x0 - nb(L, xi, uc, U_, t, -1) : nb(L, xi, uc, U_, t, +1) - x0;
+    val -= 0.5 * dt * vbar * dif / L.h;
+  }
+  return val;
+}
+
+template <typename U>
+__global__ void k_advect(Level L, Vel<U> v, double dt, const double* __restrict__ xi,
+                         double bc_in, double* __restrict__ out) {
+  const size_t n = L.ncell();
+  for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
+       c += (size_t)gridDim.x * blockDim.x) {
+    int idx[3] = {(int)(c % L.nx), (int)((c / L.nx) % L.ny), (int)(c / ((size_t)L.nx * L.ny))};
+    double div = 0.0;
+    for (int d = 0; d < L.ndim(); ++d) {
+      const U* ud = v.u[d];
+      double um = (double)ud[fidx(L, d, idx[0], idx[1], idx[2])];
+      if (um != 0.0)
+        div -= face_area(L, d, idx[0]) * um * face_value(L, v, dt, xi, bc_in, d, idx, um);
+      int p[3] = {idx[0], idx[1], idx[2]};
+      p[d] += 1;
+      double up = (double)ud[fidx(L, d, p[0], p[1], p[2])];
+      if (up != 0.0)
+        div += face_area(L, d, p[0]) * up * face_value(L, v, dt, xi, bc_in, d, p, up);
+    }
+    out[c] = xi[c] - dt * div / cell_volume(L, idx[0]);
+  }
+}
+
 // One step of NF fields (double) that share the velocities.
 //
 // Per cell and direction a face value needs only the cell value less the
@@ -260,6 +336,17 @@ sfx_status advect(sfx_ctx* c, const void* ux, const void* uy, const void* uz, do
   if (c->prec == SFX_F64)
     return bcg64(c, Vel<double>{{(const double*)ux, (const double*)uy, (const double*)uz}}, dt, P, s);
   return bcg64(c, Vel<float>{{(const float*)ux, (const float*)uy, (const float*)uz}}, dt, P, s);
+}
+
+sfx_status advect_phi(sfx_ctx* c, const void* ux, const void* uy, const void* uz, double dt,
+                      const double* xi, double bc_in, double* out, cudaStream_t s) {
+  if (c->prec != SFX_F64) return advect(c, ux, uy, uz, dt, xi, bc_in, out, s);
+  const Level& L = c->lev[0].lv;
+  const Vel<double> v{{(const double*)ux, (const double*)uy, (const double*)uz}};
+  SFX_KERNEL(c, K_ADVECT, k_advect<double>, blocks_for(L.ncell(), 256), 256, s, L, v, dt, xi, bc_in,
+             out);
+  SFX_LAUNCH_CHECK();
+  return SFX_OK;
 }
 
 sfx_status advect2(sfx_ctx* c, const double* ux, const double* uy, const double* uz, double dt,
