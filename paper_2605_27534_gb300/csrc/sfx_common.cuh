@@ -77,10 +77,13 @@ struct CellBlock {
     return (((size_t)L.nx + bx - 1) / bx) * (((size_t)L.ny + by - 1) / by) *
            (((size_t)L.nz + bz - 1) / bz);
   }
-  // the cell of this thread in block b; false past the grid
+  // the cell of this thread (or of thread t) in block b; false past the grid
   static __device__ __forceinline__ bool at(const Level& L, unsigned b, int* x) {
+    return at(L, b, x, threadIdx.x);
+  }
+  static __device__ __forceinline__ bool at(const Level& L, unsigned b, int* x, int t) {
     const unsigned nbx = (L.nx + bx - 1) / bx, nby = (L.ny + by - 1) / by;
-    const int3 l = cell(threadIdx.x);
+    const int3 l = cell(t);
     x[0] = (int)(b % nbx) * bx + l.x;
     x[1] = (int)(b / nbx % nby) * by + l.y;
     x[2] = (int)(b / nbx / nby) * bz + l.z;

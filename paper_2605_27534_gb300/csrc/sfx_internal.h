@@ -216,6 +216,7 @@ struct sfx_ctx {
   void* block_list = nullptr;        // redistancing and VoF: active blocks and their flags
   unsigned char* vofH = nullptr;     // VoF: indicator H, minus-face fluxes Q by cell
   double* vofQ = nullptr;
+  unsigned* vof_cut = nullptr;       // VoF: faces that need a plane (large grids)
   double* acdi = nullptr;            // ACDI: phi*, r, psi, unit normals
 };
 

@@ -16,59 +16,105 @@
 namespace sfx {
 namespace {
 
-// Only cells near fluid 1 change.  Where C is zero bit for bit every flux out
-// of a cell is zero, so a block of cells (32 x 4 x 4; 32 x 16 in 2D) without
-// fluid 1 in itself or an adjacent block stays as it is through the step (a
-// pass moves fluid by one cell along its direction).  On large grids the
-// blocks are classified once per step and the passes run over a list of the
-// active ones; small grids, where a launch costs more than the sweep, take
-// every block.  What bounds a pass on active blocks is the FP64 pipe
-// (velocity times dt/h, the update), so signs and the tests for empty and
-// full cells read the integer words and floats are widened without the
-// conversion instruction.  256^3 sphere of radius 64 in float: 2.45 ms per step
-// with every face and cell, 0.90 ms fresh and 1.35 ms once 500 steps have torn
-// off wisps (flux 236, update 26 us per direction, classification 94 us).
+// Only cells near fluid 1 change.  Every flux out of a cell with C <= 0 is
+// zero, so a block of cells (32 x 4 x 4; 32 x 16 in 2D) without fluid 1 in
+// itself or an adjacent block stays as it is through the step (a pass moves
+// fluid by one cell along its direction).  On large grids the blocks are
+// classified once per step and the passes run over a list of the active
+// ones; small grids, where a launch costs more than the sweep, take every
+// block.  What bounds a flux pass is the PLIC geometry (about 2000
+// instructions in a chain for a plane offset where C is within float rounding
+// of 0 or 1, as in a third of a drop's interior), so on large grids the faces
+// that need it are listed first and then taken by full warps (gathered per
+// block instead, the other warps of a block waited for the chains); signs and
+// the tests for empty and full cells read the integer words and floats are
+// widened without the conversion instruction, which issues at the FP64 rate.
+// 256^3 sphere of radius 64 in float: 2.45 ms per step with every face and
+// cell, 0.57 ms now (planes 102, other faces 42, update 24 us per direction,
+// classification 30 us), 0.85 ms after 500 steps of wisps.
 constexpr size_t kVofListCells = (size_t)1 << 20;
 
 __device__ __forceinline__ long long vbits(double v) { return __double_as_longlong(v); }
 
-// flag[b] = 1 where block b holds fluid 1; eight cells of loads in flight
+// flag[b] = 1 where block b holds fluid 1: a warp per block, its 16 rows of
+// 32 cells in flight together
 template <int ND>
-__global__ void __launch_bounds__(512) k_vof_flags(Level L, const double* __restrict__ C,
+__global__ void __launch_bounds__(256) k_vof_flags(Level L, unsigned nb, const double* __restrict__ C,
                                                    unsigned char* __restrict__ flag) {
-  int x[3];
-  const bool in = CellBlock<ND>::at(L, blockIdx.x, x);
-  const bool wet = in && vbits(C[cidx(L, x[0], x[1], x[2])]) != 0;
-  const int any = __syncthreads_or(wet);
-  if (threadIdx.x == 0) flag[blockIdx.x] = any ? 1 : 0;
+  using B = CellBlock<ND>;
+  const unsigned b = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+  if (b >= nb) return;
+  const unsigned nbx = (L.nx + B::bx - 1) / B::bx, nby = (L.ny + B::by - 1) / B::by;
+  const int i = (int)(b % nbx) * B::bx + (threadIdx.x & 31);
+  const int j0 = (int)(b / nbx % nby) * B::by, k0 = (int)(b / nbx / nby) * B::bz;
+  bool wet = false;
+  if (i < L.nx) {
+#pragma unroll
+    for (int r = 0; r < B::by * B::bz; ++r) {
+      const int j = j0 + r % B::by, k = k0 + r / B::by;
+      if (j < L.ny && k < L.nz) wet |= vbits(C[cidx(L, i, j, k)]) > 0;
+    }
+  }
+  const bool any = __any_sync(0xffffffffu, wet);
+  if ((threadIdx.x & 31) == 0) flag[b] = any ? 1 : 0;
 }
 
-// The blocks with a flagged block among themselves and their neighbours
-// (diagonals included), each with a bit per direction whose plus-side
-// neighbour block is active too; list[0] counts them.
+// act[b] = 1 where block b or a neighbour (diagonals included) is flagged
 template <int ND>
-__global__ void k_vof_list(Level L, const unsigned char* __restrict__ flag, int2* __restrict__ list) {
+__global__ void k_vof_active(Level L, const unsigned char* __restrict__ flag,
+                             unsigned char* __restrict__ act) {
   using B = CellBlock<ND>;
   const int nx = (L.nx + B::bx - 1) / B::bx, ny = (L.ny + B::by - 1) / B::by,
             nz = (L.nz + B::bz - 1) / B::bz;
   const int nb = nx * ny * nz;
-  auto active = [&](int X, int Y, int Z) {
-    if (X >= nx || Y >= ny || Z >= nz) return false;
-    for (int c = max(Z - 1, 0); c <= min(Z + 1, nz - 1); ++c)
-      for (int b = max(Y - 1, 0); b <= min(Y + 1, ny - 1); ++b)
-        for (int a = max(X - 1, 0); a <= min(X + 1, nx - 1); ++a)
-          if (flag[(c * ny + b) * nx + a]) return true;
-    return false;
-  };
   for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x) {
     const int X = b % nx, Y = b / nx % ny, Z = b / nx / ny;
-    if (!active(X, Y, Z)) continue;
+    unsigned v = 0;
+#pragma unroll
+    for (int q = 0; q < (ND == 3 ? 27 : 9); ++q) {
+      const int a = min(max(X + q % 3 - 1, 0), nx - 1), e = min(max(Y + q / 3 % 3 - 1, 0), ny - 1),
+                f = min(max(Z + q / 9 - (ND == 3), 0), nz - 1);
+      v |= flag[(f * ny + e) * nx + a];
+    }
+    act[b] = (unsigned char)v;
+  }
+}
+
+// The active blocks, each with a bit per direction whose plus-side neighbour
+// block is active too; list[0] counts them.
+template <int ND>
+__global__ void k_vof_list(Level L, const unsigned char* __restrict__ act, int2* __restrict__ list) {
+  using B = CellBlock<ND>;
+  const int nx = (L.nx + B::bx - 1) / B::bx, ny = (L.ny + B::by - 1) / B::by,
+            nz = (L.nz + B::bz - 1) / B::bz;
+  const int nb = nx * ny * nz;
+  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x) {
+    if (!act[b]) continue;
+    const int X = b % nx, Y = b / nx % ny, Z = b / nx / ny;
     int m = 0;
-    if (active(X + 1, Y, Z)) m |= 1;
-    if (active(X, Y + 1, Z)) m |= 2;
-    if (ND == 3 && active(X, Y, Z + 1)) m |= 4;
+    if (X + 1 < nx && act[b + 1]) m |= 1;
+    if (Y + 1 < ny && act[b + nx]) m |= 2;
+    if (ND == 3 && Z + 1 < nz && act[b + nx * ny]) m |= 4;
     list[1 + atomicAdd(&list[0].x, 1)] = make_int2(b, m);
   }
+}
+
+// Flux through the minus-side face of cell x in direction d (not a wall)
+// from its upwind cell's plane.
+template <typename U, typename G, int ND>
+__device__ __forceinline__ double plic_flux(const Level& L, int d, const int* x, size_t st,
+                                            const double* __restrict__ C,
+                                            const U* __restrict__ u, double dt_h) {
+  const size_t c = cidx(L, x[0], x[1], x[2]);
+  const double cf = widen(u[fidx(L, d, x[0], x[1], x[2])]) * dt_h;
+  const bool pos = vbits(cf) > 0;
+  int y[3] = {x[0], x[1], x[2]};
+  if (pos) y[d] -= 1;
+  G m[3];
+  youngs_normal(L, C, y[0], y[1], y[2], m);
+  const G cg = (G)C[pos ? c - st : c];
+  return pos ? widen(plic_slab<G>(ND, m, cg, d, G(1) - (G)cf, G(1)))
+             : -widen(plic_slab<G>(ND, m, cg, d, G(0), (G)(-cf)));
 }
 
 // Volume fraction crossing the minus-side face of every cell in direction d
@@ -81,37 +127,65 @@ template <typename U, typename G, int ND>
 __global__ void __launch_bounds__(512)
 k_vof_flux(Level L, int d, const int2* __restrict__ list, const double* __restrict__ C,
            const U* __restrict__ u, double dt_h, double* __restrict__ Q,
-           unsigned char* __restrict__ H) {
+           unsigned char* __restrict__ H, unsigned* __restrict__ cut) {
   const size_t st = d == 0 ? 1 : (d == 1 ? (size_t)L.nx : (size_t)L.nx * L.ny);
   const unsigned nb = list ? (unsigned)list[0].x : gridDim.x;
   for (unsigned q = blockIdx.x; q < nb; q += gridDim.x) {
+    const unsigned blk = list ? (unsigned)list[1 + q].x : q;
     int x[3];
-    if (!CellBlock<ND>::at(L, list ? (unsigned)list[1 + q].x : q, x)) continue;
-    const size_t c = cidx(L, x[0], x[1], x[2]);
-    const double cq = C[c];
-    if (H) H[c] = cq > 0.5 ? 1 : 0;
-    double flux = 0.0;
-    if (x[d] > 0) {
-      // both candidates for the upwind cell are loaded with u
-      const double cm = C[c - st];
-      const U uf = u[fidx(L, d, x[0], x[1], x[2])];
-      if (vbits(cm) != 0 || vbits(cq) != 0) {
-        const double cf = widen(uf) * dt_h;
-        const bool pos = vbits(cf) > 0;
-        const double cu = pos ? cm : cq;
-        if (vbits(cf) << 1 != 0 && vbits(cu) > 0) {     // a flow out of a cell with fluid
-          const int ui = pos && d == 0 ? x[0] - 1 : x[0];
-          const int uj = pos && d == 1 ? x[1] - 1 : x[1];
-          const int uk = pos && d == 2 ? x[2] - 1 : x[2];
-          G m[3] = {G(0), G(0), G(0)};
-          if (vbits(cu) < 0x3ff0000000000000LL) youngs_normal(L, C, ui, uj, uk, m);  // full: no plane
-          const G cg = (G)cu;
-          flux = pos ? widen(plic_slab<G>(ND, m, cg, d, G(1) - (G)cf, G(1)))
-                     : -widen(plic_slab<G>(ND, m, cg, d, G(0), (G)(-cf)));
+    bool plane = false;
+    size_t c = 0;
+    if (CellBlock<ND>::at(L, blk, x)) {
+      c = cidx(L, x[0], x[1], x[2]);
+      const double cq = C[c];
+      if (H) H[c] = cq > 0.5 ? 1 : 0;
+      double flux = 0.0;
+      if (x[d] > 0) {
+        // both candidates for the upwind cell are loaded with u
+        const double cm = C[c - st];
+        const U uf = u[fidx(L, d, x[0], x[1], x[2])];
+        const double cu = uf > U(0) ? cm : cq;
+        if (uf != U(0) && vbits(cu) > 0) {     // a flow out of a cell with fluid
+          const double cf = widen(uf) * dt_h;
+          // no plane in a cell that is full, in float also within rounding
+          if (!((G)cu < G(1))) {
+            const G z[3] = {G(0), G(0), G(0)};
+            flux = vbits(cf) > 0 ? widen(plic_slab<G>(ND, z, (G)cu, d, G(1) - (G)cf, G(1)))
+                                 : -widen(plic_slab<G>(ND, z, (G)cu, d, G(0), (G)(-cf)));
+          } else {
+            plane = true;
+          }
         }
       }
+      if (!plane) Q[c] = flux;
+      else if (!cut) Q[c] = plic_flux<U, G, ND>(L, d, x, st, C, u, dt_h);
     }
-    Q[c] = flux;
+    if (cut) {        // one slot of the list per lane that needs a plane
+      const unsigned full = 0xffffffffu, m = __ballot_sync(full, plane);
+      if (m) {
+        unsigned base = 0;
+        const int lane = threadIdx.x & 31, lead = __ffs(m) - 1;
+        if (lane == lead) base = atomicAdd(cut, (unsigned)__popc(m));
+        base = __shfl_sync(full, base, lead);
+        if (plane) cut[1 + base + __popc(m & ((1u << lane) - 1))] = (unsigned)c;
+      }
+    }
+  }
+}
+
+// The listed faces (cells whose minus-side face in direction d needs a
+// plane): cut[0] of them.
+template <typename U, typename G, int ND>
+__global__ void __launch_bounds__(128)
+k_vof_planes(Level L, int d, const double* __restrict__ C, const U* __restrict__ u, double dt_h,
+             const unsigned* __restrict__ cut, double* __restrict__ Q) {
+  const unsigned n = cut[0];
+  const size_t st = d == 0 ? 1 : (d == 1 ? (size_t)L.nx : (size_t)L.nx * L.ny);
+  for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
+    const unsigned c = cut[1 + q];
+    const int x[3] = {(int)(c % (unsigned)L.nx), (int)(c / (unsigned)L.nx % (unsigned)L.ny),
+                      (int)(c / (unsigned)L.nx / (unsigned)L.ny)};
+    Q[c] = plic_flux<U, G, ND>(L, d, x, st, C, u, dt_h);
   }
 }
 
@@ -152,20 +226,31 @@ sfx_status vof_impl(sfx_ctx* c, const U* const* u, double dt, int order, double*
   const size_t nb = CellBlock<ND>::count(L);
   int2* list = nullptr;
   unsigned grid = (unsigned)nb;
+  unsigned* cut = nullptr;
   if (L.ncell() >= kVofListCells) {
+    if (L.ncell() < ((size_t)1 << 32) && !c->vof_cut) {
+      SFX_CUDA(cudaMalloc((void**)&c->vof_cut, (L.ncell() + 1) * sizeof(unsigned)));
+      c->allocations.push_back(c->vof_cut);
+    }
+    cut = c->vof_cut;
     const sfx_status st = block_list(c, nb);
     if (st != SFX_OK) return st;
     list = (int2*)c->block_list;
     unsigned char* flag = (unsigned char*)(list + nb + 1);
     SFX_CUDA(cudaMemsetAsync(list, 0, sizeof(int2), s));
-    SFX_KERNEL(c, K_OTHER, k_vof_flags<ND>, (unsigned)nb, 512, s, L, C, flag);
-    SFX_KERNEL(c, K_OTHER, k_vof_list<ND>, blocks_for(nb, 128), 128, s, L, flag, list);
+    SFX_KERNEL(c, K_OTHER, k_vof_flags<ND>, (unsigned)((nb + 7) / 8), 256, s, L, (unsigned)nb, C, flag);
+    SFX_KERNEL(c, K_OTHER, k_vof_active<ND>, blocks_for(nb, 128), 128, s, L, flag, flag + nb);
+    SFX_KERNEL(c, K_OTHER, k_vof_list<ND>, blocks_for(nb, 128), 128, s, L, flag + nb, list);
     grid = (unsigned)std::min(nb, (size_t)c->sm_count * 4);
   }
   for (int q = 0; q < ND; ++q) {
     const int d = order ? ND - 1 - q : q;
+    if (cut) SFX_CUDA(cudaMemsetAsync(cut, 0, sizeof(unsigned), s));
     SFX_KERNEL(c, K_OTHER, (k_vof_flux<U, G, ND>), grid, 512, s, L, d, list, C, u[d], dt_h, c->vofQ,
-               q == 0 ? c->vofH : nullptr);
+               q == 0 ? c->vofH : nullptr, cut);
+    if (cut)
+      SFX_KERNEL(c, K_OTHER, (k_vof_planes<U, G, ND>), c->sm_count * 16, 128, s, L, d, C, u[d], dt_h,
+                 cut, c->vofQ);
     SFX_KERNEL(c, K_OTHER, (k_vof_update<U, ND>), grid, 512, s, L, d, list, u[d], dt_h, c->vofQ,
                c->vofH, C);
   }
