@@ -189,8 +189,12 @@ sfx_status sfx_ctx_create(const sfx_grid* grid, int precision, sfx_ctx** out) {
   if (st == SFX_OK) st = dalloc(c, &c->Fstar, n);
   if (st == SFX_OK) st = dalloc(c, &c->chi0, n);
   if (st == SFX_OK) st = dalloc(c, &c->chi_tmp, n);
-  c->n_partial_blocks = kTotalsBlocks;
-  if (st == SFX_OK) st = dalloc(c, &c->partials, (size_t)2 * 8 * c->n_partial_blocks);
+  if (st == SFX_OK) st = dalloc(c, &c->partials, (size_t)2 * 8 * kTotalsBlocks);
+  if (st == SFX_OK) st = dalloc(c, &c->tickets, 8);
+  if (st == SFX_OK) {
+    const cudaError_t e = cudaMemset(c->tickets, 0, 8 * sizeof(unsigned));
+    if (e != cudaSuccess) st = cuda_fail(e);
+  }
   if (st == SFX_OK) st = dalloc(c, &c->d_norms, 16);
   if (st == SFX_OK) st = dalloc(c, &c->d_sums, 8);
   if (st == SFX_OK && precision == SFX_F32) st = f32_ensure_scratch(c);

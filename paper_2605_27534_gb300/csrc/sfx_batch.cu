@@ -257,17 +257,17 @@ __global__ void k_b_corr(const BInst* __restrict__ I, int n, const int* __restri
   corr2_cell<G>(B.p, i, j, 0, H, P.rc + w, P.e2 + w, color, first, fst, Fst, fst, Fst);
 }
 
-// per-instance compensated totals: kTotBlocks blocks per instance each walk
+// per-instance compensated totals: tot_parts blocks per instance each walk
 // a share of its cells, accumulate both fields in double-float pairs and
 // combine their threads in compensated doubles ...
-constexpr int kTotBlocks = 8;
-__global__ void k_b_totals(const BInst* __restrict__ I, BPtr P) {
-  const int inst = blockIdx.x / kTotBlocks, part = blockIdx.x % kTotBlocks;
+constexpr int kTotBlocks = 16;   // at most (sfx_batch::tot_parts)
+__global__ void __launch_bounds__(256) k_b_totals(const BInst* __restrict__ I, int parts, BPtr P) {
+  const int inst = blockIdx.x / parts, part = blockIdx.x % parts;
   const BInst& B = I[inst];
   const Level& L = B.p.L;
   const ix n = (ix)L.ncell(), nx = (ix)L.nx;
   float2 acc[2] = {make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
-  for (ix c = part * blockDim.x + threadIdx.x; c < n; c += kTotBlocks * blockDim.x) {
+  for (ix c = part * blockDim.x + threadIdx.x; c < n; c += parts * blockDim.x) {
     // ring volume / (pi h^3), or 1 for planar cells (volume h^2)
     const float w = L.geom == SFX_AXISYM ? 2.0f * (float)(c % nx) + 1.0f : 1.0f;
 #pragma unroll
@@ -278,38 +278,24 @@ __global__ void k_b_totals(const BInst* __restrict__ I, BPtr P) {
       acc[fld] = df_add2(acc[fld], v);
     }
   }
-  __shared__ double ss[2][16], sc[2][16];
 #pragma unroll
   for (int fld = 0; fld < 2; ++fld) {
     double s = (double)acc[fld].x, cc = (double)acc[fld].y;
-    warp_sum_comp(s, cc);
-    if ((threadIdx.x & 31) == 0) {
-      ss[fld][threadIdx.x >> 5] = s;
-      sc[fld][threadIdx.x >> 5] = cc;
+    block_sum_comp<256>(s, cc);
+    if (threadIdx.x == 0) {
+      P.tpart[4 * (size_t)blockIdx.x + 2 * fld] = s;
+      P.tpart[4 * (size_t)blockIdx.x + 2 * fld + 1] = cc;
     }
-  }
-  __syncthreads();
-  if (threadIdx.x < 2) {
-    const int fld = threadIdx.x;
-    double a = ss[fld][0], b = sc[fld][0];
-    for (int q = 1; q < (int)(blockDim.x >> 5); ++q) {
-      double t, e;
-      two_sum(a, ss[fld][q], t, e);
-      a = t;
-      b += sc[fld][q] + e;
-    }
-    P.tpart[4 * (size_t)blockIdx.x + 2 * fld] = a;
-    P.tpart[4 * (size_t)blockIdx.x + 2 * fld + 1] = b;
   }
 }
 
 // ... and one warp per instance combines its blocks in a fixed order
-__global__ void k_b_totals_final(const BInst* __restrict__ I, int n, BPtr P) {
+__global__ void k_b_totals_final(const BInst* __restrict__ I, int n, int parts, BPtr P) {
   const int inst = blockIdx.x;
   if (inst >= n) return;
   for (int fld = 0; fld < 2; ++fld) {
     double s = 0.0, cc = 0.0;
-    for (int b = inst * kTotBlocks + threadIdx.x; b < (inst + 1) * kTotBlocks; b += blockDim.x) {
+    for (int b = inst * parts + threadIdx.x; b < (inst + 1) * parts; b += blockDim.x) {
       double t, e;
       two_sum(s, P.tpart[4 * (size_t)b + 2 * fld], t, e);
       s = t;
@@ -343,6 +329,7 @@ struct sfx_batch {
   int nb_cell = 0, nb_rf = 0, nb_zf = 0, nb_pair = 0;
   int block = 256;
   int geom = SFX_AXISYM;   // of every instance
+  int tot_parts = 1;       // blocks of partial totals per instance
   BPtr P{};
   std::vector<void*> allocs;
   // graph cache
@@ -453,8 +440,8 @@ sfx_status enqueue_step(sfx_batch* b, bool advect, float tol, cudaStream_t s) {
   SFX_CUDA(be);
   SFX_CUDA(cudaStreamUpdateCaptureDependencies(s, &cnode, nullptr, 1,
                                                cudaStreamSetCaptureDependencies));
-  k_b_totals<<<n * kTotBlocks, 256, 0, s>>>(b->dI, P);
-  k_b_totals_final<<<n, 32, 0, s>>>(b->dI, n, P);
+  k_b_totals<<<n * b->tot_parts, 256, 0, s>>>(b->dI, b->tot_parts, P);
+  k_b_totals_final<<<n, 32, 0, s>>>(b->dI, n, b->tot_parts, P);
   SFX_LAUNCH_CHECK();
   return SFX_OK;
 }
@@ -587,6 +574,11 @@ sfx_status sfx_batch_create_geom(const sfx_batch_instance* inst, int n, int geom
   if (st == SFX_OK) st = balloc(b, &P.rres, 2 * (size_t)n);
   if (st == SFX_OK) st = balloc(b, &P.mass, 2 * (size_t)n);
   if (st == SFX_OK) st = balloc(b, &P.work, 2 * (size_t)n);
+  // totals: a block's FP64 reduction costs as much as 4096 cells of pairs
+  // (512 columns of 2048 cells: 185 us with 8 blocks each, 13 us with one)
+  size_t most = 0;
+  for (const auto& q : b->hinst) most = std::max(most, (size_t)q.nr * q.nz);
+  b->tot_parts = (int)std::min((size_t)kTotBlocks, std::max((size_t)1, most / 4096));
   // block partials: at most one block per 128 cells of each instance
   const size_t maxblk = nc / 128 + (size_t)n + 1;
   if (st == SFX_OK) st = balloc(b, &P.part, 4 * maxblk);

@@ -61,6 +61,17 @@ __device__ __forceinline__ double widen(float x) {
 }
 __device__ __forceinline__ double widen(double x) { return x; }
 
+// Row r = k ny + j (64-bit division only past 2^32).
+__device__ __forceinline__ void row_jk(size_t r, int ny, int& j, int& k) {
+  if (r >> 32) {
+    k = (int)(r / (size_t)ny);
+    j = (int)(r - (size_t)k * ny);
+  } else {
+    k = (int)((unsigned)r / (unsigned)ny);
+    j = (int)((unsigned)r - (unsigned)k * (unsigned)ny);
+  }
+}
+
 // Blocks of 32 x 4 x 4 cells (32 x 16 in 2D) with 512 threads for kernels
 // whose work sits in a band around the interface: a warp holds 8 x 2 x 2
 // cells (8 x 4), so that few warps straddle the band's edge.
@@ -120,6 +131,83 @@ __device__ inline void warp_sum_comp(double& s, double& c) {
     two_sum(s, so, t, e);
     s = t;
     c = c + co + e;
+  }
+}
+
+// Compensated block reduction of (s, c) pairs in a fixed order; thread 0
+// receives the block's pair in (s, c).  NT threads per block, a multiple of
+// 32.  The first warp adds the others' pairs lane by lane and then across its
+// lanes: an FP64 instruction occupies the SM's pipe for 16 cycles however
+// few lanes it serves, and a shuffle tree in every warp cost four times as
+// many (the totals of a 128^2 grid 17 us, nearly all of it this).
+template <int NT>
+__device__ __forceinline__ void block_sum_comp(double& s, double& c) {
+  __shared__ double ss[NT], sc[NT];
+  ss[threadIdx.x] = s;
+  sc[threadIdx.x] = c;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+#pragma unroll
+    for (int q = 1; q < NT / 32; ++q) {
+      double t, e;
+      two_sum(s, ss[threadIdx.x + 32 * q], t, e);
+      s = t;
+      c += sc[threadIdx.x + 32 * q] + e;
+    }
+    warp_sum_comp(s, c);
+  }
+  __syncthreads();
+}
+
+// The pairs of `n` blocks (part[2 q], part[2 q + 1]) combined in a fixed
+// order by the first warp of a block; lane 0 receives (s, c).
+__device__ __forceinline__ void warp_combine(const double* part, int n, double& s, double& c) {
+  s = 0.0;
+  c = 0.0;
+  for (int q = threadIdx.x; q < n; q += 32) {
+    double t, e;
+    two_sum(s, part[2 * q], t, e);
+    s = t;
+    c += part[2 * q + 1] + e;
+  }
+  warp_sum_comp(s, c);
+}
+
+// A block's pair stored as block `blk` of `n` for one total; the last block
+// to do so combines them and gets true in thread 0, with the pair.  The
+// ticket returns to zero for the next launch.
+template <int NT>
+__device__ __forceinline__ bool last_block_total(double* part, int blk, int n, unsigned* ticket,
+                                                 double& s, double& c) {
+  block_sum_comp<NT>(s, c);
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+    part[2 * blk] = s;
+    part[2 * blk + 1] = c;
+    __threadfence();
+    last = atomicAdd(ticket, 1u) == (unsigned)n - 1;
+  }
+  __syncthreads();
+  if (!last || threadIdx.x >= 32) return false;
+  __threadfence();
+  warp_combine(part, n, s, c);
+  if (threadIdx.x == 0) *ticket = 0u;
+  return threadIdx.x == 0;
+}
+
+// A thread's compensated part of sum V x (blocks in x over the cells).
+__device__ __forceinline__ void totals_thread(const Level& L, const double* __restrict__ x,
+                                              double& s, double& c) {
+  const size_t n = L.ncell();
+  s = 0.0;
+  c = 0.0;
+  for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n;
+       q += (size_t)gridDim.x * blockDim.x) {
+    const int i = L.geom == SFX_AXISYM ? (int)(q % (size_t)L.nx) : 0;
+    double t, e;
+    two_sum(s, cell_volume(L, i) * x[q], t, e);
+    s = t;
+    c += e;
   }
 }
 

@@ -840,20 +840,22 @@ __global__ void __launch_bounds__(kAdvX* kAdvY)
 // Per-thread double-float accumulation of w_i (hi + lo) with w_i the cell
 // volume over its constant factor (1, or 2i+1 on rings); FP64 only across
 // threads.
-__global__ void k_total32_partials(Level L, const float2* __restrict__ x0,
-                                   const float2* __restrict__ x1, int f0,
-                                   double* __restrict__ partials) {
-  // blockIdx.y picks the field: both fields' blocks in flight together
-  const float2* __restrict__ x = blockIdx.y ? x1 : x0;
-  const int fi = f0 + (int)blockIdx.y;
+struct TotalFields32 {
+  const float2* x[8];
+};
+__global__ void __launch_bounds__(kTotalsThreads)
+k_totals32(Level L, TotalFields32 fl, double scale, double* __restrict__ partials,
+           unsigned* __restrict__ tickets, double* __restrict__ out) {
+  // blockIdx.y picks the field: all fields' blocks in flight together
+  const int fi = (int)blockIdx.y;
+  const float2* __restrict__ x = fl.x[fi];
   const size_t n = L.ncell();
-  // four independent pair accumulators: four loads in flight per thread
-  float2 acc[4] = {make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f),
-                   make_float2(0.0f, 0.0f)};
+  // two independent pair accumulators, fed by four 16-byte loads (two cells
+  // each) in flight per thread; 8-byte loads where the field is not aligned
+  float2 acc[2] = {make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
   const size_t step = (size_t)gridDim.x * blockDim.x;
-  size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  auto weighted = [&](size_t cq) {
-    float2 v = x[cq];
+  const size_t t0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  auto weighted = [&](float2 v, size_t cq) {
     if (L.geom == SFX_AXISYM) {
       float w = 2.0f * (float)(cq % L.nx) + 1.0f;
       float p = v.x * w;
@@ -862,69 +864,37 @@ __global__ void k_total32_partials(Level L, const float2* __restrict__ x0,
     }
     return v;
   };
-  // full groups of four without bounds checks (their loads issue together),
-  // then the remainder
-  for (; c + 3 * step < n; c += 4 * step) {
-    float2 v[4];
+  size_t done = 0;      // cells taken by the pair loads
+  if (((size_t)x & 15) == 0) {
+    const float4* __restrict__ x4 = reinterpret_cast<const float4*>(x);
+    const size_t n2 = n / 2;
+    size_t q = t0;
+    for (; q + 3 * step < n2; q += 4 * step) {
+      float4 v[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) v[q] = weighted(c + (size_t)q * step);
+      for (int k = 0; k < 4; ++k) v[k] = x4[q + k * step];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) acc[q] = df_add2(acc[q], v[q]);
-  }
-  for (int q = 0; c < n; c += step, ++q) acc[q & 3] = df_add2(acc[q & 3], weighted(c));
-  // each pair is exact in FP64 (hi + lo spans < 53 bits); the four are
-  // combined by compensated FP64 sums, then reduced across threads
-  double s = (double)acc[0].x + (double)acc[0].y, cc = 0.0;
-#pragma unroll
-  for (int q = 1; q < 4; ++q) {
-    double t, e;
-    two_sum(s, (double)acc[q].x + (double)acc[q].y, t, e);
-    s = t;
-    cc += e;
-  }
-  warp_sum_comp(s, cc);
-  __shared__ double ss[8], sc[8];
-  int w = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) { ss[w] = s; sc[w] = cc; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = ss[0], b = sc[0];
-    for (int q = 1; q < (int)(blockDim.x >> 5); ++q) {
-      double t, e;
-      two_sum(a, ss[q], t, e);
-      a = t;
-      b += sc[q] + e;
+      for (int k = 0; k < 4; ++k) {
+        const size_t c = 2 * (q + k * step);
+        acc[0] = df_add2(acc[0], weighted(make_float2(v[k].x, v[k].y), c));
+        acc[1] = df_add2(acc[1], weighted(make_float2(v[k].z, v[k].w), c + 1));
+      }
     }
-    partials[2 * ((size_t)fi * gridDim.x + blockIdx.x)] = a;
-    partials[2 * ((size_t)fi * gridDim.x + blockIdx.x) + 1] = b;
-  }
-}
-
-__global__ void k_total32_final(const double* __restrict__ partials, int nblk, double scale,
-                                double* __restrict__ out) {
-  const int fi = blockIdx.x;
-  double s = 0.0, cc = 0.0;
-  for (int q = threadIdx.x; q < nblk; q += blockDim.x) {
-    double t, e;
-    two_sum(s, partials[2 * ((size_t)fi * nblk + q)], t, e);
-    s = t;
-    cc += partials[2 * ((size_t)fi * nblk + q) + 1] + e;
-  }
-  warp_sum_comp(s, cc);
-  __shared__ double ss[8], sc[8];
-  int w = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) { ss[w] = s; sc[w] = cc; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = ss[0], b = sc[0];
-    for (int q = 1; q < (int)(blockDim.x >> 5); ++q) {
-      double t, e;
-      two_sum(a, ss[q], t, e);
-      a = t;
-      b += sc[q] + e;
+    for (; q < n2; q += step) {
+      const float4 v = x4[q];
+      acc[0] = df_add2(acc[0], weighted(make_float2(v.x, v.y), 2 * q));
+      acc[1] = df_add2(acc[1], weighted(make_float2(v.z, v.w), 2 * q + 1));
     }
-    out[fi] = (a + b) * scale;
+    done = 2 * n2;
   }
+  for (size_t c = done + t0; c < n; c += step) acc[0] = df_add2(acc[0], weighted(x[c], c));
+  // each pair is exact in FP64 (hi + lo spans < 53 bits); the two are
+  // combined by a compensated FP64 sum, then reduced across threads
+  double s, cc;
+  two_sum(widen(acc[0].x) + widen(acc[0].y), widen(acc[1].x) + widen(acc[1].y), s, cc);
+  if (last_block_total<kTotalsThreads>(partials + 2 * (size_t)fi * gridDim.x, blockIdx.x,
+                                       gridDim.x, tickets + fi, s, cc))
+    out[fi] = (s + cc) * scale;
 }
 
 // ------------------------------------------------------------ EOS, force
@@ -1778,15 +1748,14 @@ sfx_status advect32(sfx_ctx* c, const float* ux, const float* uy, const float* u
 
 sfx_status totals32(sfx_ctx* c, const void* const* fields, int nf, double* out, cudaStream_t s) {
   const Level& L = c->lev[0].lv;
-  const int nblk = c->n_partial_blocks;
-  for (int i = 0; i < nf; i += 2) {
-    const int m = std::min(2, nf - i);
-    SFX_KERNEL(c, K_TOTALS, k_total32_partials, dim3((unsigned)nblk, (unsigned)m), 256, s, L,
-               (const float2*)fields[i], (const float2*)fields[i + m - 1], i, c->partials);
-  }
   double h = L.h;
   double scale = L.geom == SFX_PLANAR2D ? h * h : (L.geom == SFX_CART3D ? h * h * h : kPi * h * h * h);
-  SFX_KERNEL(c, K_TOTALS, k_total32_final, nf, 256, s, c->partials, nblk, scale, c->d_sums);
+  TotalFields32 f{};
+  for (int i = 0; i < nf; ++i) f.x[i] = (const float2*)fields[i];
+  // 1024 cells per block at least: a block's FP64 reduction takes as long
+  const size_t nblk = std::min((size_t)kTotalsBlocks, (L.ncell() + 1023) / 1024);
+  SFX_KERNEL(c, K_TOTALS, k_totals32, dim3((unsigned)nblk, (unsigned)nf), kTotalsThreads, s, L, f,
+             scale, c->partials, c->tickets, c->d_sums);
   SFX_LAUNCH_CHECK();
   SFX_CUDA(cudaMemcpyAsync(c->h_sums, c->d_sums, nf * sizeof(double), cudaMemcpyDeviceToHost, s));
   SFX_CUDA(cudaStreamSynchronize(s));

@@ -12,65 +12,27 @@ namespace {
 
 constexpr int kTotThreads = kTotalsThreads;
 
-// Per-block compensated partial sums of V x for field `fi`.
-__global__ void k_total_partials(Level L, const double* __restrict__ x, int fi,
-                                 double* __restrict__ partials) {
-  const size_t n = L.ncell();
-  double s = 0.0, cc = 0.0;
-  for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
-       c += (size_t)gridDim.x * blockDim.x) {
-    double v = cell_volume(L, (int)(c % L.nx)) * x[c];
-    double t, e;
-    two_sum(s, v, t, e);
-    s = t;
-    cc += e;
-  }
-  warp_sum_comp(s, cc);
-  __shared__ double ss[kTotThreads / 32], sc[kTotThreads / 32];
-  int w = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) { ss[w] = s; sc[w] = cc; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = ss[0], b = sc[0];
-    for (int q = 1; q < kTotThreads / 32; ++q) {
-      double t, e;
-      two_sum(a, ss[q], t, e);
-      a = t;
-      b += sc[q] + e;
-    }
-    size_t o = 2 * ((size_t)fi * gridDim.x + blockIdx.x);
-    partials[o] = a;
-    partials[o + 1] = b;
-  }
+// The totals sum V x of the fields in grid.y, both stages in one launch.
+struct TotalFields {
+  const double* x[8];
+};
+__global__ void __launch_bounds__(kTotThreads)
+k_totals(Level L, TotalFields f, double* __restrict__ partials, unsigned* __restrict__ tickets,
+         double* __restrict__ out) {
+  const int fi = blockIdx.y;
+  double s, cc;
+  totals_thread(L, f.x[fi], s, cc);
+  if (last_block_total<kTotThreads>(partials + 2 * (size_t)fi * gridDim.x, blockIdx.x, gridDim.x,
+                                    tickets + fi, s, cc))
+    out[fi] = s + cc;
 }
 
-// One block per field: fixed-order combination of the block partials.
+// One block: fixed-order combination of block partials.
 __global__ void k_total_final(const double* __restrict__ partials, int nblk,
                               double* __restrict__ out) {
-  const int fi = blockIdx.x;
-  double s = 0.0, cc = 0.0;
-  for (int q = threadIdx.x; q < nblk; q += blockDim.x) {
-    size_t o = 2 * ((size_t)fi * nblk + q);
-    double t, e;
-    two_sum(s, partials[o], t, e);
-    s = t;
-    cc += partials[o + 1] + e;
-  }
-  warp_sum_comp(s, cc);
-  __shared__ double ss[kTotThreads / 32], sc[kTotThreads / 32];
-  int w = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) { ss[w] = s; sc[w] = cc; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = ss[0], b = sc[0];
-    for (int q = 1; q < kTotThreads / 32; ++q) {
-      double t, e;
-      two_sum(a, ss[q], t, e);
-      a = t;
-      b += sc[q] + e;
-    }
-    out[fi] = a + b;
-  }
+  double s, cc;
+  warp_combine(partials, nblk, s, cc);
+  if (threadIdx.x == 0) out[0] = s + cc;
 }
 
 struct EosArgs {
@@ -250,7 +212,7 @@ sfx_status marangoni_loss(sfx_ctx* c, const sfx_params* p, const double* f, cons
   const int nbp = c->adj.nblk;
   SFX_KERNEL(c, K_FORCES, k_loss_partials, nbp, kTotThreads, s, L, c->adj.force, c->adj.dm,
              grad ? c->adj.G : nullptr, c->adj.part);
-  SFX_KERNEL(c, K_FORCES, k_total_final, 1, kTotThreads, s, c->adj.part, nbp, c->adj.d_out);
+  SFX_KERNEL(c, K_FORCES, k_total_final, 1, 32, s, c->adj.part, nbp, c->adj.d_out);
   if (grad)
     SFX_KERNEL(c, K_FORCES, k_loss_grad, nb, 256, s, L, q, f, phi, c->adj.G, grad);
   SFX_LAUNCH_CHECK();
@@ -262,10 +224,10 @@ sfx_status marangoni_loss(sfx_ctx* c, const sfx_params* p, const double* f, cons
 
 sfx_status totals(sfx_ctx* c, const double* const* fields, int nf, double* out, cudaStream_t s) {
   const Level& L = c->lev[0].lv;
-  const int nblk = c->n_partial_blocks;
-  for (int i = 0; i < nf; ++i)
-    SFX_KERNEL(c, K_TOTALS, k_total_partials, nblk, kTotThreads, s, L, fields[i], i, c->partials);
-  SFX_KERNEL(c, K_TOTALS, k_total_final, nf, kTotThreads, s, c->partials, nblk, c->d_sums);
+  TotalFields f{};
+  for (int i = 0; i < nf; ++i) f.x[i] = fields[i];
+  SFX_KERNEL(c, K_TOTALS, k_totals, dim3(totals_blocks(L.ncell()), nf), kTotThreads, s, L, f,
+             c->partials, c->tickets, c->d_sums);
   SFX_LAUNCH_CHECK();
   SFX_CUDA(cudaMemcpyAsync(c->h_sums, c->d_sums, nf * sizeof(double), cudaMemcpyDeviceToHost, s));
   SFX_CUDA(cudaStreamSynchronize(s));

@@ -16,9 +16,15 @@ namespace sfx {
 
 // Launch shape of the compensated FP64 totals: blocks of partial sums and
 // threads per block.  sfx_totals and sfx_totals_noalloc both use it, so
-// they reduce in the same order and return the same bits.
+// they reduce in the same order and return the same bits.  256 cells per
+// block at least: a cell costs 8 FP64 instructions, a block's reduction 100
+// warps' worth.
 constexpr int kTotalsBlocks = 152 * 4;
 constexpr int kTotalsThreads = 256;
+inline unsigned totals_blocks(size_t n) {
+  const size_t b = (n + 255) / 256;
+  return (unsigned)(b < kTotalsBlocks ? b : kTotalsBlocks);
+}
 
 // FP32 Newton solves (single-grid and batched) evaluate the residuals in
 // FP32 until both relative residuals are below this, or for a set number
@@ -199,7 +205,7 @@ struct sfx_ctx {
   double* sigma_tmp = nullptr;
   // reductions
   double* partials = nullptr;        // block partial sums (s, c) pairs
-  int n_partial_blocks = 0;
+  unsigned* tickets = nullptr;       // blocks done per total (8), zero between launches
   unsigned long long* d_norms = nullptr;  // 16 slots (device): 0..7 the FP64 solves and the
                                           // FP32 sweeps (7: d_flag), 8..15 the FP32 Newton
                                           // solve's two norm buffers

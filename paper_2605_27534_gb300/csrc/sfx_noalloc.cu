@@ -50,59 +50,23 @@ sfx_status scratch_address(double** out) {
   return SFX_OK;
 }
 
-__global__ void k_na_partials(Level L, const double* __restrict__ x, int fi,
-                              double* __restrict__ scratch) {
-  const size_t n = L.ncell();
-  double s = 0.0, cc = 0.0;
-  for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
-       c += (size_t)gridDim.x * blockDim.x) {
-    double t, e;
-    two_sum(s, cell_volume(L, (int)(c % L.nx)) * x[c], t, e);
-    s = t;
-    cc += e;
-  }
-  warp_sum_comp(s, cc);
-  __shared__ double ws[kNaThreads / 32], wc[kNaThreads / 32];
-  const int w = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) { ws[w] = s; wc[w] = cc; }
-  __syncthreads();
+__global__ void __launch_bounds__(kNaThreads)
+k_na_partials(Level L, const double* __restrict__ x, int fi, double* __restrict__ scratch) {
+  double s, c;
+  totals_thread(L, x, s, c);
+  block_sum_comp<kNaThreads>(s, c);
   if (threadIdx.x == 0) {
-    double a = ws[0], b = wc[0];
-    for (int q = 1; q < kNaThreads / 32; ++q) {
-      double t, e;
-      two_sum(a, ws[q], t, e);
-      a = t;
-      b += wc[q] + e;
-    }
-    scratch[2 * ((size_t)fi * kNaBlocks + blockIdx.x)] = a;
-    scratch[2 * ((size_t)fi * kNaBlocks + blockIdx.x) + 1] = b;
+    double* part = scratch + 2 * ((size_t)fi * kNaBlocks + blockIdx.x);
+    part[0] = s;
+    part[1] = c;
   }
 }
 
-__global__ void k_na_final(double* __restrict__ scratch) {
+__global__ void k_na_final(double* __restrict__ scratch, int nblk) {
   const int fi = blockIdx.x;
-  double s = 0.0, cc = 0.0;
-  for (int q = threadIdx.x; q < kNaBlocks; q += blockDim.x) {
-    double t, e;
-    two_sum(s, scratch[2 * (fi * kNaBlocks + q)], t, e);
-    s = t;
-    cc += scratch[2 * (fi * kNaBlocks + q) + 1] + e;
-  }
-  warp_sum_comp(s, cc);
-  __shared__ double ws[kNaThreads / 32], wc[kNaThreads / 32];
-  const int w = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) { ws[w] = s; wc[w] = cc; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = ws[0], b = wc[0];
-    for (int q = 1; q < kNaThreads / 32; ++q) {
-      double t, e;
-      two_sum(a, ws[q], t, e);
-      a = t;
-      b += wc[q] + e;
-    }
-    scratch[2 * SFX_NOALLOC_MAX_FIELDS * kNaBlocks + fi] = a + b;
-  }
+  double s, c;
+  warp_combine(scratch + 2 * (size_t)fi * kNaBlocks, nblk, s, c);
+  if (threadIdx.x == 0) scratch[2 * SFX_NOALLOC_MAX_FIELDS * kNaBlocks + fi] = s + c;
 }
 
 bool noalloc_grid_ok(const sfx_grid* g) {
@@ -125,8 +89,9 @@ extern "C" sfx_status sfx_totals_noalloc(const sfx_grid* grid, const double* con
   if (st != SFX_OK) return st;
   cudaStream_t s = (cudaStream_t)stream;
   Level L{grid->geom, grid->nx, grid->ny, grid->nz, grid->h};
-  for (int i = 0; i < n_fields; ++i) k_na_partials<<<kNaBlocks, kNaThreads, 0, s>>>(L, fields[i], i, scratch);
-  k_na_final<<<n_fields, kNaThreads, 0, s>>>(scratch);
+  const unsigned nblk = totals_blocks(L.ncell());
+  for (int i = 0; i < n_fields; ++i) k_na_partials<<<nblk, kNaThreads, 0, s>>>(L, fields[i], i, scratch);
+  k_na_final<<<n_fields, 32, 0, s>>>(scratch, (int)nblk);
   SFX_LAUNCH_CHECK();
   SFX_CUDA(cudaMemcpyAsync(out, scratch + 2 * SFX_NOALLOC_MAX_FIELDS * kNaBlocks,
                            n_fields * sizeof(double), cudaMemcpyDeviceToHost, s));

@@ -181,27 +181,4 @@ __device__ __forceinline__ void flux_weights_T(const Level& L, const Op& op, int
   dT = sd / Vc;
 }
 
-// Compensated block reduction of (s, c) pairs; thread 0 receives the
-// block's pair in (s, c).  NT threads per block, a multiple of 32.
-template <int NT>
-__device__ __forceinline__ void block_sum_comp(double& s, double& c) {
-  warp_sum_comp(s, c);
-  __shared__ double ss[NT / 32], sc[NT / 32];
-  const int w = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) { ss[w] = s; sc[w] = c; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = ss[0], b = sc[0];
-    for (int q = 1; q < NT / 32; ++q) {
-      double t, e;
-      two_sum(a, ss[q], t, e);
-      a = t;
-      b += sc[q] + e;
-    }
-    s = a;
-    c = b;
-  }
-  __syncthreads();
-}
-
 }  // namespace sfx
