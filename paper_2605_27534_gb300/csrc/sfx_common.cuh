@@ -225,27 +225,38 @@ __device__ __forceinline__ double normal_fade(double m, double slope) {
   return m < 1e-30 ? 0.0 : fmin(fmax(m / (kNormalKappa * slope) - 1.0, 0.0), 1.0);
 }
 
-// Unit normal component n_d = (grad phi)_d / |grad phi| at cell (i,j,k):
-// centred differences, zero-gradient walls, faded out where phi is flat
-// (above).
-template <typename P>
-__device__ __forceinline__ double normal_comp(const Level& L, const P* __restrict__ phi, int i,
-                                              int j, int k, int d, double eps) {
+// Appends the indices of the lanes with `take` to list (list[0] counts), one
+// atomic per warp; every lane of the warp calls it.
+__device__ __forceinline__ void warp_append(unsigned* list, bool take, unsigned v) {
+  const unsigned m = __ballot_sync(0xffffffffu, take);
+  if (!m) return;
+  const int lane = threadIdx.x & 31, lead = __ffs(m) - 1;
+  unsigned base = 0;
+  if (lane == lead) base = atomicAdd(list, (unsigned)__popc(m));
+  base = __shfl_sync(0xffffffffu, base, lead);
+  if (take) list[1 + base + __popc(m & ((1u << lane) - 1))] = v;
+}
+
+// Unit normal grad phi / |grad phi| at cell x: centred differences,
+// zero-gradient walls, faded out where phi is flat (above).
+__device__ __forceinline__ void unit_normal64(const Level& L, const double* __restrict__ phi,
+                                              const int* x, double eps, double* n) {
   double g[3] = {0.0, 0.0, 0.0};
   const double inv2h = 0.5 / L.h;
+  const int i = x[0], j = x[1], k = x[2];
   int ip = min(i + 1, L.nx - 1), im = max(i - 1, 0);
   int jp = min(j + 1, L.ny - 1), jm = max(j - 1, 0);
-  g[0] = ((double)phi[cidx(L, ip, j, k)] - (double)phi[cidx(L, im, j, k)]) * inv2h;
-  g[1] = ((double)phi[cidx(L, i, jp, k)] - (double)phi[cidx(L, i, jm, k)]) * inv2h;
+  g[0] = (phi[cidx(L, ip, j, k)] - phi[cidx(L, im, j, k)]) * inv2h;
+  g[1] = (phi[cidx(L, i, jp, k)] - phi[cidx(L, i, jm, k)]) * inv2h;
   if (L.geom == SFX_CART3D) {
     int kp = min(k + 1, L.nz - 1), km = max(k - 1, 0);
-    g[2] = ((double)phi[cidx(L, i, j, kp)] - (double)phi[cidx(L, i, j, km)]) * inv2h;
+    g[2] = (phi[cidx(L, i, j, kp)] - phi[cidx(L, i, j, km)]) * inv2h;
   }
-  double m = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
-  const double pc = (double)phi[cidx(L, i, j, k)];
+  const double m = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
+  const double pc = phi[cidx(L, i, j, k)];
   const double slope = pc * (1.0 - pc) / eps;
   const double w = normal_fade(m, slope);
-  return w > 0.0 ? w * (g[d] / m) : 0.0;
+  for (int d = 0; d < 3; ++d) n[d] = w > 0.0 ? w * (g[d] / m) : 0.0;
 }
 
 }  // namespace sfx

@@ -1,5 +1,6 @@
 // Conserved totals (compensated, deterministic), the surface-tension EOS of
 // Sec. 2.3 and the Marangoni force of Sec. 2.4.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -41,13 +42,22 @@ struct EosArgs {
 };
 
 // Gamma = f/delta_phi where delta_phi >= 1e-3/eps, else 0; sigma in double.
-template <typename P>
+// It also empties the list of interface cells of the force behind it.
 __global__ void k_eos(size_t n, EosArgs q, const double* __restrict__ f,
-                      const P* __restrict__ phi, double* __restrict__ sigma) {
+                      const double* __restrict__ phi, double* __restrict__ sigma,
+                      unsigned* __restrict__ list) {
+  if (list && blockIdx.x == 0 && threadIdx.x == 0) list[0] = 0;
   for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
        c += (size_t)gridDim.x * blockDim.x) {
-    double p = (double)phi[c];
-    double del = p * (1.0 - p) / q.eps;
+    double p = phi[c];
+    // delta_phi well below 1e-3/eps: Gamma = 0, which every EOS takes to
+    // sigma0, without the quotients and the logarithm (FP64 pipe)
+    const double pq = p * (1.0 - p);
+    if (pq < 0.99e-3) {
+      sigma[c] = q.sigma0;
+      continue;
+    }
+    double del = pq / q.eps;
     double G = del >= 1e-3 / q.eps ? f[c] / del : 0.0;
     double x = G / q.ginf;
     double s;
@@ -73,64 +83,88 @@ __device__ __forceinline__ double eos_slope(const EosArgs& q, double G) {
   return -q.sigma0 * q.E / q.ginf * (1.0 - t * t);
 }
 
-template <typename P>
-__global__ void k_force(Level L, const P* __restrict__ phi, const double* __restrict__ C,
-                        const double* __restrict__ sigma, int dm_mode, double eps,
-                        double* __restrict__ force, double* __restrict__ dm_out) {
+// One cell of the Marangoni force with its delta_m.
+__device__ __forceinline__ void force64_cell(const Level& L, const double* __restrict__ phi,
+                                             const double* __restrict__ C,
+                                             const double* __restrict__ sigma, int dm_mode,
+                                             double eps, size_t c, double* __restrict__ force,
+                                             double* __restrict__ dm_out) {
   const size_t n = L.ncell();
   const int nd = L.ndim();
   const double inv2h = 0.5 / L.h;
-  for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
-       c += (size_t)gridDim.x * blockDim.x) {
-    int idx[3] = {(int)(c % L.nx), (int)((c / L.nx) % L.ny), (int)(c / ((size_t)L.nx * L.ny))};
-    double gs[3] = {0, 0, 0}, nn[3] = {0, 0, 0}, ndg = 0.0;
-    for (int d = 0; d < nd; ++d) {
-      int pp[3] = {idx[0], idx[1], idx[2]}, pm[3] = {idx[0], idx[1], idx[2]};
-      pp[d] = min(pp[d] + 1, L.extent(d) - 1);
-      pm[d] = max(pm[d] - 1, 0);
-      gs[d] = (sigma[cidx(L, pp[0], pp[1], pp[2])] - sigma[cidx(L, pm[0], pm[1], pm[2])]) * inv2h;
-      nn[d] = normal_comp(L, phi, idx[0], idx[1], idx[2], d, eps);
-      ndg += nn[d] * gs[d];
-    }
-    double dm;
+  int idx[3];
+  idx[0] = (int)(c % L.nx);
+  row_jk(c / L.nx, L.ny, idx[1], idx[2]);
+  double gs[3] = {0, 0, 0}, nn[3], ndg = 0.0, q = 0.0;
+  unit_normal64(L, phi, idx, eps, nn);
+  for (int d = 0; d < nd; ++d) {
+    int pp[3] = {idx[0], idx[1], idx[2]}, pm[3] = {idx[0], idx[1], idx[2]};
+    pp[d] = min(pp[d] + 1, L.extent(d) - 1);
+    pm[d] = max(pm[d] - 1, 0);
+    const size_t cp = cidx(L, pp[0], pp[1], pp[2]), cm = cidx(L, pm[0], pm[1], pm[2]);
+    gs[d] = (sigma[cp] - sigma[cm]) * inv2h;
+    ndg += nn[d] * gs[d];
     if (dm_mode == 0) {
-      double q = 0.0;
-      for (int d = 0; d < nd; ++d) {
-        int pp[3] = {idx[0], idx[1], idx[2]}, pm[3] = {idx[0], idx[1], idx[2]};
-        pp[d] = min(pp[d] + 1, L.extent(d) - 1);
-        pm[d] = max(pm[d] - 1, 0);
-        double g = (C[cidx(L, pp[0], pp[1], pp[2])] - C[cidx(L, pm[0], pm[1], pm[2])]) * inv2h;
-        q += g * g;
-      }
-      dm = sqrt(q);
-    } else {
-      double Cc = C[c];
-      // interface cells: 1e-6 < C < 1 - 1e-6 (nearer fractions are the
-      // round-off of empty or full cells)
-      if (Cc > 1e-6 && Cc < 1.0 - 1e-6) {
-        // Youngs normal: minus the (1,2,1)-weighted gradient of C
-        double m[3] = {0, 0, 0};
-        int kr = nd == 3 ? 1 : 0;
-        for (int dk = -kr; dk <= kr; ++dk)
-          for (int dj = -1; dj <= 1; ++dj)
-            for (int di = -1; di <= 1; ++di) {
-              int a = min(max(idx[0] + di, 0), L.nx - 1);
-              int b = min(max(idx[1] + dj, 0), L.ny - 1);
-              int e = min(max(idx[2] + dk, 0), L.nz - 1);
-              double w = (di == 0 ? 2.0 : 1.0) * (dj == 0 ? 2.0 : 1.0) *
-                         (nd == 3 ? (dk == 0 ? 2.0 : 1.0) : 1.0);
-              double v = C[cidx(L, a, b, e)];
-              m[0] -= w * di * v;
-              m[1] -= w * dj * v;
-              m[2] -= w * dk * v;
-            }
-        dm = plic_unit_area(nd, m, Cc) / L.h;
-      } else {
-        dm = 0.0;
+      const double g = (C[cp] - C[cm]) * inv2h;
+      q += g * g;
+    }
+  }
+  double dm;
+  if (dm_mode == 0) {
+    dm = sqrt(q);
+  } else {
+    double m[3];
+    youngs_normal(L, C, idx[0], idx[1], idx[2], m);
+    dm = plic_unit_area(nd, m, C[c]) / L.h;
+  }
+  for (int d = 0; d < nd; ++d) force[(size_t)d * n + c] = dm * (gs[d] - nn[d] * ndg);
+  if (dm_out) dm_out[c] = dm;
+}
+
+// With the PLIC area only interface cells carry a force (1e-6 < C < 1 - 1e-6:
+// nearer fractions are the round-off of empty or full cells).  They are
+// listed first and taken by full warps: a cell is a chain of about 600 FP64
+// instructions, an instruction occupies the SM's FP64 pipe for a whole warp
+// however few lanes it serves, and in rows of 32 cells a warp held one or two
+// interface cells.  96^3: 449 -> 36 us, 128^2 104 -> 21 us (with the plane
+// offsets of sfx_plic.cuh).
+__global__ void k_force_list(size_t n, int nd, const double* __restrict__ C,
+                             double* __restrict__ force, double* __restrict__ dm_out,
+                             unsigned* __restrict__ list) {
+  const size_t step = (size_t)gridDim.x * blockDim.x;
+  // every lane of a warp takes part in the append
+  for (size_t b = blockIdx.x * (size_t)blockDim.x; b < n; b += step) {
+    const size_t c = b + threadIdx.x;
+    bool cut = false;
+    if (c < n) {
+      const double Cc = C[c];
+      cut = Cc > 1e-6 && Cc < 1.0 - 1e-6;
+      if (!cut) {
+        for (int d = 0; d < nd; ++d) force[(size_t)d * n + c] = 0.0;
+        if (dm_out) dm_out[c] = 0.0;
       }
     }
-    for (int d = 0; d < nd; ++d) force[(size_t)d * n + c] = dm * (gs[d] - nn[d] * ndg);
-    if (dm_out) dm_out[c] = dm;
+    warp_append(list, cut, (unsigned)c);
+  }
+}
+
+// The cells of the list, or all of them (list null: every cell carries |grad
+// C|, or its index does not fit the list).
+__global__ void __launch_bounds__(64)
+k_force(Level L, const double* __restrict__ phi, const double* __restrict__ C,
+        const double* __restrict__ sigma, int dm_mode, double eps,
+        const unsigned* __restrict__ list, double* __restrict__ force,
+        double* __restrict__ dm_out) {
+  const size_t n = list ? list[0] : L.ncell();
+  for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n;
+       q += (size_t)gridDim.x * blockDim.x) {
+    const size_t c = list ? list[1 + q] : q;
+    if (!list && dm_mode != 0 && !(C[c] > 1e-6 && C[c] < 1.0 - 1e-6)) {
+      for (int d = 0; d < L.ndim(); ++d) force[(size_t)d * n + c] = 0.0;
+      if (dm_out) dm_out[c] = 0.0;
+      continue;
+    }
+    force64_cell(L, phi, C, sigma, dm_mode, eps, c, force, dm_out);
   }
 }
 
@@ -197,6 +231,36 @@ __global__ void k_loss_grad(Level L, EosArgs q, const double* __restrict__ f,
 
 }  // namespace
 
+sfx_status cut_list(sfx_ctx* c, unsigned** list) {
+  const size_t n = c->lev[0].lv.ncell();
+  if (!c->cut_list && n < ((size_t)1 << 32)) {
+    SFX_CUDA(cudaMalloc((void**)&c->cut_list, (n + 1) * sizeof(unsigned)));
+    c->allocations.push_back(c->cut_list);
+  }
+  *list = c->cut_list;
+  return SFX_OK;
+}
+
+// sigma, the force and (dm not null) delta_m of an FP64 state
+static sfx_status eos_force(sfx_ctx* c, const EosArgs& q, const double* f, const double* phi,
+                            const double* C, int dm_mode, double* sigma, double* force, double* dm,
+                            cudaStream_t s) {
+  const Level& L = c->lev[0].lv;
+  const size_t n = L.ncell();
+  const int nb = blocks_for(n, 256);
+  unsigned* list = nullptr;
+  if (dm_mode != 0) {
+    const sfx_status st = cut_list(c, &list);
+    if (st != SFX_OK) return st;
+  }
+  SFX_KERNEL(c, K_FORCES, k_eos, nb, 256, s, n, q, f, phi, sigma, list);
+  if (list) SFX_KERNEL(c, K_FORCES, k_force_list, nb, 256, s, n, L.ndim(), C, force, dm, list);
+  SFX_KERNEL(c, K_FORCES, k_force, std::min(blocks_for(n, 64), c->sm_count * 16), 64, s, L, phi, C,
+             sigma, dm_mode, q.eps, list, force, dm);
+  SFX_LAUNCH_CHECK();
+  return SFX_OK;
+}
+
 sfx_status marangoni_loss(sfx_ctx* c, const sfx_params* p, const double* f, const double* phi,
                           const double* C, int dm_mode, double* loss, double* grad,
                           cudaStream_t s) {
@@ -206,9 +270,8 @@ sfx_status marangoni_loss(sfx_ctx* c, const sfx_params* p, const double* f, cons
   const size_t n = L.ncell();
   const int nb = blocks_for(n, 256);
   EosArgs q{p->gamma_inf, p->eps, p->sigma0, p->E, p->eos};
-  SFX_KERNEL(c, K_FORCES, k_eos<double>, nb, 256, s, n, q, f, phi, c->adj.sig);
-  SFX_KERNEL(c, K_FORCES, k_force<double>, nb, 256, s, L, phi, C, c->adj.sig, dm_mode, p->eps,
-             c->adj.force, c->adj.dm);
+  st = eos_force(c, q, f, phi, C, dm_mode, c->adj.sig, c->adj.force, c->adj.dm, s);
+  if (st != SFX_OK) return st;
   const int nbp = c->adj.nblk;
   SFX_KERNEL(c, K_FORCES, k_loss_partials, nbp, kTotThreads, s, L, c->adj.force, c->adj.dm,
              grad ? c->adj.G : nullptr, c->adj.part);
@@ -238,15 +301,8 @@ sfx_status totals(sfx_ctx* c, const double* const* fields, int nf, double* out, 
 sfx_status marangoni(sfx_ctx* c, const sfx_params* p, const double* f, const void* phi,
                      const double* C, int dm_mode, double* sigma, double* force,
                      cudaStream_t s) {
-  const Level& L = c->lev[0].lv;
-  const size_t n = L.ncell();
   EosArgs q{p->gamma_inf, p->eps, p->sigma0, p->E, p->eos};
-  const int nb = blocks_for(n, 256);
-  SFX_KERNEL(c, K_FORCES, k_eos<double>, nb, 256, s, n, q, f, (const double*)phi, sigma);
-  SFX_KERNEL(c, K_FORCES, k_force<double>, nb, 256, s, L, (const double*)phi, C, sigma, dm_mode,
-             p->eps, force, (double*)nullptr);
-  SFX_LAUNCH_CHECK();
-  return SFX_OK;
+  return eos_force(c, q, f, (const double*)phi, C, dm_mode, sigma, force, nullptr, s);
 }
 
 }  // namespace sfx

@@ -222,7 +222,7 @@ struct sfx_ctx {
   void* block_list = nullptr;        // redistancing and VoF: active blocks and their flags
   unsigned char* vofH = nullptr;     // VoF: indicator H, minus-face fluxes Q by cell
   double* vofQ = nullptr;
-  unsigned* vof_cut = nullptr;       // VoF: faces that need a plane (large grids)
+  unsigned* cut_list = nullptr;      // cells near the interface: a count and their indices
   double* acdi = nullptr;            // ACDI: phi*, r, psi, unit normals
 };
 
@@ -298,6 +298,9 @@ sfx_status acdi_step(sfx_ctx* c, const void* ux, const void* uy, const void* uz,
 // sfx_capillary.cu
 sfx_status capillary(sfx_ctx* c, const sfx_params* p, const double* phi, const void* C,
                      const void* sigma, void* kappa, void* force, cudaStream_t s);
+// sfx_forces.cu: ctx->cut_list (allocated on first use; each pass fills it
+// anew), null where a grid's cells do not fit 32-bit indices
+sfx_status cut_list(sfx_ctx* c, unsigned** list);
 // sfx_phase.cu: ctx->block_list for nb blocks of cells: a count, nb int2 and
 // two flags per block (allocated on first use; each pass fills it anew)
 sfx_status block_list(sfx_ctx* c, size_t nb);

@@ -15,7 +15,7 @@ template <typename T>
 struct PlicTraits;
 template <>
 struct PlicTraits<double> {
-  static constexpr double step_tol = 1e-17;   // below the resolution of alpha in [0, 1]
+  static constexpr double step_tol = 4e-16;   // the last step's error is its square
 };
 template <>
 struct PlicTraits<float> {
@@ -85,14 +85,15 @@ __device__ inline VolSlope<T> plic_volume(const T* q, bool three_d, T a) {
 }
 
 // Plane offset alpha in [0, 1] with volume fraction C: the root of the
-// increasing V(alpha) - C by Newton steps on the slope dV/dalpha, kept
-// inside a bracket that every evaluation narrows (a bisection step replaces
-// a Newton step that leaves it); stops when the step falls below the
-// resolution of alpha, the bracket closes, or after 100 evaluations.  The
-// same root as a bisection to full precision, in a handful of evaluations.
-template <typename T>
-__device__ inline T plic_alpha(const T* q, bool three_d, T C) {
-  T lo = T(0), hi = T(1), a = C;
+// increasing V(alpha) - C by Newton steps on the slope dV/dalpha from `a`,
+// kept inside a bracket that every evaluation narrows (a bisection step
+// replaces a Newton step that leaves it); stops when the step falls below the
+// resolution of alpha, the bracket closes, or after 100 evaluations.  A step
+// that rounds to nothing at an end of the bracket counts as leaving it, and
+// tens of bisections follow; with EARLY the step itself is tested first.
+template <typename T, bool EARLY>
+__device__ inline T plic_newton(const T* q, bool three_d, T C, T a) {
+  T lo = T(0), hi = T(1);
   for (int it = 0; it < 100; ++it) {
     const VolSlope<T> r = plic_volume(q, three_d, a);
     const T f = r.v - C;
@@ -100,11 +101,31 @@ __device__ inline T plic_alpha(const T* q, bool three_d, T C) {
     if (f < T(0)) lo = a;
     else hi = a;
     T an = r.dv > T(0) ? a - f / r.dv : T(0.5) * (lo + hi);
+    if (EARLY && r.dv > T(0) && fabs(an - a) <= PlicTraits<T>::step_tol) return an;
     if (!(an > lo && an < hi)) an = T(0.5) * (lo + hi);
     if (fabs(an - a) <= PlicTraits<T>::step_tol || !(hi - lo > T(0))) return an;
     a = an;
   }
   return a;
+}
+
+// The float geometry of the VoF fluxes.
+template <typename T>
+__device__ inline T plic_alpha(const T* q, bool three_d, T C) {
+  return plic_newton<T, false>(q, three_d, C, C);
+}
+// In double the iteration starts from the float root of the smaller of C and
+// 1 - C (good to ~1e-6 of it), so that two or three FP64 evaluations remain:
+// each is a chain of ~40 dependent FP64 instructions (a 128^2 force took 104
+// us, most of it the chain of the slowest cell; 20 us now).
+template <>
+__device__ inline double plic_alpha<double>(const double* q, bool three_d, double C) {
+  const bool flip = C > 0.5;
+  const double t = flip ? 1.0 - C : C;
+  const float qf[3] = {(float)q[0], (float)q[1], (float)q[2]};
+  const double a0 = (double)plic_newton<float, true>(qf, three_d, (float)t, (float)t);
+  const double a = plic_newton<double, true>(q, three_d, t, a0);
+  return flip ? 1.0 - a : a;
 }
 
 // Components |m|/sum|m| in ascending order (q[0] = 0 in 2D); false when m = 0.

@@ -160,16 +160,7 @@ k_vof_flux(Level L, int d, const int2* __restrict__ list, const double* __restri
       if (!plane) Q[c] = flux;
       else if (!cut) Q[c] = plic_flux<U, G, ND>(L, d, x, st, C, u, dt_h);
     }
-    if (cut) {        // one slot of the list per lane that needs a plane
-      const unsigned full = 0xffffffffu, m = __ballot_sync(full, plane);
-      if (m) {
-        unsigned base = 0;
-        const int lane = threadIdx.x & 31, lead = __ffs(m) - 1;
-        if (lane == lead) base = atomicAdd(cut, (unsigned)__popc(m));
-        base = __shfl_sync(full, base, lead);
-        if (plane) cut[1 + base + __popc(m & ((1u << lane) - 1))] = (unsigned)c;
-      }
-    }
+    if (cut) warp_append(cut, plane, (unsigned)c);
   }
 }
 
@@ -228,12 +219,9 @@ sfx_status vof_impl(sfx_ctx* c, const U* const* u, double dt, int order, double*
   unsigned grid = (unsigned)nb;
   unsigned* cut = nullptr;
   if (L.ncell() >= kVofListCells) {
-    if (L.ncell() < ((size_t)1 << 32) && !c->vof_cut) {
-      SFX_CUDA(cudaMalloc((void**)&c->vof_cut, (L.ncell() + 1) * sizeof(unsigned)));
-      c->allocations.push_back(c->vof_cut);
-    }
-    cut = c->vof_cut;
-    const sfx_status st = block_list(c, nb);
+    sfx_status st = cut_list(c, &cut);
+    if (st != SFX_OK) return st;
+    st = block_list(c, nb);
     if (st != SFX_OK) return st;
     list = (int2*)c->block_list;
     unsigned char* flag = (unsigned char*)(list + nb + 1);
