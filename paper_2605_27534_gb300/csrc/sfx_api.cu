@@ -421,6 +421,7 @@ sfx_status sfx_set_tuning(sfx_ctx* c, int key, int value) {
   if (key == SFX_TUNE_F32_SOLVER && value >= 0 && value <= 2) {
     c->f32.solver = value;
     c->f32.predicted = 0;
+    c->f32.drift_phi = nullptr;   // the solvers keep different face arrays
     return SFX_OK;
   }
   return SFX_ERR_ARG;

@@ -60,6 +60,20 @@ __device__ __forceinline__ double widen(float x) {
                           (int)(b << 29));
 }
 __device__ __forceinline__ double widen(double x) { return x; }
+// double to float, rounded to nearest even as the conversion instruction
+// does, from the integer words (the same reason); values outside the normal
+// floats take the instruction.
+__device__ __forceinline__ float narrow(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned e = (hi >> 20) & 0x7ffu;
+  if (e - 897u < 253u) {
+    const unsigned m = ((hi & 0xfffffu) << 3) | (lo >> 29), r = lo & 0x1fffffffu;
+    unsigned v = ((e - 896u) << 23) | m;
+    if (r > 0x10000000u || (r == 0x10000000u && (m & 1u))) ++v;   // may carry into the exponent
+    return __uint_as_float((hi & 0x80000000u) | v);
+  }
+  return ((hi << 1) | lo) == 0u ? __uint_as_float(hi) : (float)x;
+}
 
 // Row r = k ny + j (64-bit division only past 2^32).
 __device__ __forceinline__ void row_jk(size_t r, int ny, int& j, int& k) {

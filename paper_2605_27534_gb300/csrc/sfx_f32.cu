@@ -40,37 +40,79 @@
 namespace sfx {
 namespace {
 
-// Drift faces of direction d in float (Bf, BF, B2) and half (H2) precision;
-// Hm (may be null): the half pair again, at the colour-packed position of
-// the cell whose minus side the face is (the layout of the tiled sweep,
-// nx even; the far wall's faces have no such cell and are not kept).
-__global__ void k_drift32(Level L, int d, const double* __restrict__ phi, float Df, float DF,
-                          float inv_eps, float* __restrict__ Bf, float* __restrict__ BF,
-                          float2* __restrict__ B2, __half2* __restrict__ H2,
-                          __half2* __restrict__ Hm) {
-  size_t n = L.nface(d);
-  int fx = L.nx + (d == 0), fy = L.ny + (d == 1);
-  for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n;
-       q += (size_t)gridDim.x * blockDim.x) {
-    int i = (int)(q % fx), j = (int)((q / fx) % fy), k = (int)(q / ((size_t)fx * fy));
-    int pos = d == 0 ? i : (d == 1 ? j : k);
-    float bf = 0.0f, bF = 0.0f;
-    if (pos > 0 && pos < L.extent(d)) {
-      int li = i - (d == 0), lj = j - (d == 1), lk = k - (d == 2);
-      const float sL = fold_phi(phi[cidx(L, li, lj, lk)]), sR = fold_phi(phi[cidx(L, i, j, k)]);
-      const float nL = normal_f32(L, phi, li, lj, lk, d, inv_eps);
-      const float nR = normal_f32(L, phi, i, j, k, d, inv_eps);
-      drift_face(sL, sR, nL, nR, Df, DF, inv_eps, bf, bF);
+// The phi-dependent arrays of a step: the folded float copy of phi, and the
+// drift faces on the minus sides of a block's cells (and on the far walls,
+// zero) as float pairs (B2) and half pairs (H2); where asked for, B_f and B_F
+// by themselves (the solvers 0 and 2) and the half pair again (Hm) at the
+// colour-packed position of the cell (the layout of the tiled sweep, nx
+// even; the far wall's faces have no such cell and are not kept).
+// Normals are formed once per cell, in shared memory with one layer on the
+// minus sides (a face per thread and direction formed two per face: six per
+// cell, sixty FP64 instructions); the FP64 differences of phi are narrowed
+// through the integer words.  157 x 131 x 117: 270 -> 57 us, 512^2 24 -> 7 us.
+struct Setup32 {
+  Level L;
+  const double* phi;
+  float Df, DF, inv_eps;
+  float* phi32;
+  float* Bf[3];
+  float* BF[3];
+  float2* B2[3];
+  __half2* H2[3];
+  __half2* Hm[3];
+};
+
+template <int ND>
+__global__ void __launch_bounds__(ND == 3 ? 512 : 128) k_setup32(Setup32 q) {
+  constexpr int BX = 32, BY = 4, BZ = ND == 3 ? 4 : 1;
+  constexpr int HX = BX + 1, HY = BY + 1, HZ = ND == 3 ? BZ + 1 : 1;
+  __shared__ float sn[ND][HZ][HY][HX], sp[HZ][HY][HX];
+  const Level& L = q.L;
+  const int x0 = blockIdx.x * BX, y0 = blockIdx.y * BY, z0 = blockIdx.z * BZ;
+  for (int t = threadIdx.x; t < HX * HY * HZ; t += blockDim.x) {
+    const int lx = t % HX, ly = t / HX % HY, lz = t / (HX * HY);
+    const int i = x0 + lx - 1, j = y0 + ly - 1, k = ND == 3 ? z0 + lz - 1 : 0;
+    float n[3] = {0.0f, 0.0f, 0.0f}, f = 0.0f;
+    if (i >= 0 && i < L.nx && j >= 0 && j < L.ny && k >= 0 && k < L.nz) {
+      normal3_f32(L, q.phi, i, j, k, q.inv_eps, n);
+      f = fold_phi(q.phi[cidx(L, i, j, k)]);
     }
-    Bf[q] = bf;
-    BF[q] = bF;
-    B2[q] = make_float2(bf, bF);
+    sp[lz][ly][lx] = f;
+#pragma unroll
+    for (int d = 0; d < ND; ++d) sn[d][lz][ly][lx] = n[d];
+  }
+  __syncthreads();
+  const int lx = threadIdx.x % BX, ly = threadIdx.x / BX % BY, lz = threadIdx.x / (BX * BY);
+  const int x[3] = {x0 + lx, y0 + ly, z0 + lz};
+  if (x[0] >= L.nx || x[1] >= L.ny || x[2] >= L.nz) return;
+  const int hz = ND == 3 ? lz + 1 : 0;
+  const float sR = sp[hz][ly + 1][lx + 1];
+  q.phi32[cidx(L, x[0], x[1], x[2])] = sR;
+#pragma unroll
+  for (int d = 0; d < ND; ++d) {
+    const int mz = hz - (ND == 3 && d == 2), my = ly + 1 - (d == 1), mx = lx + 1 - (d == 0);
+    float bf = 0.0f, bF = 0.0f;
+    if (x[d] > 0)
+      drift_face(sp[mz][my][mx], sR, sn[d][mz][my][mx], sn[d][hz][ly + 1][lx + 1], q.Df, q.DF,
+                 q.inv_eps, bf, bF);
+    const size_t f = fidx(L, d, x[0], x[1], x[2]);
     const __half2 hv = __floats2half2_rn(bf, bF);
-    H2[q] = hv;
-    if (Hm && pos < L.extent(d)) {
+    q.B2[d][f] = make_float2(bf, bF);
+    q.H2[d][f] = hv;
+    if (q.Bf[d]) {
+      q.Bf[d][f] = bf;
+      q.BF[d][f] = bF;
+    }
+    if (q.Hm[d]) {
       const size_t half = (size_t)(L.nx >> 1);
-      Hm[(size_t)((i + j + k) & 1) * half * L.ny * L.nz + ((size_t)k * L.ny + j) * half + (i >> 1)] =
-          hv;
+      q.Hm[d][(size_t)((x[0] + x[1] + x[2]) & 1) * half * L.ny * L.nz +
+              ((size_t)x[2] * L.ny + x[1]) * half + (x[0] >> 1)] = hv;
+    }
+    if (x[d] + 1 == L.extent(d)) {   // the far wall's face
+      const size_t w = fidx(L, d, x[0] + (d == 0), x[1] + (d == 1), x[2] + (d == 2));
+      q.B2[d][w] = make_float2(0.0f, 0.0f);
+      q.H2[d][w] = __floats2half2_rn(0.0f, 0.0f);
+      if (q.Bf[d]) q.Bf[d][w] = q.BF[d][w] = 0.0f;
     }
   }
 }
@@ -901,7 +943,7 @@ k_totals32(Level L, TotalFields32 fl, double scale, double* __restrict__ partial
 struct Eos32 {
   float ginf, eps, inv_eps, sigma0, E;
   int eos;
-  double ginf_d, eps_d, sigma0_d, E_d;   // the same in FP64 (near saturation)
+  double sigE_d, ginf_eps_d;   // sigma0 E and Gamma_inf/eps in FP64 (near saturation)
 };
 
 // sigma - sigma0 (kept for the gradient, where it has full relative
@@ -910,31 +952,94 @@ struct Eos32 {
 // phi, Gamma from the whole double-float pair of f, 1 - Gamma/Gamma_inf and
 // its logarithm, since float spacing in Gamma/Gamma_inf (6e-8) would be a
 // large relative error of 1 - Gamma/Gamma_inf there.  FP32 below.
+// The Langmuir term near saturation, sigma0 E ln(1 - x) with 1 - x = (a - f)/a,
+// a = Gamma_inf delta_phi: the difference, quotient and logarithm in FP64.
+// Out of line: inlined, its logarithm took the kernel to 80 registers.
+__device__ __noinline__ float eos32_saturated(double pd, float2 fc, double sigE, double ginf_eps) {
+  const double a = pd * (1.0 - pd) * ginf_eps;
+  const double t = (a - (widen(fc.x) + widen(fc.y))) / a;
+  return narrow(sigE * log(fmax(t, 1.0 - (1.0 - 1e-12))));   // x stays at 1 - 1e-12
+}
+
+// phi within 5e-4 of 0 or 1 (or outside): phi (1 - phi) is half the threshold
+// of Gamma, told from the integer words alone.
+__device__ __forceinline__ bool eos32_bulk(double pd) {
+  const long long b = __double_as_longlong(pd);
+  return b < 0x3f40624dd2f1a9fcLL || b > 0x3feffbe76c8b4396LL;
+}
+
+// Where delta_phi is below the threshold Gamma = 0 and f is not read.
+__device__ __forceinline__ float eos32_cell(const Eos32& q, double pd,
+                                            const float2* __restrict__ f, size_t c) {
+  if (eos32_bulk(pd)) return 0.0f;
+  const PhiPair ph = unfold(fold_phi(pd));
+  const float del = ph.p * ph.q * q.inv_eps;
+  if (!(del >= 1e-3f * q.inv_eps)) return 0.0f;
+  const float2 fc = f[c];
+  const float x = df_val(fc) / del / q.ginf;
+  if (q.eos == SFX_EOS_LANGMUIR) {
+    if (x > 0.5f) return eos32_saturated(pd, fc, q.sigE_d, q.ginf_eps_d);
+    return q.sigma0 * q.E * log1pf(-x);
+  }
+  if (q.eos == SFX_EOS_LINEAR) return -q.sigma0 * q.E * x;
+  return -q.sigma0 * tanhf(q.E * x);
+}
+
+// sigma - sigma0 and sigma of every cell.  It also empties the list of
+// interface cells of the force behind it.
 __global__ void k_eos32(size_t n, Eos32 q, const float2* __restrict__ f,
                         const double* __restrict__ phi, float* __restrict__ dsig,
-                        float* __restrict__ sigma) {
-  for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
-       c += (size_t)gridDim.x * blockDim.x) {
-    PhiPair ph = unfold(fold_phi(phi[c]));
-    float del = ph.p * ph.q * q.inv_eps;
-    float G = del >= 1e-3f * q.inv_eps ? df_val(f[c]) / del : 0.0f;
-    float x = G / q.ginf;
-    float ds;
-    if (q.eos == SFX_EOS_LANGMUIR) {
-      if (x > 0.5f) {
-        const double pd = phi[c];
-        const double deld = pd * (1.0 - pd) / q.eps_d;
-        const float2 fc = f[c];
-        const double xd = ((double)fc.x + (double)fc.y) / deld / q.ginf_d;
-        ds = (float)(q.sigma0_d * q.E_d * log1p(-fmin(xd, 1.0 - 1e-12)));
-      } else {
-        ds = q.sigma0 * q.E * log1pf(-x);
-      }
-    } else if (q.eos == SFX_EOS_LINEAR) {
-      ds = -q.sigma0 * q.E * x;
+                        float* __restrict__ sigma, unsigned* __restrict__ list) {
+  if (list && blockIdx.x == 0 && threadIdx.x == 0) list[0] = 0;
+  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n;
+       t += (size_t)gridDim.x * blockDim.x) {
+    const float ds = eos32_cell(q, phi[t], f, t);
+    dsig[t] = ds;
+    if (sigma) sigma[t] = q.sigma0 + ds;
+  }
+}
+
+// The same in two launches for large grids: the cells with Gamma = 0 (phi in,
+// zeros and sigma0 out, two cells per thread: bound by HBM), which lists the
+// others in `band`, and the band by full warps: near saturation a cell takes
+// about 50 FP64 instructions, and a warp of a row held a few band cells.
+// 256^3 with a saturating sphere: 150 -> 85 us.
+constexpr size_t kEosListCells = (size_t)1 << 20;
+__global__ void k_eos32_bulk(ix n, float sigma0, const double* __restrict__ phi,
+                             float* __restrict__ dsig, float* __restrict__ sigma,
+                             unsigned* __restrict__ band, unsigned* __restrict__ list) {
+  if (list && blockIdx.x == 0 && threadIdx.x == 0) list[0] = 0;
+  const ix m = (n + 1) / 2, step = gridDim.x * blockDim.x;
+  const bool vec = (((size_t)phi & 15) | ((size_t)sigma & 7)) == 0;
+  // every lane of a warp takes part in the appends
+  for (ix b = blockIdx.x * blockDim.x; b < m; b += step) {
+    const ix t = b + threadIdx.x, c = 2 * t;
+    double2 p = make_double2(0.0, 0.0);
+    if (vec && c + 1 < n) {
+      p = reinterpret_cast<const double2*>(phi)[t];
+      reinterpret_cast<float2*>(dsig)[t] = make_float2(0.0f, 0.0f);
+      if (sigma) reinterpret_cast<float2*>(sigma)[t] = make_float2(sigma0, sigma0);
     } else {
-      ds = -q.sigma0 * tanhf(q.E * x);
+      for (ix e = c; e < n && e < c + 2; ++e) {
+        (e == c ? p.x : p.y) = phi[e];
+        dsig[e] = 0.0f;
+        if (sigma) sigma[e] = sigma0;
+      }
     }
+    const bool b0 = c < n && !eos32_bulk(p.x), b1 = c + 1 < n && !eos32_bulk(p.y);
+    if (!__any_sync(0xffffffffu, b0 || b1)) continue;
+    warp_append(band, b0, c);
+    warp_append(band, b1, c + 1);
+  }
+}
+__global__ void __launch_bounds__(128)
+k_eos32_band(Eos32 q, const float2* __restrict__ f, const double* __restrict__ phi,
+             const unsigned* __restrict__ band, float* __restrict__ dsig,
+             float* __restrict__ sigma) {
+  const ix m = band[0];
+  for (ix t = blockIdx.x * blockDim.x + threadIdx.x; t < m; t += gridDim.x * blockDim.x) {
+    const ix c = band[1 + t];
+    const float ds = eos32_cell(q, phi[c], f, c);
     dsig[c] = ds;
     if (sigma) sigma[c] = q.sigma0 + ds;
   }
@@ -1071,7 +1176,53 @@ struct RowWalk {
   }
 };
 
-// blocks over (x chunk, rows); each block walks rows r = k ny + j
+// With the PLIC area (dm_mode 1) the interface cells are listed first, the
+// others' force set to zero (four cells per thread: C in, force out, bound by
+// HBM), and a second launch takes the listed cells by full warps; in rows of
+// cells a warp held a few of them and every other lane waited.  256^3: 157 ->
+// 69 us, 160^3 58 -> 33 us.
+__device__ __forceinline__ bool cut32(float C) { return C > 1e-6f && C < 1.0f - 1e-6f; }
+
+template <bool QUADS>
+__global__ void k_force32_list(ix n, int nd, const float* __restrict__ C, float* __restrict__ force,
+                               unsigned* __restrict__ list) {
+  const ix m = QUADS ? n / 4 : n, step = gridDim.x * blockDim.x;
+  // every lane of a warp takes part in the appends
+  for (ix b = blockIdx.x * blockDim.x; b < m; b += step) {
+    const ix t = b + threadIdx.x;
+    if (QUADS) {
+      const float4 v = t < m ? reinterpret_cast<const float4*>(C)[t] : make_float4(0, 0, 0, 0);
+      if (t < m)
+        for (int d = 0; d < nd; ++d)
+          reinterpret_cast<float4*>(force + (size_t)d * n)[t] = make_float4(0, 0, 0, 0);
+      const bool c0 = cut32(v.x), c1 = cut32(v.y), c2 = cut32(v.z), c3 = cut32(v.w);
+      if (!__any_sync(0xffffffffu, c0 || c1 || c2 || c3)) continue;
+      warp_append(list, c0, 4 * t);
+      warp_append(list, c1, 4 * t + 1);
+      warp_append(list, c2, 4 * t + 2);
+      warp_append(list, c3, 4 * t + 3);
+    } else {
+      const bool cut = t < m && cut32(C[t]);
+      if (t < m && !cut)
+        for (int d = 0; d < nd; ++d) force[(size_t)d * n + t] = 0.0f;
+      warp_append(list, cut, t);
+    }
+  }
+}
+
+__global__ void __launch_bounds__(64)
+k_force32_cells(Level L, const double* __restrict__ phi, const float* __restrict__ C,
+                const float* __restrict__ dsig, float inv_eps, const unsigned* __restrict__ list,
+                float* __restrict__ force) {
+  const ix m = list[0], n = (ix)L.nx * (ix)L.ny * (ix)L.nz;
+  for (ix q = blockIdx.x * blockDim.x + threadIdx.x; q < m; q += gridDim.x * blockDim.x) {
+    const ix c = list[1 + q], r = c / (ix)L.nx;
+    force32_cell(L, phi, C, dsig, 1, inv_eps, (int)(c - r * (ix)L.nx), (int)(r % (ix)L.ny),
+                 (int)(r / (ix)L.ny), c, n, force);
+  }
+}
+
+// dm_mode 0: every cell; blocks over (x chunk, rows), rows r = k ny + j
 __global__ void k_force32(Level L, const double* __restrict__ phi, const float* __restrict__ C,
                           const float* __restrict__ dsig, int dm_mode, float inv_eps,
                           float* __restrict__ force) {
@@ -1092,14 +1243,6 @@ __global__ void k_pack_df(size_t n, const double* __restrict__ in, float2* __res
     double d = in[c];
     float hi = (float)d;
     out[c] = make_float2(hi, (float)(d - (double)hi));
-  }
-}
-
-__global__ void k_fold_phi(size_t n, const double* __restrict__ phi, float* __restrict__ out) {
-  for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
-       c += (size_t)gridDim.x * blockDim.x) {
-    double p = phi[c];
-    out[c] = p <= 0.5 ? (float)p : (float)(p - 1.0);
   }
 }
 
@@ -1548,11 +1691,20 @@ sfx_status step_f32(sfx_ctx* c, const sfx_params* pr, const double* phi_in, cons
                      c->f32.drift_key[2] == pr->eps;
   const float* phi = c->f32.phi32;
   if (!reuse) {
-    SFX_KERNEL(c, K_SETUP, k_fold_phi, blocks_for(n, 256), 256, s, n, phi_in, c->f32.phi32);
-    for (int d = 0; d < nd; ++d)
-      SFX_KERNEL(c, K_SETUP, k_drift32, blocks_for(L.nface(d), 256), 256, s, L, d, phi_in,
-                 (float)pr->Df, (float)pr->DF, (float)(1.0 / pr->eps), Bf[d], BF[d],
-                 c->f32.B2[d], c->f32.H2[d], c->f32.Hm[d]);
+    Setup32 q{L, phi_in, (float)pr->Df, (float)pr->DF, (float)(1.0 / pr->eps), c->f32.phi32,
+              {}, {}, {}, {}, {}};
+    for (int d = 0; d < nd; ++d) {
+      if (c->f32.solver != 1) {
+        q.Bf[d] = Bf[d];
+        q.BF[d] = BF[d];
+      }
+      q.B2[d] = c->f32.B2[d];
+      q.H2[d] = c->f32.H2[d];
+      q.Hm[d] = c->f32.Hm[d];
+    }
+    const dim3 g((unsigned)((L.nx + 31) / 32), (unsigned)((L.ny + 3) / 4), (unsigned)((L.nz + 3) / 4));
+    if (nd == 3) SFX_KERNEL(c, K_SETUP, k_setup32<3>, g, 512, s, q);
+    else SFX_KERNEL(c, K_SETUP, k_setup32<2>, g, 128, s, q);
     SFX_LAUNCH_CHECK();
     ++c->f32.drift_epoch;
     c->f32.drift_phi = phi_in;
@@ -1770,11 +1922,34 @@ sfx_status marangoni32(sfx_ctx* c, const sfx_params* p, const float2* f, const d
   const Level& L = c->lev[0].lv;
   const size_t n = L.ncell();
   Eos32 q{(float)p->gamma_inf, (float)p->eps, (float)(1.0 / p->eps), (float)p->sigma0,
-          (float)p->E, p->eos, p->gamma_inf, p->eps, p->sigma0, p->E};
-  SFX_KERNEL(c, K_FORCES, k_eos32, blocks_for(n, 256), 256, s, n, q, f, phi, c->f32.dsig, sigma);
-  const RowGrid fg = row_grid(L, c->sm_count);
-  SFX_KERNEL(c, K_FORCES, k_force32, fg.grid, fg.block, s, L, phi, C, c->f32.dsig, dm_mode,
-             q.inv_eps, force);
+          (float)p->E, p->eos, p->sigma0 * p->E, p->gamma_inf / p->eps};
+  unsigned* list = nullptr;
+  if (dm_mode != 0 && (st = cut_list(c, &list)) != SFX_OK) return st;
+  if (n >= kEosListCells) {
+    unsigned* band = reinterpret_cast<unsigned*>(c->f32.falt);   // idle outside solvers 0 and 2
+    SFX_CUDA(cudaMemsetAsync(band, 0, sizeof(unsigned), s));
+    SFX_KERNEL(c, K_FORCES, k_eos32_bulk, blocks_for((n + 1) / 2, 256), 256, s, (ix)n, q.sigma0, phi,
+               c->f32.dsig, sigma, band, list);
+    SFX_KERNEL(c, K_FORCES, k_eos32_band, c->sm_count * 16, 128, s, q, f, phi, band, c->f32.dsig,
+               sigma);
+  } else {
+    SFX_KERNEL(c, K_FORCES, k_eos32, blocks_for(n, 256), 256, s, n, q, f, phi, c->f32.dsig, sigma,
+               list);
+  }
+  if (list) {
+    const bool quads = n % 4 == 0 && (((size_t)C | (size_t)force) & 15) == 0;
+    const int nb = blocks_for(quads ? n / 4 : n, 256), nd = L.ndim();
+    if (quads)
+      SFX_KERNEL(c, K_FORCES, k_force32_list<true>, nb, 256, s, (ix)n, nd, C, force, list);
+    else
+      SFX_KERNEL(c, K_FORCES, k_force32_list<false>, nb, 256, s, (ix)n, nd, C, force, list);
+    SFX_KERNEL(c, K_FORCES, k_force32_cells, std::min(blocks_for(n, 64), c->sm_count * 16), 64, s, L,
+               phi, C, c->f32.dsig, q.inv_eps, list, force);
+  } else {
+    const RowGrid fg = row_grid(L, c->sm_count);
+    SFX_KERNEL(c, K_FORCES, k_force32, fg.grid, fg.block, s, L, phi, C, c->f32.dsig, dm_mode,
+               q.inv_eps, force);
+  }
   SFX_LAUNCH_CHECK();
   return SFX_OK;
 }

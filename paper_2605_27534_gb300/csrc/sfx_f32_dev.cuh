@@ -85,8 +85,16 @@ __device__ __forceinline__ P2 v_lp_sub(const P2& a, const P2& b) {
 
 // ------------------------------------------------------------ drifts
 // Folded float copy of phi: phi where phi <= 1/2, phi - 1 elsewhere.
+// (Compared and narrowed through the integer words: the FP64 pipe issues at
+// 1/59 of their rate.)
 __device__ __forceinline__ float fold_phi(double p) {
-  return p <= 0.5 ? (float)p : (float)(p - 1.0);
+  const long long b = __double_as_longlong(p);
+  return b <= 0x3fe0000000000000LL ? narrow(p) : narrow(p - 1.0);   // p <= 1/2 (or below 0)
+}
+
+// a - b taken in FP64, as a float
+__device__ __forceinline__ float diff32(double a, double b) {
+  return __double_as_longlong(a) == __double_as_longlong(b) ? 0.0f : narrow(a - b);
 }
 
 // n = grad phi/|grad phi| at cell (i,j,k) (centred differences, one-sided
@@ -102,12 +110,12 @@ __device__ __forceinline__ void normal3_f32(const Level& L, const double* __rest
                                             int j, int k, float inv_eps, float* n) {
   const int ip = min(i + 1, L.nx - 1), im = max(i - 1, 0);
   const int jp = min(j + 1, L.ny - 1), jm = max(j - 1, 0);
-  const float g0 = (float)(phi[cidx(L, ip, j, k)] - phi[cidx(L, im, j, k)]);
-  const float g1 = (float)(phi[cidx(L, i, jp, k)] - phi[cidx(L, i, jm, k)]);
+  const float g0 = diff32(phi[cidx(L, ip, j, k)], phi[cidx(L, im, j, k)]);
+  const float g1 = diff32(phi[cidx(L, i, jp, k)], phi[cidx(L, i, jm, k)]);
   float g2 = 0.0f;
   if (L.geom == SFX_CART3D) {
     const int kp = min(k + 1, L.nz - 1), km = max(k - 1, 0);
-    g2 = (float)(phi[cidx(L, i, j, kp)] - phi[cidx(L, i, j, km)]);
+    g2 = diff32(phi[cidx(L, i, j, kp)], phi[cidx(L, i, j, km)]);
   }
   n[0] = n[1] = n[2] = 0.0f;
   const float mx = fmaxf(fabsf(g0), fmaxf(fabsf(g1), fabsf(g2)));

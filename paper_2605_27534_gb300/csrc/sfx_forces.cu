@@ -50,13 +50,15 @@ __global__ void k_eos(size_t n, EosArgs q, const double* __restrict__ f,
   for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
        c += (size_t)gridDim.x * blockDim.x) {
     double p = phi[c];
-    // delta_phi well below 1e-3/eps: Gamma = 0, which every EOS takes to
-    // sigma0, without the quotients and the logarithm (FP64 pipe)
-    const double pq = p * (1.0 - p);
-    if (pq < 0.99e-3) {
+    // phi within 5e-4 of 0 or 1 (or outside): delta_phi is half of 1e-3/eps,
+    // Gamma = 0 and every EOS gives sigma0, told from the integer words
+    // without the quotients and the logarithm (FP64 pipe)
+    const long long b = __double_as_longlong(p);
+    if (b < 0x3f40624dd2f1a9fcLL || b > 0x3feffbe76c8b4396LL) {
       sigma[c] = q.sigma0;
       continue;
     }
+    const double pq = p * (1.0 - p);
     double del = pq / q.eps;
     double G = del >= 1e-3 / q.eps ? f[c] / del : 0.0;
     double x = G / q.ginf;

@@ -74,3 +74,25 @@ def test_force_from_the_list_against_the_oracle(sfx, geom, shape, kind, dm_mode)
         assert (out[:, (C32 <= 1e-6) | (C32 >= 1 - 1e-6)] == 0).all()
     if kind != "edges":     # there a float Youngs normal may cancel to nothing
         assert np.abs(out - F_o.reshape(n)).max() < 1e-4 * max(np.abs(F_o).max(), 1e-300)
+
+
+def test_eos_of_large_float_grids_takes_the_band(sfx):
+    """2^20 cells and more: the cells with Gamma = 0 and the band around the
+    interface in two launches; an odd count of cells, Gamma up to and past
+    saturation, phi at both ends of the threshold."""
+    import torch
+    g = W.Grid(W.PLANAR, 1031, 1025, 1, 1.0 / 1031)
+    p = W.Params(eps=0.75 * g.h)
+    rng = np.random.default_rng(6)
+    phi = rng.choice([0.0, 1e-4, 5e-4, 9.9e-4, 1.01e-3, 0.1, 0.5, 0.9, 1 - 1.01e-3, 1 - 9.9e-4,
+                      0.9995, 1.0], g.shape)
+    f = rng.choice([0.0, 0.3, 0.499, 0.501, 0.9, 0.999999, 1.0, 1.3], g.shape) * phi * (1 - phi) / p.eps
+    C = np.zeros(g.shape)
+    want, _ = oracle.marangoni(g, p, f, phi, C, 1)
+    ctx = sfx.Context.for_grid(g, sfx.SFX_F32)
+    s = dev(np.full(g.shape, np.nan), torch.float32)
+    F = torch.empty((2,) + g.shape, device="cuda")
+    ctx.sfx_marangoni_force(p, ctx.sfx_df_pack(dev(f)), dev(phi), dev(C, torch.float32), s, F)
+    # the logarithm of 1 - x at x = 0.999999 from a pair of 48 bits: 1e-8;
+    # sigma in float (values down to sigma0 (1 + E ln 1e-12) = -4.5)
+    assert np.abs(host(s) - want).max() < 1e-6 and (host(F) == 0).all()
