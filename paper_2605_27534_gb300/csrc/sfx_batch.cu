@@ -17,6 +17,7 @@
 
 #include "sfx_df.cuh"
 #include "sfx_f32_dev.cuh"
+#include "sfx_block2d.cuh"
 #include "sfx_internal.h"
 
 namespace sfx {
@@ -257,6 +258,27 @@ __global__ void k_b_corr(const BInst* __restrict__ I, int n, const int* __restri
   corr2_cell<G>(B.p, i, j, 0, H, P.rc + w, P.e2 + w, color, first, fst, Fst, fst, Fst);
 }
 
+// all sweeps of an iteration on 2D tiles (sfx_block2d.cuh); blocks over the
+// tiles of every instance, ty rows each
+template <int G>
+__global__ void __launch_bounds__(kT2Threads)
+k_b_corr_tiles(const BInst* __restrict__ I, int n, const int* __restrict__ pre, int ty, int sweeps,
+               BPtr P) {
+  const int inst = find_inst(pre, n, blockIdx.x);
+  if (!P.active[inst]) return;
+  const BInst& B = I[inst];
+  const Level& L = B.p.L;
+  const int tx = L.nx <= kT2Width ? L.nx + (L.nx & 1) : kT2Width - 4 * sweeps;
+  const int nx = (L.nx + tx - 1) / tx, t = blockIdx.x - pre[inst];
+  float2* f = P.f + B.coff;
+  float2* F = P.F + B.coff;
+  corr_tile2d<G>(B.p, (t % nx) * tx, (t / nx) * ty, tx, ty, sweeps, P.H2[0] + B.rfoff,
+                 P.H2[1] + B.zfoff, P.rc + B.poff, P.e2 + B.poff, [&](ix c, float2 e) {
+                   f[c] = df_add(f[c], e.x);
+                   F[c] = df_add(F[c], e.y);
+                 });
+}
+
 // per-instance compensated totals: tot_parts blocks per instance each walk
 // a share of its cells, accumulate both fields in double-float pairs and
 // combine their threads in compensated doubles ...
@@ -327,6 +349,9 @@ struct sfx_batch {
   int* pre_zf = nullptr;
   int* pre_pair = nullptr;
   int nb_cell = 0, nb_rf = 0, nb_zf = 0, nb_pair = 0;
+  int* pre_tile = nullptr;   // tiles of all sweeps in one launch, of tile_ty rows
+  int nb_tile = 0, tile_ty = 0, tile_sweeps = 0;   // (tile_ty 0: colour launches)
+  size_t tile_smem = 0;
   int block = 256;
   int geom = SFX_AXISYM;   // of every instance
   int tot_parts = 1;       // blocks of partial totals per instance
@@ -382,6 +407,38 @@ sfx_status build_prefix(sfx_batch* b) {
   return SFX_OK;
 }
 
+// Tiles of the current number of sweeps (before a capture).
+sfx_status build_tiles(sfx_batch* b) {
+  if (b->tile_sweeps == b->sweeps) return SFX_OK;
+  struct Ext {
+    int nx, ny;
+  };
+  std::vector<Ext> g;
+  for (const auto& q : b->hinst) g.push_back(Ext{q.nr, q.nz});
+  int dev = 0, sms = 152;
+  SFX_CUDA(cudaGetDevice(&dev));
+  SFX_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int ty = tile2d_rows(g.data(), b->n, b->sweeps, sms);
+  size_t smem = 0;
+  std::vector<int> pre(1, 0);
+  for (const Ext& e : g) {
+    const Tile2D t = tile2d_of(e.nx, std::max(ty, 1), b->sweeps);
+    smem = std::max(smem, tile2d_smem(e.nx, e.ny, t, b->sweeps));
+    pre.push_back(pre.back() + ((e.nx + t.tx - 1) / t.tx) * ((e.ny + t.ty - 1) / t.ty));
+    if (ty == 0) break;
+  }
+  if (ty > 0) {
+    SFX_CUDA(cudaMemcpy(b->pre_tile, pre.data(), pre.size() * sizeof(int), cudaMemcpyHostToDevice));
+    auto tiles = b->geom == SFX_AXISYM ? &k_b_corr_tiles<SFX_AXISYM> : &k_b_corr_tiles<SFX_PLANAR2D>;
+    SFX_CUDA(cudaFuncSetAttribute(tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kT2Smem));
+  }
+  b->tile_ty = ty;
+  b->tile_smem = smem;
+  b->nb_tile = pre.back();
+  b->tile_sweeps = b->sweeps;
+  return SFX_OK;
+}
+
 // Enqueue one batched step on s under stream capture: the set-up kernels,
 // the Newton iterations as the body of a conditional while node (run again
 // while an instance is active and the budget lasts, so a step whose
@@ -428,7 +485,11 @@ sfx_status enqueue_step(sfx_batch* b, bool advect, float tol, cudaStream_t s) {
   resid<<<b->nb_cell, bs, 0, sb>>>(b->dI, n, b->pre_cell, P);
   k_b_flags<<<n, 256, 0, sb>>>(n, b->pre_cell, P, tol, b->fast);
   // the residual pass did the first red half-sweep
-  for (int q = 0; q < b->sweeps; ++q)
+  if (b->tile_ty > 0) {
+    auto tiles = axi ? &k_b_corr_tiles<SFX_AXISYM> : &k_b_corr_tiles<SFX_PLANAR2D>;
+    tiles<<<b->nb_tile, kT2Threads, b->tile_smem, sb>>>(b->dI, n, b->pre_tile, b->tile_ty, b->sweeps, P);
+  }
+  for (int q = 0; q < b->sweeps && b->tile_ty == 0; ++q)
     for (int color = (q == 0 ? 1 : 0); color < 2; ++color)
       corr<<<b->nb_pair, bs, 0, sb>>>(b->dI, n, b->pre_pair, P, color, q == 0 ? 1 : 0,
                                       q == b->sweeps - 1 && color == 1 ? 1 : 0);
@@ -464,6 +525,8 @@ sfx_status ensure_graph(sfx_batch* b, const void* phi, const void* ur, const voi
   b->P.uz = (const float*)uz;
   b->P.f = (float2*)f;
   b->P.F = (float2*)F;
+  const sfx_status ts = build_tiles(b);
+  if (ts != SFX_OK) return ts;
   if (!b->cap) SFX_CUDA(cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking));
   cudaGraph_t g = nullptr;
   SFX_CUDA(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
@@ -557,6 +620,7 @@ sfx_status sfx_batch_create_geom(const sfx_batch_instance* inst, int n, int geom
   if (st == SFX_OK) st = balloc(b, &b->pre_rf, (size_t)n + 1);
   if (st == SFX_OK) st = balloc(b, &b->pre_zf, (size_t)n + 1);
   if (st == SFX_OK) st = balloc(b, &b->pre_pair, (size_t)n + 1);
+  if (st == SFX_OK) st = balloc(b, &b->pre_tile, (size_t)n + 1);
   if (st == SFX_OK) st = balloc(b, &P.phi32, nc);
   if (st == SFX_OK) st = balloc(b, &P.fs, nc);
   if (st == SFX_OK) st = balloc(b, &P.Fs, nc);

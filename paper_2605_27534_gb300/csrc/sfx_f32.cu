@@ -34,6 +34,7 @@
 #include "sfx_df.cuh"
 #include "sfx_f32_dev.cuh"
 #include "sfx_internal.h"
+#include "sfx_block2d.cuh"
 #include "sfx_tiled.cuh"
 #include "sfx_advect3.cuh"
 
@@ -474,6 +475,22 @@ k_corr2_32(Nw32 p, const __half2* __restrict__ Hx, const __half2* __restrict__ H
   corr2_load<G>(p, i2, j, k2, H, rc, e2, color, first, b);
   corr2_apply<G>(p, a, e2, fst, Fst, fsrc, Fsrc);
   corr2_apply<G>(p, b, e2, fst, Fst, fsrc, Fsrc);
+}
+
+// All sweeps of an iteration on 2D tiles (sfx_block2d.cuh); the state becomes
+// src + correction.
+template <int G>
+__global__ void __launch_bounds__(kT2Threads)
+k_corr2_tile2d(Nw32 p, int tx, int ty, int sweeps, const __half2* __restrict__ Hx,
+               const __half2* __restrict__ Hy, const float4* __restrict__ rc,
+               const float2* __restrict__ e2, float2* fst, float2* Fst, const float2* fsrc,
+               const float2* Fsrc, const int* __restrict__ done) {
+  if (done && *done) return;
+  corr_tile2d<G>(p, blockIdx.x * tx, blockIdx.y * ty, tx, ty, sweeps, Hx, Hy, rc, e2,
+                 [&](ix c, float2 e) {
+                   fst[c] = df_add(fsrc[c], e.x);
+                   Fst[c] = df_add(Fsrc[c], e.y);
+                 });
 }
 
 // The Newton kernels of one geometry (the branches on the geometry in the
@@ -1530,6 +1547,20 @@ sfx_status solve_newton32(sfx_ctx* c, const Nw32& p, const float* phi, float* co
     const sfx_status ts = tiled_sweep_prepare(c);
     if (ts != SFX_OK) return ts;
   }
+  // 2D grids: all sweeps of an iteration in one launch
+  Tile2D t2;
+  size_t t2smem = 0;
+  decltype(&k_corr2_tile2d<SFX_AXISYM>) tile2d = nullptr;
+  if (L.ndim() == 2 && mgl < 2) {
+    const int ty = tile2d_rows(&L, 1, sweeps, c->sm_count);
+    if (ty > 0) {
+      t2 = tile2d_of(L.nx, ty, sweeps);
+      t2smem = tile2d_smem(L.nx, L.ny, t2, sweeps);
+      tile2d = L.geom == SFX_AXISYM ? &k_corr2_tile2d<SFX_AXISYM> : &k_corr2_tile2d<SFX_PLANAR2D>;
+      SFX_CUDA(cudaFuncSetAttribute(tile2d, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)kT2Smem));
+    }
+  }
   // the incremental residual needs the previous correction kept: on the
   // tiled path the two correction buffers alternate, the residual pass of
   // an iteration writing the first red half-sweep into the buffer that the
@@ -1620,6 +1651,12 @@ sfx_status solve_newton32(sfx_ctx* c, const Nw32& p, const float* phi, float* co
       SFX_KERNEL(c, K_SMOOTH_FINE, (k_corr2_32<SFX_CART3D, 1>), grd1, blk, s, p, c->f32.H2[0],
                  c->f32.H2[1], Hz, c->f32.rc, ebuf[in], 1, 0, fc, Fc, fsrc, Fsrc, flag);
       efin = in;
+    } else if (tile2d) {
+      const dim3 g((unsigned)((L.nx + t2.tx - 1) / t2.tx), (unsigned)((L.ny + t2.ty - 1) / t2.ty));
+      prof_before(c, K_SMOOTH_FINE, s);
+      tile2d<<<g, kT2Threads, t2smem, s>>>(p, t2.tx, t2.ty, sweeps, c->f32.H2[0], c->f32.H2[1],
+                                           c->f32.rc, c->f32.e2, fc, Fc, fsrc, Fsrc, flag);
+      prof_after(c, K_SMOOTH_FINE, s);
     } else {
       for (int q = 0; q < sweeps; ++q)
         for (int color = (q == 0 ? 1 : 0); color < 2; ++color) {

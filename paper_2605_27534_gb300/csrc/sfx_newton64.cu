@@ -28,6 +28,7 @@
 #include <cmath>
 #include <cstring>
 
+#include "sfx_block2d.cuh"
 #include "sfx_f32_dev.cuh"
 #include "sfx_internal.h"
 
@@ -358,6 +359,21 @@ k_corr64(Nw32 p, const __half2* __restrict__ Hx, const __half2* __restrict__ Hy,
   }
 }
 
+// All sweeps of an iteration on 2D tiles (sfx_block2d.cuh).
+template <int G>
+__global__ void __launch_bounds__(kT2Threads)
+k_corr64_tile2d(Nw32 p, int tx, int ty, int sweeps, const __half2* __restrict__ Hx,
+                const __half2* __restrict__ Hy, const float4* __restrict__ rc,
+                const float2* __restrict__ e2, double* fst, double* Fst, const double* fsrc,
+                const double* Fsrc, const int* __restrict__ stop) {
+  if (*stop) return;
+  corr_tile2d<G>(p, blockIdx.x * tx, blockIdx.y * ty, tx, ty, sweeps, Hx, Hy, rc, e2,
+                 [&](ix c, float2 e) {
+                   fst[c] = fsrc[c] + widen(e.x);
+                   Fst[c] = Fsrc[c] + widen(e.y);
+                 });
+}
+
 // Launch shape of the residual: x chunks of up to 256 threads, and rows in
 // turn, eight blocks per SM.
 struct Rows {
@@ -423,6 +439,14 @@ sfx_status solve(sfx_ctx* c, const Newton64& q, double* f, double* F, bool from_
   const Rows rg = rows_of(L, c->sm_count);
   const dim3 blk(128), grd((unsigned)(((L.nx + 1) / 2 + 127) / 128), (unsigned)L.ny, (unsigned)L.nz);
   const int cap = std::min(o->max_cycles, kMaxNewton);
+  Tile2D t2;
+  size_t t2smem = 0;
+  if (G != SFX_CART3D && (t2.ty = tile2d_rows(&L, 1, sweeps, c->sm_count)) > 0) {
+    t2 = tile2d_of(L.nx, t2.ty, sweeps);
+    t2smem = tile2d_smem(L.nx, L.ny, t2, sweeps);
+    SFX_CUDA(cudaFuncSetAttribute(k_corr64_tile2d<G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)kT2Smem));
+  }
   *conv = false;
   SFX_CUDA(cudaMemsetAsync(ctl, 0, sizeof(Ctl64), s));
   float first = 0.0f;
@@ -434,7 +458,14 @@ sfx_status solve(sfx_ctx* c, const Newton64& q, double* f, double* F, bool from_
       SFX_KERNEL(c, K_RESIDUAL, k_resid64<G>, rg.grid, rg.block, s, q, fa, Fa, tol, ctl,
                  S.report + 8 * (it & 1));
       SFX_CUDA(cudaEventRecord(S.ev[it & 1], s));
-      for (int w = 0; w < sweeps; ++w)
+      if (t2.ty > 0) {
+        const dim3 g((unsigned)((L.nx + t2.tx - 1) / t2.tx), (unsigned)((L.ny + t2.ty - 1) / t2.ty));
+        prof_before(c, K_SMOOTH_FINE, s);
+        k_corr64_tile2d<G><<<g, kT2Threads, t2smem, s>>>(q.p, t2.tx, t2.ty, sweeps, q.H[0], q.H[1],
+                                                         q.rc, q.e2, f, F, fa, Fa, &ctl->stop);
+        prof_after(c, K_SMOOTH_FINE, s);
+      }
+      for (int w = 0; w < sweeps && t2.ty == 0; ++w)
         for (int color = w == 0 ? 1 : 0; color < 2; ++color) {
           const bool add = w == sweeps - 1 && color == 1;
           SFX_KERNEL(c, K_SMOOTH_FINE, k_corr64<G>, grd, blk, s, q.p, q.H[0], q.H[1], q.H[2], q.rc,
