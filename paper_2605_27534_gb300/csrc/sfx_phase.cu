@@ -30,41 +30,23 @@ template <typename T> __device__ __forceinline__ T tiny_pos();
 template <> __device__ __forceinline__ double tiny_pos<double>() { return 1e-300; }
 template <> __device__ __forceinline__ float tiny_pos<float>() { return 1e-30f; }
 
-// One Jacobi update of chi at a cell from its own chi0 (s0) and iterate
-// (x0) and those of its neighbours along each direction (the cell itself at
-// a wall): Godunov upwind |grad chi| away from the interface, the
-// Russo-Smereka sub-cell fix in cells where chi0 changes sign.
+// Whether chi0 (s0 here, zm and zp its neighbours', the cell's own past a wall)
+// changes sign against a face neighbour, and then the sub-cell distance
+// h chi0/|Delta chi0|.
 template <typename T>
-__device__ __forceinline__ T redist_update(int nd, T s0, T x0, const T* z0m, const T* z0p,
-                                           const T* xm, const T* xp, const bool* hasm,
-                                           const bool* hasp, T h, T invh, T dtau, T dtau_h) {
-  const T sg = s0 > (T)0 ? (T)1 : (s0 < (T)0 ? (T)-1 : (T)0);
+__device__ __forceinline__ bool redist_cut(int nd, T s0, const T* zm, const T* zp, const bool* hasm,
+                                           const bool* hasp, T h, T& dist) {
   bool cut = false;
-  T gsum = 0, dsum = 0;
+  T dsum = 0;
   for (int d = 0; d < nd; ++d) {
-    if ((hasm[d] && s0 * z0m[d] < (T)0) || (hasp[d] && s0 * z0p[d] < (T)0)) cut = true;
-    // sub-cell estimate of |grad chi0| h along d
-    T q = fabs(z0p[d] - z0m[d]) * (T)0.5;
-    q = fmax(q, fabs(z0p[d] - s0));
-    q = fmax(q, fabs(s0 - z0m[d]));
+    if ((hasm[d] && s0 * zm[d] < (T)0) || (hasp[d] && s0 * zp[d] < (T)0)) cut = true;
+    T q = fabs(zp[d] - zm[d]) * (T)0.5;
+    q = fmax(q, fabs(zp[d] - s0));
+    q = fmax(q, fabs(s0 - zm[d]));
     dsum += q * q;
-    // Godunov upwind gradient of the current iterate
-    const T bwd = (x0 - xm[d]) * invh, fwd = (xp[d] - x0) * invh;
-    T t;
-    if (sg > (T)0) {
-      const T ap = fmax(bwd, (T)0), bm = fmin(fwd, (T)0);
-      t = fmax(ap * ap, bm * bm);
-    } else {
-      const T am = fmin(bwd, (T)0), bp = fmax(fwd, (T)0);
-      t = fmax(am * am, bp * bp);
-    }
-    gsum += t;
   }
-  if (cut) {
-    const T dchi = fmax(sqrt(dsum), (T)tiny_pos<T>());
-    return x0 - dtau_h * (sg * fabs(x0) - h * s0 / dchi);
-  }
-  return x0 - dtau * sg * (sqrt(gsum) - (T)1);
+  if (cut) dist = h * s0 / fmax(sqrt(dsum), (T)tiny_pos<T>());
+  return cut;
 }
 
 // ------------------------------------------------- redistancing by blocks
@@ -336,87 +318,119 @@ __global__ void __launch_bounds__(512) k_rd_finish(Level L, RdGrid R, T dtau, in
 // (kRdX + 2 kRdK) x (kRdY + 2 kRdK) window of chi0 and the iterate into
 // shared memory and updates a window that shrinks by one cell per step, so
 // that after `steps` steps its kRdX x kRdY core holds exactly the values of
-// `steps` single-step launches (the same update of the same operands).
+// `steps` single-step launches (the same update of the same operands).  A
+// thread keeps its column of the window (80 columns of 12 rows in turn) and
+// what does not change with the steps: the sign of chi0, or where chi0
+// changes sign the sub-cell distance.  One block per SM at 512^2, so the
+// steps are bound by the latency of few warps: 960 threads instead of 256,
+// 38 -> 16 us per launch at 512^2 (three launches).  `first`: chi0 and the iterate are formed from
+// C here.
 constexpr int kRdX = 64, kRdY = 32, kRdK = 8;
 constexpr int kRdWX = kRdX + 2 * kRdK, kRdWY = kRdY + 2 * kRdK;
+constexpr int kRdRows = 12, kRdPer = kRdWY / kRdRows;
+static_assert(kRdWY % kRdRows == 0, "rows per thread");
 
-__global__ void __launch_bounds__(256)
-    k_redistance_fused2d(Level L, float dtau, const float* __restrict__ chi0,
-                         const float* __restrict__ cin, float* __restrict__ cout, int steps) {
+__global__ void __launch_bounds__(kRdWX* kRdRows)
+    k_redistance_fused2d(Level L, float dtau, const double* __restrict__ C, bool first,
+                         float* __restrict__ chi0, const float* __restrict__ cin,
+                         float* __restrict__ cout, double* __restrict__ chi, int steps) {
   __shared__ float sz[kRdWY][kRdWX];
   __shared__ float sx[2][kRdWY][kRdWX];
   const float h = (float)L.h, invh = (float)(1.0 / L.h), dtau_h = dtau / h;
-  const int gx0 = blockIdx.x * kRdX - kRdK, gy0 = blockIdx.y * kRdY - kRdK;
-  for (int q = threadIdx.x; q < kRdWX * kRdWY; q += blockDim.x) {
-    const int lx = q % kRdWX, ly = q / kRdWX;
-    const int gx = gx0 + lx, gy = gy0 + ly;
+  const int lx = threadIdx.x % kRdWX, ty = threadIdx.x / kRdWX;
+  const int gx = blockIdx.x * kRdX - kRdK + lx, gy0 = blockIdx.y * kRdY - kRdK;
+  const bool inx = gx >= 0 && gx < L.nx;
+#pragma unroll
+  for (int q = 0; q < kRdPer; ++q) {
+    const int ly = ty + q * kRdRows, gy = gy0 + ly;
     float z = 0.0f, x = 0.0f;
-    if (gx >= 0 && gx < L.nx && gy >= 0 && gy < L.ny) {
-      const unsigned c = (unsigned)gy * (unsigned)L.nx + (unsigned)gx;
-      z = chi0[c];
-      x = cin[c];
+    if (inx && gy >= 0 && gy < L.ny) {
+      const size_t c = (size_t)gy * L.nx + gx;
+      if (first) {
+        z = x = (float)(2.0 * L.h * (C[c] - 0.5));
+        // the core's values of chi0, for the launches after this one
+        if (lx >= kRdK && lx < kRdK + kRdX && ly >= kRdK && ly < kRdK + kRdY) chi0[c] = z;
+      } else {
+        z = chi0[c];
+        x = cin[c];
+      }
     }
     sz[ly][lx] = z;
     sx[0][ly][lx] = x;
   }
   __syncthreads();
+  const bool hm = gx > 0, hp = gx + 1 < L.nx;
+  float s[kRdPer], dist[kRdPer];     // sign of chi0; the sub-cell distance where it is cut
+  unsigned cut = 0;
+#pragma unroll
+  for (int q = 0; q < kRdPer; ++q) {
+    const int ly = ty + q * kRdRows, gy = gy0 + ly;
+    s[q] = dist[q] = 0.0f;
+    if (!inx || gy < 0 || gy >= L.ny || lx < 1 || lx >= kRdWX - 1 || ly < 1 || ly >= kRdWY - 1) continue;
+    const float s0 = sz[ly][lx];
+    const bool hasm[2] = {hm, gy > 0}, hasp[2] = {hp, gy + 1 < L.ny};
+    const float zm[2] = {hm ? sz[ly][lx - 1] : s0, gy > 0 ? sz[ly - 1][lx] : s0};
+    const float zp[2] = {hp ? sz[ly][lx + 1] : s0, gy + 1 < L.ny ? sz[ly + 1][lx] : s0};
+    s[q] = s0 > 0.0f ? 1.0f : (s0 < 0.0f ? -1.0f : 0.0f);
+    if (redist_cut<float>(2, s0, zm, zp, hasm, hasp, h, dist[q])) cut |= 1u << q;
+  }
   int cur = 0;
   for (int st = 0; st < steps; ++st) {
     // cells at least st + 1 away from the window edge can be updated
-    const int lo = st + 1, nxw = kRdWX - 2 * lo, nyw = kRdWY - 2 * lo;
-    for (int q = threadIdx.x; q < nxw * nyw; q += blockDim.x) {
-      const int lx = lo + q % nxw, ly = lo + q / nxw;
-      const int gx = gx0 + lx, gy = gy0 + ly;
-      if (gx < 0 || gx >= L.nx || gy < 0 || gy >= L.ny) continue;
-      bool hasm[2] = {gx > 0, gy > 0}, hasp[2] = {gx + 1 < L.nx, gy + 1 < L.ny};
-      const float s0 = sz[ly][lx], x0 = sx[cur][ly][lx];
-      float z0m[2], z0p[2], xm[2], xp[2];
-      z0m[0] = hasm[0] ? sz[ly][lx - 1] : s0;
-      z0p[0] = hasp[0] ? sz[ly][lx + 1] : s0;
-      z0m[1] = hasm[1] ? sz[ly - 1][lx] : s0;
-      z0p[1] = hasp[1] ? sz[ly + 1][lx] : s0;
-      xm[0] = hasm[0] ? sx[cur][ly][lx - 1] : x0;
-      xp[0] = hasp[0] ? sx[cur][ly][lx + 1] : x0;
-      xm[1] = hasm[1] ? sx[cur][ly - 1][lx] : x0;
-      xp[1] = hasp[1] ? sx[cur][ly + 1][lx] : x0;
-      sx[cur ^ 1][ly][lx] = redist_update<float>(2, s0, x0, z0m, z0p, xm, xp, hasm, hasp, h, invh,
-                                                 dtau, dtau_h);
+    const int lo = st + 1;
+    if (inx && lx >= lo && lx < kRdWX - lo) {
+#pragma unroll
+      for (int q = 0; q < kRdPer; ++q) {
+        const int ly = ty + q * kRdRows, gy = gy0 + ly;
+        if (ly < lo || ly >= kRdWY - lo || gy < 0 || gy >= L.ny) continue;
+        const float x0 = sx[cur][ly][lx];
+        float v;
+        if (cut >> q & 1) {
+          v = x0 - dtau_h * (s[q] * fabsf(x0) - dist[q]);
+        } else {
+          const float xm[2] = {hm ? sx[cur][ly][lx - 1] : x0, gy > 0 ? sx[cur][ly - 1][lx] : x0};
+          const float xp[2] = {hp ? sx[cur][ly][lx + 1] : x0,
+                               gy + 1 < L.ny ? sx[cur][ly + 1][lx] : x0};
+          v = s[q] == 0.0f ? x0 : rd_step<2>(s[q], x0, xm, xp, invh, dtau);
+        }
+        sx[cur ^ 1][ly][lx] = v;
+      }
     }
     __syncthreads();
     cur ^= 1;
   }
-  for (int q = threadIdx.x; q < kRdX * kRdY; q += blockDim.x) {
-    const int lx = kRdK + q % kRdX, ly = kRdK + q / kRdX;
-    const int gx = gx0 + lx, gy = gy0 + ly;
-    if (gx < L.nx && gy < L.ny) cout[(unsigned)gy * (unsigned)L.nx + (unsigned)gx] = sx[cur][ly][lx];
+  if (lx < kRdK || lx >= kRdK + kRdX || !inx) return;
+#pragma unroll
+  for (int q = 0; q < kRdPer; ++q) {
+    const int ly = ty + q * kRdRows, gy = gy0 + ly;
+    if (ly < kRdK || ly >= kRdK + kRdY || gy < 0 || gy >= L.ny) continue;
+    const size_t c = (size_t)gy * L.nx + gx;
+    if (chi) chi[c] = (double)sx[cur][ly][lx];      // the last launch
+    else cout[c] = sx[cur][ly][lx];
   }
 }
 
-// SFX_F32 contexts iterate the redistancing in FP32 (their solution depends
-// on phi only to ~1e-8 through it): chi0 and the float iterate.
-__global__ void k_chi0_32(size_t n, double h, const double* __restrict__ C,
-                          float* __restrict__ chi0, float* __restrict__ chi) {
-  for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
-       c += (size_t)gridDim.x * blockDim.x) {
-    const float v = (float)(2.0 * h * (C[c] - 0.5));
-    chi0[c] = v;
-    chi[c] = v;
-  }
-}
-
-__global__ void k_widen(size_t n, const float* __restrict__ x, double* __restrict__ y) {
-  for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
-       c += (size_t)gridDim.x * blockDim.x)
-    y[c] = (double)x[c];
-}
-
-__global__ void k_phi_delta64(size_t n, double eps, const double* __restrict__ chi,
-                              double* __restrict__ phi, double* __restrict__ delta) {
-  for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
-       c += (size_t)gridDim.x * blockDim.x) {
-    const double p = phi_of(chi[c], eps);
-    phi[c] = p;
-    if (delta) delta[c] = p * (1.0 - p) / eps;
+// phi and delta from chi.  Far from the interface chi holds one value over
+// whole blocks, so a block's first cell is evaluated once and its value
+// shared: only the band pays an FP64 tanh per cell.
+__global__ void __launch_bounds__(256)
+k_phi_delta64(size_t n, double eps, const double* __restrict__ chi, double* __restrict__ phi,
+              double* __restrict__ delta) {
+  __shared__ double sx, sp;
+  for (size_t b = blockIdx.x * (size_t)blockDim.x; b < n; b += (size_t)gridDim.x * blockDim.x) {
+    const size_t c = b + threadIdx.x;
+    const double x = c < n ? chi[c] : 0.0;
+    if (threadIdx.x == 0) {
+      sx = x;
+      sp = phi_of(x, eps);
+    }
+    __syncthreads();
+    if (c < n) {
+      const double p = same_bits(x, sx) ? sp : phi_of(x, eps);
+      phi[c] = p;
+      if (delta) delta[c] = p * (1.0 - p) / eps;
+    }
+    __syncthreads();
   }
 }
 
@@ -484,15 +498,21 @@ sfx_status phase_field_build(sfx_ctx* c, const double* C, double* chi, void* phi
     float* b = c->chi32 + 2 * n;
     if (L.ndim() == 3)
       return redistance_blocks<float, 3>(c, C, z0, a, b, chi, ph, de, iters, dtau, eps, s);
-    SFX_KERNEL(c, K_PHASE, k_chi0_32, nb, 256, s, n, L.h, C, z0, a);
-    // kRdK steps per launch
+    // kRdK steps per launch; the first forms chi0, the last writes chi (with
+    // no step at all, chi0 itself; in place of C only after every block has
+    // read it)
     const dim3 fg((unsigned)((L.nx + kRdX - 1) / kRdX), (unsigned)((L.ny + kRdY - 1) / kRdY));
-    for (int it = 0; it < iters; it += kRdK) {
-      const int steps = std::min(kRdK, iters - it);
-      SFX_KERNEL(c, K_PHASE, k_redistance_fused2d, fg, 256, s, L, (float)dtau, z0, a, b, steps);
+    int it = 0;
+    bool first = true, last_in_scratch = false;
+    do {
+      const int steps = first && chi == C ? 0 : std::min(kRdK, iters - it);
+      it += steps;
+      SFX_KERNEL(c, K_PHASE, k_redistance_fused2d, fg, kRdWX * kRdRows, s, L, (float)dtau, C, first,
+                 z0, a, b, it == iters && !(first && chi == C) ? chi : nullptr, steps);
+      last_in_scratch = it == iters && first && chi == C;
+      first = false;
       std::swap(a, b);
-    }
-    SFX_KERNEL(c, K_PHASE, k_widen, nb, 256, s, n, a, chi);
+    } while (it < iters || last_in_scratch);
     SFX_KERNEL(c, K_PHASE, k_phi_delta64, nb, 256, s, n, eps, chi, ph, de);
     SFX_LAUNCH_CHECK();
     return SFX_OK;

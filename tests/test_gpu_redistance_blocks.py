@@ -66,9 +66,12 @@ def test_redistance_blocks_against_the_oracle(sfx, geom, shape, kind):
         same = Cd.clone()               # chi in place of C
         ctx.sfx_phase_field_build(same, same, phi, None, iters=iters, dtau=dtau, eps=eps)
         assert np.array_equal(host(same), host(chi))
-    if geom == W.CART3D:                # the float iterate
-        ctx = sfx.Context.for_grid(g, sfx.SFX_F32)
-        ctx.sfx_set_tuning(sfx._lib.SFX_TUNE_F32_REDIST, 1)
-        chi_o, phi_o, _ = oracle.phase_field_build(g, C, 24, dtau, eps)
-        ctx.sfx_phase_field_build(Cd, chi, phi, None, iters=24, dtau=dtau, eps=eps)
+    ctx = sfx.Context.for_grid(g, sfx.SFX_F32)     # the float iterate
+    ctx.sfx_set_tuning(sfx._lib.SFX_TUNE_F32_REDIST, 1)
+    for iters in (0, 3, 24):
+        chi_o, phi_o, _ = oracle.phase_field_build(g, C, iters, dtau, eps)
+        ctx.sfx_phase_field_build(Cd, chi, phi, None, iters=iters, dtau=dtau, eps=eps)
         assert rel_err(host(chi), chi_o) < 1e-5
+        same = Cd.clone()
+        ctx.sfx_phase_field_build(same, same, phi, None, iters=iters, dtau=dtau, eps=eps)
+        assert np.array_equal(host(same), host(chi))
