@@ -157,7 +157,9 @@ void sfx_ctx_destroy(sfx_ctx* c) {
   if (c->adj.h_out) cudaFreeHost(c->adj.h_out);
   if (c->adj.h_nrm) cudaFreeHost(c->adj.h_nrm);
   if (c->adj.relax) cudaGraphExecDestroy(c->adj.relax);
+  if (c->adj.h_ctl) cudaFreeHost(c->adj.h_ctl);
   if (c->adj.cap) cudaStreamDestroy(c->adj.cap);
+  if (c->adj.cap_body) cudaStreamDestroy(c->adj.cap_body);
   delete c;
 }
 

@@ -150,8 +150,8 @@ struct AdjScratch {
   double* nf = nullptr;           // adjoint unknowns nu_f, nu_F
   double* nF = nullptr;
   double* sig = nullptr;          // sigma of the loss
+  double* dm = nullptr;           // delta_m per cell (2D solve: lam_F, and lam_f in sig)
   double* force = nullptr;        // ndim x N
-  double* dm = nullptr;           // delta_m per cell
   double* G = nullptr;            // dL/d(grad sigma), ndim x N
   double* part = nullptr;         // block partial sums, 5 quantities
   int nblk = 0;
@@ -159,13 +159,17 @@ struct AdjScratch {
   double* h_out = nullptr;
   unsigned long long* d_nrm = nullptr;   // 2 max-norm slots and mirror
   unsigned long long* h_nrm = nullptr;
+  double* U = nullptr;            // 2D: 12 x N table of the solve (shares force, G)
   float4* K = nullptr;            // FP32 relaxation: inverse 2x2 block per cell
-  float* W = nullptr;             // 12 x N neighbour weights (6 per field)
+  float* W = nullptr;             // neighbour weights, 2 ndim x N per field (3D: 6 per field)
   float2* r = nullptr;            // FP64 residual rounded to float
-  float2* e = nullptr;            // correction (e_f, e_F)
-  // the relaxation of one defect-correction check (e = 0, the colour
-  // sweeps, nu += e) as a CUDA graph: one launch instead of 2 S + 2
-  cudaStream_t cap = nullptr;     // private stream the graph is captured on
+  float2* e = nullptr;            // correction (e_f, e_F); 2D: two of them
+  void* ctl = nullptr;            // 2D: state of the solve (device) and mirror
+  void* h_ctl = nullptr;
+  // 3D: the relaxation of one defect-correction check (e = 0, the colour
+  // sweeps, nu += e) as a CUDA graph; 2D: the whole solve
+  cudaStream_t cap = nullptr;     // private streams the graph is captured on
+  cudaStream_t cap_body = nullptr;
   cudaGraphExec_t relax = nullptr;
   int relax_sweeps = 0;           // S of the captured graph
 };
