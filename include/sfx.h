@@ -604,9 +604,10 @@ sfx_status sfx_profile_read(sfx_ctx* ctx, int kind, long long* launches,
    did work, where the library can tell: the residual passes of the FP32
    Newton solve (SFX_K_RESIDUAL, SFX_K_RESID_FAST, SFX_K_RESID_INCR), of
    which each iteration launches every kind and all but one return at once,
-   counted from the residual
-   kind recorded with the iteration's norms (iterations whose norms the
-   solve read); -1 for the other kinds.  SFX_ERR_ARG on a bad kind. */
+   counted from the residual kind recorded with the iteration's norms
+   (iterations whose norms the solve read; a 2D solve whose residual is one
+   launch of either kind counts it as SFX_K_RESIDUAL); -1 for the other
+   kinds.  SFX_ERR_ARG on a bad kind. */
 sfx_status sfx_profile_work(sfx_ctx* ctx, int kind, long long* working);
 
 #ifdef __cplusplus

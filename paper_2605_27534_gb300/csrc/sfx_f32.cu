@@ -1433,6 +1433,64 @@ __global__ void k_flag32(unsigned int* __restrict__ nrm, const unsigned int* __r
   }
 }
 
+// The residual pass of an iteration on a 2D grid whose sweeps are one launch:
+// of the kind chosen on the device, with the test of k_flag32 and the host's
+// report in the last block.  flag: see k_flag32; [8..11] the norms, [12] the
+// finished blocks, all zero at the start of a solve and after each pass.
+// rho > 0 tries a predicted start as k_pred_check32 does: a rejected one is
+// not tested or reported, and the pass that follows the restart runs only
+// where flag[2] says so (`retry`).  At 128^2 .. 512^2 an iteration was seven
+// calls (two memory operations, both residual kinds, the test, the copy of the
+// norms, the sweeps), some 20 us of host time around 12-18 us of work; now it
+// is three.  24 steps of 256^2 within an 8-step gradient: 10.5 -> 7.8 ms; a
+// moving step of 512^2: 481 -> 391 us.
+template <int G>
+__global__ void __launch_bounds__(256, 4)
+k_resid2d_32(Nw32 p, const float* __restrict__ phi, const float2* __restrict__ B2x,
+             const float2* __restrict__ B2y, const float2* __restrict__ fin,
+             const float2* __restrict__ Fin, const float2* __restrict__ fst,
+             const float2* __restrict__ Fst, float4* __restrict__ rc, float2* __restrict__ e2,
+             float tol, float rho, int retry, int fast_max, int* flag, unsigned int* report) {
+  if (flag[0] || (retry && flag[2])) return;
+  const int kind = fast_max <= 0 ? 1 : flag[4];
+  const Level& L = p.L;
+  float m[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  const float2* B2[3] = {B2x, B2y, nullptr};
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < L.nx)
+    for (ix j = blockIdx.y; j < (ix)L.ny; j += gridDim.y) {
+      const ix c = j * (ix)L.nx + (ix)i;
+      if (kind == 0) resid32_cell<G>(p, i, (int)j, 0, c, phi, B2, fin, Fin, fst, Fst, rc, m, e2);
+      else resid2_cell<G>(p, i, (int)j, 0, c, phi, B2, fin, Fin, fst, Fst, rc, m, e2);
+    }
+  unsigned int* nrm = (unsigned int*)flag + 8;
+  resid_norms(m, nrm);
+  if (threadIdx.x < 4) __threadfence();
+  __syncthreads();
+  if (threadIdx.x) return;
+  const int blocks = (int)(gridDim.x * gridDim.y);
+  if (atomicAdd(flag + 12, 1) != blocks - 1) return;
+  __threadfence();
+  float v[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    v[q] = __uint_as_float(atomicExch(nrm + q, 0u));
+    report[q] = __float_as_uint(v[q]);
+  }
+  report[4] = (unsigned int)kind;
+  flag[12] = 0;
+  if (rho > 0.0f) {
+    const bool good = v[0] <= rho * v[1] && v[2] <= rho * v[3];   // false for NaN
+    flag[2] = good ? 1 : 0;
+    if (!good) return;
+  }
+  if (kind == 1) {
+    if (v[0] <= tol * v[1] && v[2] <= tol * v[3]) flag[0] = 1;
+  } else if (++flag[5] >= fast_max || (v[0] <= kFastSwitch * v[1] && v[2] <= kFastSwitch * v[3])) {
+    flag[4] = 1;
+  }
+}
+
 __global__ void k_set32(int* __restrict__ p, int v) {
   if (threadIdx.x == 0) *p = v;
 }
@@ -1464,18 +1522,6 @@ __global__ void k_restore32(size_t n, const int* __restrict__ ok, const float2* 
 
 // Initial guess of the Newton iteration: x* plus the implicit increment of
 // the previous step (a smooth solution changes little from step to step).
-// (f, F) <- (f*, F*) when the Newton solve converged at its first check
-// (flag[1] = 1): its state updates then never ran.
-__global__ void k_copy_if_first32(size_t n, const int* __restrict__ flag,
-                                  const float2* __restrict__ fs, const float2* __restrict__ Fs,
-                                  float2* __restrict__ f, float2* __restrict__ F) {
-  if (!(flag[0] && flag[1] == 1)) return;
-  for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
-       c += (size_t)gridDim.x * blockDim.x) {
-    f[c] = fs[c];
-    F[c] = Fs[c];
-  }
-}
 __global__ void k_predict32(size_t n, const float2* __restrict__ fs, const float2* __restrict__ Fs,
                             const float* __restrict__ df, const float* __restrict__ dF,
                             float2* __restrict__ f, float2* __restrict__ F) {
@@ -1575,8 +1621,10 @@ sfx_status solve_newton32(sfx_ctx* c, const Nw32& p, const float* phi, float* co
   int efin = 1;   // buffer of the last correction added to the state
   // flag[4] = 1: pair residuals from the first iteration (no FP32 passes)
   const int fast_max = c->f32.fast_resid;
-  SFX_CUDA(cudaMemsetAsync(flag, 0, 8 * sizeof(int), s));
-  if (fast_max <= 0) SFX_KERNEL(c, K_OTHER, k_set32, 1, 32, s, flag + 4, 1);
+  const bool merged = tile2d != nullptr;   // the 2D iteration of three calls
+  const auto resid2d = L.geom == SFX_AXISYM ? &k_resid2d_32<SFX_AXISYM> : &k_resid2d_32<SFX_PLANAR2D>;
+  SFX_CUDA(cudaMemsetAsync(flag, 0, 16 * sizeof(int), s));
+  if (fast_max <= 0 && !merged) SFX_KERNEL(c, K_OTHER, k_set32, 1, 32, s, flag + 4, 1);
   // Each iteration: the residual pass (which also does the first red
   // half-sweep of the correction, from zero), a device-side convergence
   // test, then the rest of the red-black sweeps, the last black one adding
@@ -1589,7 +1637,7 @@ sfx_status solve_newton32(sfx_ctx* c, const Nw32& p, const float* phi, float* co
   int it = 0, done_it = 0;
   for (it = 1; it <= o->max_cycles; ++it) {
     unsigned int* nbuf = dn + 8 * (it & 1);
-    SFX_CUDA(cudaMemsetAsync(nbuf, 0, 8 * sizeof(unsigned int), s));
+    if (!merged) SFX_CUDA(cudaMemsetAsync(nbuf, 0, 8 * sizeof(unsigned int), s));
     // from_star: the first iterate is x* itself, read from (f*, F*); the
     // first state update writes x* + e into (f, F), so no copy precedes it
     const bool star = from_star && it == 1;
@@ -1598,27 +1646,37 @@ sfx_status solve_newton32(sfx_ctx* c, const Nw32& p, const float* phi, float* co
     // the FP32 or the pair residual pass, as chosen on the device
     const int etgt = tiled ? 1 - efin : 0;
     float2* e2t = ebuf[etgt];
-    SFX_KERNEL(c, K_RESID_FAST, nk.fast, rg.grid, rg.block, s, p, phi, B2[0], B2[1], B2[2], fsrc,
-               Fsrc, fs, Fs, c->f32.rc, nbuf, e2t, flag, flag + 4);
-    pair_pass(fsrc, Fsrc, nbuf, e2t, flag);
-    if (incr_ok && it > 1)
-      SFX_KERNEL(c, K_RESID_INCR, nk.incr, rg.grid, rg.block, s, p, phi, B2[0], B2[1], B2[2],
-                 ebuf[efin], c->f32.rc, nbuf, e2t, flag, flag + 4);
-    if (it == 1 && predicted) {
-      // keep the predicted start only if its residual is already small;
-      // otherwise restart from x* (both launches return at once when kept)
-      int* ok = flag + 2;
-      const float rho = c->f32.predict_rho;
-      SFX_KERNEL(c, K_OTHER, k_pred_check32, 1, 32, s, nbuf, rho, ok);
-      SFX_KERNEL(c, K_SETUP, k_restore32, nb, 256, s, n, ok, fs, Fs, fc, Fc);
-      SFX_KERNEL(c, K_RESID_FAST, nk.fast, rg.grid, rg.block, s, p, phi, B2[0], B2[1], B2[2],
-                 fc, Fc, fs, Fs, c->f32.rc, nbuf, e2t, ok, flag + 4);
-      pair_pass(fc, Fc, nbuf, e2t, ok);
+    if (merged) {
+      const bool tried = predicted && it == 1;
+      for (int retry = 0; retry <= (tried ? 1 : 0); ++retry) {
+        if (retry) SFX_KERNEL(c, K_SETUP, k_restore32, nb, 256, s, n, flag + 2, fs, Fs, fc, Fc);
+        SFX_KERNEL(c, K_RESIDUAL, resid2d, rg.grid, rg.block, s, p, phi, B2[0], B2[1], fsrc, Fsrc,
+                   fs, Fs, c->f32.rc, e2t, tolf, tried && !retry ? c->f32.predict_rho : 0.0f, retry,
+                   fast_max, flag, hn + 8 * (it & 1));
+      }
+    } else {
+      SFX_KERNEL(c, K_RESID_FAST, nk.fast, rg.grid, rg.block, s, p, phi, B2[0], B2[1], B2[2], fsrc,
+                 Fsrc, fs, Fs, c->f32.rc, nbuf, e2t, flag, flag + 4);
+      pair_pass(fsrc, Fsrc, nbuf, e2t, flag);
+      if (incr_ok && it > 1)
+        SFX_KERNEL(c, K_RESID_INCR, nk.incr, rg.grid, rg.block, s, p, phi, B2[0], B2[1], B2[2],
+                   ebuf[efin], c->f32.rc, nbuf, e2t, flag, flag + 4);
+      if (it == 1 && predicted) {
+        // keep the predicted start only if its residual is already small;
+        // otherwise restart from x* (both launches return at once when kept)
+        int* ok = flag + 2;
+        const float rho = c->f32.predict_rho;
+        SFX_KERNEL(c, K_OTHER, k_pred_check32, 1, 32, s, nbuf, rho, ok);
+        SFX_KERNEL(c, K_SETUP, k_restore32, nb, 256, s, n, ok, fs, Fs, fc, Fc);
+        SFX_KERNEL(c, K_RESID_FAST, nk.fast, rg.grid, rg.block, s, p, phi, B2[0], B2[1], B2[2],
+                   fc, Fc, fs, Fs, c->f32.rc, nbuf, e2t, ok, flag + 4);
+        pair_pass(fc, Fc, nbuf, e2t, ok);
+      }
+      SFX_KERNEL(c, K_OTHER, k_flag32, 1, 32, s, nbuf, dn + 8 * ((it - 1) & 1), tolf, it, fast_max,
+                 incr_ok, flag);
+      SFX_CUDA(cudaMemcpyAsync(hn + 8 * (it & 1), nbuf, 8 * sizeof(unsigned int),
+                               cudaMemcpyDeviceToHost, s));
     }
-    SFX_KERNEL(c, K_OTHER, k_flag32, 1, 32, s, nbuf, dn + 8 * ((it - 1) & 1), tolf, it, fast_max,
-               incr_ok, flag);
-    SFX_CUDA(cudaMemcpyAsync(hn + 8 * (it & 1), nbuf, 8 * sizeof(unsigned int),
-                             cudaMemcpyDeviceToHost, s));
     SFX_CUDA(cudaEventRecord(c->f32.ev[it & 1], s));
     if (mgl >= 2) {
       // a V-cycle on the correction: finish the first sweep, pre - 1 more
@@ -1672,7 +1730,7 @@ sfx_status solve_newton32(sfx_ctx* c, const Nw32& p, const float* phi, float* co
       SFX_CUDA(cudaEventSynchronize(c->f32.ev[prev & 1]));
       const unsigned int* hb = hn + 8 * (prev & 1);
       if (hb[1] == kTimeoutBits) return SFX_ERR_TIMEOUT;
-      ++c->prof.work[hb[4] <= 2u ? hb[4] : 0];   // the residual kind of iteration prev
+      ++c->prof.work[merged ? 1 : hb[4] <= 2u ? hb[4] : 0];   // the residual kind of iteration prev
       memcpy(nrm, hb, 4 * sizeof(float));
       for (int q = 0; q < 4; ++q)
         if (!std::isfinite(nrm[q])) return SFX_ERR_NONFINITE;
@@ -1683,18 +1741,13 @@ sfx_status solve_newton32(sfx_ctx* c, const Nw32& p, const float* phi, float* co
       }
     }
   }
-  if (from_star) {
-    // converged at the first check: x* was the answer and was never copied
-    SFX_KERNEL(c, K_SETUP, k_copy_if_first32, nb, 256, s, n, flag, fs, Fs, fc, Fc);
-    SFX_LAUNCH_CHECK();
-  }
   if (!*conv) {
     // the last iteration's residuals
     SFX_CUDA(cudaStreamSynchronize(s));
     const int last = std::min(it, o->max_cycles);
     const unsigned int* hb = hn + 8 * (last & 1);
     if (hb[1] == kTimeoutBits) return SFX_ERR_TIMEOUT;
-    ++c->prof.work[hb[4] <= 2u ? hb[4] : 0];   // the residual kind of the last iteration
+    ++c->prof.work[merged ? 1 : hb[4] <= 2u ? hb[4] : 0];   // the residual kind of the last iteration
     if (tiled) {
       int err = 0;
       SFX_CUDA(cudaMemcpy(&err, flag + 3, sizeof(int), cudaMemcpyDeviceToHost));
@@ -1705,6 +1758,11 @@ sfx_status solve_newton32(sfx_ctx* c, const Nw32& p, const float* phi, float* co
       if (!std::isfinite(nrm[q])) return SFX_ERR_NONFINITE;
     if (hb[4] >= 1u && nrm[0] <= tolf * nrm[1] && nrm[2] <= tolf * nrm[3]) *conv = true;
     done_it = last;
+  }
+  if (from_star && *conv && done_it == 1) {
+    // converged at the first check: x* was the answer and was never copied
+    SFX_CUDA(cudaMemcpyAsync(fc, fs, n * sizeof(float2), cudaMemcpyDeviceToDevice, s));
+    SFX_CUDA(cudaMemcpyAsync(Fc, Fs, n * sizeof(float2), cudaMemcpyDeviceToDevice, s));
   }
   *iters = done_it;
   return SFX_OK;
@@ -2027,7 +2085,7 @@ sfx_status f32_ensure_scratch(sfx_ctx* c) {
   if ((st = get(n * sizeof(float), (void**)&c->f32.phi32)) != SFX_OK) return st;
   if ((st = get(n * sizeof(float), (void**)&c->f32.inc_f)) != SFX_OK) return st;
   if ((st = get(n * sizeof(float), (void**)&c->f32.inc_F)) != SFX_OK) return st;
-  if ((st = get(8 * sizeof(int), (void**)&c->f32.flag)) != SFX_OK) return st;
+  if ((st = get(16 * sizeof(int), (void**)&c->f32.flag)) != SFX_OK) return st;
   if ((st = get(n * sizeof(float2), (void**)&c->f32.falt)) != SFX_OK) return st;
   if ((st = get(n * sizeof(float2), (void**)&c->f32.Falt)) != SFX_OK) return st;
   // the Newton work arrays are colour-packed: 2 planes of ny nz ceil(nx/2)

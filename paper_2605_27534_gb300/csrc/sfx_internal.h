@@ -105,7 +105,8 @@ struct F32Scratch {
   float* phi32 = nullptr;           // folded float copy of phi
   int* flag = nullptr;              // convergence flag, iteration, prediction kept,
                                     // a tiled sweep that gave up waiting, residual
-                                    // kind (0 FP32, else pair), FP32 passes so far
+                                    // kind (0 FP32, else pair), FP32 passes so far;
+                                    // [8..12] norms and blocks of the 2D residual pass
   int fast_resid = 2;               // FP32 residual passes at most per Newton solve
   bool adv_staged = true;           // 3D advection from shared-memory planes
   bool incr_resid = true;           // incremental FP32 residuals after a pair pass (tiled path)
