@@ -191,6 +191,15 @@ __device__ inline T plic_slab(int nd, const T* m, T C, int d, T a, T b) {
   return plic_below(nd, n, alpha, d, rb) - plic_below(nd, n, alpha, d, ra);
 }
 
+// double to T, a float without the conversion instruction (FP64 pipe; 27 of
+// them per face)
+template <typename T>
+__device__ __forceinline__ T to_real(double x);
+template <>
+__device__ __forceinline__ double to_real<double>(double x) { return x; }
+template <>
+__device__ __forceinline__ float to_real<float>(double x) { return narrow(x); }
+
 // Youngs normal: minus the (1,2,1)-weighted gradient of C over the
 // 3x3(x3) block around (i,j,k), zero-gradient walls.
 template <typename T>
@@ -207,7 +216,7 @@ __device__ inline void youngs_normal(const Level& L, const double* __restrict__ 
         const int e = min(max(k + dk, 0), L.nz - 1);
         const T w = (di == 0 ? T(2) : T(1)) * (dj == 0 ? T(2) : T(1)) *
                     (nd == 3 ? (dk == 0 ? T(2) : T(1)) : T(1));
-        const T v = (T)C[cidx(L, a, b, e)];
+        const T v = to_real<T>(C[cidx(L, a, b, e)]);
         m[0] -= w * di * v;
         m[1] -= w * dj * v;
         m[2] -= w * dk * v;

@@ -30,8 +30,11 @@ namespace {
 // the tests for empty and full cells read the integer words and floats are
 // widened without the conversion instruction, which issues at the FP64 rate.
 // 256^3 sphere of radius 64 in float: 2.45 ms per step with every face and
-// cell, 0.57 ms now (planes 102, other faces 42, update 24 us per direction,
-// classification 30 us), 0.85 ms after 500 steps of wisps.
+// cell, 0.46 ms now (planes 69, other faces 39, update 24 us per direction,
+// classification 30 us), 0.70 ms after 500 steps of wisps.  The geometry is
+// inlined once per kernel, for the flow in either direction: twice, its code
+// did not fit the instruction cache (planes 102 us; small grids, where a pass
+// lasts one chain, 28 us instead of 24).
 constexpr size_t kVofListCells = (size_t)1 << 20;
 
 __device__ __forceinline__ long long vbits(double v) { return __double_as_longlong(v); }
@@ -112,9 +115,10 @@ __device__ __forceinline__ double plic_flux(const Level& L, int d, const int* x,
   if (pos) y[d] -= 1;
   G m[3];
   youngs_normal(L, C, y[0], y[1], y[2], m);
-  const G cg = (G)C[pos ? c - st : c];
-  return pos ? widen(plic_slab<G>(ND, m, cg, d, G(1) - (G)cf, G(1)))
-             : -widen(plic_slab<G>(ND, m, cg, d, G(0), (G)(-cf)));
+  const G g = (G)cf;
+  const double v = widen(plic_slab<G>(ND, m, (G)C[pos ? c - st : c], d, pos ? G(1) - g : G(0),
+                                      pos ? G(1) : -g));
+  return pos ? v : -v;
 }
 
 // Volume fraction crossing the minus-side face of every cell in direction d
@@ -129,13 +133,16 @@ k_vof_flux(Level L, int d, const int2* __restrict__ list, const double* __restri
            const U* __restrict__ u, double dt_h, double* __restrict__ Q,
            unsigned char* __restrict__ H, unsigned* __restrict__ cut) {
   const size_t st = d == 0 ? 1 : (d == 1 ? (size_t)L.nx : (size_t)L.nx * L.ny);
-  const unsigned nb = list ? (unsigned)list[0].x : gridDim.x;
-  for (unsigned q = blockIdx.x; q < nb; q += gridDim.x) {
+  // blocks of fewer threads take a share of a cell block each
+  const unsigned sub = (unsigned)CellBlock<ND>::threads / blockDim.x, step = gridDim.x / sub;
+  const int t = (int)(blockIdx.x % sub * blockDim.x + threadIdx.x);
+  const unsigned nb = list ? (unsigned)list[0].x : step;
+  for (unsigned q = blockIdx.x / sub; q < nb; q += step) {
     const unsigned blk = list ? (unsigned)list[1 + q].x : q;
     int x[3];
     bool plane = false;
     size_t c = 0;
-    if (CellBlock<ND>::at(L, blk, x)) {
+    if (CellBlock<ND>::at(L, blk, x, t)) {
       c = cidx(L, x[0], x[1], x[2]);
       const double cq = C[c];
       if (H) H[c] = cq > 0.5 ? 1 : 0;
@@ -149,9 +156,10 @@ k_vof_flux(Level L, int d, const int2* __restrict__ list, const double* __restri
           const double cf = widen(uf) * dt_h;
           // no plane in a cell that is full, in float also within rounding
           if (!((G)cu < G(1))) {
-            const G z[3] = {G(0), G(0), G(0)};
-            flux = vbits(cf) > 0 ? widen(plic_slab<G>(ND, z, (G)cu, d, G(1) - (G)cf, G(1)))
-                                 : -widen(plic_slab<G>(ND, z, (G)cu, d, G(0), (G)(-cf)));
+            // (plic_slab of a cell with C >= 1; a NaN is no fraction: C (b - a))
+            const G g = (G)cf, w = vbits(cf) > 0 ? G(1) - (G(1) - g) : -g;
+            flux = widen((G)cu >= G(1) ? w : (G)cu * w);
+            if (vbits(cf) <= 0) flux = -flux;
           } else {
             plane = true;
           }
@@ -234,8 +242,9 @@ sfx_status vof_impl(sfx_ctx* c, const U* const* u, double dt, int order, double*
   for (int q = 0; q < ND; ++q) {
     const int d = order ? ND - 1 - q : q;
     if (cut) SFX_CUDA(cudaMemsetAsync(cut, 0, sizeof(unsigned), s));
-    SFX_KERNEL(c, K_OTHER, (k_vof_flux<U, G, ND>), grid, 512, s, L, d, list, C, u[d], dt_h, c->vofQ,
-               q == 0 ? c->vofH : nullptr, cut);
+    // without a list a block lasts as long as its longest chain: small ones
+    SFX_KERNEL(c, K_OTHER, (k_vof_flux<U, G, ND>), list ? grid : 4 * grid, list ? 512 : 128, s, L, d,
+               list, C, u[d], dt_h, c->vofQ, q == 0 ? c->vofH : nullptr, cut);
     if (cut)
       SFX_KERNEL(c, K_OTHER, (k_vof_planes<U, G, ND>), c->sm_count * 16, 128, s, L, d, C, u[d], dt_h,
                  cut, c->vofQ);
