@@ -14,8 +14,8 @@
 // (columns tx < kA3X - 1), shares them through shared memory, and carries
 // the z face on the plus side of its cell to the next plane.  Each face
 // value comes from bcg_face2 and each cell sums its fluxes in the order of
-// advect_cell2, so the result is bitwise that of k_advect2t_32 and of the
-// batched kernels.
+// k_advect2t_32 and of the batched kernels, so the result is theirs bit for
+// bit.
 #pragma once
 
 #include "sfx_df.cuh"

@@ -30,7 +30,10 @@ struct BInst {
   size_t poff;                  // offset of the colour-packed Newton work arrays
 };
 
-// block -> instance through a prefix table of block counts
+// block -> instance through a prefix table of block counts (the kernels that
+// run once per phi; those of the step read a table of (instance, block of
+// the instance): the search's dependent loads cost a block of 256 cells as
+// much as its cells)
 __device__ __forceinline__ int find_inst(const int* __restrict__ pre, int n, int b) {
   int lo = 0, hi = n;   // pre[lo] <= b < pre[hi]
   while (hi - lo > 1) {
@@ -61,7 +64,10 @@ struct BPtr {
   float* rres;            // 2 per instance: last relative residuals
   double* mass;           // 2 per instance
   unsigned long long* work;   // 2 per instance: residual passes, sweep groups
-  int* loop;              // Newton iterations done in the current step
+  int* loop;              // [0] Newton iterations done in the current step, [1] instances
+                          // that finished this iteration's test, [2] of them still active,
+                          // [3] active at its start
+  int* done;              // per instance: blocks of the running pass that finished
   float* part;            // per cell block: the 4 residual maxima
   double* tpart;          // per cell block: (s, c) compensated sums of f and F
 };
@@ -93,43 +99,107 @@ __global__ void k_b_drift(const BInst* __restrict__ I, int n, const int* __restr
   P.H2[dir][fo + q] = __floats2half2_rn(bf, bF);
 }
 
-__global__ void k_b_advect(const BInst* __restrict__ I, int n, const int* __restrict__ pre, BPtr P) {
-  const int inst = find_inst(pre, n, blockIdx.x);
-  const BInst& B = I[inst];
+// Advection with every face evaluated once: a block takes a tile of up to 31
+// columns and as many rows as its threads cover, each thread the faces on
+// the minus side of its cell; the last column and row give the tile's plus
+// faces (as a plane of k_advect2t_32, bit for bit).  64 cylindrical grids
+// of 3.2e6 cells: 101 -> 96 us (the arithmetic of the limited slopes).
+constexpr int kBAdv = 256;
+struct AdvTile {
+  int wx, wy;                // threads across and up; cells wx - 1 by wy - 1
+};
+__host__ __device__ __forceinline__ AdvTile adv_tile(int nx) {
+  const int wx = (nx < 31 ? nx : 31) + 1;
+  return AdvTile{wx, kBAdv / wx};
+}
+__global__ void __launch_bounds__(kBAdv, 8)
+k_b_advect(const BInst* __restrict__ I, const int2* __restrict__ map, BPtr P) {
+  __shared__ float4 sx[kBAdv], sy[kBAdv];
+  const int2 m = map[blockIdx.x];
+  const BInst& B = I[m.x];
   const Level& L = B.p.L;
-  const size_t c = (size_t)(blockIdx.x - pre[inst]) * blockDim.x + threadIdx.x;
-  if (c >= L.ncell()) return;
-  Adv32 A{L, B.dt, B.p.invh, {P.ur + B.rfoff, P.uz + B.zfoff, nullptr}};
-  const int i = (int)((ix)c % (ix)L.nx), j = (int)((ix)c / (ix)L.nx);
-  advect_cell2(A, P.f + B.coff, P.F + B.coff, B.bc_f, B.bc_F, i, j, 0, (ix)c, P.fs[B.coff + c],
-               P.Fs[B.coff + c]);
+  const AdvTile T = adv_tile(L.nx);
+  const int tiles = (L.nx + T.wx - 2) / (T.wx - 1), t = threadIdx.x;
+  const int tx = t % T.wx, ty = t / T.wx;
+  const int i = m.y % tiles * (T.wx - 1) + tx, j = m.y / tiles * (T.wy - 1) + ty;
+  const Adv32 A{L, B.dt, B.p.invh, {P.ur + B.rfoff, P.uz + B.zfoff, nullptr}};
+  const float2 *f = P.f + B.coff, *F = P.F + B.coff;
+  const float wxm = wr_face(L.geom, i), wy = wz_face(L.geom, i);
+  float4 qx = make_float4(0.0f, 0.0f, 0.0f, 0.0f), qy = qx;
+  float ux = 0.0f, uy = 0.0f;
+  if (ty < T.wy && i <= L.nx && j < L.ny) {
+    int fc[3] = {i, j, 0};
+    ux = A.u[0][fidx32(L, 0, i, j, 0)];
+    qx = face_flux2(A, f, F, B.bc_f, B.bc_F, 0, fc, ux, wxm);
+  }
+  if (ty < T.wy && i < L.nx && j <= L.ny) {
+    int fc[3] = {i, j, 0};
+    uy = A.u[1][fidx32(L, 1, i, j, 0)];
+    qy = face_flux2(A, f, F, B.bc_f, B.bc_F, 1, fc, uy, wy);
+  }
+  sx[t] = qx;
+  sy[t] = qy;
+  __syncthreads();
+  if (tx >= T.wx - 1 || ty >= T.wy - 1 || i >= L.nx || j >= L.ny) return;
+  float2 S1 = make_float2(0.0f, 0.0f), S2 = S1;
+  if (ux != 0.0f) acc_face(S1, S2, qx, false);
+  if (A.u[0][fidx32(L, 0, i + 1, j, 0)] != 0.0f) acc_face(S1, S2, sx[t + 1], true);
+  if (uy != 0.0f) acc_face(S1, S2, qy, false);
+  if (A.u[1][fidx32(L, 1, i, j + 1, 0)] != 0.0f) acc_face(S1, S2, sy[t + T.wx], true);
+  float2 i1 = df_mul_f(df_mul_f(S1, -A.dt), A.invh);
+  float2 i2 = df_mul_f(df_mul_f(S2, -A.dt), A.invh);
+  if (L.geom == SFX_AXISYM) {
+    i1 = df_div_f(i1, wz_face(L.geom, i));
+    i2 = df_div_f(i2, wz_face(L.geom, i));
+  }
+  const ix c = cidx32(L, i, j, 0);
+  P.fs[B.coff + c] = df_add2(f[c], i1);
+  P.Fs[B.coff + c] = df_add2(F[c], i2);
 }
 
 // folded float copy of phi, and the start of the step
-__global__ void k_b_fold(const BInst* __restrict__ I, int n, const int* __restrict__ pre, BPtr P) {
-  const int inst = find_inst(pre, n, blockIdx.x);
-  const BInst& B = I[inst];
-  const size_t c = (size_t)(blockIdx.x - pre[inst]) * blockDim.x + threadIdx.x;
-  if (c >= B.p.L.ncell()) return;
-  P.phi32[B.coff + c] = fold_phi(P.phi[B.coff + c]);
+__global__ void k_b_fold(const BInst* __restrict__ I, const int2* __restrict__ map, int per, BPtr P) {
+  const int2 m = map[blockIdx.x];
+  const BInst& B = I[m.x];
+  const size_t n = B.p.L.ncell(), c0 = (size_t)m.y * per * blockDim.x + threadIdx.x;
+  for (int u = 0; u < per; ++u) {
+    const size_t c = c0 + (size_t)u * blockDim.x;
+    if (c < n) P.phi32[B.coff + c] = fold_phi(P.phi[B.coff + c]);
+  }
 }
 
-// state <- post-advection fields (the Newton iteration starts there)
-__global__ void k_b_copy(const BInst* __restrict__ I, int n, const int* __restrict__ pre, BPtr P,
-                         int from_star) {
-  const int inst = find_inst(pre, n, blockIdx.x);
-  const BInst& B = I[inst];
-  const size_t c = (size_t)(blockIdx.x - pre[inst]) * blockDim.x + threadIdx.x;
-  if (c >= B.p.L.ncell()) return;
-  const size_t g = B.coff + c;
-  if (from_star) { P.f[g] = P.fs[g]; P.F[g] = P.Fs[g]; }
-  else { P.fs[g] = P.f[g]; P.Fs[g] = P.F[g]; }
+// How a step starts.  kCopied: (f, F) and (f*, F*) hold the start before the
+// first iteration.  Where the tiles of an iteration write the state, no copy
+// precedes it: kStar (after advection) reads the first iterate from (f*, F*),
+// kState (no flow) reads (f*, F*) from the state, and the first state update
+// completes the other pair.
+enum { kCopied = 0, kStar = 1, kState = 2 };
+
+// state <- post-advection fields, or the reverse; with `first` set, of the
+// instances that converged at their first test only (their update never ran)
+__global__ void k_b_copy(const BInst* __restrict__ I, const int2* __restrict__ map, int per, BPtr P,
+                         int from_star, int first) {
+  const int2 m = map[blockIdx.x];
+  if (first && (P.active[m.x] || P.iters[m.x] != 1)) return;
+  const BInst& B = I[m.x];
+  const size_t n = B.p.L.ncell(), c0 = (size_t)m.y * per * blockDim.x + threadIdx.x;
+  for (int u = 0; u < per; ++u) {
+    const size_t c = c0 + (size_t)u * blockDim.x;
+    if (c >= n) return;
+    const size_t g = B.coff + c;
+    if (from_star) { P.f[g] = P.fs[g]; P.F[g] = P.Fs[g]; }
+    else { P.fs[g] = P.f[g]; P.Fs[g] = P.F[g]; }
+  }
 }
 
 __global__ void k_b_init(int n, BPtr P, int fast) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0) *P.loop = 0;
+  if (i == 0) {
+    P.loop[0] = P.loop[1] = P.loop[2] = 0;
+    P.loop[3] = n;
+  }
   if (i >= n) return;
+  P.done[i] = 0;
   P.active[i] = 1;
   P.iters[i] = 0;
   P.rkind[2 * i] = fast > 0 ? 0 : 1;
@@ -137,55 +207,75 @@ __global__ void k_b_init(int n, BPtr P, int fast) {
   for (int q = 0; q < 4; ++q) P.norms[4 * i + q] = 0u;
 }
 
+// The residuals of the active instances, with the convergence test of an
+// instance in its last block and the decision about another iteration in the
+// last instance's (a launch of their own each before: 6 us of every
+// iteration).  A thread takes `per` cells, so that the set-up of a block (its
+// instance's parameters) is shared, and 64 registers leave two thirds more
+// threads on an SM; `start`: see kCopied.  64 cylindrical grids of 3.2e6 cells:
+// 101 + 6 -> 76 us, 512 columns of 2048 cells 38 + 5 -> 29 us (one cell per
+// thread 105 and 39, four 76 and 31).
 // G: the geometry of every instance of the batch (compile time, as in the
 // single-grid Newton kernels, so that both run the same cell arithmetic)
 template <int G>
-__global__ void k_b_resid(const BInst* __restrict__ I, int n, const int* __restrict__ pre, BPtr P) {
-  const int inst = find_inst(pre, n, blockIdx.x);
+__global__ void __launch_bounds__(512, 2)
+k_b_resid(const BInst* __restrict__ I, const int2* __restrict__ map,
+                          const int* __restrict__ pre, int per, BPtr P, int start, float tol,
+                          int fast, int max_it, cudaGraphConditionalHandle loop) {
+  const int2 mp = map[blockIdx.x];
+  const int inst = mp.x;
   if (!P.active[inst]) return;
   const BInst& B = I[inst];
   const Level& L = B.p.L;
-  const size_t c = (size_t)(blockIdx.x - pre[inst]) * blockDim.x + threadIdx.x;
+  const ix n = (ix)L.ncell(), nx = (ix)L.nx, bs = blockDim.x;
+  const int it = P.loop[0] + 1;
+  // the FP32 residual for the instance's first iterations (the kind is
+  // the same for every block of an instance)
+  const int kind = P.rkind[2 * inst];
+  const size_t o = B.coff, w = B.poff;
+  const float2* B2[3] = {P.B2[0] + B.rfoff, P.B2[1] + B.zfoff, nullptr};
+  const float2 *fs = P.fs + o, *Fs = P.Fs + o, *f = P.f + o, *F = P.F + o;
+  if (it == 1 && start == kStar) f = fs, F = Fs;
+  if (it == 1 && start == kState) fs = f, Fs = F;
   float m[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-  if (c < L.ncell()) {
-    const int i = (int)((ix)c % (ix)L.nx), j = (int)((ix)c / (ix)L.nx);
-    const float2* B2[3] = {P.B2[0] + B.rfoff, P.B2[1] + B.zfoff, nullptr};
-    const size_t o = B.coff, w = B.poff;
-    // the FP32 residual for the instance's first iterations (the kind is
-    // the same for every block of an instance)
-    if (P.rkind[2 * inst] == 0)
-      resid32_cell<G>(B.p, i, j, 0, c, P.phi32 + o, B2, P.f + o, P.F + o, P.fs + o, P.Fs + o,
-                      P.rc + w, m, P.e2 + w);
+  ix c = (ix)mp.y * (ix)per * bs + threadIdx.x;
+  int i = (int)(c % nx), j = (int)(c / nx);
+  const int di = (int)(bs % nx), dj = (int)(bs / nx);
+  for (int u = 0; u < per && c < n; ++u, c += bs) {
+    if (kind == 0)
+      resid32_cell<G>(B.p, i, j, 0, c, P.phi32 + o, B2, f, F, fs, Fs, P.rc + w, m, P.e2 + w);
     else
-      resid2_cell<G>(B.p, i, j, 0, c, P.phi32 + o, B2, P.f + o, P.F + o, P.fs + o, P.Fs + o,
-                     P.rc + w, m, P.e2 + w);
+      resid2_cell<G>(B.p, i, j, 0, c, P.phi32 + o, B2, f, F, fs, Fs, P.rc + w, m, P.e2 + w);
+    i += di;
+    j += dj;
+    if (i >= L.nx) i -= L.nx, ++j;
   }
-  // block maxima; the flags kernel combines the blocks of each instance
+  // block maxima; the instance's last block combines its blocks
   __shared__ float wm[4][16];
+  __shared__ bool last;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const float v = warp_max(m[q]);
     if ((threadIdx.x & 31) == 0) wm[q][threadIdx.x >> 5] = v;
   }
   __syncthreads();
+  const int warps = (int)(blockDim.x >> 5);
   if (threadIdx.x < 4) {
     float v = 0.0f;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v = fmaxf(v, wm[threadIdx.x][w]);
+    for (int q = 0; q < warps; ++q) v = fmaxf(v, wm[threadIdx.x][q]);
     P.part[4 * (size_t)blockIdx.x + threadIdx.x] = v;
+    __threadfence();
   }
-}
-
-// convergence test of the current iteration: one block per instance still
-// active combines the residual maxima of the instance's blocks
-__global__ void k_b_flags(int n, const int* __restrict__ pre, BPtr P, float tol, int fast) {
-  const int i = blockIdx.x;
-  if (i >= n || !P.active[i]) return;
-  const int it = *P.loop + 1;
+  __syncthreads();
+  const int b0 = pre[inst], b1 = pre[inst + 1];
+  if (threadIdx.x == 0) last = atomicAdd(&P.done[inst], 1) == b1 - b0 - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
   float mx[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-  for (int b = pre[i] + threadIdx.x; b < pre[i + 1]; b += blockDim.x)
+  for (int b = b0 + (int)threadIdx.x; b < b1; b += (int)blockDim.x)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) mx[q] = fmaxf(mx[q], P.part[4 * (size_t)b + q]);
-  __shared__ float wm[4][8];
+    for (int q = 0; q < 4; ++q) mx[q] = fmaxf(mx[q], __ldcg(&P.part[4 * (size_t)b + q]));
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     mx[q] = warp_max(mx[q]);
@@ -193,37 +283,36 @@ __global__ void k_b_flags(int n, const int* __restrict__ pre, BPtr P, float tol,
   }
   __syncthreads();
   if (threadIdx.x != 0) return;
-  for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
+  P.done[inst] = 0;
+  for (int q = 1; q < warps; ++q)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) mx[q] = fmaxf(mx[q], wm[q][w]);
+    for (int k = 0; k < 4; ++k) mx[k] = fmaxf(mx[k], wm[k][q]);
   const float rf = mx[0], bf = mx[1], rF = mx[2], bF = mx[3];
-  P.rres[2 * i] = rf / fmaxf(bf, 1e-30f);
-  P.rres[2 * i + 1] = rF / fmaxf(bF, 1e-30f);
-  P.iters[i] = it;
-  P.work[2 * i] += 1;
-  if (P.rkind[2 * i] != 0 && rf <= tol * bf && rF <= tol * bF) {
-    P.active[i] = 0;   // converged on a pair residual: stop here
-    return;
+  P.rres[2 * inst] = rf / fmaxf(bf, 1e-30f);
+  P.rres[2 * inst + 1] = rF / fmaxf(bF, 1e-30f);
+  P.iters[inst] = it;
+  P.work[2 * inst] += 1;
+  if (kind != 0 && rf <= tol * bf && rF <= tol * bF) {
+    P.active[inst] = 0;   // converged on a pair residual: stop here
+  } else {
+    P.work[2 * inst + 1] += 1;   // the sweeps run
+    // after `fast` FP32 passes, or once the residuals are small, the pair
+    // residual (as the single-grid solve switches)
+    if (kind == 0 && (++P.rkind[2 * inst + 1] >= fast ||
+                      (rf <= kFastResidSwitch * bf && rF <= kFastResidSwitch * bF)))
+      P.rkind[2 * inst] = 1;
+    atomicAdd(&P.loop[2], 1);
   }
-  P.work[2 * i + 1] += 1;   // the sweeps run
-  // after `fast` FP32 passes, or once the residuals are small, the pair
-  // residual (as the single-grid solve switches)
-  if (P.rkind[2 * i] == 0 && (++P.rkind[2 * i + 1] >= fast ||
-                              (rf <= kFastResidSwitch * bf && rF <= kFastResidSwitch * bF)))
-    P.rkind[2 * i] = 1;
-}
-
-// end of an iteration: count it, and let the step's loop run again while
-// an instance is active and the iteration budget lasts
-__global__ void k_b_next(int n, BPtr P, int max_it, cudaGraphConditionalHandle loop) {
-  int any = 0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) any |= P.active[i];
-  any = __syncthreads_or(any);
-  if (threadIdx.x == 0) {
-    const int done = *P.loop + 1;
-    *P.loop = done;
-    cudaGraphSetConditional(loop, (any && done < max_it) ? 1u : 0u);
-  }
+  // the last instance: count the iteration, and let the step's loop run
+  // again while an instance is active and the iteration budget lasts
+  __threadfence();
+  if (atomicAdd(&P.loop[1], 1) != P.loop[3] - 1) return;
+  __threadfence();
+  const int any = atomicExch(&P.loop[2], 0);
+  P.loop[3] = any;
+  P.loop[1] = 0;
+  P.loop[0] = it;
+  cudaGraphSetConditional(loop, (any && it < max_it) ? 1u : 0u);
 }
 
 // one colour of the coupled correction sweep; blocks over half-rows
@@ -262,20 +351,22 @@ __global__ void k_b_corr(const BInst* __restrict__ I, int n, const int* __restri
 // tiles of every instance, ty rows each
 template <int G>
 __global__ void __launch_bounds__(kT2Threads)
-k_b_corr_tiles(const BInst* __restrict__ I, int n, const int* __restrict__ pre, int ty, int sweeps,
-               BPtr P) {
-  const int inst = find_inst(pre, n, blockIdx.x);
-  if (!P.active[inst]) return;
-  const BInst& B = I[inst];
+k_b_corr_tiles(const BInst* __restrict__ I, const int2* __restrict__ map, int ty, int sweeps,
+               BPtr P, int start) {
+  const int2 m = map[blockIdx.x];
+  if (!P.active[m.x]) return;
+  const int first = P.loop[0] == 1 ? start : kCopied;   // (counted by the residual pass)
+  const BInst& B = I[m.x];
   const Level& L = B.p.L;
   const int tx = L.nx <= kT2Width ? L.nx + (L.nx & 1) : kT2Width - 4 * sweeps;
-  const int nx = (L.nx + tx - 1) / tx, t = blockIdx.x - pre[inst];
-  float2* f = P.f + B.coff;
-  float2* F = P.F + B.coff;
+  const int nx = (L.nx + tx - 1) / tx, t = m.y;
+  float2 *f = P.f + B.coff, *F = P.F + B.coff, *fs = P.fs + B.coff, *Fs = P.Fs + B.coff;
   corr_tile2d<G>(B.p, (t % nx) * tx, (t / nx) * ty, tx, ty, sweeps, P.H2[0] + B.rfoff,
                  P.H2[1] + B.zfoff, P.rc + B.poff, P.e2 + B.poff, [&](ix c, float2 e) {
-                   f[c] = df_add(f[c], e.x);
-                   F[c] = df_add(F[c], e.y);
+                   const float2 a = first == kStar ? fs[c] : f[c], b = first == kStar ? Fs[c] : F[c];
+                   if (first == kState) fs[c] = a, Fs[c] = b;
+                   f[c] = df_add(a, e.x);
+                   F[c] = df_add(b, e.y);
                  });
 }
 
@@ -288,6 +379,7 @@ __global__ void __launch_bounds__(256) k_b_totals(const BInst* __restrict__ I, i
   const BInst& B = I[inst];
   const Level& L = B.p.L;
   const ix n = (ix)L.ncell(), nx = (ix)L.nx;
+  __shared__ bool last;
   float2 acc[2] = {make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
   for (ix c = part * blockDim.x + threadIdx.x; c < n; c += parts * blockDim.x) {
     // ring volume / (pi h^3), or 1 for planar cells (volume h^2)
@@ -309,28 +401,30 @@ __global__ void __launch_bounds__(256) k_b_totals(const BInst* __restrict__ I, i
       P.tpart[4 * (size_t)blockIdx.x + 2 * fld + 1] = cc;
     }
   }
-}
-
-// ... and one warp per instance combines its blocks in a fixed order
-__global__ void k_b_totals_final(const BInst* __restrict__ I, int n, int parts, BPtr P) {
-  const int inst = blockIdx.x;
-  if (inst >= n) return;
+  // ... and the first warp of the instance's last block combines the blocks
+  // in a fixed order
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(&P.done[inst], 1) == parts - 1;
+    if (last) P.done[inst] = 0;
+  }
+  __syncthreads();
+  if (!last || threadIdx.x >= 32) return;
+  __threadfence();
   for (int fld = 0; fld < 2; ++fld) {
     double s = 0.0, cc = 0.0;
-    for (int b = inst * parts + threadIdx.x; b < (inst + 1) * parts; b += blockDim.x) {
+    for (int b = inst * parts + (int)threadIdx.x; b < (inst + 1) * parts; b += 32) {
       double t, e;
-      two_sum(s, P.tpart[4 * (size_t)b + 2 * fld], t, e);
+      two_sum(s, __ldcg(&P.tpart[4 * (size_t)b + 2 * fld]), t, e);
       s = t;
-      cc += P.tpart[4 * (size_t)b + 2 * fld + 1] + e;
+      cc += __ldcg(&P.tpart[4 * (size_t)b + 2 * fld + 1]) + e;
     }
     warp_sum_comp(s, cc);
-    if (threadIdx.x == 0) {
-      const Level& L = I[inst].p.L;
-      const double h = L.h;
-      P.mass[2 * inst + fld] = (s + cc) * (L.geom == SFX_AXISYM ? kPi * h * h * h : h * h);
-    }
+    if (threadIdx.x == 0)
+      P.mass[2 * inst + fld] = (s + cc) * (L.geom == SFX_AXISYM ? kPi * L.h * L.h * L.h : L.h * L.h);
   }
 }
+
 
 }  // namespace
 }  // namespace sfx
@@ -344,12 +438,16 @@ struct sfx_batch {
   size_t ncell = 0, nrf = 0, nzf = 0, npack = 0;
   std::vector<size_t> coff, rfoff, zfoff;
   BInst* dI = nullptr;
-  int* pre_cell = nullptr;   // blocks of `block` threads over cells
+  int* pre_cell = nullptr;   // blocks of `block` threads, `per` cells each
+  int2* map_cell = nullptr;  // (instance, its block) of those blocks,
+  int2* map_adv = nullptr;   // of the advection tiles
+  int2* map_tile = nullptr;  // and of the correction tiles
+  int per = 1, nb_adv = 0;
   int* pre_rf = nullptr;
   int* pre_zf = nullptr;
   int* pre_pair = nullptr;
   int nb_cell = 0, nb_rf = 0, nb_zf = 0, nb_pair = 0;
-  int* pre_tile = nullptr;   // tiles of all sweeps in one launch, of tile_ty rows
+  // tiles of all sweeps in one launch, of tile_ty rows
   int nb_tile = 0, tile_ty = 0, tile_sweeps = 0;   // (tile_ty 0: colour launches)
   size_t tile_smem = 0;
   int block = 256;
@@ -387,16 +485,27 @@ sfx_status balloc(sfx_batch* b, T** p, size_t n) {
 // prefix tables of blocks per instance for the current block size
 sfx_status build_prefix(sfx_batch* b) {
   const int bs = b->block;
+  int dev = 0, sms = 152;
+  SFX_CUDA(cudaGetDevice(&dev));
+  SFX_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  // cells per thread: 8, 4 or 2 where that leaves 768 threads per SM (6 split
+  // columns of 2048 cells unevenly: 33 instead of 29 us)
+  b->per = 8;
+  while (b->per > 1 && b->ncell < (size_t)sms * 768 * b->per) b->per /= 2;
+  const size_t cells = (size_t)bs * b->per;
+  std::vector<int2> mc;
   std::vector<int> pc(b->n + 1), pr(b->n + 1), pz(b->n + 1), pp(b->n + 1);
   pc[0] = pr[0] = pz[0] = pp[0] = 0;
   for (int i = 0; i < b->n; ++i) {
     const Level& L = b->hI[i].p.L;
-    pc[i + 1] = pc[i] + (int)((L.ncell() + bs - 1) / bs);
+    pc[i + 1] = pc[i] + (int)((L.ncell() + cells - 1) / cells);
+    for (int q = pc[i]; q < pc[i + 1]; ++q) mc.push_back(make_int2(i, q - pc[i]));
     pr[i + 1] = pr[i] + (int)((L.nface(0) + bs - 1) / bs);
     pz[i + 1] = pz[i] + (int)((L.nface(1) + bs - 1) / bs);
     pp[i + 1] = pp[i] + (int)(((size_t)((L.nx + 1) / 2) * L.ny + bs - 1) / bs);
   }
   b->nb_cell = pc[b->n];
+  SFX_CUDA(cudaMemcpy(b->map_cell, mc.data(), mc.size() * sizeof(int2), cudaMemcpyHostToDevice));
   b->nb_rf = pr[b->n];
   b->nb_zf = pz[b->n];
   b->nb_pair = pp[b->n];
@@ -410,6 +519,7 @@ sfx_status build_prefix(sfx_batch* b) {
 // Tiles of the current number of sweeps (before a capture).
 sfx_status build_tiles(sfx_batch* b) {
   if (b->tile_sweeps == b->sweeps) return SFX_OK;
+  b->tile_sweeps = 0;
   struct Ext {
     int nx, ny;
   };
@@ -418,23 +528,27 @@ sfx_status build_tiles(sfx_batch* b) {
   int dev = 0, sms = 152;
   SFX_CUDA(cudaGetDevice(&dev));
   SFX_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  std::vector<int2> map;
   const int ty = tile2d_rows(g.data(), b->n, b->sweeps, sms);
   size_t smem = 0;
-  std::vector<int> pre(1, 0);
-  for (const Ext& e : g) {
-    const Tile2D t = tile2d_of(e.nx, std::max(ty, 1), b->sweeps);
+  for (int q = 0; q < b->n && ty > 0; ++q) {
+    const Ext& e = g[q];
+    const Tile2D t = tile2d_of(e.nx, ty, b->sweeps);
     smem = std::max(smem, tile2d_smem(e.nx, e.ny, t, b->sweeps));
-    pre.push_back(pre.back() + ((e.nx + t.tx - 1) / t.tx) * ((e.ny + t.ty - 1) / t.ty));
-    if (ty == 0) break;
+    const int tiles = ((e.nx + t.tx - 1) / t.tx) * ((e.ny + t.ty - 1) / t.ty);
+    for (int k = 0; k < tiles; ++k) map.push_back(make_int2(q, k));
   }
   if (ty > 0) {
-    SFX_CUDA(cudaMemcpy(b->pre_tile, pre.data(), pre.size() * sizeof(int), cudaMemcpyHostToDevice));
+    if (b->map_tile) SFX_CUDA(cudaFree(b->map_tile));
+    b->map_tile = nullptr;
+    SFX_CUDA(cudaMalloc((void**)&b->map_tile, map.size() * sizeof(int2)));
+    SFX_CUDA(cudaMemcpy(b->map_tile, map.data(), map.size() * sizeof(int2), cudaMemcpyHostToDevice));
     auto tiles = b->geom == SFX_AXISYM ? &k_b_corr_tiles<SFX_AXISYM> : &k_b_corr_tiles<SFX_PLANAR2D>;
     SFX_CUDA(cudaFuncSetAttribute(tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kT2Smem));
   }
   b->tile_ty = ty;
   b->tile_smem = smem;
-  b->nb_tile = pre.back();
+  b->nb_tile = (int)map.size();
   b->tile_sweeps = b->sweeps;
   return SFX_OK;
 }
@@ -448,16 +562,14 @@ sfx_status enqueue_step(sfx_batch* b, bool advect, float tol, cudaStream_t s) {
   BPtr& P = b->P;
   k_b_init<<<(n + 127) / 128, 128, 0, s>>>(n, P, b->fast);
   if (!b->reuse_phi) {
-    k_b_fold<<<b->nb_cell, bs, 0, s>>>(b->dI, n, b->pre_cell, P);
+    k_b_fold<<<b->nb_cell, bs, 0, s>>>(b->dI, b->map_cell, b->per, P);
     k_b_drift<<<b->nb_rf, bs, 0, s>>>(b->dI, n, b->pre_rf, 0, P);
     k_b_drift<<<b->nb_zf, bs, 0, s>>>(b->dI, n, b->pre_zf, 1, P);
   }
-  if (advect) {
-    k_b_advect<<<b->nb_cell, bs, 0, s>>>(b->dI, n, b->pre_cell, P);
-    k_b_copy<<<b->nb_cell, bs, 0, s>>>(b->dI, n, b->pre_cell, P, 1);
-  } else {
-    k_b_copy<<<b->nb_cell, bs, 0, s>>>(b->dI, n, b->pre_cell, P, 0);
-  }
+  if (advect) k_b_advect<<<b->nb_adv, kBAdv, 0, s>>>(b->dI, b->map_adv, P);
+  const int start = b->tile_ty == 0 ? kCopied : advect ? kStar : kState;
+  if (start == kCopied)
+    k_b_copy<<<b->nb_cell, bs, 0, s>>>(b->dI, b->map_cell, b->per, P, advect ? 1 : 0, 0);
   SFX_LAUNCH_CHECK();
   // the while node, after everything captured so far
   cudaStreamCaptureStatus cs;
@@ -482,18 +594,18 @@ sfx_status enqueue_step(sfx_batch* b, bool advect, float tol, cudaStream_t s) {
   const bool axi = b->geom == SFX_AXISYM;
   auto resid = axi ? &k_b_resid<SFX_AXISYM> : &k_b_resid<SFX_PLANAR2D>;
   auto corr = axi ? &k_b_corr<SFX_AXISYM> : &k_b_corr<SFX_PLANAR2D>;
-  resid<<<b->nb_cell, bs, 0, sb>>>(b->dI, n, b->pre_cell, P);
-  k_b_flags<<<n, 256, 0, sb>>>(n, b->pre_cell, P, tol, b->fast);
+  resid<<<b->nb_cell, bs, 0, sb>>>(b->dI, b->map_cell, b->pre_cell, b->per, P, start, tol, b->fast,
+                                   b->max_it, loop);
   // the residual pass did the first red half-sweep
   if (b->tile_ty > 0) {
     auto tiles = axi ? &k_b_corr_tiles<SFX_AXISYM> : &k_b_corr_tiles<SFX_PLANAR2D>;
-    tiles<<<b->nb_tile, kT2Threads, b->tile_smem, sb>>>(b->dI, n, b->pre_tile, b->tile_ty, b->sweeps, P);
+    tiles<<<b->nb_tile, kT2Threads, b->tile_smem, sb>>>(b->dI, b->map_tile, b->tile_ty, b->sweeps, P,
+                                                        start);
   }
   for (int q = 0; q < b->sweeps && b->tile_ty == 0; ++q)
     for (int color = (q == 0 ? 1 : 0); color < 2; ++color)
       corr<<<b->nb_pair, bs, 0, sb>>>(b->dI, n, b->pre_pair, P, color, q == 0 ? 1 : 0,
                                       q == b->sweeps - 1 && color == 1 ? 1 : 0);
-  k_b_next<<<1, 256, 0, sb>>>(n, P, b->max_it, loop);
   const cudaError_t le = cudaGetLastError();
   cudaGraph_t body_out = nullptr;
   const cudaError_t be = cudaStreamEndCapture(sb, &body_out);
@@ -501,8 +613,9 @@ sfx_status enqueue_step(sfx_batch* b, bool advect, float tol, cudaStream_t s) {
   SFX_CUDA(be);
   SFX_CUDA(cudaStreamUpdateCaptureDependencies(s, &cnode, nullptr, 1,
                                                cudaStreamSetCaptureDependencies));
+  if (start == kStar)
+    k_b_copy<<<b->nb_cell, bs, 0, s>>>(b->dI, b->map_cell, b->per, P, 1, 1);
   k_b_totals<<<n * b->tot_parts, 256, 0, s>>>(b->dI, b->tot_parts, P);
-  k_b_totals_final<<<n, 32, 0, s>>>(b->dI, n, b->tot_parts, P);
   SFX_LAUNCH_CHECK();
   return SFX_OK;
 }
@@ -620,7 +733,6 @@ sfx_status sfx_batch_create_geom(const sfx_batch_instance* inst, int n, int geom
   if (st == SFX_OK) st = balloc(b, &b->pre_rf, (size_t)n + 1);
   if (st == SFX_OK) st = balloc(b, &b->pre_zf, (size_t)n + 1);
   if (st == SFX_OK) st = balloc(b, &b->pre_pair, (size_t)n + 1);
-  if (st == SFX_OK) st = balloc(b, &b->pre_tile, (size_t)n + 1);
   if (st == SFX_OK) st = balloc(b, &P.phi32, nc);
   if (st == SFX_OK) st = balloc(b, &P.fs, nc);
   if (st == SFX_OK) st = balloc(b, &P.Fs, nc);
@@ -634,7 +746,8 @@ sfx_status sfx_batch_create_geom(const sfx_batch_instance* inst, int n, int geom
   if (st == SFX_OK) st = balloc(b, &P.rkind, 2 * (size_t)n);
   if (st == SFX_OK) st = balloc(b, &P.active, (size_t)n);
   if (st == SFX_OK) st = balloc(b, &P.iters, (size_t)n);
-  if (st == SFX_OK) st = balloc(b, &P.loop, (size_t)1);
+  if (st == SFX_OK) st = balloc(b, &P.loop, (size_t)4);
+  if (st == SFX_OK) st = balloc(b, &P.done, (size_t)n);
   if (st == SFX_OK) st = balloc(b, &P.rres, 2 * (size_t)n);
   if (st == SFX_OK) st = balloc(b, &P.mass, 2 * (size_t)n);
   if (st == SFX_OK) st = balloc(b, &P.work, 2 * (size_t)n);
@@ -646,6 +759,20 @@ sfx_status sfx_batch_create_geom(const sfx_batch_instance* inst, int n, int geom
   // block partials: at most one block per 128 cells of each instance
   const size_t maxblk = nc / 128 + (size_t)n + 1;
   if (st == SFX_OK) st = balloc(b, &P.part, 4 * maxblk);
+  if (st == SFX_OK) st = balloc(b, &b->map_cell, maxblk);
+  std::vector<int2> ma;
+  for (int i = 0; i < n; ++i) {
+    const Level& L = b->hI[i].p.L;
+    const AdvTile T = adv_tile(L.nx);
+    const int tiles = ((L.nx + T.wx - 2) / (T.wx - 1)) * ((L.ny + T.wy - 2) / (T.wy - 1));
+    for (int k = 0; k < tiles; ++k) ma.push_back(make_int2(i, k));
+  }
+  b->nb_adv = (int)ma.size();
+  if (st == SFX_OK) st = balloc(b, &b->map_adv, ma.size());
+  if (st == SFX_OK) {
+    cudaError_t e = cudaMemcpy(b->map_adv, ma.data(), ma.size() * sizeof(int2), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) st = cuda_fail(e);
+  }
   if (st == SFX_OK) st = balloc(b, &P.tpart, 4 * (size_t)n * kTotBlocks);
   if (st == SFX_OK) {
     cudaError_t e = cudaMemset(P.work, 0, 2 * (size_t)n * sizeof(unsigned long long));
@@ -670,6 +797,7 @@ void sfx_batch_destroy(sfx_batch* b) {
   if (b->cap) cudaStreamDestroy(b->cap);
   if (b->cap_body) cudaStreamDestroy(b->cap_body);
   for (void* p : b->allocs) cudaFree(p);
+  cudaFree(b->map_tile);
   delete b;
 }
 
@@ -727,7 +855,7 @@ sfx_status sfx_batch_step(sfx_batch* b, const void* phi, const void* ur, const v
     // phi declared static: its folded copy and the drifts once, outside the graph
     cudaStream_t s = (cudaStream_t)stream;
     const int n = b->n, bs = b->block;
-    k_b_fold<<<b->nb_cell, bs, 0, s>>>(b->dI, n, b->pre_cell, b->P);
+    k_b_fold<<<b->nb_cell, bs, 0, s>>>(b->dI, b->map_cell, b->per, b->P);
     k_b_drift<<<b->nb_rf, bs, 0, s>>>(b->dI, n, b->pre_rf, 0, b->P);
     k_b_drift<<<b->nb_zf, bs, 0, s>>>(b->dI, n, b->pre_zf, 1, b->P);
     SFX_LAUNCH_CHECK();

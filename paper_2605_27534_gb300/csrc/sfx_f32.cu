@@ -810,26 +810,10 @@ __global__ void k_advect32(Adv32 A, const float2* __restrict__ x, float bc_in,
 // (i0 + tx, j0 + ty) of the current plane (the last column and row give the
 // tile's plus faces) and shares them through shared memory; the z face on
 // the plus side of its cell is carried into the next plane as that plane's
-// minus face.  Each face term is the weighted pair flux w u v of
-// advect_cell2 and the cell sums them in its order (minus then plus face,
-// x, y, z), so the result is bitwise that of advect_cell2 (the batched
-// kernels).
+// minus face.  The cell sums the weighted pair fluxes w u v in a fixed order
+// (minus then plus face, x, y, z), as the batched kernel does: bitwise the
+// same result.
 constexpr int kAdvX = 32, kAdvY = 8, kAdvZ = 8;
-
-// weighted pair fluxes of one face for both fields: (f.hi, f.lo, F.hi, F.lo)
-__device__ __forceinline__ float4 face_flux2(const Adv32& A, const float2* __restrict__ x1,
-                                             const float2* __restrict__ x2, float bc1, float bc2,
-                                             int d, int* fc, float u, float w) {
-  if (u == 0.0f) return make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-  float v1, v2;
-  face32v2(A, x1, x2, bc1, bc2, d, fc, u, v1, v2);
-  float pr = __fmul_rn(u, v1);
-  const float2 a = df_mul_f(make_float2(pr, fmaf(u, v1, -pr)), w);
-  pr = __fmul_rn(u, v2);
-  const float2 b = df_mul_f(make_float2(pr, fmaf(u, v2, -pr)), w);
-  return make_float4(a.x, a.y, b.x, b.y);
-}
-
 
 __global__ void __launch_bounds__(kAdvX* kAdvY)
     k_advect2t_32(Adv32 A, const float2* __restrict__ f, const float2* __restrict__ F,

@@ -1004,47 +1004,18 @@ __device__ __forceinline__ void acc_face(float2& S1, float2& S2, float4 q, bool 
   }
 }
 
-// advect_cell for two fields sharing the face geometry (bitwise the same
-// per field).
-__device__ __forceinline__ void advect_cell2(const Adv32& A, const float2* __restrict__ x1,
+// weighted pair fluxes of one face for both fields: (f.hi, f.lo, F.hi, F.lo)
+__device__ __forceinline__ float4 face_flux2(const Adv32& A, const float2* __restrict__ x1,
                                              const float2* __restrict__ x2, float bc1, float bc2,
-                                             int i, int j, int k, ix c, float2& o1,
-                                             float2& o2) {
-  const Level& L = A.L;
-  int idx[3] = {i, j, k};
-  float2 S1 = make_float2(0.0f, 0.0f), S2 = make_float2(0.0f, 0.0f);
-  for (int d = 0; d < L.ndim(); ++d) {
-    int pp[3] = {idx[0], idx[1], idx[2]};
-    pp[d] += 1;
-    const float um = A.u[d][fidx(L, d, idx[0], idx[1], idx[2])];
-    const float up = A.u[d][fidx(L, d, pp[0], pp[1], pp[2])];
-    const float wm = d == 0 ? wr_face(L.geom, idx[0]) : (d == 1 ? wz_face(L.geom, idx[0]) : 1.0f);
-    const float wp = d == 0 ? wr_face(L.geom, idx[0] + 1) : wm;
-    if (um != 0.0f) {
-      float v1, v2;
-      face32v2(A, x1, x2, bc1, bc2, d, idx, um, v1, v2);
-      float pr = __fmul_rn(um, v1);
-      S1 = df_sub2(S1, df_mul_f(make_float2(pr, fmaf(um, v1, -pr)), wm));
-      pr = __fmul_rn(um, v2);
-      S2 = df_sub2(S2, df_mul_f(make_float2(pr, fmaf(um, v2, -pr)), wm));
-    }
-    if (up != 0.0f) {
-      float v1, v2;
-      face32v2(A, x1, x2, bc1, bc2, d, pp, up, v1, v2);
-      float pr = __fmul_rn(up, v1);
-      S1 = df_add2(S1, df_mul_f(make_float2(pr, fmaf(up, v1, -pr)), wp));
-      pr = __fmul_rn(up, v2);
-      S2 = df_add2(S2, df_mul_f(make_float2(pr, fmaf(up, v2, -pr)), wp));
-    }
-  }
-  float2 i1 = df_mul_f(df_mul_f(S1, -A.dt), A.invh);
-  float2 i2 = df_mul_f(df_mul_f(S2, -A.dt), A.invh);
-  if (L.geom == SFX_AXISYM) {
-    i1 = df_div_f(i1, wz_face(L.geom, idx[0]));
-    i2 = df_div_f(i2, wz_face(L.geom, idx[0]));
-  }
-  o1 = df_add2(x1[c], i1);
-  o2 = df_add2(x2[c], i2);
+                                             int d, int* fc, float u, float w) {
+  if (u == 0.0f) return make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  float v1, v2;
+  face32v2(A, x1, x2, bc1, bc2, d, fc, u, v1, v2);
+  float pr = __fmul_rn(u, v1);
+  const float2 a = df_mul_f(make_float2(pr, fmaf(u, v1, -pr)), w);
+  pr = __fmul_rn(u, v2);
+  const float2 b = df_mul_f(make_float2(pr, fmaf(u, v2, -pr)), w);
+  return make_float4(a.x, a.y, b.x, b.y);
 }
 
 }  // namespace
