@@ -6,8 +6,13 @@ the loss L = sum_c V_c |F_Ma,c|^2 of the final Marangoni force; its backward
 is the hand-written discrete adjoint of the library (sfx_adjoint_step,
 sfx_marangoni_loss, sfx_f_from_gamma), giving dL/dGamma0 and dL/dtheta for
 theta = (k_a, k_d, D_f, D_F).  The forward keeps a checkpoint of the state
-every K steps; the backward recomputes each segment of K steps from its
-checkpoint and walks it backwards.  The forward may run in an SFX_F32
+every K steps and every state of the last segment, which the backward walks
+first; the backward recomputes each earlier segment of K steps from its
+checkpoint and walks it backwards.  (The backward holds the states of one
+segment at a time in any case.  Recomputing the last one, once for its end
+and once for its states, ran every step of a rollout within K steps three
+times: eight steps at 256x256 with their gradient 7.65 -> 4.4 ms.)  The
+forward may run in an SFX_F32
 context (double-float state); the adjoint always works in FP64 on the
 recomputed states.  Every step of the computation runs in libsfx kernels.
 """
@@ -74,17 +79,21 @@ class SurfactantRollout(torch.autograd.Function):
         f, F = _to_state(ctx, f0), _to_state(ctx, setup.F0)
         checkpoints = [(f.clone(), F.clone())]
         done = 0
-        while done < setup.nsteps:
-            n = min(setup.K, setup.nsteps - done)
-            _forward_steps(setup, ps, f, F, n)
-            done += n
-            if done < setup.nsteps:
-                checkpoints.append((f.clone(), F.clone()))
+        while setup.nsteps - done > setup.K:
+            _forward_steps(setup, ps, f, F, setup.K)
+            done += setup.K
+            checkpoints.append((f.clone(), F.clone()))
+        last = []
+        for _ in range(setup.nsteps - done):
+            _forward_steps(setup, ps, f, F, 1)
+            if any(fctx.needs_input_grad):
+                last.append((f.clone(), F.clone()))
         L, _ = ctx.sfx_marangoni_loss(ps, _to_double(ctx, f), setup.phi, setup.C, setup.dm_mode,
                                       grad=False)
         fctx.setup = setup
         fctx.ps = ps
         fctx.checkpoints = checkpoints
+        fctx.last = last
         fctx.theta_device = theta.device
         fctx.theta_dtype = theta.dtype
         return torch.tensor(L, dtype=torch.float64)
@@ -96,23 +105,23 @@ class SurfactantRollout(torch.autograd.Function):
         ctx = setup.context
         o = default_opts(tol=setup.adj_tol, max_cycles=1000, nu1=10, nu2=10)
         # the final state, for dL/df
-        last_f, last_F = (t.clone() for t in fctx.checkpoints[-1])
-        rem = setup.nsteps - setup.K * (len(fctx.checkpoints) - 1)
-        _forward_steps(setup, ps, last_f, last_F, rem)
+        last_f = (fctx.last or fctx.checkpoints)[-1][0]
         _, gf = ctx.sfx_marangoni_loss(ps, _to_double(ctx, last_f), setup.phi, setup.C,
                                        setup.dm_mode, grad=True)
         lam_f = gf * float(gL)
         lam_F = torch.zeros_like(lam_f)
         dtheta = [0.0, 0.0, 0.0, 0.0]
         for s in range(len(fctx.checkpoints) - 1, -1, -1):
-            n = min(setup.K, setup.nsteps - s * setup.K)
-            f, F = (t.clone() for t in fctx.checkpoints[s])
-            states = []
-            for _ in range(n):
-                _forward_steps(setup, ps, f, F, 1)
-                states.append((_to_double(ctx, f).clone(), _to_double(ctx, F).clone()))
+            states = fctx.last
+            if s < len(fctx.checkpoints) - 1:
+                f, F = (t.clone() for t in fctx.checkpoints[s])
+                states = []
+                for _ in range(setup.K):
+                    _forward_steps(setup, ps, f, F, 1)
+                    states.append((f.clone(), F.clone()))
             for f1, F1 in reversed(states):
-                ctx.sfx_adjoint_step(ps, setup.phi, f1, F1, setup.dt, lam_f, lam_F, dtheta, o)
+                ctx.sfx_adjoint_step(ps, setup.phi, _to_double(ctx, f1), _to_double(ctx, F1),
+                                     setup.dt, lam_f, lam_F, dtheta, o)
         dgamma = ctx.sfx_f_from_gamma(lam_f, setup.phi, ps.eps)
         dth = torch.tensor(dtheta, dtype=fctx.theta_dtype, device=fctx.theta_device)
         return dgamma, dth, None
