@@ -66,8 +66,13 @@ __device__ __forceinline__ bool redist_cut(int nd, T s0, const T* zm, const T* z
 // costs one FP64 minimum, subtraction, maximum, product and sum per
 // direction and a root; the sub-cell distance is formed once (aux), and
 // a warp whose cells all equal their neighbours (compared as bits) only
-// adds dtau.  192^3 sphere of radius 48, 24 steps: 31.5 ms stepping every
-// cell from its definition, 1.87 ms with active blocks.
+// adds dtau.  Blocks differ in cost (those in the band against flat ones) and
+// the FP64 pipe idles in a last wave: a step takes resident blocks of 128
+// threads, a quarter of a cell block each, 66 us at 192^3 (four blocks of 512
+// threads per SM, of which three fit: 78 us, the SMs active 71 % of it; minima
+// of the differences in the integer words instead of the FP64 pipe: 86 us).
+// 192^3 sphere of radius 48, 24 steps: 31.5 ms stepping every cell from its
+// definition, 1.59 ms with active blocks.
 constexpr int kBx = 32;
 template <int ND>
 using RdBlk = CellBlock<ND>;   // (rows of 32 cells per warp stepped 1.6 times as many warps)
@@ -174,7 +179,8 @@ __global__ void k_rd_list(RdGrid R, const unsigned char* __restrict__ act, int2*
 // Godunov gradient.  With y = s x the upwind difference along a direction is
 // max(0, y0 - min(y-, y+)) (the larger of the two one-sided squares), so a
 // direction costs a minimum, a subtraction and one fused multiply-add; signs
-// are tested and flipped in the integer words.
+// are tested and flipped in the integer words.  A neighbour that is NaN adds
+// no slope, as in the definition's maxima with 0.
 template <int ND>
 __device__ __forceinline__ double rd_step(double a, double x0, const double* xm, const double* xp,
                                           double invh, double dtau) {
@@ -185,8 +191,8 @@ __device__ __forceinline__ double rd_step(double a, double x0, const double* xm,
   for (int d = 0; d < ND; ++d) {
     const double ym = __longlong_as_double(__double_as_longlong(xm[d]) ^ sb);
     const double yp = __longlong_as_double(__double_as_longlong(xp[d]) ^ sb);
-    double m = y0 - (ym < yp ? ym : yp);
-    if (__double_as_longlong(m) < 0) m = 0.0;
+    double m = y0 - fmin(ym, yp);
+    if ((unsigned)__double2hiint(m) > 0x7ff00000u) m = 0.0;   // negative or NaN
     g = fma(m, m, g);
   }
   const double y = fma(-dtau, fma(sqrt(g), invh, -1.0), y0);
@@ -230,12 +236,14 @@ __global__ void __launch_bounds__(512) k_rd_step(Level L, RdGrid R, T dtau,
                                                  const T* __restrict__ cin, T* __restrict__ cout) {
   using B = RdBlk<ND>;
   const T h = (T)L.h, invh = (T)(1.0 / L.h), dtau_h = dtau / h;
-  const int3 lc = B::cell(threadIdx.x);
+  // blocks of fewer threads take a share of a cell block each
+  const int sub = B::threads / (int)blockDim.x, step = (int)gridDim.x / sub;
+  const int3 lc = B::cell((int)(blockIdx.x % sub * blockDim.x + threadIdx.x));
   const int lx = lc.x, ly = lc.y, lz = lc.z;
   const int lo[3] = {lx, ly, lz}, last[3] = {kBx - 1, B::by - 1, B::bz - 1};
   const size_t st[3] = {1, (size_t)L.nx, (size_t)L.nx * L.ny};
   const int count = list[0].x;
-  for (int q = blockIdx.x; q < count; q += gridDim.x) {
+  for (int q = (int)blockIdx.x / sub; q < count; q += step) {
     const int2 e = list[1 + q];
     const int b = e.x;
     const int i = (b % R.nbx) * kBx + lx, j = (b / R.nbx % R.nby) * B::by + ly,
@@ -452,9 +460,12 @@ static sfx_status redistance_blocks(sfx_ctx* c, const double* C, T* aux, T* a, T
   int2* list = (int2*)c->block_list;
   unsigned char* f0 = (unsigned char*)(list + nb + 1);
   unsigned char* f1 = f0 + nb;
-  // blocks of 512 threads in turn over the list, two to three per SM
   const int full = (int)std::min(nb, (size_t)c->sm_count * 64);
-  const int grid = (int)std::min(nb, (size_t)c->sm_count * 4);
+  // a step: resident blocks of 128 threads, each with a quarter of a cell
+  // block in turn (12 to an SM fit by registers)
+  constexpr int kStepThreads = 128;
+  const size_t sub = B::threads / kStepThreads;
+  const int grid = (int)std::min(nb * sub, (size_t)c->sm_count * 12 / sub * sub);
   const int sg = (int)std::min((nb + 255) / 256, (size_t)c->sm_count * 8);
   SFX_CUDA(cudaMemsetAsync(list, 0, sizeof(int2), s));
   SFX_KERNEL(c, K_PHASE, (k_rd_init<T, ND>), full, 512, s, L, R, C, aux, a, f0);
@@ -466,7 +477,7 @@ static sfx_status redistance_blocks(sfx_ctx* c, const double* C, T* aux, T* a, T
   }
   SFX_KERNEL(c, K_PHASE, k_rd_list, sg, 256, s, R, fi, list);
   for (int it = 0; it < iters; ++it) {
-    SFX_KERNEL(c, K_PHASE, (k_rd_step<T, ND>), grid, 512, s, L, R, (T)dtau, list, aux, a, b);
+    SFX_KERNEL(c, K_PHASE, (k_rd_step<T, ND>), grid, kStepThreads, s, L, R, (T)dtau, list, aux, a, b);
     std::swap(a, b);
   }
   SFX_KERNEL(c, K_PHASE, (k_rd_finish<T, ND>), full, 512, s, L, R, (T)dtau, iters, eps, fi, C, a,
