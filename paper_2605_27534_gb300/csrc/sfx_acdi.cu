@@ -25,9 +25,9 @@
 //     where phi saturates, and the surfactant step divides by phi + eta).
 // A cell that is not marked has |grad psi| < kAcdiKappa, so its normal is 0
 // whatever its last bits.  160^3 sphere: psi, normal and update 1.91 ms with
-// every cell in FP64 and six faces of a root and a quotient each, 0.42 ms with
-// a band of nine cells marked, 1.08 ms once the profile has spread over 96 % of
-// the box (cells 0.39, normals 0.14, update 0.51 ms).
+// every cell in FP64 and six faces of a root and a quotient each; now, with the
+// marks, 0.28 ms with a band of nine cells marked, 0.74 ms once the profile has
+// spread (after 40 steps: cells 0.29, normals 0.11, update 0.30 ms).
 //
 // SFX_F64 contexts (BITS) keep every rounding of the definition: on a plateau
 // of phi its last bits set how far the normal of the forces is faded in, and
@@ -61,6 +61,13 @@ __global__ void k_acdi_psi32(size_t n, const double* __restrict__ ps, float scal
     const float b = fminf(fmaxf((float)(1.0 - p), 0.0f), 1.0f);
     psi[c] = scale * logf(__fdividef(a + (float)kAcdiVeps, b + (float)kAcdiVeps));
   }
+}
+
+// fmin(fmax(v, 0), 1), NaN included, without the FP64 pipe
+__device__ __forceinline__ double clip01(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  if (b > 0x7ff0000000000000ULL) return 0.0;   // below 0 or NaN
+  return b < 0x3ff0000000000000ULL ? v : 1.0;
 }
 
 template <int ND>
@@ -112,7 +119,7 @@ __global__ void k_acdi_cell(Level L, const unsigned char* __restrict__ mark,
 #pragma unroll
   for (int q = 0; q < 2 * ND; ++q) any |= mark[o[q]];
   if (!any) return;
-  const double p = fmin(fmax(ps[c], 0.0), 1.0);
+  const double p = clip01(ps[c]);
   const double rc = (p + kAcdiVeps) / (1.0 - p + kAcdiVeps);
   g[c] = BITS ? rc : sqrt(rc);
   psi[c] = eps * log(rc);
@@ -189,60 +196,109 @@ __global__ void k_acdi_update_bits(Level L, const unsigned char* __restrict__ ma
     div += s * w * af;
   }
   const double v = pc + dt * div * invh;
-  phi[c] = clip ? fmin(fmax(v, 0.0), 1.0) : v;
+  phi[c] = clip ? clip01(v) : v;
 }
 
 // phi = phi* + dt/V sum_f (+-) A_f a_f; wall faces carry nothing and the
 // axis face has zero area.  k1 = dt zeta eps/h^2, k2 = dt zeta/(2h): with s =
 // r_L^(1/2) r_R^(1/2) and nbar = (n_L + n_R)/2 a face's sharpening flux
-// zeta/4 w_f nbar is zeta s/(1 + s)^2 (n_L + n_R)/2.
+// zeta/4 w_f nbar_f is zeta s/(1 + s)^2 (n_L + n_R)/2.
+//
+// A face's s/(1 + s)^2 costs a quotient, and six faces per cell took 84 of
+// the pass's FP64 instructions, so a block evaluates each face once: a thread
+// the minus sides of its cell, 272 threads (48 in 2D) the block's far sides,
+// both factors of the product handed over through shared memory (a cell still
+// fuses it into its own sum, so the bits are those of six faces per cell).
+// Rows of 40 doubles keep the two rows of a half warp in different banks.
+// 160^3 after 40 steps: 425 -> 304 us; after one 180 -> 145 us (with two instead
+// of three blocks per SM 335 and 165; clipping on the FP64 pipe 319 and 160).
 template <int ND, bool AXI>
-__global__ void k_acdi_update(Level L, const unsigned char* __restrict__ mark,
-                              const double* __restrict__ ps, const double* __restrict__ g,
-                              const double* __restrict__ nv, double k1, double k2, int clip,
-                              double* __restrict__ phi) {
+__global__ void __launch_bounds__(512, 3)
+k_acdi_update(Level L, const unsigned char* __restrict__ mark, const double* __restrict__ ps,
+              const double* __restrict__ g, const double* __restrict__ nv, double k1, double k2,
+              int clip, double* __restrict__ phi) {
+  using B = CellBlock<ND>;
+  constexpr int kRow = 40, kRows = ND == 3 ? B::by * (B::bz + 1) : B::by + 1;
+  __shared__ double sa[ND][kRows * kRow], sn[ND][kRows * kRow];
+  const size_t n = L.ncell();
+  const size_t st[3] = {1, (size_t)L.nx, (size_t)L.nx * L.ny};
+  const int3 l = B::cell(threadIdx.x);
   int x[3];
-  if (!CellBlock<ND>::at(L, blockIdx.x, x)) return;
-  const size_t c = cidx(L, x[0], x[1], x[2]), n = L.ncell();
+  const bool in = B::at(L, blockIdx.x, x);
+  const size_t c = in ? cidx(L, x[0], x[1], x[2]) : 0;
   // face area over V/h of the radial faces
   double wr[2] = {1.0, 1.0};
   if (AXI) {
     wr[0] = (double)(2 * x[0]) / (double)(2 * x[0] + 1);
     wr[1] = (double)(2 * x[0] + 2) / (double)(2 * x[0] + 1);
   }
-  size_t o[2 * ND];
-  bool has[2 * ND];
-  neighbours<ND>(L, x, c, o, has);
-  const double pc = ps[c];
-  double lap = 0.0, div = 0.0;
-#pragma unroll
-  for (int q = 0; q < 2 * ND; ++q) {
-    const double dp = ps[o[q]] - pc;      // 0 at a wall
-    lap = AXI && q < 2 ? fma(wr[q], dp, lap) : lap + dp;
-  }
-  const int mc = mark[c];
-  int mo[2 * ND], any = mc;
-#pragma unroll
-  for (int q = 0; q < 2 * ND; ++q) {
-    mo[q] = has[q] ? mark[o[q]] : 0;
-    any |= mo[q];
-  }
-  if (any) {
-    const double gc = g[c];
+  int any = 0;
+  double pc = 0.0, lap = 0.0, div = 0.0;
+  if (in) {
+    size_t o[2 * ND];
+    bool has[2 * ND];
+    neighbours<ND>(L, x, c, o, has);
+    any = mark[c];
+    pc = ps[c];
 #pragma unroll
     for (int q = 0; q < 2 * ND; ++q) {
-      if (!has[q] || !(mc | mo[q])) continue;
-      const double* nd = nv + (size_t)(q / 2) * n;
-      const double nn = (mc ? nd[c] : 0.0) + (mo[q] ? nd[o[q]] : 0.0);
-      const double u = 1.0 / fma(gc, g[o[q]], 1.0);   // 1/(1 + s); s/(1 + s)^2 = u - u^2
-      double a = fma(-u, u, u);
+      any |= mark[o[q]];
+      const double dp = ps[o[q]] - pc;      // 0 at a wall
+      lap = AXI && q < 2 ? fma(wr[q], dp, lap) : lap + dp;
+    }
+  }
+  const auto slot = [](int d, int lx, int ly, int lz) {
+    return (lz * (B::by + (d == 1)) + ly) * kRow + lx;
+  };
+  // s/(1 + s)^2 and n_L + n_R of the minus side of cell y in direction d
+  const auto face = [&](int d, int yx, int yy, int yz, int at) {
+    double a = 0.0, nn = 0.0;
+    const int yd = d == 0 ? yx : (d == 1 ? yy : yz);
+    if (yd > 0 && yx < L.nx && yy < L.ny && yz < L.nz) {
+      const size_t r = cidx(L, yx, yy, yz), m = r - st[d];
+      const int mr = mark[r], mm = mark[m];
+      if (mr | mm) {
+        const double* nd = nv + (size_t)d * n;
+        nn = (mr ? nd[r] : 0.0) + (mm ? nd[m] : 0.0);
+        const double u = 1.0 / fma(g[r], g[m], 1.0);   // 1/(1 + s); s/(1 + s)^2 = u - u^2
+        a = fma(-u, u, u);
+      }
+    }
+    sa[d][at] = a;
+    sn[d][at] = nn;
+  };
+  const bool sharp = __syncthreads_or(any);
+  if (sharp) {
+#pragma unroll
+    for (int d = 0; d < ND; ++d) face(d, x[0], x[1], x[2], slot(d, l.x, l.y, l.z));
+    const int x0 = x[0] - l.x, y0 = x[1] - l.y, z0 = x[2] - l.z, t = threadIdx.x;
+    constexpr int fy = B::bx * B::bz, fz = ND == 3 ? B::bx * B::by : 0;
+    if (t < fy) {
+      const int a = t % B::bx, e = t / B::bx;
+      face(1, x0 + a, y0 + B::by, z0 + e, slot(1, a, B::by, e));
+    } else if (t < fy + fz) {
+      const int a = (t - fy) % B::bx, e = (t - fy) / B::bx;
+      face(ND - 1, x0 + a, y0 + e, z0 + B::bz, slot(ND - 1, a, e, B::bz));
+    } else if (t < fy + fz + B::by * B::bz) {
+      const int a = (t - fy - fz) % B::by, e = (t - fy - fz) / B::by;
+      face(0, x0 + B::bx, y0 + a, z0 + e, slot(0, B::bx, a, e));
+    }
+    __syncthreads();
+  }
+  if (!in) return;
+  if (any) {
+#pragma unroll
+    for (int q = 0; q < 2 * ND; ++q) {
+      const int d = q / 2, p = q & 1;
+      const int at = slot(d, l.x + (p && d == 0), l.y + (p && d == 1), l.z + (p && d == 2));
+      double a = sa[d][at];
       if (AXI && q < 2) a *= wr[q];
-      div = fma(q & 1 ? -a : a, nn, div);
+      div = fma(p ? -a : a, sn[d][at], div);
     }
   }
   double v = fma(k1, lap, pc);
   if (any) v = fma(k2, div, v);
-  phi[c] = clip ? fmin(fmax(v, 0.0), 1.0) : v;
+  phi[c] = clip ? clip01(v) : v;
 }
 
 template <int ND, bool AXI>
