@@ -16,6 +16,12 @@
 // value comes from bcg_face2 and each cell sums its fluxes in the order of
 // k_advect2t_32 and of the batched kernels, so the result is theirs bit for
 // bit.
+//
+// What bounds it is issue (28 warp instructions per cell), once the loads are
+// out of the way: a thread holds its entries of the next plane in registers
+// while the block evaluates this one (64 registers, four blocks per SM; loaded
+// and stored in one go the block waited for them at its barrier on every
+// plane).  256^3: 498 -> 469 us, 157 x 131 x 117: 112 -> 89 us.
 #pragma once
 
 #include "sfx_df.cuh"
@@ -25,7 +31,6 @@ namespace sfx {
 namespace {
 
 constexpr int kA3X = 32, kA3Y = 8;        // threads; cells (kA3X - 1) x (kA3Y - 1)
-constexpr int kA3Z = 16;                  // planes per block
 constexpr int kVX = kA3X + 3, kVY = kA3Y + 3;   // values: x [ox - 2, + kVX), y [oy - 2, + kVY)
 constexpr int kUX = kA3X + 1, kUY = kA3Y + 1;   // velocities: x [ox - 1, + kUX), y [oy - 1, + kUY)
 constexpr int kA3Ring = 4;                // planes k - 1 .. k + 2 (and k0 - 2 first)
@@ -69,34 +74,52 @@ __device__ __forceinline__ Adv3Stage adv3_stage_init(const Level& L, int ox, int
   return S;
 }
 
-// Stage plane m (values clamped to the grid, velocities zero outside it).
-__device__ __forceinline__ void adv3_stage(const Adv32& A, const Adv3Stage& S,
-                                           const float2* __restrict__ f,
-                                           const float2* __restrict__ F, Adv3Plane& P, int m) {
+// A thread's entries of plane m (values clamped to the grid, velocities zero
+// outside it), held in registers between their load and their place in the
+// ring.
+struct Adv3Regs {
+  float2 f[2], F[2];
+  float u[3][2];
+};
+__device__ __forceinline__ void adv3_load(const Adv32& A, const Adv3Stage& S,
+                                          const float2* __restrict__ f,
+                                          const float2* __restrict__ F, int m, Adv3Regs& q) {
   const Level& L = A.L;
   const unsigned plane = (unsigned)L.nx * (unsigned)L.ny;
   const unsigned vz = (unsigned)min(max(m, 0), L.nz - 1) * plane;
-  float2* pv = &P.v[0][0];
 #pragma unroll
   for (int r = 0; r < 2; ++r)
     if (S.vpos[r] >= 0) {
       const unsigned c = vz + S.vbase[r];
-      pv[S.vpos[r]] = make_float2(df_val(f[c]), df_val(F[c]));
+      q.f[r] = f[c];
+      q.F[r] = F[c];
     }
   const bool m_in = m >= 0 && m < L.nz, mz_in = m >= 0 && m <= L.nz;
   const unsigned zx = (unsigned)m * (unsigned)L.ny * (unsigned)(L.nx + 1);
   const unsigned zy = (unsigned)m * (unsigned)(L.ny + 1) * (unsigned)L.nx;
   const unsigned zz = (unsigned)m * plane;
+#pragma unroll
+  for (int r = 0; r < 2; ++r)
+    if (S.upos[r] >= 0) {
+      q.u[0][r] = (m_in && S.uin[0][r]) ? A.u[0][zx + S.ubase[0][r]] : 0.0f;
+      q.u[1][r] = (m_in && S.uin[1][r]) ? A.u[1][zy + S.ubase[1][r]] : 0.0f;
+      q.u[2][r] = (mz_in && S.uin[2][r]) ? A.u[2][zz + S.ubase[2][r]] : 0.0f;
+    }
+}
+__device__ __forceinline__ void adv3_put(const Adv3Stage& S, const Adv3Regs& q, Adv3Plane& P) {
+  float2* pv = &P.v[0][0];
   float* px = &P.ux[0][0];
   float* py = &P.uy[0][0];
   float* pz = &P.uz[0][0];
 #pragma unroll
-  for (int r = 0; r < 2; ++r)
+  for (int r = 0; r < 2; ++r) {
+    if (S.vpos[r] >= 0) pv[S.vpos[r]] = make_float2(df_val(q.f[r]), df_val(q.F[r]));
     if (S.upos[r] >= 0) {
-      px[S.upos[r]] = (m_in && S.uin[0][r]) ? A.u[0][zx + S.ubase[0][r]] : 0.0f;
-      py[S.upos[r]] = (m_in && S.uin[1][r]) ? A.u[1][zy + S.ubase[1][r]] : 0.0f;
-      pz[S.upos[r]] = (mz_in && S.uin[2][r]) ? A.u[2][zz + S.ubase[2][r]] : 0.0f;
+      px[S.upos[r]] = q.u[0][r];
+      py[S.upos[r]] = q.u[1][r];
+      pz[S.upos[r]] = q.u[2][r];
     }
+  }
 }
 
 // The weighted pair fluxes u v of one face for both fields, (f.hi, f.lo,
@@ -137,7 +160,9 @@ __device__ __forceinline__ float4 adv3_face(const Adv32& A, Slot R, float bc1, f
   return make_float4(p1, fmaf(u, v1, -p1), p2, fmaf(u, v2, -p2));
 }
 
-__global__ void __launch_bounds__(kA3X* kA3Y)
+// ZC planes per block (a constant: the loop's slots and offsets fold)
+template <int ZC>
+__global__ void __launch_bounds__(kA3X* kA3Y, 4)
 k_advect3s_32(Adv32 A, const float2* __restrict__ f, const float2* __restrict__ F, float bc_f,
               float bc_F, float2* __restrict__ fo, float2* __restrict__ Fo) {
   __shared__ Adv3Plane ring[kA3Ring];
@@ -147,12 +172,17 @@ k_advect3s_32(Adv32 A, const float2* __restrict__ f, const float2* __restrict__ 
   const int tx = threadIdx.x % kA3X, ty = threadIdx.x / kA3X;
   const int ox = blockIdx.x * (kA3X - 1), oy = blockIdx.y * (kA3Y - 1);
   const int i = ox + tx, j = oy + ty;
-  const int k0 = blockIdx.z * kA3Z, k1 = min(k0 + kA3Z, L.nz);
+  const int k0 = blockIdx.z * ZC, k1 = min(k0 + ZC, L.nz);
   const bool cell = tx < kA3X - 1 && ty < kA3Y - 1 && i < L.nx && j < L.ny;
-  auto R = [&](int m) -> Adv3Plane& { return ring[(m - k0 + 2 * kA3Ring) & (kA3Ring - 1)]; };
+  auto R = [&](int m) -> Adv3Plane& { return ring[m & (kA3Ring - 1)]; };
   const Adv3Stage St = adv3_stage_init(L, ox, oy);
   // planes k0 - 2 .. k0 + 1 for the first z face and the first plane
-  for (int m = k0 - 2; m <= k0 + 1; ++m) adv3_stage(A, St, f, F, R(m), m);
+  Adv3Regs pre;
+  for (int m = k0 - 2; m <= k0 + 1; ++m) {
+    adv3_load(A, St, f, F, m, pre);
+    adv3_put(St, pre, R(m));
+  }
+  adv3_load(A, St, f, F, k0 + 2, pre);
   __syncthreads();
   float4 zm = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   float uzm = 0.0f;
@@ -164,8 +194,16 @@ k_advect3s_32(Adv32 A, const float2* __restrict__ f, const float2* __restrict__ 
   for (int k = k0; k < k1; ++k) {
     // plane k + 2 into the slot plane k - 2 left (last read in step k - 1:
     // step k reads planes k - 1 .. k + 2)
-    adv3_stage(A, St, f, F, R(k + 2), k + 2);
+    adv3_put(St, pre, R(k + 2));
     __syncthreads();
+    // on their way while plane k is evaluated
+    if (k + 1 < k1) adv3_load(A, St, f, F, k + 3, pre);
+    float2 fc = make_float2(0.0f, 0.0f), Fc = fc;
+    if (cell) {
+      const ix c = cidx32(L, i, j, k);
+      fc = f[c];
+      Fc = F[c];
+    }
     const Adv3Plane& P = R(k);
     float4 qx = make_float4(0.0f, 0.0f, 0.0f, 0.0f), qy = qx;
     if (ty < kA3Y - 1 && i <= L.nx && j < L.ny)
@@ -192,11 +230,24 @@ k_advect3s_32(Adv32 A, const float2* __restrict__ f, const float2* __restrict__ 
       const float2 i1 = df_mul_f(df_mul_f(S1, -A.dt), A.invh);
       const float2 i2 = df_mul_f(df_mul_f(S2, -A.dt), A.invh);
       const ix c = cidx32(L, i, j, k);
-      fo[c] = df_add2(f[c], i1);
-      Fo[c] = df_add2(F[c], i2);
+      fo[c] = df_add2(fc, i1);
+      Fo[c] = df_add2(Fc, i2);
     }
     __syncthreads();
   }
+}
+
+// Planes per block: 16, which amortise the planes staged ahead of a chunk and
+// leave the scheduler many blocks to even out; 8 or 4 where the grid would
+// not fill the chip's four blocks per SM once.  64^3: 29 us with 16, 19
+// with 4; 40 x 33 x 50: 29 and 10.  (Chunks of one wave on large grids: 421
+// against 362 us at 232^3; a chunk known at run time: 488 against 469 us at
+// 256^3.)
+inline int advect3s_chunk(const Level& L, int sms) {
+  const long long tiles = (long long)((L.nx + kA3X - 2) / (kA3X - 1)) *
+                          ((L.ny + kA3Y - 2) / (kA3Y - 1));
+  const long long slots = 4LL * sms, z = (tiles * L.nz + slots - 1) / slots;
+  return z > 8 ? 16 : (z > 4 ? 8 : 4);
 }
 
 }  // namespace

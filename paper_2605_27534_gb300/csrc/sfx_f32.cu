@@ -1808,11 +1808,13 @@ sfx_status step_f32(sfx_ctx* c, const sfx_params* pr, const double* phi_in, cons
                   (unsigned)((L.ny + kAdvY - 2) / (kAdvY - 1)),
                   L.geom == SFX_CART3D ? (unsigned)((L.nz + kAdvZ - 1) / kAdvZ) : 1u);
     if (L.geom == SFX_CART3D && c->f32.adv_staged) {
+      const int zc = advect3s_chunk(L, c->sm_count);
       const dim3 a3((unsigned)((L.nx + kA3X - 2) / (kA3X - 1)),
                     (unsigned)((L.ny + kA3Y - 2) / (kA3Y - 1)),
-                    (unsigned)((L.nz + kA3Z - 1) / kA3Z));
-      SFX_KERNEL(c, K_ADVECT, k_advect3s_32, a3, kA3X * kA3Y, s, A, f, F, (float)pr->bc_f,
-                 (float)pr->bc_F, fs, Fs);
+                    (unsigned)((L.nz + zc - 1) / zc));
+      const auto adv = zc == 16 ? &k_advect3s_32<16> : (zc == 8 ? &k_advect3s_32<8> : &k_advect3s_32<4>);
+      SFX_KERNEL(c, K_ADVECT, adv, a3, kA3X * kA3Y, s, A, f, F, (float)pr->bc_f, (float)pr->bc_F,
+                 fs, Fs);
     } else {
       SFX_KERNEL(c, K_ADVECT, k_advect2t_32, ag, kAdvX * kAdvY, s, A, f, F, (float)pr->bc_f,
                  (float)pr->bc_F, fs, Fs);
