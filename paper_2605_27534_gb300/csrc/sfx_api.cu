@@ -198,7 +198,6 @@ sfx_status sfx_ctx_create(const sfx_grid* grid, int precision, sfx_ctx** out) {
     if (e != cudaSuccess) st = cuda_fail(e);
   }
   if (st == SFX_OK) st = dalloc(c, &c->d_norms, 16);
-  if (st == SFX_OK) st = dalloc(c, &c->d_sums, 8);
   if (st == SFX_OK && precision == SFX_F32) st = f32_ensure_scratch(c);
   if (st == SFX_OK) {
     c->d_flag = (int*)(c->d_norms + 7);

@@ -1504,15 +1504,26 @@ __global__ void k_restore32(size_t n, const int* __restrict__ ok, const float2* 
   }
 }
 
-// Initial guess of the Newton iteration: x* plus the implicit increment of
-// the previous step (a smooth solution changes little from step to step).
-__global__ void k_predict32(size_t n, const float2* __restrict__ fs, const float2* __restrict__ Fs,
-                            const float* __restrict__ df, const float* __restrict__ dF,
-                            float2* __restrict__ f, float2* __restrict__ F) {
+// The start of a Newton solve: x* = x without a flow (`keep`), the initial
+// guess x* plus the implicit increment of the previous step where one predicts
+// it (df not null; a smooth solution changes little from step to step), and
+// the solve's flags.  One launch: two copies, a memory operation and the
+// prediction took some 15 us of a no-flow step, 2 us of it work.
+__global__ void k_start32(size_t n, bool keep, float2* fs, float2* Fs, const float* __restrict__ df,
+                          const float* __restrict__ dF, float2* f, float2* F,
+                          int* __restrict__ flag) {
+  if (blockIdx.x == 0 && threadIdx.x < 16) flag[threadIdx.x] = 0;
   for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
        c += (size_t)gridDim.x * blockDim.x) {
-    f[c] = df_add(fs[c], df[c]);
-    F[c] = df_add(Fs[c], dF[c]);
+    const float2 a = keep ? f[c] : fs[c], b = keep ? F[c] : Fs[c];
+    if (keep) {
+      fs[c] = a;
+      Fs[c] = b;
+    }
+    if (df) {
+      f[c] = df_add(a, df[c]);
+      F[c] = df_add(b, dF[c]);
+    }
   }
 }
 
@@ -1552,7 +1563,7 @@ RowGrid row_grid(const Level& L, int sms) {
 sfx_status solve_newton32(sfx_ctx* c, const Nw32& p, const float* phi, float* const* Bf,
                           float* const* BF, float2*& fc, float2*& fo, float2*& Fc, float2*& Fo,
                           const float2* fs, const float2* Fs, const sfx_solve_opts* o,
-                          bool predicted, bool from_star, int mgl, const Mg32Coef& kc,
+                          bool predicted, bool from_star, bool flags_clear, int mgl, const Mg32Coef& kc,
                           int* iters, bool* conv, float* nrm, cudaStream_t s) {
   const Level& L = p.L;
   const size_t n = L.ncell();
@@ -1607,7 +1618,7 @@ sfx_status solve_newton32(sfx_ctx* c, const Nw32& p, const float* phi, float* co
   const int fast_max = c->f32.fast_resid;
   const bool merged = tile2d != nullptr;   // the 2D iteration of three calls
   const auto resid2d = L.geom == SFX_AXISYM ? &k_resid2d_32<SFX_AXISYM> : &k_resid2d_32<SFX_PLANAR2D>;
-  SFX_CUDA(cudaMemsetAsync(flag, 0, 16 * sizeof(int), s));
+  if (!flags_clear) SFX_CUDA(cudaMemsetAsync(flag, 0, 16 * sizeof(int), s));
   if (fast_max <= 0 && !merged) SFX_KERNEL(c, K_OTHER, k_set32, 1, 32, s, flag + 4, 1);
   // Each iteration: the residual pass (which also does the first red
   // half-sweep of the correction, from zero), a device-side convergence
@@ -1820,15 +1831,17 @@ sfx_status step_f32(sfx_ctx* c, const sfx_params* pr, const double* phi_in, cons
                  (float)pr->bc_F, fs, Fs);
     }
     SFX_LAUNCH_CHECK();
-  } else {
+  } else if (c->f32.solver != 1) {
     SFX_CUDA(cudaMemcpyAsync(fs, f, n * sizeof(float2), cudaMemcpyDeviceToDevice, s));
     SFX_CUDA(cudaMemcpyAsync(Fs, F, n * sizeof(float2), cudaMemcpyDeviceToDevice, s));
   }
   // the Newton solver starts from x* in place (no copy into f, F)
   const bool from_star = ux && !predict && c->f32.solver == 1;
-  if (predict) {
-    SFX_KERNEL(c, K_SETUP, k_predict32, blocks_for(n, 256), 256, s, n, fs, Fs, c->f32.inc_f,
-               c->f32.inc_F, f, F);
+  const bool start = c->f32.solver == 1 && (predict || !ux);
+  if (start) {
+    SFX_KERNEL(c, K_SETUP, k_start32, blocks_for(n, 256), 256, s, n, !ux, fs, Fs,
+               predict ? c->f32.inc_f : nullptr, predict ? c->f32.inc_F : nullptr, f, F,
+               c->f32.flag);
     SFX_LAUNCH_CHECK();
   } else if (ux && !from_star) {
     SFX_CUDA(cudaMemcpyAsync(f, fs, n * sizeof(float2), cudaMemcpyDeviceToDevice, s));
@@ -1873,7 +1886,7 @@ sfx_status step_f32(sfx_ctx* c, const sfx_params* pr, const double* phi_in, cons
                                     : sor_omega(pr->DF, dt, L.h, pr->eps, L.ndim());
       }
       const Mg32Coef kc{(float)pr->Df, (float)pr->DF, pf.inv_dt, pf.kd, pr->literal_upwind};
-      st = solve_newton32(c, pw, phi, Bf, BF, fc, fo, Fc, Fo, fs, Fs, o, predict, from_star, mgl,
+      st = solve_newton32(c, pw, phi, Bf, BF, fc, fo, Fc, Fo, fs, Fs, o, predict, from_star, start, mgl,
                           kc, &it, &dconv, dn, s);
     } else {
       st = solve_dc32(c, pf, pF, phi, Bf, BF, fc, fo, Fc, Fo, fs, Fs, o, &it, &dconv, dn, s);
@@ -1988,9 +2001,8 @@ sfx_status totals32(sfx_ctx* c, const void* const* fields, int nf, double* out, 
   // 1024 cells per block at least: a block's FP64 reduction takes as long
   const size_t nblk = std::min((size_t)kTotalsBlocks, (L.ncell() + 1023) / 1024);
   SFX_KERNEL(c, K_TOTALS, k_totals32, dim3((unsigned)nblk, (unsigned)nf), kTotalsThreads, s, L, f,
-             scale, c->partials, c->tickets, c->d_sums);
+             scale, c->partials, c->tickets, c->h_sums);
   SFX_LAUNCH_CHECK();
-  SFX_CUDA(cudaMemcpyAsync(c->h_sums, c->d_sums, nf * sizeof(double), cudaMemcpyDeviceToHost, s));
   SFX_CUDA(cudaStreamSynchronize(s));
   memcpy(out, c->h_sums, nf * sizeof(double));
   return SFX_OK;

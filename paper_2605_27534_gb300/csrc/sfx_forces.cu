@@ -292,9 +292,8 @@ sfx_status totals(sfx_ctx* c, const double* const* fields, int nf, double* out, 
   TotalFields f{};
   for (int i = 0; i < nf; ++i) f.x[i] = fields[i];
   SFX_KERNEL(c, K_TOTALS, k_totals, dim3(totals_blocks(L.ncell()), nf), kTotThreads, s, L, f,
-             c->partials, c->tickets, c->d_sums);
+             c->partials, c->tickets, c->h_sums);
   SFX_LAUNCH_CHECK();
-  SFX_CUDA(cudaMemcpyAsync(c->h_sums, c->d_sums, nf * sizeof(double), cudaMemcpyDeviceToHost, s));
   SFX_CUDA(cudaStreamSynchronize(s));
   memcpy(out, c->h_sums, nf * sizeof(double));
   return SFX_OK;

@@ -215,8 +215,8 @@ struct sfx_ctx {
                                           // FP32 sweeps (7: d_flag), 8..15 the FP32 Newton
                                           // solve's two norm buffers
   unsigned long long* h_norms = nullptr;  // pinned mirror
-  double* d_sums = nullptr;          // compensated totals (device)
-  double* h_sums = nullptr;          // pinned mirror
+  double* h_sums = nullptr;          // compensated totals (pinned host memory, written by the
+                                     // reduction itself: a copy behind it took 5 us of a step)
   int* d_flag = nullptr;
   std::vector<void*> allocations;
   sfx::Prof prof;
@@ -293,7 +293,9 @@ sfx_status drift_faces64(sfx_ctx* c, const double* phi, double Df, double DF, do
 // from_star).  It ends with *conv false when it should be left to the Picard
 // solver.
 bool newton64_eligible(const sfx_ctx* c, const sfx_params* p, double dt, const sfx_solve_opts* o);
-sfx_status newton64_prepare(sfx_ctx* c, const sfx_params* p, const double* phi, cudaStream_t s);
+// `copy`: (f*, F*) = (f, F) too (no flow).
+sfx_status newton64_prepare(sfx_ctx* c, const sfx_params* p, const double* phi, const double* f,
+                            const double* F, bool copy, cudaStream_t s);
 sfx_status newton64_solve(sfx_ctx* c, const sfx_params* p, double* f, double* F, double dt,
                           bool from_star, const sfx_solve_opts* o, int* iters, double* rel,
                           bool* conv, cudaStream_t s);

@@ -42,8 +42,10 @@ namespace {
 // per thread and direction took two normals per face).  Where phi is flat
 // bit for bit the normal is zero and costs no FP64 arithmetic.
 // Optional outputs: H2 the faces in half precision, c1 = r_a/(phi + eta) and
-// finf = Gamma_inf phi (1 - phi)/eps per cell.
+// finf = Gamma_inf phi (1 - phi)/eps per cell, and what a solve starts with
+// (a memory operation and two copies of their own took 10 us of a 128^2 step).
 constexpr int kSX = 32, kSY = 4;
+constexpr int kCtlWords = 8;   // of Ctl64
 
 struct Setup64 {
   Level L;
@@ -54,6 +56,10 @@ struct Setup64 {
   __half2* H[3];
   double* c1;
   double* finf;
+  // the start of a solve: its control words cleared, x* = x without a flow
+  int* ctl;
+  const double* x[2];
+  double* xs[2];
 };
 
 __device__ __forceinline__ bool bits_eq(double a, double b) {
@@ -98,6 +104,8 @@ __global__ void __launch_bounds__(kSX * kSY * (ND == 3 ? 4 : 1)) k_setup64(Setup
   __shared__ double sn[ND][HZ][HY][HX];
   const Level& L = q.L;
   const int x0 = blockIdx.x * kSX, y0 = blockIdx.y * kSY, z0 = blockIdx.z * BZ;
+  if (q.ctl && (blockIdx.x | blockIdx.y | blockIdx.z) == 0 && threadIdx.x < kCtlWords)
+    q.ctl[threadIdx.x] = 0;
   const double inv2h = 0.5 / L.h, inv_eps = 1.0 / q.eps;
   for (int t = threadIdx.x; t < HX * HY * HZ; t += blockDim.x) {
     const int lx = t % HX, ly = t / HX % HY, lz = t / (HX * HY);
@@ -144,6 +152,10 @@ __global__ void __launch_bounds__(kSX * kSY * (ND == 3 ? 4 : 1)) k_setup64(Setup
     q.c1[c] = q.ka / (p + q.eta);
     q.finf[c] = q.ginf * (p * (1.0 - p)) * inv_eps;
   }
+  if (q.xs[0]) {
+    q.xs[0][c] = q.x[0][c];
+    q.xs[1][c] = q.x[1][c];
+  }
 }
 
 // --------------------------------------------------------------- residual
@@ -171,6 +183,7 @@ struct Ctl64 {
   int stop;              // its correction has been added: no further sweeps
   int iter;              // iterations evaluated
 };
+static_assert(sizeof(Ctl64) == kCtlWords * sizeof(int), "control words");
 
 // (1/h) sum of +-G over the cell's faces of one field, G = D (a_R - a_L)/h
 // + B a_up.  The diffusive part is gathered as D/h (sum of neighbours -
@@ -448,7 +461,6 @@ sfx_status solve(sfx_ctx* c, const Newton64& q, double* f, double* F, bool from_
                                   (int)kT2Smem));
   }
   *conv = false;
-  SFX_CUDA(cudaMemsetAsync(ctl, 0, sizeof(Ctl64), s));
   float first = 0.0f;
   // the host reads an iteration's norms while the GPU works on the next one
   for (int it = 1; it <= cap + 1; ++it) {
@@ -508,7 +520,7 @@ sfx_status solve(sfx_ctx* c, const Newton64& q, double* f, double* F, bool from_
 sfx_status drift_faces64(sfx_ctx* c, const double* phi, double Df, double DF, double eps,
                          double* const* Bf, double* const* BF, cudaStream_t s) {
   const Level& L = c->lev[0].lv;
-  Setup64 q{L, phi, Df, DF, eps, 0.0, 0.0, 0.0, {}, {}, {}, nullptr, nullptr};
+  Setup64 q{L, phi, Df, DF, eps, 0.0, 0.0, 0.0, {}, {}, {}, nullptr, nullptr, nullptr, {}, {}};
   for (int d = 0; d < L.ndim(); ++d) {
     q.Bf[d] = Bf[d];
     q.BF[d] = BF[d];
@@ -533,14 +545,16 @@ bool newton64_eligible(const sfx_ctx* c, const sfx_params* p, double dt, const s
          nz <= 65535 && std::max(p->Df, p->DF) * dt <= L.h * L.h;
 }
 
-// Drift faces (into the finest level's arrays) and the coefficients of the
-// Newton solve.
-sfx_status newton64_prepare(sfx_ctx* c, const sfx_params* p, const double* phi, cudaStream_t s) {
+// Drift faces (into the finest level's arrays), the coefficients of the Newton
+// solve and its cleared control words.
+sfx_status newton64_prepare(sfx_ctx* c, const sfx_params* p, const double* phi, const double* f,
+                            const double* F, bool copy, cudaStream_t s) {
   sfx_status st = ensure(c);
   if (st != SFX_OK) return st;
   const Level& L = c->lev[0].lv;
   LevelData& D = c->lev[0];
-  Setup64 q{L, phi, p->Df, p->DF, p->eps, p->ka, p->eta, p->gamma_inf, {}, {}, {}, D.lam, D.b};
+  Setup64 q{L, phi, p->Df, p->DF, p->eps, p->ka, p->eta, p->gamma_inf, {}, {}, {}, D.lam, D.b,
+            (int*)c->n64.ctl, {f, F}, {copy ? c->fstar : nullptr, copy ? c->Fstar : nullptr}};
   for (int d = 0; d < L.ndim(); ++d) {
     q.Bf[d] = D.B[0][d];
     q.BF[d] = D.B[1][d];

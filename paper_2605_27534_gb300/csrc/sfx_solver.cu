@@ -582,7 +582,7 @@ sfx_status step_impl(sfx_ctx* c, const sfx_params* p, const double* phi, const v
   const size_t n = L.ncell();
   // drift faces of both problems (phi is fixed over the step)
   const bool newton = newton64_eligible(c, p, dt, o);
-  sfx_status ds = newton ? newton64_prepare(c, p, phi, s)
+  sfx_status ds = newton ? newton64_prepare(c, p, phi, f, F, !ux, s)
                          : drift_faces64(c, phi, p->Df, p->DF, p->eps, c->lev[0].B[0],
                                          c->lev[0].B[1], s);
   if (ds != SFX_OK) return ds;
@@ -591,7 +591,7 @@ sfx_status step_impl(sfx_ctx* c, const sfx_params* p, const double* phi, const v
     const sfx_status st = advect2(c, (const double*)ux, (const double*)uy, (const double*)uz, dt, f,
                                   F, p->bc_f, p->bc_F, c->fstar, c->Fstar, s);
     if (st != SFX_OK) return st;
-  } else {
+  } else if (!newton) {
     SFX_CUDA(cudaMemcpyAsync(c->fstar, f, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
     SFX_CUDA(cudaMemcpyAsync(c->Fstar, F, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
   }
