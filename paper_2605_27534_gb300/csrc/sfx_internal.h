@@ -308,8 +308,8 @@ sfx_status capillary(sfx_ctx* c, const sfx_params* p, const double* phi, const v
 // sfx_forces.cu: ctx->cut_list (allocated on first use; each pass fills it
 // anew), null where a grid's cells do not fit 32-bit indices
 sfx_status cut_list(sfx_ctx* c, unsigned** list);
-// sfx_phase.cu: ctx->block_list for nb blocks of cells: a count, nb int2 and
-// two flags per block (allocated on first use; each pass fills it anew)
+// sfx_phase.cu: ctx->block_list for nb blocks of cells: a count, nb int2, six
+// doubles and two flags per block at least (allocated on first use; each pass fills it anew)
 sfx_status block_list(sfx_ctx* c, size_t nb);
 // sfx_vof.cu
 sfx_status vof_advect(sfx_ctx* c, const void* ux, const void* uy, const void* uz, double dt,

@@ -26,6 +26,13 @@ __device__ __forceinline__ double phi_of(double chi, double eps) {
   return 0.5 * (1.0 - tanh(chi / (2.0 * eps)));
 }
 
+__device__ __forceinline__ bool same_bits(double a, double b) {
+  return __double_as_longlong(a) == __double_as_longlong(b);
+}
+__device__ __forceinline__ bool same_bits(float a, float b) {
+  return __float_as_int(a) == __float_as_int(b);
+}
+
 template <typename T> __device__ __forceinline__ T tiny_pos();
 template <> __device__ __forceinline__ double tiny_pos<double>() { return 1e-300; }
 template <> __device__ __forceinline__ float tiny_pos<float>() { return 1e-30f; }
@@ -72,7 +79,7 @@ __device__ __forceinline__ bool redist_cut(int nd, T s0, const T* zm, const T* z
 // threads per SM, of which three fit: 78 us, the SMs active 71 % of it; minima
 // of the differences in the integer words instead of the FP64 pipe: 86 us).
 // 192^3 sphere of radius 48, 24 steps: 31.5 ms stepping every cell from its
-// definition, 1.59 ms with active blocks.
+// definition, 1.59 ms with active blocks (the whole phase field 1.93 ms).
 constexpr int kBx = 32;
 template <int ND>
 using RdBlk = CellBlock<ND>;   // (rows of 32 cells per warp stepped 1.6 times as many warps)
@@ -88,13 +95,38 @@ template <typename T>
 __device__ __forceinline__ T rd_inf();
 template <> __device__ __forceinline__ double rd_inf<double>() { return __longlong_as_double(0x7ff0000000000000LL); }
 template <> __device__ __forceinline__ float rd_inf<float>() { return __int_as_float(0x7f800000); }
+// an infinity of x's sign, 0 where x is 0 or NaN (doubles by their integer
+// words)
+__device__ __forceinline__ double signed_inf(double x) {
+  const long long b = __double_as_longlong(x), m = b & 0x7fffffffffffffffLL;
+  if (m == 0 || m > 0x7ff0000000000000LL) return 0.0;
+  return __longlong_as_double(0x7ff0000000000000LL | (b ^ m));
+}
+__device__ __forceinline__ float signed_inf(float x) {
+  return x > 0.0f ? rd_inf<float>() : (x < 0.0f ? -rd_inf<float>() : 0.0f);
+}
+
+// What a uniform field of C = 0 and of C = 1 gives after all steps.
+struct RdUniform {
+  double chi[2], phi[2], delta[2];
+};
+
+template <typename T>
+__device__ __forceinline__ T rd_uniform(double h, double C, T dtau, int iters) {
+  T x = (T)(2.0 * h * (C - 0.5));
+  const T sg = x > (T)0 ? (T)1 : (x < (T)0 ? (T)-1 : (T)0);
+  for (int q = 0; q < iters; ++q) x = x + dtau * sg;
+  return x;
+}
 
 // chi0 (the first iterate) and aux of every cell; rough[b] = 1 where a cell
-// of block b differs from a face neighbour in C.
+// of block b differs from a face neighbour in C.  The last block also fills
+// uni for the last pass.
 template <typename T, int ND>
 __global__ void __launch_bounds__(512) k_rd_init(Level L, RdGrid R, const double* __restrict__ C,
                                                  T* __restrict__ aux, T* __restrict__ chi,
-                                                 unsigned char* __restrict__ rough) {
+                                                 unsigned char* __restrict__ rough, T dtau,
+                                                 int iters, double eps, RdUniform* uni) {
   using B = RdBlk<ND>;
   const int nb = R.nbx * R.nby * R.nbz;
   const int3 lc = B::cell(threadIdx.x);
@@ -126,7 +158,7 @@ __global__ void __launch_bounds__(512) k_rd_init(Level L, RdGrid R, const double
           q[d] = fmax(fmax(fabs(zp - zm) * (T)0.5, fabs(zp - s0)), fabs(s0 - zm));
         }
       }
-      T a = s0 > (T)0 ? rd_inf<T>() : (s0 < (T)0 ? -rd_inf<T>() : (T)0);
+      T a = signed_inf(s0);
       if (cut) {
         T dsum = 0;
 #pragma unroll
@@ -138,6 +170,12 @@ __global__ void __launch_bounds__(512) k_rd_init(Level L, RdGrid R, const double
     }
     diff = __syncthreads_or(diff);
     if (threadIdx.x == 0) rough[b] = diff ? 1 : 0;
+  }
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x < 2) {
+    const double x = (double)rd_uniform<T>(L.h, (double)threadIdx.x, dtau, iters), p = phi_of(x, eps);
+    uni->chi[threadIdx.x] = x;
+    uni->phi[threadIdx.x] = p;
+    uni->delta[threadIdx.x] = p * (1.0 - p) / eps;
   }
 }
 
@@ -213,12 +251,6 @@ __device__ __forceinline__ float rd_step(float a, float x0, const float* xm, con
   return x0 - dtau * sg * (sqrtf(g) - 1.0f);
 }
 
-__device__ __forceinline__ bool same_bits(double a, double b) {
-  return __double_as_longlong(a) == __double_as_longlong(b);
-}
-__device__ __forceinline__ bool same_bits(float a, float b) {
-  return __float_as_int(a) == __float_as_int(b);
-}
 __device__ __forceinline__ bool is_inf_bits(double a) {
   return (__double_as_longlong(a) & 0x7fffffffffffffffLL) == 0x7ff0000000000000LL;
 }
@@ -278,10 +310,15 @@ __global__ void __launch_bounds__(512) k_rd_step(Level L, RdGrid R, T dtau,
 
 // chi, phi and delta (may be null) of every cell: active blocks from the
 // iterate, the others from `iters` steps of a uniform field, taken once per
-// block.
+// block.  A tanh and two quotients are some sixty FP64 instructions, and
+// half of the cells of active blocks are out of the interface's reach (the
+// blocks are long in x, the reach is a distance in the 1-norm): those hold
+// one of the two values of uni, and warps of them evaluate nothing.  192^3:
+// 350 -> 181 us.
 template <typename T, int ND>
 __global__ void __launch_bounds__(512) k_rd_finish(Level L, RdGrid R, T dtau, int iters, double eps,
                                                    const unsigned char* __restrict__ act,
+                                                   const RdUniform* __restrict__ uni,
                                                    const double* C, const T* it, double* chi,
                                                    double* phi, double* delta) {
   using B = RdBlk<ND>;
@@ -289,16 +326,22 @@ __global__ void __launch_bounds__(512) k_rd_finish(Level L, RdGrid R, T dtau, in
   const int nb = R.nbx * R.nby * R.nbz;
   const int3 lc = B::cell(threadIdx.x);
   const int lx = lc.x, ly = lc.y, lz = lc.z;
+  const RdUniform U = *uni;
   for (int b = blockIdx.x; b < nb; b += gridDim.x) {
     const int i0 = (b % R.nbx) * kBx, j0 = (b / R.nbx % R.nby) * B::by, k0 = b / R.nbx / R.nby * B::bz;
     const bool active = act[b];
     if (!active && threadIdx.x == 0) {
-      T x = (T)(2.0 * L.h * (C[cidx(L, i0, j0, k0)] - 0.5));
-      const T sg = x > (T)0 ? (T)1 : (x < (T)0 ? (T)-1 : (T)0);
-      for (int q = 0; q < iters; ++q) x = x + dtau * sg;
-      u[0] = (double)x;
-      u[1] = phi_of(u[0], eps);
-      u[2] = u[1] * (1.0 - u[1]) / eps;
+      const double c0 = C[cidx(L, i0, j0, k0)];
+      const int one = same_bits(c0, 1.0);
+      if (one || same_bits(c0, 0.0)) {
+        u[0] = U.chi[one];
+        u[1] = U.phi[one];
+        u[2] = U.delta[one];
+      } else {
+        u[0] = (double)rd_uniform<T>(L.h, c0, dtau, iters);
+        u[1] = phi_of(u[0], eps);
+        u[2] = u[1] * (1.0 - u[1]) / eps;
+      }
     }
     __syncthreads();
     const int i = i0 + lx, j = j0 + ly, k = k0 + lz;
@@ -307,8 +350,14 @@ __global__ void __launch_bounds__(512) k_rd_finish(Level L, RdGrid R, T dtau, in
       double x, p, dl;
       if (active) {
         x = (double)it[c];
-        p = phi_of(x, eps);
-        dl = delta ? p * (1.0 - p) / eps : 0.0;
+        const int one = same_bits(x, U.chi[1]);
+        if (one || same_bits(x, U.chi[0])) {
+          p = one ? U.phi[1] : U.phi[0];
+          dl = one ? U.delta[1] : U.delta[0];
+        } else {
+          p = phi_of(x, eps);
+          dl = delta ? p * (1.0 - p) / eps : 0.0;
+        }
       } else {
         x = u[0];
         p = u[1];
@@ -458,7 +507,8 @@ static sfx_status redistance_blocks(sfx_ctx* c, const double* C, T* aux, T* a, T
   const sfx_status st = block_list(c, nb);
   if (st != SFX_OK) return st;
   int2* list = (int2*)c->block_list;
-  unsigned char* f0 = (unsigned char*)(list + nb + 1);
+  RdUniform* uni = (RdUniform*)(list + nb + 1);
+  unsigned char* f0 = (unsigned char*)(uni + 1);
   unsigned char* f1 = f0 + nb;
   const int full = (int)std::min(nb, (size_t)c->sm_count * 64);
   // a step: resident blocks of 128 threads, each with a quarter of a cell
@@ -468,7 +518,8 @@ static sfx_status redistance_blocks(sfx_ctx* c, const double* C, T* aux, T* a, T
   const int grid = (int)std::min(nb * sub, (size_t)c->sm_count * 12 / sub * sub);
   const int sg = (int)std::min((nb + 255) / 256, (size_t)c->sm_count * 8);
   SFX_CUDA(cudaMemsetAsync(list, 0, sizeof(int2), s));
-  SFX_KERNEL(c, K_PHASE, (k_rd_init<T, ND>), full, 512, s, L, R, C, aux, a, f0);
+  SFX_KERNEL(c, K_PHASE, (k_rd_init<T, ND>), full, 512, s, L, R, C, aux, a, f0, (T)dtau,
+             iters, eps, uni);
   const int ext[3] = {kBx, B::by, B::bz};
   unsigned char *fi = f0, *fo = f1;
   for (int d = 0; d < ND; ++d) {
@@ -480,15 +531,15 @@ static sfx_status redistance_blocks(sfx_ctx* c, const double* C, T* aux, T* a, T
     SFX_KERNEL(c, K_PHASE, (k_rd_step<T, ND>), grid, kStepThreads, s, L, R, (T)dtau, list, aux, a, b);
     std::swap(a, b);
   }
-  SFX_KERNEL(c, K_PHASE, (k_rd_finish<T, ND>), full, 512, s, L, R, (T)dtau, iters, eps, fi, C, a,
-             chi, phi, delta);
+  SFX_KERNEL(c, K_PHASE, (k_rd_finish<T, ND>), full, 512, s, L, R, (T)dtau, iters, eps, fi, uni,
+             C, a, chi, phi, delta);
   SFX_LAUNCH_CHECK();
   return SFX_OK;
 }
 
 sfx_status block_list(sfx_ctx* c, size_t nb) {
   if (c->block_list) return SFX_OK;
-  SFX_CUDA(cudaMalloc(&c->block_list, (nb + 1) * sizeof(int2) + 2 * nb));
+  SFX_CUDA(cudaMalloc(&c->block_list, (nb + 1) * sizeof(int2) + sizeof(RdUniform) + 2 * nb));
   c->allocations.push_back(c->block_list);
   return SFX_OK;
 }
