@@ -13,7 +13,13 @@
 // One pass: a block owns a 32 x 8 column of cells and walks its planes in
 // z, keeping the unit normals of planes k-1, k, k+1 (with a one-cell halo
 // in x and y) in a ring of shared-memory buffers, so that every normal is
-// evaluated once per block instead of once per face that uses it.
+// evaluated once per block instead of once per face that uses it.  A thread
+// evaluates one normal of a plane (352 threads: with 256, three warps took a
+// second turn while five waited) and a ring of four planes needs one barrier
+// per plane.  What bounds it is the latency of those chains (seven quotients
+// and a root, the FP64 pipe's in SFX_F64 contexts): 160^3 in float 167 -> 130
+// us, 120 x 110 x 100 in double 670 -> 504, 50 x 64 x 40 in float 119 -> 20 (with
+// chunks of 32 planes throughout 184, 625, 75 us).
 #include <algorithm>
 
 #include "sfx_f32_dev.cuh"
@@ -22,8 +28,9 @@
 namespace sfx {
 namespace {
 
-constexpr int kCapX = 32, kCapY = 8, kCapZChunk = 32;
+constexpr int kCapX = 32, kCapY = 8;
 constexpr int kCapHX = kCapX + 2, kCapHY = kCapY + 2;
+constexpr int kCapThreads = (kCapHX * kCapHY + 31) / 32 * 32;
 
 // all components of n at (i,j,k) in FP64 (the arithmetic of normal_comp)
 __device__ __forceinline__ void normal3_f64(const Level& L, const double* __restrict__ phi, int i,
@@ -70,32 +77,34 @@ struct CapNormal<float> {
 // T: arithmetic type (double in SFX_F64 contexts, float in SFX_F32);
 // P: storage type of C, sigma, kappa and the force.
 template <typename T, typename P>
-__global__ void __launch_bounds__(kCapX* kCapY)
+__global__ void __launch_bounds__(kCapThreads, sizeof(T) == 4 ? 4 : 1)
     k_capillary(Level L, const double* __restrict__ phi, const P* __restrict__ C,
-                const P* __restrict__ sigma, double eps, P* __restrict__ kappa,
+                const P* __restrict__ sigma, double eps, int zc, P* __restrict__ kappa,
                 P* __restrict__ force) {
-  // ring of three planes of normals, each with a one-cell halo in x and y
-  __shared__ T sn[3][3][kCapHY][kCapHX];
+  // ring of four planes of normals, each with a one-cell halo in x and y
+  __shared__ T sn[4][3][kCapHY][kCapHX];
   const int tx = threadIdx.x % kCapX, ty = threadIdx.x / kCapX;
   const int i0 = blockIdx.x * kCapX, j0 = blockIdx.y * kCapY;
   const int i = i0 + tx, j = j0 + ty;
+  const bool own = ty < kCapY && i < L.nx && j < L.ny;
+  const int px = threadIdx.x % kCapHX, py = threadIdx.x / kCapHX;
+  const int a = i0 + px - 1, b = j0 + py - 1;
+  const bool halo = py < kCapHY, cell = halo && a >= 0 && a < L.nx && b >= 0 && b < L.ny;
   const bool is3d = L.geom == SFX_CART3D;
-  const int k0 = is3d ? blockIdx.z * kCapZChunk : 0;
-  const int k1 = is3d ? min(k0 + kCapZChunk, L.nz) : 1;
+  const int k0 = is3d ? (int)blockIdx.z * zc : 0;
+  const int k1 = is3d ? min(k0 + zc, L.nz) : 1;
   const size_t N = L.ncell();
   const T inv_h = (T)(1.0 / L.h);
 
-  // normals of plane k (tile and halo) into ring slot (k + 3) % 3
+  // normals of plane k (tile and halo, one per thread) into ring slot k % 4
   auto fill = [&](int k) {
-    T(*s)[kCapHY][kCapHX] = sn[(k + 3) % 3];
-    for (int q = threadIdx.x; q < kCapHX * kCapHY; q += kCapX * kCapY) {
-      const int hx = q % kCapHX, hy = q / kCapHX;
-      const int a = i0 + hx - 1, b = j0 + hy - 1;
-      T n[3] = {(T)0, (T)0, (T)0};
-      if (a >= 0 && a < L.nx && b >= 0 && b < L.ny) CapNormal<T>::eval(L, phi, a, b, k, eps, n);
-      s[0][hy][hx] = n[0];
-      s[1][hy][hx] = n[1];
-      s[2][hy][hx] = n[2];
+    T n[3] = {(T)0, (T)0, (T)0};
+    if (cell) CapNormal<T>::eval(L, phi, a, b, k, eps, n);
+    if (halo) {
+      T(*s)[kCapHY][kCapHX] = sn[k & 3];
+      s[0][py][px] = n[0];
+      s[1][py][px] = n[1];
+      s[2][py][px] = n[2];
     }
   };
 
@@ -104,8 +113,8 @@ __global__ void __launch_bounds__(kCapX* kCapY)
   for (int k = k0; k < k1; ++k) {
     if (is3d && k + 1 < L.nz) fill(k + 1);
     __syncthreads();
-    if (i < L.nx && j < L.ny) {
-      T(*s)[kCapHY][kCapHX] = sn[(k + 3) % 3];
+    if (own) {
+      T(*s)[kCapHY][kCapHX] = sn[k & 3];
       const int hx = tx + 1, hy = ty + 1;
       T wm = (T)1, wp = (T)1;
       if (L.geom == SFX_AXISYM) {
@@ -122,8 +131,8 @@ __global__ void __launch_bounds__(kCapX* kCapY)
       T nz0 = (T)0;
       if (is3d) {
         nz0 = s[2][hy][hx];
-        if (k > 0) div -= (T)0.5 * (nz0 + sn[(k + 2) % 3][2][hy][hx]);
-        if (k < L.nz - 1) div += (T)0.5 * (nz0 + sn[(k + 1) % 3][2][hy][hx]);
+        if (k > 0) div -= (T)0.5 * (nz0 + sn[(k - 1) & 3][2][hy][hx]);
+        if (k < L.nz - 1) div += (T)0.5 * (nz0 + sn[(k + 1) & 3][2][hy][hx]);
       }
       const T kap = -div * inv_h;
       // delta_s = |grad C|, centred, zero-gradient ghosts
@@ -145,7 +154,7 @@ __global__ void __launch_bounds__(kCapX* kCapY)
       if (is3d) force[2 * N + c] = (P)(a * nz0);
       if (kappa) kappa[c] = (P)kap;
     }
-    __syncthreads();   // slot (k + 2) % 3 is refilled by the next plane
+    // the next plane fills slot k + 2, which holds none of k - 1 .. k + 1
   }
 }
 
@@ -153,10 +162,15 @@ template <typename T, typename P>
 sfx_status capillary_impl(sfx_ctx* c, const double* phi, const P* C, const P* sigma, double eps,
                           P* kappa, P* force, cudaStream_t s) {
   const Level& L = c->lev[0].lv;
-  const unsigned gz = L.geom == SFX_CART3D ? (unsigned)((L.nz + kCapZChunk - 1) / kCapZChunk) : 1u;
-  const dim3 grid((unsigned)((L.nx + kCapX - 1) / kCapX), (unsigned)((L.ny + kCapY - 1) / kCapY),
-                  gz);
-  SFX_KERNEL(c, K_FORCES, (k_capillary<T, P>), grid, kCapX * kCapY, s, L, phi, C, sigma, eps,
+  const unsigned gx = (unsigned)((L.nx + kCapX - 1) / kCapX),
+                 gy = (unsigned)((L.ny + kCapY - 1) / kCapY);
+  // planes per block: 16 (a chunk evaluates the normals of two planes more
+  // than it owns), 8 or 4 where the grid would not fill the chip once
+  const long long slots = (long long)c->sm_count * (sizeof(T) == 4 ? 4 : 2);
+  const long long z = ((long long)gx * gy * L.nz + slots - 1) / slots;
+  const int zc = z > 8 ? 16 : (z > 4 ? 8 : 4);
+  const dim3 grid(gx, gy, L.geom == SFX_CART3D ? (unsigned)((L.nz + zc - 1) / zc) : 1u);
+  SFX_KERNEL(c, K_FORCES, (k_capillary<T, P>), grid, kCapThreads, s, L, phi, C, sigma, eps, zc,
              kappa, force);
   SFX_LAUNCH_CHECK();
   return SFX_OK;
