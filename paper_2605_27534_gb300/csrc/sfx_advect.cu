@@ -138,7 +138,7 @@ struct AdvFields {
 };
 
 template <typename U, int G, int NF, int TY>
-__global__ void __launch_bounds__(kAX * TY, NF == 1 ? 2 : 1)
+__global__ void __launch_bounds__(kAX * TY, (NF == 1 ? 2 : 1) * (G == SFX_CART3D ? 16 / TY : 1))
 k_bcg64(Level L, Vel<U> v, double dt, AdvFields<NF> P, int zc) {
   constexpr int ND = G == SFX_CART3D ? 3 : 2;
   __shared__ double sA[NF][TY][kAX], sS[NF][TY][kAX], sF[NF][TY][kAX];
@@ -285,34 +285,54 @@ k_bcg64(Level L, Vel<U> v, double dt, AdvFields<NF> P, int zc) {
   }
 }
 
+// The 3D tiling: rows per block (16 or 8) and planes per chunk.  A block's
+// rows times planes (a chunk steps about 1.5 planes more than it owns) are the
+// FP64 work of its SM, so what decides is the most of it that an SM gets,
+// over how well its resident warps keep the pipe busy (measured: 80 % with 32
+// warp-fields, so w/(w + 8)).  40 x 33 x 50, both fields: six tiles of 16
+// rows in chunks of 8 planes 142 us, as chosen here 51; 50 x 64 x 40, one field
+// with float velocities: 79 and 39; 160^3 and 96^3 keep 16 rows, 40 and 20 planes.
+struct Tiling {
+  int ty, zc;
+};
+inline Tiling bcg64_tiling(const Level& L, int nf, int sms) {
+  Tiling best{16, L.nz};
+  double cost = 0.0;
+  for (int ty = 16; ty >= 8; ty -= 8) {
+    const long long tiles = (long long)((L.nx + kAX - 3) / (kAX - 2)) * ((L.ny + ty - 3) / (ty - 2));
+    const int fit = (nf == 1 ? 2 : 1) * (16 / ty);      // blocks resident on an SM
+    for (int n = 1; n <= std::min(L.nz, 64); ++n) {
+      const int z = (L.nz + n - 1) / n;
+      const long long per = (tiles * ((L.nz + z - 1) / z) + sms - 1) / sms;
+      const double w = (double)(std::min<long long>(per, fit) * ty * nf);
+      const double t = (double)(per * ty) * (z + 1.5) * (w + 8.0) / w;
+      if (cost == 0.0 || t < cost) cost = t, best = {ty, z};
+    }
+  }
+  return best;
+}
+
+template <typename U, int G, int NF, int TY>
+void launch_bcg64(sfx_ctx* c, const Vel<U>& v, double dt, const AdvFields<NF>& P, int zc,
+                  cudaStream_t s) {
+  const Level& L = c->lev[0].lv;
+  const dim3 g((unsigned)((L.nx + kAX - 3) / (kAX - 2)), (unsigned)((L.ny + TY - 3) / (TY - 2)),
+               (unsigned)((L.nz + zc - 1) / zc));
+  SFX_KERNEL(c, K_ADVECT, (k_bcg64<U, G, NF, TY>), g, dim3(kAX, TY), s, L, v, dt, P, zc);
+}
+
 template <typename U, int NF>
 sfx_status bcg64(sfx_ctx* c, const Vel<U>& v, double dt, const AdvFields<NF>& P, cudaStream_t s) {
   const Level& L = c->lev[0].lv;
-  const int gx = (L.nx + kAX - 3) / (kAX - 2);
   if (L.geom == SFX_CART3D) {
-    // chunks of planes: a chunk steps two planes more than it owns, so the
-    // fewest waves times (planes + 2) decides (512 threads per block, the
-    // kernel's NF blocks per SM), eight planes at least
-    constexpr int TY = 16;
-    const int gy = (L.ny + TY - 3) / (TY - 2);
-    const long long tiles = (long long)gx * gy, slots = (long long)c->sm_count * (NF == 1 ? 2 : 1);
-    int zc = L.nz;
-    long long best = -1;
-    for (int n = 1; n <= std::max(1, L.nz / 8); ++n) {
-      const int z = (L.nz + n - 1) / n;
-      const long long cost = (tiles * ((L.nz + z - 1) / z) + slots - 1) / slots * (z + 2);
-      if (best < 0 || cost < best) best = cost, zc = z;
-    }
-    const dim3 g(gx, gy, (L.nz + zc - 1) / zc);
-    SFX_KERNEL(c, K_ADVECT, (k_bcg64<U, SFX_CART3D, NF, TY>), g, dim3(kAX, TY), s, L, v, dt, P, zc);
-  } else {
+    const Tiling t = bcg64_tiling(L, NF, c->sm_count);
+    if (t.ty == 16) launch_bcg64<U, SFX_CART3D, NF, 16>(c, v, dt, P, t.zc, s);
+    else launch_bcg64<U, SFX_CART3D, NF, 8>(c, v, dt, P, t.zc, s);
+  } else if (L.geom == SFX_AXISYM) {
     // shallower tiles: 2D grids are small and want more blocks
-    constexpr int TY = 8;
-    const dim3 g(gx, (L.ny + TY - 3) / (TY - 2));
-    if (L.geom == SFX_AXISYM)
-      SFX_KERNEL(c, K_ADVECT, (k_bcg64<U, SFX_AXISYM, NF, TY>), g, dim3(kAX, TY), s, L, v, dt, P, 1);
-    else
-      SFX_KERNEL(c, K_ADVECT, (k_bcg64<U, SFX_PLANAR2D, NF, TY>), g, dim3(kAX, TY), s, L, v, dt, P, 1);
+    launch_bcg64<U, SFX_AXISYM, NF, 8>(c, v, dt, P, 1, s);
+  } else {
+    launch_bcg64<U, SFX_PLANAR2D, NF, 8>(c, v, dt, P, 1, s);
   }
   SFX_LAUNCH_CHECK();
   return SFX_OK;
