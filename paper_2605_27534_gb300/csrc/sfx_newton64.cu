@@ -242,22 +242,21 @@ k_resid64(Newton64 q, const double* __restrict__ f, const double* __restrict__ F
   if (ctl->done) {
     // every block sees done (set by an earlier launch); the sweeps behind
     // this launch return too
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) ctl->stop = 1;
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->stop = 1;
     return;
   }
   const Level& L = q.p.L;
   float m[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const ix rows = (ix)L.ny * (ix)L.nz;
-  double w[2] = {1.0, 1.0};
-  if (G == SFX_AXISYM) {
-    const double iv = 1.0 / (double)(2 * i + 1);
-    w[0] = (double)(2 * i) * iv;
-    w[1] = i + 1 < L.nx ? (double)(2 * i + 2) * iv : 0.0;
-  }
-  for (ix r = blockIdx.y; r < rows && i < L.nx; r += gridDim.y) {
-    const int j = (int)(r % (ix)L.ny), k = (int)(r / (ix)L.ny);
-    const ix c = r * (ix)L.nx + (ix)i;
+  const ix cells = (ix)L.ncell();
+  for (ix c = blockIdx.x * blockDim.x + threadIdx.x; c < cells; c += gridDim.x * blockDim.x) {
+    const ix r = c / (ix)L.nx;
+    const int i = (int)(c - r * (ix)L.nx), j = (int)(r % (ix)L.ny), k = (int)(r / (ix)L.ny);
+    double w[2] = {1.0, 1.0};
+    if (G == SFX_AXISYM) {
+      const double iv = 1.0 / (double)(2 * i + 1);
+      w[0] = (double)(2 * i) * iv;
+      w[1] = i + 1 < L.nx ? (double)(2 * i + 2) * iv : 0.0;
+    }
     bool has[6];
     ix nbi[6];
     gather6<G>(L, i, j, k, c, has, nbi);
@@ -319,7 +318,7 @@ k_resid64(Newton64 q, const double* __restrict__ f, const double* __restrict__ F
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0)
-    last = atomicAdd(&ctl->blocks, 1u) == gridDim.x * gridDim.y - 1;
+    last = atomicAdd(&ctl->blocks, 1u) == gridDim.x - 1;
   __syncthreads();
   if (!last || threadIdx.x != 0) return;
   __threadfence();
@@ -387,20 +386,18 @@ k_corr64_tile2d(Nw32 p, int tx, int ty, int sweeps, const __half2* __restrict__ 
                  });
 }
 
-// Launch shape of the residual: x chunks of up to 256 threads, and rows in
-// turn, eight blocks per SM.
-struct Rows {
-  dim3 grid, block;
+// Launch shape of the residual: cells in turn (rows of warps left the lanes
+// past a row's end idle while the FP64 pipe took their slots: 65 x 70 x 60
+// 36 -> 26 us, 300 x 400 16.2 -> 12.7, 96^3 73.4 -> 71.3), blocks of 256
+// threads, eight per SM; of 128 where that is less than one cell per thread,
+// to even out over the SMs.
+struct Shape {
+  unsigned grid, block;
 };
-Rows rows_of(const Level& L, int sms) {
-  Rows g;
-  const int tx = L.nx >= 256 ? 256 : ((L.nx + 31) / 32) * 32;
-  const int xb = (L.nx + tx - 1) / tx;
-  const long long rows = (long long)L.ny * L.nz;
-  const long long want = std::max(1LL, ((long long)sms * 2048 / tx) / xb);
-  g.block = dim3(tx);
-  g.grid = dim3(xb, (unsigned)std::min(rows, std::min(want, 65535LL)));
-  return g;
+Shape shape_of(const Level& L, int sms) {
+  const size_t n = L.ncell();
+  const unsigned block = n >= (size_t)sms * 2048 ? 256 : 128;
+  return {(unsigned)std::min((n + block - 1) / block, (size_t)sms * 2048 / block), block};
 }
 
 sfx_status ensure(sfx_ctx* c) {
@@ -449,7 +446,7 @@ sfx_status solve(sfx_ctx* c, const Newton64& q, double* f, double* F, bool from_
   Ctl64* ctl = (Ctl64*)S.ctl;
   const int sweeps = std::max(1, o->nu1 + o->nu2);
   const float tol = (float)o->tol;
-  const Rows rg = rows_of(L, c->sm_count);
+  const Shape rg = shape_of(L, c->sm_count);
   const dim3 blk(128), grd((unsigned)(((L.nx + 1) / 2 + 127) / 128), (unsigned)L.ny, (unsigned)L.nz);
   const int cap = std::min(o->max_cycles, kMaxNewton);
   Tile2D t2;
