@@ -40,7 +40,9 @@ namespace {
 // minus sides of a block's cells, from unit normals formed once per cell in
 // shared memory (the block's cells and one layer on the minus sides; a face
 // per thread and direction took two normals per face).  Where phi is flat
-// bit for bit the normal is zero and costs no FP64 arithmetic.
+// bit for bit the normal is zero and costs no FP64 arithmetic; in 3D a warp is
+// a box of 8 x 2 x 2 cells, fewer of which touch the band of phi than rows of
+// 32 do (96^3: 98 -> 90 us, 65 x 70 x 60: 60 -> 44; FP64 pipe 76 % busy).
 // Optional outputs: H2 the faces in half precision, c1 = r_a/(phi + eta) and
 // finf = Gamma_inf phi (1 - phi)/eps per cell, and what a solve starts with
 // (a memory operation and two copies of their own took 10 us of a 128^2 step).
@@ -107,17 +109,31 @@ __global__ void __launch_bounds__(kSX * kSY * (ND == 3 ? 4 : 1)) k_setup64(Setup
   if (q.ctl && (blockIdx.x | blockIdx.y | blockIdx.z) == 0 && threadIdx.x < kCtlWords)
     q.ctl[threadIdx.x] = 0;
   const double inv2h = 0.5 / L.h, inv_eps = 1.0 / q.eps;
-  for (int t = threadIdx.x; t < HX * HY * HZ; t += blockDim.x) {
-    const int lx = t % HX, ly = t / HX % HY, lz = t / (HX * HY);
+  // the normal of the cell (lx, ly, lz) of the block's box with its minus layers
+  auto normal = [&](int lx, int ly, int lz) {
     const int x[3] = {x0 + lx - 1, y0 + ly - 1, ND == 3 ? z0 + lz - 1 : 0};
     double n[ND] = {};
     if (x[0] >= 0 && x[0] < L.nx && x[1] >= 0 && x[1] < L.ny && x[2] >= 0 && x[2] < L.nz)
       unit_normal<ND>(L, q.phi, x, inv2h, inv_eps, n);
 #pragma unroll
     for (int d = 0; d < ND; ++d) sn[d][lz][ly][lx] = n[d];
+  };
+  int lx = threadIdx.x % kSX, ly = threadIdx.x / kSX % kSY, lz = threadIdx.x / (kSX * kSY);
+  if (ND == 3) {
+    const int3 l = CellBlock<3>::cell(threadIdx.x);
+    lx = l.x, ly = l.y, lz = l.z;
+    normal(lx + 1, ly + 1, lz + 1);
+    const int t = threadIdx.x;
+    if (t < kSX * kSY) normal(1 + t % kSX, 1 + t / kSX, 0);
+    else if (t < kSX * (kSY + BZ + 1)) normal(1 + t % kSX, 0, t / kSX - kSY);
+    else if (t < kSX * (kSY + BZ + 1) + HY * HZ) {
+      const int e = t - kSX * (kSY + BZ + 1);
+      normal(0, e % HY, e / HY);
+    }
+  } else {
+    for (int t = threadIdx.x; t < HX * HY; t += blockDim.x) normal(t % HX, t / HX, 0);
   }
   __syncthreads();
-  const int lx = threadIdx.x % kSX, ly = threadIdx.x / kSX % kSY, lz = threadIdx.x / (kSX * kSY);
   const int x[3] = {x0 + lx, y0 + ly, z0 + lz};
   if (x[0] >= L.nx || x[1] >= L.ny || x[2] >= L.nz) return;
   const size_t st[3] = {1, (size_t)L.nx, (size_t)L.nx * L.ny};
