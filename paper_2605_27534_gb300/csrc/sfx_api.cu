@@ -193,6 +193,7 @@ sfx_status sfx_ctx_create(const sfx_grid* grid, int precision, sfx_ctx** out) {
   if (st == SFX_OK) st = dalloc(c, &c->chi_tmp, n);
   if (st == SFX_OK) st = dalloc(c, &c->partials, (size_t)2 * 8 * kTotalsBlocks);
   if (st == SFX_OK) st = dalloc(c, &c->tickets, 8);
+  if (st == SFX_OK) st = block_list(c);
   if (st == SFX_OK) {
     const cudaError_t e = cudaMemset(c->tickets, 0, 8 * sizeof(unsigned));
     if (e != cudaSuccess) st = cuda_fail(e);

@@ -2016,8 +2016,7 @@ sfx_status marangoni32(sfx_ctx* c, const sfx_params* p, const float2* f, const d
   const size_t n = L.ncell();
   Eos32 q{(float)p->gamma_inf, (float)p->eps, (float)(1.0 / p->eps), (float)p->sigma0,
           (float)p->E, p->eos, p->sigma0 * p->E, p->gamma_inf / p->eps};
-  unsigned* list = nullptr;
-  if (dm_mode != 0 && (st = cut_list(c, &list)) != SFX_OK) return st;
+  unsigned* list = dm_mode != 0 ? cut_list(c, s) : nullptr;
   if (n >= kEosListCells) {
     unsigned* band = reinterpret_cast<unsigned*>(c->f32.falt);   // idle outside solvers 0 and 2
     SFX_CUDA(cudaMemsetAsync(band, 0, sizeof(unsigned), s));

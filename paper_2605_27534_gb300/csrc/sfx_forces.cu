@@ -233,14 +233,18 @@ __global__ void k_loss_grad(Level L, EosArgs q, const double* __restrict__ f,
 
 }  // namespace
 
-sfx_status cut_list(sfx_ctx* c, unsigned** list) {
+unsigned* cut_list(sfx_ctx* c, cudaStream_t s) {
   const size_t n = c->lev[0].lv.ncell();
-  if (!c->cut_list && n < ((size_t)1 << 32)) {
-    SFX_CUDA(cudaMalloc((void**)&c->cut_list, (n + 1) * sizeof(unsigned)));
-    c->allocations.push_back(c->cut_list);
+  cudaStreamCaptureStatus cap;
+  if (c->cut_list || n >= ((size_t)1 << 32)) return c->cut_list;
+  void* p = nullptr;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
+      cudaMalloc(&p, (n + 1) * sizeof(unsigned)) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
   }
-  *list = c->cut_list;
-  return SFX_OK;
+  c->allocations.push_back(p);
+  return c->cut_list = (unsigned*)p;
 }
 
 // sigma, the force and (dm not null) delta_m of an FP64 state
@@ -250,11 +254,7 @@ static sfx_status eos_force(sfx_ctx* c, const EosArgs& q, const double* f, const
   const Level& L = c->lev[0].lv;
   const size_t n = L.ncell();
   const int nb = blocks_for(n, 256);
-  unsigned* list = nullptr;
-  if (dm_mode != 0) {
-    const sfx_status st = cut_list(c, &list);
-    if (st != SFX_OK) return st;
-  }
+  unsigned* list = dm_mode != 0 ? cut_list(c, s) : nullptr;
   SFX_KERNEL(c, K_FORCES, k_eos, nb, 256, s, n, q, f, phi, sigma, list);
   if (list) SFX_KERNEL(c, K_FORCES, k_force_list, nb, 256, s, n, L.ndim(), C, force, dm, list);
   SFX_KERNEL(c, K_FORCES, k_force, std::min(blocks_for(n, 64), c->sm_count * 16), 64, s, L, phi, C,

@@ -292,6 +292,7 @@ sfx_status drift_faces64(sfx_ctx* c, const double* phi, double Df, double DF, do
 // faces and coefficients first; the first iterate is (f, F), or (f*, F*) with
 // from_star).  It ends with *conv false when it should be left to the Picard
 // solver.
+bool newton64_scratch(sfx_ctx* c);
 bool newton64_eligible(const sfx_ctx* c, const sfx_params* p, double dt, const sfx_solve_opts* o);
 // `copy`: (f*, F*) = (f, F) too (no flow).
 sfx_status newton64_prepare(sfx_ctx* c, const sfx_params* p, const double* phi, const double* f,
@@ -306,11 +307,13 @@ sfx_status acdi_step(sfx_ctx* c, const void* ux, const void* uy, const void* uz,
 sfx_status capillary(sfx_ctx* c, const sfx_params* p, const double* phi, const void* C,
                      const void* sigma, void* kappa, void* force, cudaStream_t s);
 // sfx_forces.cu: ctx->cut_list (allocated on first use; each pass fills it
-// anew), null where a grid's cells do not fit 32-bit indices
-sfx_status cut_list(sfx_ctx* c, unsigned** list);
-// sfx_phase.cu: ctx->block_list for nb blocks of cells: a count, nb int2, six
-// doubles and two flags per block at least (allocated on first use; each pass fills it anew)
-sfx_status block_list(sfx_ctx* c, size_t nb);
+// anew), null where a grid's cells do not fit 32-bit indices, no memory is
+// left for it or its first use is within a stream capture: the passes then
+// take every cell in turn
+unsigned* cut_list(sfx_ctx* c, cudaStream_t s);
+// sfx_phase.cu: allocates ctx->block_list: for the nb blocks of cells a count,
+// nb int2, six doubles and two flags per block (each pass fills it anew)
+sfx_status block_list(sfx_ctx* c);
 // sfx_vof.cu
 sfx_status vof_advect(sfx_ctx* c, const void* ux, const void* uy, const void* uz, double dt,
                       int order, double* C, cudaStream_t s);

@@ -422,8 +422,10 @@ sfx_status ensure(sfx_ctx* c) {
   const Level& L = c->lev[0].lv;
   const size_t np = 2 * (size_t)L.ny * L.nz * ((L.nx + 1) / 2);
   auto get = [&](size_t bytes, void** p) -> sfx_status {
-    SFX_CUDA(cudaMalloc(p, bytes));
-    c->allocations.push_back(*p);
+    if (*p) return SFX_OK;
+    void* m = nullptr;
+    SFX_CUDA(cudaMalloc(&m, bytes));
+    c->allocations.push_back(*p = m);
     return SFX_OK;
   };
   sfx_status st;
@@ -558,12 +560,18 @@ bool newton64_eligible(const sfx_ctx* c, const sfx_params* p, double dt, const s
          nz <= 65535 && std::max(p->Df, p->DF) * dt <= L.h * L.h;
 }
 
+// The work arrays of the Newton solve; where there is no memory for them the
+// Picard solver, which needs none, takes the step.
+bool newton64_scratch(sfx_ctx* c) {
+  if (ensure(c) == SFX_OK) return true;
+  cudaGetLastError();
+  return false;
+}
+
 // Drift faces (into the finest level's arrays), the coefficients of the Newton
 // solve and its cleared control words.
 sfx_status newton64_prepare(sfx_ctx* c, const sfx_params* p, const double* phi, const double* f,
                             const double* F, bool copy, cudaStream_t s) {
-  sfx_status st = ensure(c);
-  if (st != SFX_OK) return st;
   const Level& L = c->lev[0].lv;
   LevelData& D = c->lev[0];
   Setup64 q{L, phi, p->Df, p->DF, p->eps, p->ka, p->eta, p->gamma_inf, {}, {}, {}, D.lam, D.b,

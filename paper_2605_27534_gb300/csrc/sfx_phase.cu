@@ -504,8 +504,6 @@ static sfx_status redistance_blocks(sfx_ctx* c, const double* C, T* aux, T* a, T
   using B = RdBlk<ND>;
   const RdGrid R{(L.nx + kBx - 1) / kBx, (L.ny + B::by - 1) / B::by, (L.nz + B::bz - 1) / B::bz};
   const size_t nb = (size_t)R.nbx * R.nby * R.nbz;
-  const sfx_status st = block_list(c, nb);
-  if (st != SFX_OK) return st;
   int2* list = (int2*)c->block_list;
   RdUniform* uni = (RdUniform*)(list + nb + 1);
   unsigned char* f0 = (unsigned char*)(uni + 1);
@@ -537,8 +535,9 @@ static sfx_status redistance_blocks(sfx_ctx* c, const double* C, T* aux, T* a, T
   return SFX_OK;
 }
 
-sfx_status block_list(sfx_ctx* c, size_t nb) {
-  if (c->block_list) return SFX_OK;
+sfx_status block_list(sfx_ctx* c) {
+  const Level& L = c->lev[0].lv;
+  const size_t nb = L.ndim() == 3 ? CellBlock<3>::count(L) : CellBlock<2>::count(L);
   SFX_CUDA(cudaMalloc(&c->block_list, (nb + 1) * sizeof(int2) + sizeof(RdUniform) + 2 * nb));
   c->allocations.push_back(c->block_list);
   return SFX_OK;

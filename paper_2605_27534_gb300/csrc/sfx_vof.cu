@@ -227,10 +227,7 @@ sfx_status vof_impl(sfx_ctx* c, const U* const* u, double dt, int order, double*
   unsigned grid = (unsigned)nb;
   unsigned* cut = nullptr;
   if (L.ncell() >= kVofListCells) {
-    sfx_status st = cut_list(c, &cut);
-    if (st != SFX_OK) return st;
-    st = block_list(c, nb);
-    if (st != SFX_OK) return st;
+    cut = cut_list(c, s);
     list = (int2*)c->block_list;
     unsigned char* flag = (unsigned char*)(list + nb + 1);
     SFX_CUDA(cudaMemsetAsync(list, 0, sizeof(int2), s));
