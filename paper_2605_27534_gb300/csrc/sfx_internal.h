@@ -293,7 +293,8 @@ sfx_status drift_faces64(sfx_ctx* c, const double* phi, double Df, double DF, do
 // from_star).  It ends with *conv false when it should be left to the Picard
 // solver.
 bool newton64_scratch(sfx_ctx* c);
-bool newton64_eligible(const sfx_ctx* c, const sfx_params* p, double dt, const sfx_solve_opts* o);
+bool newton64_eligible(const sfx_ctx* c, const sfx_params* p, double dt, const sfx_solve_opts* o,
+                       bool flow);
 // `copy`: (f*, F*) = (f, F) too (no flow).
 sfx_status newton64_prepare(sfx_ctx* c, const sfx_params* p, const double* phi, const double* f,
                             const double* F, bool copy, cudaStream_t s);

@@ -581,7 +581,7 @@ sfx_status step_impl(sfx_ctx* c, const sfx_params* p, const double* phi, const v
   const Level& L = c->lev[0].lv;
   const size_t n = L.ncell();
   // drift faces of both problems (phi is fixed over the step)
-  const bool newton = newton64_eligible(c, p, dt, o) && newton64_scratch(c);
+  const bool newton = newton64_eligible(c, p, dt, o, ux != nullptr) && newton64_scratch(c);
   sfx_status ds = newton ? newton64_prepare(c, p, phi, f, F, !ux, s)
                          : drift_faces64(c, phi, p->Df, p->DF, p->eps, c->lev[0].B[0],
                                          c->lev[0].B[1], s);
