@@ -785,7 +785,10 @@ def vof_run(a, dev, steps, warmup=3, n=256):
             "roofline": {"bound": "hbm", "achieved": ab / (ms * 1e-3) / 1e9,
                          "peak": peaks["hbm_gbs"], "unit": "GB/s",
                          "frac": ab / (ms * 1e-3) / 1e9 / peaks["hbm_gbs"],
-                         "bytes_per_step": ab, "kernels": "indicator + 3 x (flux + update)"},
+                         "bytes_per_step": ab, "kernels": "block flags + 3 x (flux + planes + update)",
+                         "note": "bytes of passes over every cell of the grid; the passes "
+                                 "take only the blocks that hold or touch fluid, so the "
+                                 "fraction may exceed 1"},
             "sum_C_rel_change": float(Cd.sum().item()) / m0 - 1.0}
 
 

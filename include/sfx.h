@@ -200,8 +200,8 @@ sfx_status sfx_vof_advect(sfx_ctx* ctx, const void* ux, const void* uy, const vo
    |grad phi| < 1e-30.  f and F
    (state layout of the context) are updated in place; phi is double, the
    velocities are in the context precision.  SFX_F64 contexts with
-   opts->mg_levels = 0 and max(Df, DF) dt/h^2 <= 1 solve the coupled system
-   by Newton defect correction instead (FP64 state and residuals, the
+   opts->mg_levels = 0 and max(Df, DF) dt/h^2 <= 1 (planar grids: and no
+   velocities) solve the coupled system by Newton defect correction instead (FP64 state and residuals, the
    correction relaxed by nu1 + nu2 FP32 red-black sweeps with a 2x2 block
    solve per cell) and fall back to Picard iteration where it does not
    converge; stats then count its iterations.  SFX_F32 contexts solve the
