@@ -1758,6 +1758,7 @@ sfx_status solve_newton32(sfx_ctx* c, const Nw32& p, const float* phi, float* co
     // converged at the first check: x* was the answer and was never copied
     SFX_CUDA(cudaMemcpyAsync(fc, fs, n * sizeof(float2), cudaMemcpyDeviceToDevice, s));
     SFX_CUDA(cudaMemcpyAsync(Fc, Fs, n * sizeof(float2), cudaMemcpyDeviceToDevice, s));
+    SFX_CUDA(cudaStreamSynchronize(s));   // the state is final when a step returns
   }
   *iters = done_it;
   return SFX_OK;
@@ -1894,6 +1895,7 @@ sfx_status step_f32(sfx_ctx* c, const sfx_params* pr, const double* phi_in, cons
     if (st != SFX_OK) return st;
     if (fc != f) SFX_CUDA(cudaMemcpyAsync(f, fc, n * sizeof(float2), cudaMemcpyDeviceToDevice, s));
     if (Fc != F) SFX_CUDA(cudaMemcpyAsync(F, Fc, n * sizeof(float2), cudaMemcpyDeviceToDevice, s));
+    if (!stats && (fc != f || Fc != F)) SFX_CUDA(cudaStreamSynchronize(s));
     if (c->f32.predict && c->f32.solver == 1 && dconv) {
       SFX_KERNEL(c, K_SETUP, k_increment32, blocks_for(n, 256), 256, s, n, fs, Fs, f, F,
                  c->f32.inc_f, c->f32.inc_F);
@@ -1966,6 +1968,7 @@ sfx_status step_f32(sfx_ctx* c, const sfx_params* pr, const double* phi_in, cons
   c->f32.predicted = conv ? (it == first ? it - 1 : it) : 0;
   if (fc != f) SFX_CUDA(cudaMemcpyAsync(f, fc, n * sizeof(float2), cudaMemcpyDeviceToDevice, s));
   if (Fc != F) SFX_CUDA(cudaMemcpyAsync(F, Fc, n * sizeof(float2), cudaMemcpyDeviceToDevice, s));
+  if (!stats && (fc != f || Fc != F)) SFX_CUDA(cudaStreamSynchronize(s));
   if (stats) {
     stats->picard = it > o->max_cycles ? o->max_cycles : it;
     stats->vcycles = 2 * stats->picard * sweeps;

@@ -604,6 +604,9 @@ sfx_status step_impl(sfx_ctx* c, const sfx_params* p, const double* phi, const v
     sfx_status st = newton64_solve(c, p, f, F, dt, ux != nullptr, o, &it, res, &conv, s);
     if (st != SFX_OK) return st;
     cycles = 2 * it * std::max(1, o->nu1 + o->nu2);
+    // it reports before the sweeps that add its last correction have run; the
+    // state is final on return (with statistics the totals wait for it)
+    if (conv && !stats) SFX_CUDA(cudaStreamSynchronize(s));
   }
   if (!conv) {
     if (ux || newton) {
