@@ -228,7 +228,9 @@ k_b_resid(const BInst* __restrict__ I, const int2* __restrict__ map,
   const BInst& B = I[inst];
   const Level& L = B.p.L;
   const ix n = (ix)L.ncell(), nx = (ix)L.nx, bs = blockDim.x;
-  const int it = P.loop[0] + 1;
+  // both before this block counts as finished: the last instance writes them
+  // once every active instance has counted
+  const int it = P.loop[0] + 1, live = P.loop[3];
   // the FP32 residual for the instance's first iterations (the kind is
   // the same for every block of an instance)
   const int kind = P.rkind[2 * inst];
@@ -306,7 +308,7 @@ k_b_resid(const BInst* __restrict__ I, const int2* __restrict__ map,
   // the last instance: count the iteration, and let the step's loop run
   // again while an instance is active and the iteration budget lasts
   __threadfence();
-  if (atomicAdd(&P.loop[1], 1) != P.loop[3] - 1) return;
+  if (atomicAdd(&P.loop[1], 1) != live - 1) return;
   __threadfence();
   const int any = atomicExch(&P.loop[2], 0);
   P.loop[3] = any;
