@@ -351,6 +351,14 @@ k_resid64(Newton64 q, const double* __restrict__ f, const double* __restrict__ F
   __threadfence_system();
 }
 
+// The correction of a cell as it is added to the state: after a passed test
+// none that is not finite (the sweeps overflow float where 1/dt is beyond
+// 1e19; no residual follows that would see it).
+__device__ __forceinline__ float2 added(float2 e, const Ctl64* __restrict__ ctl) {
+  if (fabsf(e.x) <= 3.0e38f && fabsf(e.y) <= 3.0e38f) return e;
+  return ctl->done ? make_float2(0.0f, 0.0f) : e;
+}
+
 // One colour of the correction sweep (corr2_load, corr2_apply); the last
 // black colour of an iteration (fst not null) adds the corrections of the
 // cell and of the red cell that shares its pair to the FP64 state.
@@ -359,8 +367,8 @@ __global__ void __launch_bounds__(128)
 k_corr64(Nw32 p, const __half2* __restrict__ Hx, const __half2* __restrict__ Hy,
          const __half2* __restrict__ Hz, const float4* __restrict__ rc, float2* __restrict__ e2,
          int color, int first, double* fst, double* Fst, const double* fsrc, const double* Fsrc,
-         const int* __restrict__ stop) {
-  if (*stop) return;
+         const Ctl64* __restrict__ ctl) {
+  if (ctl->stop) return;
   const Level& L = p.L;
   const int j = blockIdx.y, k = blockIdx.z;
   const __half2* H[3] = {Hx, Hy, Hz};
@@ -374,14 +382,14 @@ k_corr64(Nw32 p, const __half2* __restrict__ Hx, const __half2* __restrict__ Hy,
   if (!fst) return;
   const RBIdx rb = rb_index(L, i, j, k);
   if (in) {
-    const float2 e = e2[a.own];
+    const float2 e = added(e2[a.own], ctl);
     fst[a.c] = fsrc[a.c] + (double)e.x;
     Fst[a.c] = Fsrc[a.c] + (double)e.y;
   }
   const int ir = i ^ 1;     // the pair's red cell (also of a row's odd tail)
   if (ir < L.nx) {
     const ix cr = cidx32(L, ir, j, k);
-    const float2 e = e2[(ix)(1 - color) * rb.plane + rb.pos];
+    const float2 e = added(e2[(ix)(1 - color) * rb.plane + rb.pos], ctl);
     fst[cr] = fsrc[cr] + (double)e.x;
     Fst[cr] = Fsrc[cr] + (double)e.y;
   }
@@ -393,10 +401,11 @@ __global__ void __launch_bounds__(kT2Threads)
 k_corr64_tile2d(Nw32 p, int tx, int ty, int sweeps, const __half2* __restrict__ Hx,
                 const __half2* __restrict__ Hy, const float4* __restrict__ rc,
                 const float2* __restrict__ e2, double* fst, double* Fst, const double* fsrc,
-                const double* Fsrc, const int* __restrict__ stop) {
-  if (*stop) return;
+                const double* Fsrc, const Ctl64* __restrict__ ctl) {
+  if (ctl->stop) return;
   corr_tile2d<G>(p, blockIdx.x * tx, blockIdx.y * ty, tx, ty, sweeps, Hx, Hy, rc, e2,
                  [&](ix c, float2 e) {
+                   e = added(e, ctl);
                    fst[c] = fsrc[c] + widen(e.x);
                    Fst[c] = Fsrc[c] + widen(e.y);
                  });
@@ -452,6 +461,8 @@ void launch_setup(sfx_ctx* c, const Setup64& q, cudaStream_t s) {
   SFX_KERNEL(c, K_SETUP, k_setup64<ND>, g, kSX * kSY * BZ, s, q);
 }
 
+constexpr double kHalfMax = 65504.0;   // the largest half
+
 // Iterations after which a solve that still converges slowly is handed to
 // the Picard solver.
 constexpr int kMaxNewton = 30;
@@ -489,7 +500,7 @@ sfx_status solve(sfx_ctx* c, const Newton64& q, double* f, double* F, bool from_
         const dim3 g((unsigned)((L.nx + t2.tx - 1) / t2.tx), (unsigned)((L.ny + t2.ty - 1) / t2.ty));
         prof_before(c, K_SMOOTH_FINE, s);
         k_corr64_tile2d<G><<<g, kT2Threads, t2smem, s>>>(q.p, t2.tx, t2.ty, sweeps, q.H[0], q.H[1],
-                                                         q.rc, q.e2, f, F, fa, Fa, &ctl->stop);
+                                                         q.rc, q.e2, f, F, fa, Fa, ctl);
         prof_after(c, K_SMOOTH_FINE, s);
       }
       for (int w = 0; w < sweeps && t2.ty == 0; ++w)
@@ -497,7 +508,7 @@ sfx_status solve(sfx_ctx* c, const Newton64& q, double* f, double* F, bool from_
           const bool add = w == sweeps - 1 && color == 1;
           SFX_KERNEL(c, K_SMOOTH_FINE, k_corr64<G>, grd, blk, s, q.p, q.H[0], q.H[1], q.H[2], q.rc,
                      q.e2, color, w == 0 ? 1 : 0, add ? f : nullptr, add ? F : nullptr, fa, Fa,
-                     &ctl->stop);
+                     ctl);
         }
       SFX_LAUNCH_CHECK();
     }
@@ -550,7 +561,9 @@ sfx_status drift_faces64(sfx_ctx* c, const double* phi, double Df, double DF, do
 // multigrid depth and max(D) dt/h^2 <= 1, where relaxation alone converges
 // (0.15-0.5 per sweep); beyond it, and where the caller names a number of
 // levels, the Picard solver's V-cycles are the better ones.  Its work arrays
-// index with 32 bits and its launches put rows in grid y.
+// index with 32 bits and its launches put rows in grid y.  The sweeps' drift
+// faces are half precision and at most D/eps: larger ones are left to the
+// Picard solver as well.
 // Planar steps with a flow stay with the Picard solver too: at tol = 1e-10 its
 // states there carry an error of up to 4e-9 in the force (of 30 circles of 50
 // to 512 cells a side, rotating, a third above 1e-9), and programs that
@@ -563,8 +576,10 @@ bool newton64_eligible(const sfx_ctx* c, const sfx_params* p, double dt, const s
   const size_t nx = L.nx, ny = L.ny, nz = L.nz;
   const size_t most = std::max({(nx + 1) * ny * nz, nx * (ny + 1) * nz, nx * ny * (nz + 1),
                                 2 * ny * nz * ((nx + 1) / 2)});
-  return c->prec == SFX_F64 && o->mg_levels == 0 && !(flow && L.geom == SFX_PLANAR2D) && most < ((size_t)1 << 31) && ny <= 65535 &&
-         nz <= 65535 && std::max(p->Df, p->DF) * dt <= L.h * L.h;
+  const double D = std::max(p->Df, p->DF);
+  return c->prec == SFX_F64 && o->mg_levels == 0 && !(flow && L.geom == SFX_PLANAR2D) &&
+         most < ((size_t)1 << 31) && ny <= 65535 && nz <= 65535 && D * dt <= L.h * L.h &&
+         D <= kHalfMax * p->eps;
 }
 
 // The work arrays of the Newton solve; where there is no memory for them the
