@@ -233,10 +233,10 @@ __global__ void k_loss_grad(Level L, EosArgs q, const double* __restrict__ f,
 
 }  // namespace
 
-unsigned* cut_list(sfx_ctx* c, cudaStream_t s) {
+unsigned* cell_list(sfx_ctx* c, unsigned** slot, cudaStream_t s) {
   const size_t n = c->lev[0].lv.ncell();
   cudaStreamCaptureStatus cap;
-  if (c->cut_list || n >= ((size_t)1 << 32)) return c->cut_list;
+  if (*slot || n >= ((size_t)1 << 32)) return *slot;
   void* p = nullptr;
   if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
       cudaMalloc(&p, (n + 1) * sizeof(unsigned)) != cudaSuccess) {
@@ -244,7 +244,7 @@ unsigned* cut_list(sfx_ctx* c, cudaStream_t s) {
     return nullptr;
   }
   c->allocations.push_back(p);
-  return c->cut_list = (unsigned*)p;
+  return *slot = (unsigned*)p;
 }
 
 // sigma, the force and (dm not null) delta_m of an FP64 state
@@ -254,7 +254,7 @@ static sfx_status eos_force(sfx_ctx* c, const EosArgs& q, const double* f, const
   const Level& L = c->lev[0].lv;
   const size_t n = L.ncell();
   const int nb = blocks_for(n, 256);
-  unsigned* list = dm_mode != 0 ? cut_list(c, s) : nullptr;
+  unsigned* list = dm_mode != 0 ? cell_list(c, &c->force_list, s) : nullptr;
   SFX_KERNEL(c, K_FORCES, k_eos, nb, 256, s, n, q, f, phi, sigma, list);
   if (list) SFX_KERNEL(c, K_FORCES, k_force_list, nb, 256, s, n, L.ndim(), C, force, dm, list);
   SFX_KERNEL(c, K_FORCES, k_force, std::min(blocks_for(n, 64), c->sm_count * 16), 64, s, L, phi, C,

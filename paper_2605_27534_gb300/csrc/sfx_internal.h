@@ -224,10 +224,15 @@ struct sfx_ctx {
   sfx::AdjScratch adj;
   sfx::N64Scratch n64;
   float* chi32 = nullptr;            // SFX_F32 redistancing: chi0, two iterates
-  void* block_list = nullptr;        // redistancing and VoF: active blocks and their flags
-  unsigned char* vofH = nullptr;     // VoF: indicator H, minus-face fluxes Q by cell
+  // Each call has its own scratch: calls of one context on different streams
+  // may overlap as long as they are different calls.
+  void* block_list = nullptr;        // redistancing: active blocks and their flags
+  unsigned char* vofH = nullptr;     // VoF: indicator H, minus-face fluxes Q by cell,
   double* vofQ = nullptr;
-  unsigned* cut_list = nullptr;      // cells near the interface: a count and their indices
+  void* vof_blocks = nullptr;        // on large grids active blocks with their flags
+  unsigned* vof_cut = nullptr;       // and the faces that need a plane (cell_list)
+  unsigned* force_list = nullptr;    // Marangoni force: interface cells (cell_list),
+  unsigned* eos_band = nullptr;      // FP32 EOS: cells with Gamma > 0 (cell_list)
   double* acdi = nullptr;            // ACDI: phi*, r, psi, unit normals
 };
 
@@ -307,11 +312,12 @@ sfx_status acdi_step(sfx_ctx* c, const void* ux, const void* uy, const void* uz,
 // sfx_capillary.cu
 sfx_status capillary(sfx_ctx* c, const sfx_params* p, const double* phi, const void* C,
                      const void* sigma, void* kappa, void* force, cudaStream_t s);
-// sfx_forces.cu: ctx->cut_list (allocated on first use; each pass fills it
-// anew), null where a grid's cells do not fit 32-bit indices, no memory is
-// left for it or its first use is within a stream capture: the passes then
-// take every cell in turn
-unsigned* cut_list(sfx_ctx* c, cudaStream_t s);
+// sfx_forces.cu: a list of cells of the context (`slot`: a count and their
+// indices, filled anew by each pass), allocated on first use; null where a
+// grid's cells do not fit 32-bit indices, no memory is left for it or its
+// first use is within a stream capture: the passes then take every cell in
+// turn
+unsigned* cell_list(sfx_ctx* c, unsigned** slot, cudaStream_t s);
 // sfx_phase.cu: allocates ctx->block_list: for the nb blocks of cells a count,
 // nb int2, six doubles and two flags per block (each pass fills it anew)
 sfx_status block_list(sfx_ctx* c);

@@ -226,9 +226,9 @@ sfx_status vof_impl(sfx_ctx* c, const U* const* u, double dt, int order, double*
   int2* list = nullptr;
   unsigned grid = (unsigned)nb;
   unsigned* cut = nullptr;
-  if (L.ncell() >= kVofListCells) {
-    cut = cut_list(c, s);
-    list = (int2*)c->block_list;
+  if (c->vof_blocks) {
+    cut = cell_list(c, &c->vof_cut, s);
+    list = (int2*)c->vof_blocks;
     unsigned char* flag = (unsigned char*)(list + nb + 1);
     SFX_CUDA(cudaMemsetAsync(list, 0, sizeof(int2), s));
     SFX_KERNEL(c, K_OTHER, k_vof_flags<ND>, (unsigned)((nb + 7) / 8), 256, s, L, (unsigned)nb, C, flag);
@@ -257,13 +257,25 @@ sfx_status vof_impl(sfx_ctx* c, const U* const* u, double dt, int order, double*
 sfx_status vof_advect(sfx_ctx* c, const void* ux, const void* uy, const void* uz, double dt,
                       int order, double* C, cudaStream_t s) {
   const Level& L = c->lev[0].lv;
+  const bool three = L.ndim() == 3;
   if (!c->vofH) {
     SFX_CUDA(cudaMalloc((void**)&c->vofH, L.ncell()));
     c->allocations.push_back(c->vofH);
+  }
+  if (!c->vofQ) {
     SFX_CUDA(cudaMalloc((void**)&c->vofQ, L.ncell() * sizeof(double)));
     c->allocations.push_back(c->vofQ);
+    // (without memory for the list every block is taken)
+    const size_t nb = three ? CellBlock<3>::count(L) : CellBlock<2>::count(L);
+    if (L.ncell() >= kVofListCells) {
+      if (cudaMalloc(&c->vof_blocks, (nb + 1) * sizeof(int2) + 2 * nb) == cudaSuccess) {
+        c->allocations.push_back(c->vof_blocks);
+      } else {
+        c->vof_blocks = nullptr;
+        cudaGetLastError();
+      }
+    }
   }
-  const bool three = L.ndim() == 3;
   if (c->prec == SFX_F32) {
     const float* u[3] = {(const float*)ux, (const float*)uy, (const float*)uz};
     return three ? vof_impl<float, float, 3>(c, u, dt, order, C, s)
