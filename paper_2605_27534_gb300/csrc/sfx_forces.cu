@@ -42,11 +42,8 @@ struct EosArgs {
 };
 
 // Gamma = f/delta_phi where delta_phi >= 1e-3/eps, else 0; sigma in double.
-// It also empties the list of interface cells of the force behind it.
 __global__ void k_eos(size_t n, EosArgs q, const double* __restrict__ f,
-                      const double* __restrict__ phi, double* __restrict__ sigma,
-                      unsigned* __restrict__ list) {
-  if (list && blockIdx.x == 0 && threadIdx.x == 0) list[0] = 0;
+                      const double* __restrict__ phi, double* __restrict__ sigma) {
   for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
        c += (size_t)gridDim.x * blockDim.x) {
     double p = phi[c];
@@ -123,51 +120,69 @@ __device__ __forceinline__ void force64_cell(const Level& L, const double* __res
   if (dm_out) dm_out[c] = dm;
 }
 
+// |grad C| instead of the PLIC area (dm_mode 0): every cell carries a force.
+__global__ void __launch_bounds__(256)
+k_force(Level L, const double* __restrict__ phi, const double* __restrict__ C,
+        const double* __restrict__ sigma, double eps, double* __restrict__ force,
+        double* __restrict__ dm_out) {
+  const size_t n = L.ncell();
+  for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
+       c += (size_t)gridDim.x * blockDim.x)
+    force64_cell(L, phi, C, sigma, 0, eps, c, force, dm_out);
+}
+
 // With the PLIC area only interface cells carry a force (1e-6 < C < 1 - 1e-6:
-// nearer fractions are the round-off of empty or full cells).  They are
-// listed first and taken by full warps: a cell is a chain of about 600 FP64
-// instructions, an instruction occupies the SM's FP64 pipe for a whole warp
-// however few lanes it serves, and in rows of 32 cells a warp held one or two
-// interface cells.  96^3: 449 -> 36 us, 128^2 104 -> 21 us (with the plane
-// offsets of sfx_plic.cuh).
-__global__ void k_force_list(size_t n, int nd, const double* __restrict__ C,
-                             double* __restrict__ force, double* __restrict__ dm_out,
-                             unsigned* __restrict__ list) {
-  const size_t step = (size_t)gridDim.x * blockDim.x;
-  // every lane of a warp takes part in the append
-  for (size_t b = blockIdx.x * (size_t)blockDim.x; b < n; b += step) {
-    const size_t c = b + threadIdx.x;
+// nearer fractions are the round-off of empty or full cells).  A block gathers
+// those of its 512 cells and takes them by full warps: a cell is a chain of
+// about 600 FP64 instructions, an instruction occupies the SM's FP64 pipe for a
+// whole warp however few lanes it serves, and in rows of 32 cells a warp held
+// one or two interface cells.  The gathered cells stay in shared memory: the
+// call has no scratch, so that calls on different streams may overlap.  With
+// the EOS: 96^3 533 -> 130 us, 160^3 1874 -> 250, 128^2 109 -> 46 (a list of the
+// context's cells: 119, 221, 50; boxes of 1024 and 2048 cells 140-167 at 96^3,
+// of 256 cells 128-146: what is left is the chains of the fullest SMs).
+template <int ND>
+__global__ void __launch_bounds__(128)
+k_force_cut(Level L, const double* __restrict__ phi, const double* __restrict__ C,
+            const double* __restrict__ sigma, double eps, double* __restrict__ force,
+            double* __restrict__ dm_out) {
+  using B = CellBlock<ND>;
+  __shared__ unsigned short list[B::threads];
+  __shared__ unsigned count;
+  const size_t n = L.ncell();
+  const unsigned nbx = (L.nx + B::bx - 1) / B::bx, nby = (L.ny + B::by - 1) / B::by;
+  const int x0 = (int)(blockIdx.x % nbx) * B::bx, y0 = (int)(blockIdx.x / nbx % nby) * B::by,
+            z0 = (int)(blockIdx.x / nbx / nby) * B::bz;
+  const auto cell = [&](int t) {
+    return cidx(L, x0 + t % B::bx, y0 + t / B::bx % B::by, z0 + t / (B::bx * B::by));
+  };
+  if (threadIdx.x == 0) count = 0;
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int t = threadIdx.x; t < B::threads; t += 128) {   // rows of cells
     bool cut = false;
-    if (c < n) {
+    if (x0 + t % B::bx < L.nx && y0 + t / B::bx % B::by < L.ny &&
+        z0 + t / (B::bx * B::by) < L.nz) {
+      const size_t c = cell(t);
       const double Cc = C[c];
       cut = Cc > 1e-6 && Cc < 1.0 - 1e-6;
       if (!cut) {
-        for (int d = 0; d < nd; ++d) force[(size_t)d * n + c] = 0.0;
+#pragma unroll
+        for (int d = 0; d < ND; ++d) force[(size_t)d * n + c] = 0.0;
         if (dm_out) dm_out[c] = 0.0;
       }
     }
-    warp_append(list, cut, (unsigned)c);
+    const unsigned m = __ballot_sync(0xffffffffu, cut);
+    if (!m) continue;
+    unsigned base = 0;
+    if (lane == 0) base = atomicAdd(&count, (unsigned)__popc(m));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (cut) list[base + __popc(m & ((1u << lane) - 1))] = (unsigned short)t;
   }
-}
-
-// The cells of the list, or all of them (list null: every cell carries |grad
-// C|, or its index does not fit the list).
-__global__ void __launch_bounds__(64)
-k_force(Level L, const double* __restrict__ phi, const double* __restrict__ C,
-        const double* __restrict__ sigma, int dm_mode, double eps,
-        const unsigned* __restrict__ list, double* __restrict__ force,
-        double* __restrict__ dm_out) {
-  const size_t n = list ? list[0] : L.ncell();
-  for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n;
-       q += (size_t)gridDim.x * blockDim.x) {
-    const size_t c = list ? list[1 + q] : q;
-    if (!list && dm_mode != 0 && !(C[c] > 1e-6 && C[c] < 1.0 - 1e-6)) {
-      for (int d = 0; d < L.ndim(); ++d) force[(size_t)d * n + c] = 0.0;
-      if (dm_out) dm_out[c] = 0.0;
-      continue;
-    }
-    force64_cell(L, phi, C, sigma, dm_mode, eps, c, force, dm_out);
-  }
+  __syncthreads();
+  for (unsigned q = threadIdx.x; q < count; q += 128)
+    force64_cell(L, phi, C, sigma, 1, eps, cell(list[q]), force, dm_out);
 }
 
 // Loss L = sum_c V_c |F_Ma,c|^2: block partials of the sum and, when G is
@@ -254,11 +269,15 @@ static sfx_status eos_force(sfx_ctx* c, const EosArgs& q, const double* f, const
   const Level& L = c->lev[0].lv;
   const size_t n = L.ncell();
   const int nb = blocks_for(n, 256);
-  unsigned* list = dm_mode != 0 ? cell_list(c, &c->force_list, s) : nullptr;
-  SFX_KERNEL(c, K_FORCES, k_eos, nb, 256, s, n, q, f, phi, sigma, list);
-  if (list) SFX_KERNEL(c, K_FORCES, k_force_list, nb, 256, s, n, L.ndim(), C, force, dm, list);
-  SFX_KERNEL(c, K_FORCES, k_force, std::min(blocks_for(n, 64), c->sm_count * 16), 64, s, L, phi, C,
-             sigma, dm_mode, q.eps, list, force, dm);
+  SFX_KERNEL(c, K_FORCES, k_eos, nb, 256, s, n, q, f, phi, sigma);
+  if (dm_mode == 0)
+    SFX_KERNEL(c, K_FORCES, k_force, nb, 256, s, L, phi, C, sigma, q.eps, force, dm);
+  else if (L.ndim() == 3)
+    SFX_KERNEL(c, K_FORCES, k_force_cut<3>, (unsigned)CellBlock<3>::count(L), 128, s, L, phi, C,
+               sigma, q.eps, force, dm);
+  else
+    SFX_KERNEL(c, K_FORCES, k_force_cut<2>, (unsigned)CellBlock<2>::count(L), 128, s, L, phi, C,
+               sigma, q.eps, force, dm);
   SFX_LAUNCH_CHECK();
   return SFX_OK;
 }

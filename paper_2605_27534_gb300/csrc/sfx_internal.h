@@ -231,8 +231,8 @@ struct sfx_ctx {
   double* vofQ = nullptr;
   void* vof_blocks = nullptr;        // on large grids active blocks with their flags
   unsigned* vof_cut = nullptr;       // and the faces that need a plane (cell_list)
-  unsigned* force_list = nullptr;    // Marangoni force: interface cells (cell_list),
-  unsigned* eos_band = nullptr;      // FP32 EOS: cells with Gamma > 0 (cell_list)
+  unsigned* force_list = nullptr;    // FP32 Marangoni force: interface cells (cell_list)
+  unsigned* eos_band = nullptr;      // and cells with Gamma > 0 (cell_list)
   double* acdi = nullptr;            // ACDI: phi*, r, psi, unit normals
 };
 

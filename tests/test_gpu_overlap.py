@@ -65,3 +65,37 @@ def test_calls_of_one_context_overlap(geom, shape, prec):
         torch.cuda.synchronize()
         for o, w in zip(outs, want):
             assert all(torch.equal(a, b) for a, b in zip(o, w))
+
+
+@pytest.mark.parametrize("shape", [(40, 44, 50), (1, 300, 310)])
+def test_fp64_forces_of_one_context_overlap(shape):
+    """The FP64 force has no scratch: two of them, of different fractions."""
+    import paper_2605_27534_gb300 as sfx
+    import torch
+    nz, ny, nx = shape
+    g = W.Grid(W.CART3D if nz > 1 else W.PLANAR, nx, ny, nz, 1.0 / max(shape))
+    p = W.Params(eps=0.75 * g.h)
+    rng = np.random.default_rng(5)
+    phi = dev(rng.uniform(0.02, 0.98, shape))
+    f = dev(0.4 * rng.uniform(0, 1, shape) * 0.2 / p.eps)
+    C = [dev(np.where(rng.uniform(size=shape) < w, rng.uniform(0.1, 0.9, shape), 0.0)) for w in (0.02, 0.4)]
+    ctx = sfx.Context.for_grid(g, sfx.SFX_F64)
+    sigma = [torch.empty_like(phi) for _ in C]
+    force = [torch.empty((g.ndim,) + shape, dtype=torch.float64, device="cuda") for _ in C]
+    streams = [torch.cuda.Stream() for _ in C]
+
+    def call(k):
+        ctx.sfx_marangoni_force(p, f, phi, C[k], sigma[k], force[k])
+
+    for k in (0, 1):
+        call(k)
+    torch.cuda.synchronize()
+    want = [t.clone() for t in force]
+    torch.cuda.synchronize()
+    for _ in range(40):
+        for _ in range(4):
+            for k in (0, 1):
+                with torch.cuda.stream(streams[k]):
+                    call(k)
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(force, want))
