@@ -1181,7 +1181,10 @@ struct RowWalk {
 // others' force set to zero (four cells per thread: C in, force out, bound by
 // HBM), and a second launch takes the listed cells by full warps; in rows of
 // cells a warp held a few of them and every other lane waited.  256^3: 157 ->
-// 69 us, 160^3 58 -> 33 us.
+// 69 us, 160^3 58 -> 33 us.  On small grids the launch costs more than that
+// saves (with the EOS: 512^2 27 us in rows, 30 with a list, 60 x 70 x 65 30 and
+// 36, 128^2 24 and 29; 96^3 50 and 41), so they take every cell in rows.
+constexpr size_t kForceListCells = (size_t)1 << 19;
 __device__ __forceinline__ bool cut32(float C) { return C > 1e-6f && C < 1.0f - 1e-6f; }
 
 template <bool QUADS>
@@ -1223,7 +1226,8 @@ k_force32_cells(Level L, const double* __restrict__ phi, const float* __restrict
   }
 }
 
-// dm_mode 0: every cell; blocks over (x chunk, rows), rows r = k ny + j
+// Every cell (dm_mode 0, and small grids); blocks over (x chunk, rows), rows
+// r = k ny + j
 __global__ void k_force32(Level L, const double* __restrict__ phi, const float* __restrict__ C,
                           const float* __restrict__ dsig, int dm_mode, float inv_eps,
                           float* __restrict__ force) {
@@ -2019,7 +2023,7 @@ sfx_status marangoni32(sfx_ctx* c, const sfx_params* p, const float2* f, const d
   const size_t n = L.ncell();
   Eos32 q{(float)p->gamma_inf, (float)p->eps, (float)(1.0 / p->eps), (float)p->sigma0,
           (float)p->E, p->eos, p->sigma0 * p->E, p->gamma_inf / p->eps};
-  unsigned* list = dm_mode != 0 ? cell_list(c, &c->force_list, s) : nullptr;
+  unsigned* list = dm_mode != 0 && n >= kForceListCells ? cell_list(c, &c->force_list, s) : nullptr;
   unsigned* band = n >= kEosListCells ? cell_list(c, &c->eos_band, s) : nullptr;
   if (band) {
     SFX_CUDA(cudaMemsetAsync(band, 0, sizeof(unsigned), s));
