@@ -131,6 +131,10 @@ k_force(Level L, const double* __restrict__ phi, const double* __restrict__ C,
     force64_cell(L, phi, C, sigma, 0, eps, c, force, dm_out);
 }
 
+__device__ __forceinline__ bool finite_bits(double x) {
+  return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u;
+}
+
 // With the PLIC area only interface cells carry a force (1e-6 < C < 1 - 1e-6:
 // nearer fractions are the round-off of empty or full cells).  A block gathers
 // those of its 512 cells and takes them by full warps: a cell is a chain of
@@ -138,7 +142,7 @@ k_force(Level L, const double* __restrict__ phi, const double* __restrict__ C,
 // whole warp however few lanes it serves, and in rows of 32 cells a warp held
 // one or two interface cells.  The gathered cells stay in shared memory: the
 // call has no scratch, so that calls on different streams may overlap.  With
-// the EOS: 96^3 533 -> 130 us, 160^3 1874 -> 250, 128^2 109 -> 46 (a list of the
+// the EOS: 96^3 533 -> 133 us, 160^3 1874 -> 252, 128^2 109 -> 46 (a list of the
 // context's cells: 119, 221, 50; boxes of 1024 and 2048 cells 140-167 at 96^3,
 // of 256 cells 128-146: what is left is the chains of the fullest SMs).
 template <int ND>
@@ -168,8 +172,18 @@ k_force_cut(Level L, const double* __restrict__ phi, const double* __restrict__ 
       const double Cc = C[c];
       cut = Cc > 1e-6 && Cc < 1.0 - 1e-6;
       if (!cut) {
+        // delta_m = 0 times a gradient of sigma that is not finite is NaN
+        const int x[3] = {x0 + t % B::bx, y0 + t / B::bx % B::by, z0 + t / (B::bx * B::by)};
+        const size_t st[3] = {1, (size_t)L.nx, (size_t)L.nx * L.ny};
+        bool finite = true;
 #pragma unroll
-        for (int d = 0; d < ND; ++d) force[(size_t)d * n + c] = 0.0;
+        for (int d = 0; d < ND; ++d) {
+          finite &= finite_bits(sigma[x[d] + 1 < L.extent(d) ? c + st[d] : c]);
+          finite &= finite_bits(sigma[x[d] > 0 ? c - st[d] : c]);
+        }
+        const double v = finite ? 0.0 : __longlong_as_double(0x7ff8000000000000LL);
+#pragma unroll
+        for (int d = 0; d < ND; ++d) force[(size_t)d * n + c] = v;
         if (dm_out) dm_out[c] = 0.0;
       }
     }
