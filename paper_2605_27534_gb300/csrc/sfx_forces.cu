@@ -82,6 +82,10 @@ __device__ __forceinline__ double eos_slope(const EosArgs& q, double G) {
   return -q.sigma0 * q.E / q.ginf * (1.0 - t * t);
 }
 
+// Interface cells of the PLIC area: nearer fractions are the round-off of empty
+// or full cells.
+__device__ __forceinline__ bool plic_cell(double C) { return C > 1e-6 && C < 1.0 - 1e-6; }
+
 // One cell of the Marangoni force with its delta_m.
 __device__ __forceinline__ void force64_cell(const Level& L, const double* __restrict__ phi,
                                              const double* __restrict__ C,
@@ -114,7 +118,7 @@ __device__ __forceinline__ void force64_cell(const Level& L, const double* __res
   } else {
     double m[3];
     youngs_normal(L, C, idx[0], idx[1], idx[2], m);
-    dm = plic_unit_area(nd, m, C[c]) / L.h;
+    dm = plic_cell(C[c]) ? plic_unit_area(nd, m, C[c]) / L.h : 0.0;
   }
   for (int d = 0; d < nd; ++d) force[(size_t)d * n + c] = dm * (gs[d] - nn[d] * ndg);
   if (dm_out) dm_out[c] = dm;
@@ -135,10 +139,8 @@ __device__ __forceinline__ bool finite_bits(double x) {
   return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u;
 }
 
-// With the PLIC area only interface cells carry a force (1e-6 < C < 1 - 1e-6:
-// nearer fractions are the round-off of empty or full cells).  A block gathers
-// those of its 512 cells and takes them by full warps: a cell is a chain of
-// about 600 FP64 instructions, an instruction occupies the SM's FP64 pipe for a
+// With the PLIC area only interface cells carry a force.  A block gathers those
+// of its 512 cells and takes them by full warps: a cell is a chain of about 600 FP64 instructions, an instruction occupies the SM's FP64 pipe for a
 // whole warp however few lanes it serves, and in rows of 32 cells a warp held
 // one or two interface cells.  The gathered cells stay in shared memory: the
 // call has no scratch, so that calls on different streams may overlap.  With
@@ -169,21 +171,26 @@ k_force_cut(Level L, const double* __restrict__ phi, const double* __restrict__ 
     if (x0 + t % B::bx < L.nx && y0 + t / B::bx % B::by < L.ny &&
         z0 + t / (B::bx * B::by) < L.nz) {
       const size_t c = cell(t);
-      const double Cc = C[c];
-      cut = Cc > 1e-6 && Cc < 1.0 - 1e-6;
+      cut = plic_cell(C[c]);
       if (!cut) {
-        // delta_m = 0 times a gradient of sigma that is not finite is NaN
+        // delta_m = 0 times a gradient or a normal that is not finite is NaN:
+        // those cells are evaluated as well
         const int x[3] = {x0 + t % B::bx, y0 + t / B::bx % B::by, z0 + t / (B::bx * B::by)};
         const size_t st[3] = {1, (size_t)L.nx, (size_t)L.nx * L.ny};
         bool finite = true;
 #pragma unroll
         for (int d = 0; d < ND; ++d) {
-          finite &= finite_bits(sigma[x[d] + 1 < L.extent(d) ? c + st[d] : c]);
-          finite &= finite_bits(sigma[x[d] > 0 ? c - st[d] : c]);
+          const size_t cp = x[d] + 1 < L.extent(d) ? c + st[d] : c, cm = x[d] > 0 ? c - st[d] : c;
+          finite &= finite_bits(sigma[cp]);
+          finite &= finite_bits(sigma[cm]);
+          finite &= finite_bits(phi[cp]);
+          finite &= finite_bits(phi[cm]);
         }
-        const double v = finite ? 0.0 : __longlong_as_double(0x7ff8000000000000LL);
+        cut = !finite;
+      }
+      if (!cut) {
 #pragma unroll
-        for (int d = 0; d < ND; ++d) force[(size_t)d * n + c] = v;
+        for (int d = 0; d < ND; ++d) force[(size_t)d * n + c] = 0.0;
         if (dm_out) dm_out[c] = 0.0;
       }
     }
