@@ -39,6 +39,12 @@ constexpr size_t kVofListCells = (size_t)1 << 20;
 
 __device__ __forceinline__ long long vbits(double v) { return __double_as_longlong(v); }
 
+// a cell that may give fluid: C > 0, or NaN of either sign
+__device__ __forceinline__ bool wet(double C) {
+  const long long b = vbits(C);
+  return b > 0 || (unsigned long long)b > 0xfff0000000000000ULL;
+}
+
 // flag[b] = 1 where block b holds fluid 1: a warp per block, its 16 rows of
 // 32 cells in flight together
 template <int ND>
@@ -50,15 +56,15 @@ __global__ void __launch_bounds__(256) k_vof_flags(Level L, unsigned nb, const d
   const unsigned nbx = (L.nx + B::bx - 1) / B::bx, nby = (L.ny + B::by - 1) / B::by;
   const int i = (int)(b % nbx) * B::bx + (threadIdx.x & 31);
   const int j0 = (int)(b / nbx % nby) * B::by, k0 = (int)(b / nbx / nby) * B::bz;
-  bool wet = false;
+  bool any = false;
   if (i < L.nx) {
 #pragma unroll
     for (int r = 0; r < B::by * B::bz; ++r) {
       const int j = j0 + r % B::by, k = k0 + r / B::by;
-      if (j < L.ny && k < L.nz) wet |= vbits(C[cidx(L, i, j, k)]) > 0;
+      if (j < L.ny && k < L.nz) any |= wet(C[cidx(L, i, j, k)]);
     }
   }
-  const bool any = __any_sync(0xffffffffu, wet);
+  any = __any_sync(0xffffffffu, any);
   if ((threadIdx.x & 31) == 0) flag[b] = any ? 1 : 0;
 }
 
@@ -152,7 +158,7 @@ k_vof_flux(Level L, int d, const int2* __restrict__ list, const double* __restri
         const double cm = C[c - st];
         const U uf = u[fidx(L, d, x[0], x[1], x[2])];
         const double cu = uf > U(0) ? cm : cq;
-        if (uf != U(0) && vbits(cu) > 0) {     // a flow out of a cell with fluid
+        if (uf != U(0) && wet(cu)) {           // a flow out of a cell with fluid
           const double cf = widen(uf) * dt_h;
           // no plane in a cell that is full, in float also within rounding
           if (!((G)cu < G(1))) {
