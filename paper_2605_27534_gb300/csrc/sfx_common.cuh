@@ -98,7 +98,7 @@ struct CellBlock {
                                (w >> 3) * 2 + (l >> 4))
                    : make_int3((w & 3) * 8 + (l & 7), (w >> 2) * 4 + (l >> 3), 0);
   }
-  static size_t count(const Level& L) {
+  static __host__ __device__ __forceinline__ size_t count(const Level& L) {
     return (((size_t)L.nx + bx - 1) / bx) * (((size_t)L.ny + by - 1) / by) *
            (((size_t)L.nz + bz - 1) / bz);
   }

@@ -45,6 +45,60 @@ __device__ __forceinline__ bool wet(double C) {
   return b > 0 || (unsigned long long)b > 0xfff0000000000000ULL;
 }
 
+__device__ __forceinline__ bool finite_bits(float x) {
+  return (__float_as_uint(x) & 0x7f800000u) != 0x7f800000u;
+}
+__device__ __forceinline__ bool finite_bits(double x) {
+  return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u;
+}
+__device__ __forceinline__ bool positive(double x) {   // false for NaN
+  return (unsigned long long)vbits(x) - 1ULL < 0x7ff0000000000000ULL;
+}
+
+template <typename U>
+struct VofVel {
+  const U* u[3];
+};
+
+// list[0].y = 1 where a velocity is not finite: H (c_+ - c_-) of its cells is
+// NaN then, with H = 0 too, and the passes behind it visit every block.  Block
+// b of nb.
+template <typename U, int ND>
+__device__ __forceinline__ void vof_finite(const Level& L, const VofVel<U>& v, unsigned b,
+                                           unsigned nb, int2* __restrict__ list) {
+  constexpr int per = 16 / sizeof(U);
+  struct alignas(16) Pack {
+    U x[per];
+  };
+  bool ok = true;
+  const size_t t0 = (size_t)b * blockDim.x + threadIdx.x, step = (size_t)nb * blockDim.x;
+  for (int d = 0; d < ND; ++d) {
+    const U* u = v.u[d];
+    const size_t n = L.nface(d), m = ((size_t)u & 15) == 0 ? n / per : 0;
+    size_t t = t0;
+    for (; t + 7 * step < m; t += 8 * step) {
+      Pack q[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) q[k] = reinterpret_cast<const Pack*>(u)[t + k * step];
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+#pragma unroll
+        for (int e = 0; e < per; ++e) ok &= finite_bits(q[k].x[e]);
+    }
+    for (; t < m; t += step) {
+      const Pack q = reinterpret_cast<const Pack*>(u)[t];
+#pragma unroll
+      for (int e = 0; e < per; ++e) ok &= finite_bits(q.x[e]);
+    }
+    for (t = m * per + t0; t < n; t += step) ok &= finite_bits(u[t]);
+  }
+  if (!ok) list[0].y = 1;
+}
+template <typename U, int ND>
+__global__ void __launch_bounds__(128) k_vof_finite(Level L, VofVel<U> v, int2* list) {
+  vof_finite<U, ND>(L, v, blockIdx.x, gridDim.x, list);
+}
+
 // flag[b] = 1 where block b holds fluid 1: a warp per block, its 16 rows of
 // 32 cells in flight together
 template <int ND>
@@ -89,23 +143,27 @@ __global__ void k_vof_active(Level L, const unsigned char* __restrict__ flag,
   }
 }
 
-// The active blocks, each with a bit per direction whose plus-side neighbour
-// block is active too; list[0] counts them.
+// A bit per direction whose plus-side neighbour of block b is active too.
 template <int ND>
-__global__ void k_vof_list(Level L, const unsigned char* __restrict__ act, int2* __restrict__ list) {
+__device__ __forceinline__ int vof_plus(const Level& L, const unsigned char* __restrict__ act,
+                                        int b) {
   using B = CellBlock<ND>;
   const int nx = (L.nx + B::bx - 1) / B::bx, ny = (L.ny + B::by - 1) / B::by,
             nz = (L.nz + B::bz - 1) / B::bz;
-  const int nb = nx * ny * nz;
-  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x) {
-    if (!act[b]) continue;
-    const int X = b % nx, Y = b / nx % ny, Z = b / nx / ny;
-    int m = 0;
-    if (X + 1 < nx && act[b + 1]) m |= 1;
-    if (Y + 1 < ny && act[b + nx]) m |= 2;
-    if (ND == 3 && Z + 1 < nz && act[b + nx * ny]) m |= 4;
-    list[1 + atomicAdd(&list[0].x, 1)] = make_int2(b, m);
-  }
+  const int X = b % nx, Y = b / nx % ny, Z = b / nx / ny;
+  int m = 0;
+  if (X + 1 < nx && act[b + 1]) m |= 1;
+  if (Y + 1 < ny && act[b + nx]) m |= 2;
+  if (ND == 3 && Z + 1 < nz && act[b + nx * ny]) m |= 4;
+  return m;
+}
+
+// The active blocks with those bits; list[0].x counts them.
+template <int ND>
+__global__ void k_vof_list(Level L, const unsigned char* __restrict__ act, int2* __restrict__ list) {
+  const int nb = (int)CellBlock<ND>::count(L);
+  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x)
+    if (act[b]) list[1 + atomicAdd(&list[0].x, 1)] = make_int2(b, vof_plus<ND>(L, act, b));
 }
 
 // Flux through the minus-side face of cell x in direction d (not a wall)
@@ -116,7 +174,7 @@ __device__ __forceinline__ double plic_flux(const Level& L, int d, const int* x,
                                             const U* __restrict__ u, double dt_h) {
   const size_t c = cidx(L, x[0], x[1], x[2]);
   const double cf = widen(u[fidx(L, d, x[0], x[1], x[2])]) * dt_h;
-  const bool pos = vbits(cf) > 0;
+  const bool pos = positive(cf);
   int y[3] = {x[0], x[1], x[2]};
   if (pos) y[d] -= 1;
   G m[3];
@@ -142,9 +200,10 @@ k_vof_flux(Level L, int d, const int2* __restrict__ list, const double* __restri
   // blocks of fewer threads take a share of a cell block each
   const unsigned sub = (unsigned)CellBlock<ND>::threads / blockDim.x, step = gridDim.x / sub;
   const int t = (int)(blockIdx.x % sub * blockDim.x + threadIdx.x);
-  const unsigned nb = list ? (unsigned)list[0].x : step;
+  const bool every = list && list[0].y;   // NaN may come from any block (vof_finite)
+  const unsigned nb = !list ? step : every ? (unsigned)CellBlock<ND>::count(L) : (unsigned)list[0].x;
   for (unsigned q = blockIdx.x / sub; q < nb; q += step) {
-    const unsigned blk = list ? (unsigned)list[1 + q].x : q;
+    const unsigned blk = list && !every ? (unsigned)list[1 + q].x : q;
     int x[3];
     bool plane = false;
     size_t c = 0;
@@ -163,9 +222,9 @@ k_vof_flux(Level L, int d, const int2* __restrict__ list, const double* __restri
           // no plane in a cell that is full, in float also within rounding
           if (!((G)cu < G(1))) {
             // (plic_slab of a cell with C >= 1; a NaN is no fraction: C (b - a))
-            const G g = (G)cf, w = vbits(cf) > 0 ? G(1) - (G(1) - g) : -g;
+            const G g = (G)cf, w = positive(cf) ? G(1) - (G(1) - g) : -g;
             flux = widen((G)cu >= G(1) ? w : (G)cu * w);
-            if (vbits(cf) <= 0) flux = -flux;
+            if (!positive(cf)) flux = -flux;
           } else {
             plane = true;
           }
@@ -179,14 +238,20 @@ k_vof_flux(Level L, int d, const int2* __restrict__ list, const double* __restri
 }
 
 // The listed faces (cells whose minus-side face in direction d needs a
-// plane): cut[0] of them.
+// plane): cut[0] of them.  In the first direction the first `look` blocks read
+// the velocities instead (vof_finite): the chains of the planes leave HBM idle.
 template <typename U, typename G, int ND>
 __global__ void __launch_bounds__(128)
 k_vof_planes(Level L, int d, const double* __restrict__ C, const U* __restrict__ u, double dt_h,
-             const unsigned* __restrict__ cut, double* __restrict__ Q) {
-  const unsigned n = cut[0];
+             const unsigned* __restrict__ cut, double* __restrict__ Q, unsigned look, VofVel<U> v,
+             int2* __restrict__ list) {
+  if (blockIdx.x < look) {
+    vof_finite<U, ND>(L, v, blockIdx.x, look, list);
+    return;
+  }
+  const unsigned n = cut[0], blocks = gridDim.x - look;
   const size_t st = d == 0 ? 1 : (d == 1 ? (size_t)L.nx : (size_t)L.nx * L.ny);
-  for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
+  for (unsigned q = (blockIdx.x - look) * blockDim.x + threadIdx.x; q < n; q += blocks * blockDim.x) {
     const unsigned c = cut[1 + q];
     const int x[3] = {(int)(c % (unsigned)L.nx), (int)(c / (unsigned)L.nx % (unsigned)L.ny),
                       (int)(c / (unsigned)L.nx / (unsigned)L.ny)};
@@ -196,28 +261,37 @@ k_vof_planes(Level L, int d, const double* __restrict__ C, const U* __restrict__
 
 template <typename U, int ND>
 __global__ void __launch_bounds__(512)
-k_vof_update(Level L, int d, const int2* __restrict__ list, const U* __restrict__ u, double dt_h,
+k_vof_update(Level L, int d, bool first, const int2* __restrict__ list,
+             const unsigned char* __restrict__ act, const U* __restrict__ u, double dt_h,
              const double* __restrict__ Q, const unsigned char* __restrict__ H,
              double* __restrict__ C) {
   using B = CellBlock<ND>;
   const size_t st = d == 0 ? 1 : (d == 1 ? (size_t)L.nx : (size_t)L.nx * L.ny);
-  const unsigned nb = list ? (unsigned)list[0].x : gridDim.x;
   const int ext = d == 0 ? B::bx : (d == 1 ? B::by : B::bz);
+  const bool every = list && list[0].y, all = !list || every;   // velocities may not be finite
+  const unsigned nb = !list ? gridDim.x : every ? (unsigned)B::count(L) : (unsigned)list[0].x;
   for (unsigned q = blockIdx.x; q < nb; q += gridDim.x) {
-    const int2 e = list ? list[1 + q] : make_int2((int)q, 7);
+    // (the fluxes of the first direction took the active blocks only)
+    const int2 e = !list || (every && !first) ? make_int2((int)q, 7)
+                   : every ? make_int2((int)q, vof_plus<ND>(L, act, (int)q)) : list[1 + q];
+    const bool active = !every || act[q], fluxes = active || !first;
     int x[3];
     if (!B::at(L, (unsigned)e.x, x)) continue;
     const size_t c = cidx(L, x[0], x[1], x[2]);
     // no flux through the far wall and into an inactive block
     const bool plus = x[d] + 1 < L.extent(d) && (x[d] % ext + 1 < ext || (e.y >> d & 1));
-    const double Qm = Q[c], Qp = plus ? Q[c + st] : 0.0;
-    const bool h = H[c] != 0;
-    if (!h && ((vbits(Qm) | vbits(Qp)) << 1) == 0) continue;
+    const double Qm = fluxes ? Q[c] : 0.0, Qp = fluxes && plus ? Q[c + st] : 0.0;
+    const bool h = active && H[c] != 0;
+    const bool flux = ((vbits(Qm) | vbits(Qp)) << 1) != 0;
+    if (!h && !all && !flux) continue;
     double v = C[c] - (Qp - Qm);
-    if (h) {
+    if (h || all) {
       const size_t fm = fidx(L, d, x[0], x[1], x[2]);
       const size_t fp = fidx(L, d, x[0] + (d == 0), x[1] + (d == 1), x[2] + (d == 2));
-      v += widen(u[fp]) * dt_h - widen(u[fm]) * dt_h;
+      const U um = u[fm], up = u[fp];
+      if (h) v += widen(up) * dt_h - widen(um) * dt_h;
+      else if (!finite_bits(up) || !finite_bits(um)) v = __longlong_as_double(0x7ff8000000000000LL);
+      else if (!flux) continue;
     }
     C[c] = v;
   }
@@ -232,10 +306,13 @@ sfx_status vof_impl(sfx_ctx* c, const U* const* u, double dt, int order, double*
   int2* list = nullptr;
   unsigned grid = (unsigned)nb;
   unsigned* cut = nullptr;
+  const unsigned char* act = nullptr;
+  const VofVel<U> v{{u[0], u[1], u[2]}};
   if (c->vof_blocks) {
     cut = cell_list(c, &c->vof_cut, s);
     list = (int2*)c->vof_blocks;
     unsigned char* flag = (unsigned char*)(list + nb + 1);
+    act = flag + nb;
     SFX_CUDA(cudaMemsetAsync(list, 0, sizeof(int2), s));
     SFX_KERNEL(c, K_OTHER, k_vof_flags<ND>, (unsigned)((nb + 7) / 8), 256, s, L, (unsigned)nb, C, flag);
     SFX_KERNEL(c, K_OTHER, k_vof_active<ND>, blocks_for(nb, 128), 128, s, L, flag, flag + nb);
@@ -248,11 +325,14 @@ sfx_status vof_impl(sfx_ctx* c, const U* const* u, double dt, int order, double*
     // without a list a block lasts as long as its longest chain: small ones
     SFX_KERNEL(c, K_OTHER, (k_vof_flux<U, G, ND>), list ? grid : 4 * grid, list ? 512 : 128, s, L, d,
                list, C, u[d], dt_h, c->vofQ, q == 0 ? c->vofH : nullptr, cut);
+    const unsigned look = list && q == 0 ? (unsigned)c->sm_count * 2 : 0;
     if (cut)
-      SFX_KERNEL(c, K_OTHER, (k_vof_planes<U, G, ND>), c->sm_count * 16, 128, s, L, d, C, u[d], dt_h,
-                 cut, c->vofQ);
-    SFX_KERNEL(c, K_OTHER, (k_vof_update<U, ND>), grid, 512, s, L, d, list, u[d], dt_h, c->vofQ,
-               c->vofH, C);
+      SFX_KERNEL(c, K_OTHER, (k_vof_planes<U, G, ND>), c->sm_count * 16 + look, 128, s, L, d, C, u[d],
+                 dt_h, cut, c->vofQ, look, v, list);
+    else if (look)
+      SFX_KERNEL(c, K_OTHER, (k_vof_finite<U, ND>), look, 128, s, L, v, list);
+    SFX_KERNEL(c, K_OTHER, (k_vof_update<U, ND>), grid, 512, s, L, d, q == 0, list, act, u[d],
+               dt_h, c->vofQ, c->vofH, C);
   }
   SFX_LAUNCH_CHECK();
   return SFX_OK;

@@ -49,3 +49,21 @@ def test_a_nan_fraction_counts_by_value(shape, where, prec):
         assert g.sum() > 1 and (where == "full" or (g == want).all())
         got.append(g)
     assert (got[0] == got[1]).all()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("value", [np.nan, -np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("where", ["dry", "wall"])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_a_velocity_that_is_not_finite_reaches_empty_cells(shape, where, value, prec):
+    """H (c_+ - c_-) is not a number with H = 0 either."""
+    nz, ny, nx = shape
+
+    def change(C, u):
+        for d, a in enumerate(u):
+            at = [nz // 3, 3, 2]
+            if where == "wall":
+                at[2 - d] = a.shape[2 - d] - 1
+            a[tuple(at)] = value
+    got, want = _run(shape, change, prec)
+    assert want.sum() > 1 and (got == want).all()
