@@ -92,9 +92,12 @@ __device__ __forceinline__ float fold_phi(double p) {
   return b <= 0x3fe0000000000000LL ? narrow(p) : narrow(p - 1.0);   // p <= 1/2 (or below 0)
 }
 
-// a - b taken in FP64, as a float
+// a - b taken in FP64, as a float (NaN where both are the same infinity or NaN)
 __device__ __forceinline__ float diff32(double a, double b) {
-  return __double_as_longlong(a) == __double_as_longlong(b) ? 0.0f : narrow(a - b);
+  return __double_as_longlong(a) == __double_as_longlong(b) &&
+                 ((unsigned)__double2hiint(a) & 0x7ff00000u) != 0x7ff00000u
+             ? 0.0f
+             : narrow(a - b);
 }
 
 // n = grad phi/|grad phi| at cell (i,j,k) (centred differences, one-sided
