@@ -73,6 +73,13 @@ __device__ __forceinline__ void unit_normal(const Level& L, const double* __rest
                                             const int* x, double inv2h, double inv_eps, double* n) {
   const size_t st[3] = {1, (size_t)L.nx, (size_t)L.nx * L.ny};
   const size_t c = cidx(L, x[0], x[1], x[2]);
+  const double pc = phi[c];
+  if (((unsigned)__double2hiint(pc) & 0x7ff00000u) == 0x7ff00000u) {
+    // the drift of its faces, a multiple of phi, is not a number
+#pragma unroll
+    for (int d = 0; d < ND; ++d) n[d] = pc - pc;
+    return;
+  }
   double a[ND], b[ND];
   bool flat = true;
 #pragma unroll
@@ -89,7 +96,7 @@ __device__ __forceinline__ void unit_normal(const Level& L, const double* __rest
     a[d] = (a[d] - b[d]) * inv2h;
     m2 = fma(a[d], a[d], m2);
   }
-  const double m = sqrt(m2), pc = phi[c];
+  const double m = sqrt(m2);
   const double slope = kNormalKappa * (pc * (1.0 - pc) * inv_eps);
   // phi outside [0, 1] has no profile slope: no direction either
   if (m < 1e-30 || !(slope >= 0.0) || !(m > slope)) return;
