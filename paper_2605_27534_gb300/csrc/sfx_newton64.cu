@@ -98,8 +98,8 @@ __device__ __forceinline__ void unit_normal(const Level& L, const double* __rest
   }
   const double m = sqrt(m2);
   const double slope = kNormalKappa * (pc * (1.0 - pc) * inv_eps);
-  // phi outside [0, 1] has no profile slope: no direction either
-  if (m < 1e-30 || !(slope >= 0.0) || !(m > slope)) return;
+  // phi outside [0, 1], and -0, has no profile slope: no direction either
+  if (m < 1e-30 || __double_as_longlong(slope) < 0 || !(m > slope)) return;
   const double w = m >= 2.0 * slope ? 1.0 : m / slope - 1.0;
   const double s = w / m;
 #pragma unroll

@@ -41,3 +41,18 @@ def test_faces_of_a_bad_cell_are_not_a_number(geom, shape, bad, prec):
     for v in out:      # (next to an infinity the normal is inf/inf as well)
         got = np.isnan(host(v))
         assert got[want].all() and (np.isinf(bad) or (got == want).all())
+
+
+@pytest.mark.parametrize("geom,shape", [(W.PLANAR, (1, 20, 33)), (W.CART3D, (9, 14, 35))])
+def test_phi_of_minus_zero_has_no_normal(geom, shape):
+    """phi (1 - phi) = -0 there: |grad phi| over it is below any threshold (as
+    the oracle's normals and those of the forces have it)."""
+    import paper_2605_27534_gb300 as sfx
+    g, p, phi, f, F, dt = _problem(geom, shape)
+    phi[:, ::3, ::2] = -0.0
+    fo, Fo, _ = oracle.surfactant_step(g, p, phi, f, F, dt, 1e-13)
+    ctx = sfx.Context.for_grid(g, sfx.SFX_F64)
+    fd, Fd = dev(f), dev(F)
+    st = ctx.sfx_surfactant_step(p, dev(phi), fd, Fd, dt, opts=sfx.default_opts(tol=1e-13))
+    # both solve to 1e-13 of a right-hand side that is x/dt here (no exchange)
+    assert st.converged and rel_err(host(fd), fo) < 1e-12 and rel_err(host(Fd), Fo) < 1e-12
