@@ -36,6 +36,9 @@ __device__ __forceinline__ bool same_bits(float a, float b) {
 template <typename T> __device__ __forceinline__ T tiny_pos();
 template <> __device__ __forceinline__ double tiny_pos<double>() { return 1e-300; }
 template <> __device__ __forceinline__ float tiny_pos<float>() { return 1e-30f; }
+template <typename T> __device__ __forceinline__ T least_pos();
+template <> __device__ __forceinline__ double least_pos<double>() { return __longlong_as_double(1); }
+template <> __device__ __forceinline__ float least_pos<float>() { return __int_as_float(1); }
 
 // Whether chi0 (s0 here, zm and zp its neighbours', the cell's own past a wall)
 // changes sign against a face neighbour, and then the sub-cell distance
@@ -164,6 +167,8 @@ __global__ void __launch_bounds__(512) k_rd_init(Level L, RdGrid R, const double
 #pragma unroll
         for (int d = 0; d < ND; ++d) dsum += q[d] * q[d];
         a = (T)L.h * s0 / fmax(sqrt(dsum), (T)tiny_pos<T>());
+        // 0 (next to an infinite C) stands for chi0 = 0: the smallest distance
+        if (a == (T)0) a = s0 > (T)0 ? least_pos<T>() : -least_pos<T>();
       }
       aux[c] = a;
       chi[c] = s0;
