@@ -139,18 +139,18 @@ struct AdvFields {
 
 template <typename U, int G, int NF, int TY>
 __global__ void __launch_bounds__(kAX * TY, (NF == 1 ? 2 : 1) * (G == SFX_CART3D ? 16 / TY : 1))
-k_bcg64(Level L, Vel<U> v, double dt, AdvFields<NF> P, int zc) {
+k_bcg64(Level L, Vel<U> v, double dt, AdvFields<NF> P, int zc, unsigned yb, unsigned zb) {
   constexpr int ND = G == SFX_CART3D ? 3 : 2;
   __shared__ double sA[NF][TY][kAX], sS[NF][TY][kAX], sF[NF][TY][kAX];
   const unsigned full = 0xffffffffu;
   const int tx = threadIdx.x, ty = threadIdx.y;
-  const int i = blockIdx.x * (kAX - 2) + tx - 1, j = blockIdx.y * (TY - 2) + ty - 1;
+  const int i = blockIdx.x * (kAX - 2) + tx - 1, j = (int)(yb + blockIdx.y) * (TY - 2) + ty - 1;
   const bool cell = i >= 0 && i < L.nx && j >= 0 && j < L.ny;
   // minus-side faces of the cell, and the far walls' (of cells nx and ny)
   const bool fx = i >= 0 && i <= L.nx && j >= 0 && j < L.ny && tx > 0;
   const bool fy = j >= 0 && j <= L.ny && i >= 0 && i < L.nx && ty > 0;
   const bool inner = cell && tx > 0 && tx < kAX - 1 && ty > 0 && ty < TY - 1;
-  const int k0 = ND == 3 ? blockIdx.z * zc : 0, k1 = ND == 3 ? min(k0 + zc, L.nz) : 1;
+  const int k0 = ND == 3 ? (int)(zb + blockIdx.z) * zc : 0, k1 = ND == 3 ? min(k0 + zc, L.nz) : 1;
   const double dth = dt / L.h, kk = 0.25 * dth;
   // a radial face's area over V/h
   double wm = 1.0, wp = 1.0;
@@ -316,9 +316,11 @@ template <typename U, int G, int NF, int TY>
 void launch_bcg64(sfx_ctx* c, const Vel<U>& v, double dt, const AdvFields<NF>& P, int zc,
                   cudaStream_t s) {
   const Level& L = c->lev[0].lv;
-  const dim3 g((unsigned)((L.nx + kAX - 3) / (kAX - 2)), (unsigned)((L.ny + TY - 3) / (TY - 2)),
-               (unsigned)((L.nz + zc - 1) / zc));
-  SFX_KERNEL(c, K_ADVECT, (k_bcg64<U, G, NF, TY>), g, dim3(kAX, TY), s, L, v, dt, P, zc);
+  grid_parts((unsigned)((L.nx + kAX - 3) / (kAX - 2)), (unsigned)((L.ny + TY - 3) / (TY - 2)),
+             (unsigned)((L.nz + zc - 1) / zc), [&](dim3 g, unsigned yb, unsigned zb) {
+               SFX_KERNEL(c, K_ADVECT, (k_bcg64<U, G, NF, TY>), g, dim3(kAX, TY), s, L, v, dt, P, zc,
+                          yb, zb);
+             });
 }
 
 template <typename U, int NF>

@@ -32,7 +32,7 @@ constexpr int kCapX = 32, kCapY = 8;
 constexpr int kCapHX = kCapX + 2, kCapHY = kCapY + 2;
 constexpr int kCapThreads = (kCapHX * kCapHY + 31) / 32 * 32;
 
-// all components of n at (i,j,k) in FP64 (the arithmetic of normal_comp)
+// all components of n at (i,j,k) in FP64
 __device__ __forceinline__ void normal3_f64(const Level& L, const double* __restrict__ phi, int i,
                                             int j, int k, double eps, double* n) {
   const double inv2h = 0.5 / L.h;
@@ -168,7 +168,8 @@ sfx_status capillary_impl(sfx_ctx* c, const double* phi, const P* C, const P* si
   // than it owns), 8 or 4 where the grid would not fill the chip once
   const long long slots = (long long)c->sm_count * (sizeof(T) == 4 ? 4 : 2);
   const long long z = ((long long)gx * gy * L.nz + slots - 1) / slots;
-  const int zc = z > 8 ? 16 : (z > 4 ? 8 : 4);
+  int zc = z > 8 ? 16 : (z > 4 ? 8 : 4);
+  while (((long long)L.nz + zc - 1) / zc > 65535) zc *= 2;
   const dim3 grid(gx, gy, L.geom == SFX_CART3D ? (unsigned)((L.nz + zc - 1) / zc) : 1u);
   SFX_KERNEL(c, K_FORCES, (k_capillary<T, P>), grid, kCapThreads, s, L, phi, C, sigma, eps, zc,
              kappa, force);

@@ -64,12 +64,12 @@ struct Setup32 {
 };
 
 template <int ND>
-__global__ void __launch_bounds__(ND == 3 ? 512 : 128) k_setup32(Setup32 q) {
+__global__ void __launch_bounds__(ND == 3 ? 512 : 128) k_setup32(Setup32 q, unsigned yb, unsigned zb) {
   constexpr int BX = 32, BY = 4, BZ = ND == 3 ? 4 : 1;
   constexpr int HX = BX + 1, HY = BY + 1, HZ = ND == 3 ? BZ + 1 : 1;
   __shared__ float sn[ND][HZ][HY][HX], sp[HZ][HY][HX];
   const Level& L = q.L;
-  const int x0 = blockIdx.x * BX, y0 = blockIdx.y * BY, z0 = blockIdx.z * BZ;
+  const int x0 = blockIdx.x * BX, y0 = (int)(yb + blockIdx.y) * BY, z0 = (int)(zb + blockIdx.z) * BZ;
   for (int t = threadIdx.x; t < HX * HY * HZ; t += blockDim.x) {
     const int lx = t % HX, ly = t / HX % HY, lz = t / (HX * HY);
     const int i = x0 + lx - 1, j = y0 + ly - 1, k = ND == 3 ? z0 + lz - 1 : 0;
@@ -1797,9 +1797,11 @@ sfx_status step_f32(sfx_ctx* c, const sfx_params* pr, const double* phi_in, cons
       q.H2[d] = c->f32.H2[d];
       q.Hm[d] = c->f32.Hm[d];
     }
-    const dim3 g((unsigned)((L.nx + 31) / 32), (unsigned)((L.ny + 3) / 4), (unsigned)((L.nz + 3) / 4));
-    if (nd == 3) SFX_KERNEL(c, K_SETUP, k_setup32<3>, g, 512, s, q);
-    else SFX_KERNEL(c, K_SETUP, k_setup32<2>, g, 128, s, q);
+    grid_parts((unsigned)((L.nx + 31) / 32), (unsigned)((L.ny + 3) / 4), (unsigned)((L.nz + 3) / 4),
+               [&](dim3 g, unsigned yb, unsigned zb) {
+                 if (nd == 3) SFX_KERNEL(c, K_SETUP, k_setup32<3>, g, 512, s, q, yb, zb);
+                 else SFX_KERNEL(c, K_SETUP, k_setup32<2>, g, 128, s, q, yb, zb);
+               });
     SFX_LAUNCH_CHECK();
     ++c->f32.drift_epoch;
     c->f32.drift_phi = phi_in;

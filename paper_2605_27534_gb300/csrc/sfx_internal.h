@@ -356,6 +356,15 @@ sfx_status marangoni32(sfx_ctx* c, const sfx_params* p, const float2* f, const d
 sfx_status df_pack(const double* in, void* out, size_t n, cudaStream_t s);
 sfx_status df_unpack(const void* in, double* out, size_t n, cudaStream_t s);
 
+// A launch has 65535 blocks in y and in z at most: launch(grid, y0, z0) for the
+// parts of a grid of blocks, which start at block (0, y0, z0).
+template <class Launch>
+inline void grid_parts(unsigned x, unsigned y, unsigned z, Launch launch) {
+  for (unsigned z0 = 0; z0 < z; z0 += 65535)
+    for (unsigned y0 = 0; y0 < y; y0 += 65535)
+      launch(dim3(x, y - y0 < 65535 ? y - y0 : 65535, z - z0 < 65535 ? z - z0 : 65535), y0, z0);
+}
+
 inline int blocks_for(size_t n, int threads) {
   size_t b = (n + threads - 1) / threads;
   if (b > 152 * 64) b = 152 * 64;

@@ -107,13 +107,14 @@ __device__ __forceinline__ void unit_normal(const Level& L, const double* __rest
 }
 
 template <int ND>
-__global__ void __launch_bounds__(kSX * kSY * (ND == 3 ? 4 : 1)) k_setup64(Setup64 q) {
+__global__ void __launch_bounds__(kSX * kSY * (ND == 3 ? 4 : 1)) k_setup64(Setup64 q, unsigned yb, unsigned zb) {
   constexpr int BZ = ND == 3 ? 4 : 1;
   constexpr int HX = kSX + 1, HY = kSY + 1, HZ = ND == 3 ? BZ + 1 : 1;
   __shared__ double sn[ND][HZ][HY][HX];
   const Level& L = q.L;
-  const int x0 = blockIdx.x * kSX, y0 = blockIdx.y * kSY, z0 = blockIdx.z * BZ;
-  if (q.ctl && (blockIdx.x | blockIdx.y | blockIdx.z) == 0 && threadIdx.x < kCtlWords)
+  const int x0 = blockIdx.x * kSX, y0 = (int)(yb + blockIdx.y) * kSY,
+            z0 = (int)(zb + blockIdx.z) * BZ;
+  if (q.ctl && (x0 | y0 | z0) == 0 && threadIdx.x < kCtlWords)
     q.ctl[threadIdx.x] = 0;
   const double inv2h = 0.5 / L.h, inv_eps = 1.0 / q.eps;
   // the normal of the cell (lx, ly, lz) of the block's box with its minus layers
@@ -463,9 +464,10 @@ template <int ND>
 void launch_setup(sfx_ctx* c, const Setup64& q, cudaStream_t s) {
   const Level& L = q.L;
   constexpr int BZ = ND == 3 ? 4 : 1;
-  const dim3 g((unsigned)((L.nx + kSX - 1) / kSX), (unsigned)((L.ny + kSY - 1) / kSY),
-               (unsigned)((L.nz + BZ - 1) / BZ));
-  SFX_KERNEL(c, K_SETUP, k_setup64<ND>, g, kSX * kSY * BZ, s, q);
+  grid_parts((unsigned)((L.nx + kSX - 1) / kSX), (unsigned)((L.ny + kSY - 1) / kSY),
+             (unsigned)((L.nz + BZ - 1) / BZ), [&](dim3 g, unsigned yb, unsigned zb) {
+               SFX_KERNEL(c, K_SETUP, k_setup64<ND>, g, kSX * kSY * BZ, s, q, yb, zb);
+             });
 }
 
 constexpr double kHalfMax = 65504.0;   // the largest half
