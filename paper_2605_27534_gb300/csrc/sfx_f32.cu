@@ -2025,8 +2025,12 @@ sfx_status marangoni32(sfx_ctx* c, const sfx_params* p, const float2* f, const d
   const size_t n = L.ncell();
   Eos32 q{(float)p->gamma_inf, (float)p->eps, (float)(1.0 / p->eps), (float)p->sigma0,
           (float)p->E, p->eos, p->sigma0 * p->E, p->gamma_inf / p->eps};
-  unsigned* list = dm_mode != 0 && n >= kForceListCells ? cell_list(c, &c->force_list, s) : nullptr;
-  unsigned* band = n >= kEosListCells ? cell_list(c, &c->eos_band, s) : nullptr;
+  static_assert(kForceListCells <= kEosListCells, "one allocation for both lists");
+  const bool large = n >= kEosListCells;
+  unsigned* list = large || (dm_mode != 0 && n >= kForceListCells)
+                       ? cell_list(c, &c->force_list, large ? 2 : 1, s) : nullptr;
+  unsigned* band = large && list ? list + n + 1 : nullptr;
+  if (dm_mode == 0) list = nullptr;
   if (band) {
     SFX_CUDA(cudaMemsetAsync(band, 0, sizeof(unsigned), s));
     SFX_KERNEL(c, K_FORCES, k_eos32_bulk, blocks_for((n + 1) / 2, 256), 256, s, (ix)n, q.sigma0, phi,

@@ -269,13 +269,13 @@ __global__ void k_loss_grad(Level L, EosArgs q, const double* __restrict__ f,
 
 }  // namespace
 
-unsigned* cell_list(sfx_ctx* c, unsigned** slot, cudaStream_t s) {
+unsigned* cell_list(sfx_ctx* c, unsigned** slot, int lists, cudaStream_t s) {
   const size_t n = c->lev[0].lv.ncell();
   cudaStreamCaptureStatus cap;
   if (*slot || n >= ((size_t)1 << 32)) return *slot;
   void* p = nullptr;
   if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
-      cudaMalloc(&p, (n + 1) * sizeof(unsigned)) != cudaSuccess) {
+      cudaMalloc(&p, lists * (n + 1) * sizeof(unsigned)) != cudaSuccess) {
     cudaGetLastError();
     return nullptr;
   }

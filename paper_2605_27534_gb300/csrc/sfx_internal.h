@@ -231,8 +231,8 @@ struct sfx_ctx {
   double* vofQ = nullptr;
   void* vof_blocks = nullptr;        // on large grids active blocks with their flags
   unsigned* vof_cut = nullptr;       // and the faces that need a plane (cell_list)
-  unsigned* force_list = nullptr;    // FP32 Marangoni force: interface cells (cell_list)
-  unsigned* eos_band = nullptr;      // and cells with Gamma > 0 (cell_list)
+  unsigned* force_list = nullptr;    // FP32 Marangoni force: interface cells, and on large
+                                     // grids cells with Gamma > 0 behind them (cell_list)
   double* acdi = nullptr;            // ACDI: phi*, r, psi, unit normals
 };
 
@@ -312,12 +312,12 @@ sfx_status acdi_step(sfx_ctx* c, const void* ux, const void* uy, const void* uz,
 // sfx_capillary.cu
 sfx_status capillary(sfx_ctx* c, const sfx_params* p, const double* phi, const void* C,
                      const void* sigma, void* kappa, void* force, cudaStream_t s);
-// sfx_forces.cu: a list of cells of the context (`slot`: a count and their
-// indices, filled anew by each pass), allocated on first use; null where a
-// grid's cells do not fit 32-bit indices, no memory is left for it or its
-// first use is within a stream capture: the passes then take every cell in
+// sfx_forces.cu: `lists` lists of cells of the context (`slot`: for each a count
+// and their indices, filled anew by each pass), allocated on first use; null
+// where a grid's cells do not fit 32-bit indices, no memory is left for it or
+// its first use is within a stream capture: the passes then take every cell in
 // turn
-unsigned* cell_list(sfx_ctx* c, unsigned** slot, cudaStream_t s);
+unsigned* cell_list(sfx_ctx* c, unsigned** slot, int lists, cudaStream_t s);
 // sfx_phase.cu: allocates ctx->block_list: for the nb blocks of cells a count,
 // nb int2, six doubles and two flags per block (each pass fills it anew)
 sfx_status block_list(sfx_ctx* c);

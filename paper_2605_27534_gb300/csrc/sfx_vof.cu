@@ -309,7 +309,7 @@ sfx_status vof_impl(sfx_ctx* c, const U* const* u, double dt, int order, double*
   const unsigned char* act = nullptr;
   const VofVel<U> v{{u[0], u[1], u[2]}};
   if (c->vof_blocks) {
-    cut = cell_list(c, &c->vof_cut, s);
+    cut = cell_list(c, &c->vof_cut, 1, s);
     list = (int2*)c->vof_blocks;
     unsigned char* flag = (unsigned char*)(list + nb + 1);
     act = flag + nb;
