@@ -242,6 +242,13 @@ __device__ __forceinline__ double flux64(const Newton64& q, double Doh, const do
   return fma(Doh, fma(-cnt, a, S), T) * q.invh;
 }
 
+// What a cell of f* or F* adds to the norm of the right-hand side at least: a
+// field that is not zero but vanishes in float has a norm below the host's
+// range, not one of 0, which its residual of 0 would pass.
+__device__ __forceinline__ float nonzero_norm(double x) {
+  return (((unsigned)__double2hiint(x) << 1) | (unsigned)__double2loint(x)) != 0u ? 1e-30f : 0.0f;
+}
+
 // The system may have several solutions.  The exchange is bilinear, so the
 // difference (df, dF) of two solutions solves the linearised system at their
 // mean, with U = u + r_d and v there; its columns are dominated by their
@@ -328,8 +335,10 @@ k_resid64(Newton64 q, const double* __restrict__ f, const double* __restrict__ F
     const float idt = (float)q.inv_dt;
     m[0] = fmaxf(m[0], fabsf(rf));
     m[1] = fmaxf(m[1], fabsf(__fmaf_rn((float)fst, idt, __fmul_rn(u, (float)finf))));
+    m[1] = fmaxf(m[1], nonzero_norm(fst));
     m[2] = fmaxf(m[2], fabsf(rF));
     m[3] = fmaxf(m[3], fabsf(__fmaf_rn((float)Fst, idt, __fmul_rn((float)q.kd, (float)fc))));
+    m[3] = fmaxf(m[3], nonzero_norm(Fst));
     // off the branch (above): as a non-finite norm
     const float U = __fadd_rn(u, (float)q.kd);
     if (!(fabsf(rf) <= 3.0e38f) || !(fabsf(rF) <= 3.0e38f) || U < -0.45f * idt ||
