@@ -505,7 +505,7 @@ sfx_status solve(sfx_ctx* c, const Newton64& q, double* f, double* F, bool from_
                                   (int)kT2Smem));
   }
   *conv = false;
-  float first = 0.0f;
+  float first = 0.0f, back[3] = {0.0f, 0.0f, 0.0f};   // the first residual; the last three
   // the host reads an iteration's norms while the GPU works on the next one
   for (int it = 1; it <= cap + 1; ++it) {
     if (it <= cap) {
@@ -555,6 +555,15 @@ sfx_status solve(sfx_ctx* c, const Newton64& q, double* f, double* F, bool from_
     const float worst = (float)std::max(rel[0], rel[1]);
     if (prev == 1) first = worst;
     if (worst > 1e3f * std::max(first, 1.0f)) return SFX_OK;   // diverging
+    // at the best of its last three rates it would not get there: stalled (at
+    // the rounding of the residual, for a tolerance below it) or too slow
+    if (prev >= 6) {
+      const double rate = std::min({worst / back[0], back[0] / back[1], back[1] / back[2]});
+      if (!(rate < 0.999) || prev + std::log(o->tol / worst) / std::log(rate) > cap + 1) return SFX_OK;
+    }
+    back[2] = back[1];
+    back[1] = back[0];
+    back[0] = worst;
   }
   return SFX_OK;
 }
