@@ -7,14 +7,15 @@ is the hand-written discrete adjoint of the library (sfx_adjoint_step,
 sfx_marangoni_loss, sfx_f_from_gamma), giving dL/dGamma0 and dL/dtheta for
 theta = (k_a, k_d, D_f, D_F).  The forward keeps a checkpoint of the state
 every K steps and every state of the last segment, which the backward walks
-first; the backward recomputes each earlier segment of K steps from its
-checkpoint and walks it backwards.  (The backward holds the states of one
-segment at a time in any case.  Recomputing the last one, once for its end
-and once for its states, ran every step of a rollout within K steps three
-times: eight steps at 256x256 with their gradient 7.65 -> 4.4 ms.)  The
-forward may run in an SFX_F32
-context (double-float state); the adjoint always works in FP64 on the
-recomputed states.  Every step of the computation runs in libsfx kernels.
+first, freeing each state behind its step (a second backward of a retained
+graph recomputes them); the backward recomputes each earlier segment of K steps
+from its checkpoint and walks it in the same way.  An open graph so holds its
+checkpoints and the states of at most K steps, and its backward never more than
+that.  (Recomputing the last segment, once for its end and once for its states,
+ran every step of a rollout within K steps three times: eight steps at 256x256
+with their gradient 7.65 -> 4.4 ms.)  The forward may run in an SFX_F32
+context (double-float state); the adjoint always works in FP64 on these
+states.  Every step of the computation runs in libsfx kernels.
 """
 from __future__ import annotations
 
@@ -58,6 +59,16 @@ def _forward_steps(setup: RolloutSetup, ps: Params, f, F, n):
         # no stats: the step then skips its totals and their host wait (a
         # step that fails to converge still raises)
         ctx.sfx_surfactant_step(ps, setup.phi, f, F, setup.dt, opts=o, stats=False)
+
+
+def _segment(setup: RolloutSetup, ps: Params, start, n):
+    """The states after each of n steps from the checkpoint `start`."""
+    f, F = (t.clone() for t in start)
+    states = []
+    for _ in range(n):
+        _forward_steps(setup, ps, f, F, 1)
+        states.append((f.clone(), F.clone()))
+    return states
 
 
 def _to_state(ctx, x):
@@ -104,22 +115,22 @@ class SurfactantRollout(torch.autograd.Function):
         setup, ps = fctx.setup, fctx.ps
         ctx = setup.context
         o = default_opts(tol=setup.adj_tol, max_cycles=1000, nu1=10, nu2=10)
+        last, fctx.last = fctx.last, None
+        if last is None:           # a second backward of the same graph
+            last = _segment(setup, ps, fctx.checkpoints[-1],
+                            setup.nsteps - (len(fctx.checkpoints) - 1) * setup.K)
         # the final state, for dL/df
-        last_f = (fctx.last or fctx.checkpoints)[-1][0]
+        last_f = (last or fctx.checkpoints)[-1][0]
         _, gf = ctx.sfx_marangoni_loss(ps, _to_double(ctx, last_f), setup.phi, setup.C,
                                        setup.dm_mode, grad=True)
         lam_f = gf * float(gL)
         lam_F = torch.zeros_like(lam_f)
         dtheta = [0.0, 0.0, 0.0, 0.0]
         for s in range(len(fctx.checkpoints) - 1, -1, -1):
-            states = fctx.last
-            if s < len(fctx.checkpoints) - 1:
-                f, F = (t.clone() for t in fctx.checkpoints[s])
-                states = []
-                for _ in range(setup.K):
-                    _forward_steps(setup, ps, f, F, 1)
-                    states.append((f.clone(), F.clone()))
-            for f1, F1 in reversed(states):
+            states = last if s == len(fctx.checkpoints) - 1 else \
+                _segment(setup, ps, fctx.checkpoints[s], setup.K)
+            while states:          # (frees each state behind its step)
+                f1, F1 = states.pop()
                 ctx.sfx_adjoint_step(ps, setup.phi, _to_double(ctx, f1), _to_double(ctx, F1),
                                      setup.dt, lam_f, lam_F, dtheta, o)
         dgamma = ctx.sfx_f_from_gamma(lam_f, setup.phi, ps.eps)
