@@ -91,3 +91,18 @@ def test_residual_schedule_text(bench, fast, incr, tiled, want):
     text = bench.residual_schedule(_Opts(fast, incr, tiled), True)
     assert text.endswith(want), text
     assert bench.residual_schedule(_Opts(fast, incr, tiled), False) == "pair arithmetic"
+
+
+def test_vof_bytes_count_the_blocks_that_hold_or_touch_fluid(bench):
+    """Ragged grid of 3 x 4 x 3 blocks of 32 x 4 x 4 cells: one cell of fluid in
+    the block in the middle makes 27 of them active, in the corner block 8; a dry
+    grid pays the passes over every cell only."""
+    torch = pytest.importorskip("torch")
+    C = torch.zeros(10, 15, 70, dtype=torch.float64)
+    every = 20.0 * C.numel()
+    assert bench.vof_bytes(C) == every
+    C[5, 5, 40] = 0.25
+    assert bench.vof_bytes(C) == every + 148.0 * 512 * 27
+    C[5, 5, 40] = 0.0
+    C[9, 14, 69] = 1.0
+    assert bench.vof_bytes(C) == every + 148.0 * 512 * 8
