@@ -209,6 +209,18 @@ k_bcg64(Level L, Vel<U> v, double dt, AdvFields<NF> P, int zc, unsigned yb, unsi
           A[q][d] = x0;
         }
       }
+      // no slopes, but a velocity that is not finite times 0 is a transverse term
+      if (flat) {
+        bool ok = finite_bits(v.u[0][c + (size_t)k * L.ny + j]);
+        ok &= finite_bits(v.u[0][c + (size_t)k * L.ny + j + 1]);
+        ok &= finite_bits(v.u[1][c + (size_t)k * L.nx]);
+        ok &= finite_bits(v.u[1][c + (size_t)k * L.nx + L.nx]);
+        if (ND == 3) {
+          ok &= finite_bits(v.u[2][c]);
+          ok &= finite_bits(v.u[2][c + sz]);
+        }
+        flat = ok;
+      }
       if (!flat) {
         // mean velocities of the cell: dt/(2h) vbar
         kv[0] = (widen(v.u[0][c + (size_t)k * L.ny + j]) + widen(v.u[0][c + (size_t)k * L.ny + j + 1])) * kk;

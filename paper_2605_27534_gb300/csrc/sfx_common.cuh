@@ -75,6 +75,14 @@ __device__ __forceinline__ float narrow(double x) {
   return ((hi << 1) | lo) == 0u ? __uint_as_float(hi) : (float)x;
 }
 
+// neither NaN nor infinite, from the integer words
+__device__ __forceinline__ bool finite_bits(float x) {
+  return (__float_as_uint(x) & 0x7f800000u) != 0x7f800000u;
+}
+__device__ __forceinline__ bool finite_bits(double x) {
+  return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u;
+}
+
 // Row r = k ny + j (64-bit division only past 2^32).
 __device__ __forceinline__ void row_jk(size_t r, int ny, int& j, int& k) {
   if (r >> 32) {

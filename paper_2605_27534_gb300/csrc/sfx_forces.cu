@@ -135,10 +135,6 @@ k_force(Level L, const double* __restrict__ phi, const double* __restrict__ C,
     force64_cell(L, phi, C, sigma, 0, eps, c, force, dm_out);
 }
 
-__device__ __forceinline__ bool finite_bits(double x) {
-  return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u;
-}
-
 // With the PLIC area only interface cells carry a force.  A block gathers those
 // of its 512 cells and takes them by full warps: a cell is a chain of about 600 FP64 instructions, an instruction occupies the SM's FP64 pipe for a
 // whole warp however few lanes it serves, and in rows of 32 cells a warp held

@@ -45,12 +45,6 @@ __device__ __forceinline__ bool wet(double C) {
   return b > 0 || (unsigned long long)b > 0xfff0000000000000ULL;
 }
 
-__device__ __forceinline__ bool finite_bits(float x) {
-  return (__float_as_uint(x) & 0x7f800000u) != 0x7f800000u;
-}
-__device__ __forceinline__ bool finite_bits(double x) {
-  return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u;
-}
 __device__ __forceinline__ bool positive(double x) {   // false for NaN
   return (unsigned long long)vbits(x) - 1ULL < 0x7ff0000000000000ULL;
 }
