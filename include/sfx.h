@@ -18,7 +18,14 @@
  *   by sfx_ctx_destroy.
  * Streams.  `stream` is a cudaStream_t passed as void* (NULL = legacy default
  *   stream).  Work is enqueued on it in order.  Calls that report statistics
- *   or iterate to a tolerance synchronise with that stream before returning.
+ *   or iterate to a tolerance synchronise with that stream before returning,
+ *   with stats = NULL too: the fields are final then.  A context serves one
+ *   host thread at a time.  Its calls on different streams may overlap if they
+ *   are different calls, each of which has its own scratch (and two
+ *   sfx_advect, two sfx_capillary_force, or in SFX_F64 two
+ *   sfx_marangoni_force, which have none); not two of one kind, and not two of
+ *   those that solve, reduce or differentiate (steps, sfx_mg_solve,
+ *   sfx_totals, sfx_cfl_dt, sfx_adjoint_*, sfx_marangoni_loss).
  * Errors.  Every call returns an sfx_status; nothing is thrown across the
  *   ABI.  sfx_status_string() names a status.  On SFX_ERR_ARG nothing was
  *   enqueued.  On SFX_ERR_NOT_CONVERGED the fields hold the last iterate and
@@ -184,7 +191,10 @@ sfx_status sfx_mg_solve(sfx_ctx* ctx, double D, const double* Bx,
    |c_f| <= 1/2.  Walls carry no flux.  C: double, in place; velocities in
    the context precision; SFX_F32 contexts evaluate the PLIC geometry of the
    fluxes in FP32 (fluxes to ~1e-7, C still conserved exactly).  Planar 2D and 3D (SFX_ERR_ARG for axisymmetric
-   grids).  The context allocates two scratch arrays on first use. */
+   grids).  A face or cell value that is not finite makes the cells that the
+   formula takes it into NaN, empty ones (0 times it) included.  The context
+   allocates its scratch on first use (9 bytes per cell; on grids of 2^20 cells
+   and more 4 more and a block list). */
 sfx_status sfx_vof_advect(sfx_ctx* ctx, const void* ux, const void* uy, const void* uz,
                           double dt, int order, double* C, void* stream);
 
@@ -200,11 +210,13 @@ sfx_status sfx_vof_advect(sfx_ctx* ctx, const void* ux, const void* uy, const vo
    |grad phi| < 1e-30.  f and F
    (state layout of the context) are updated in place; phi is double, the
    velocities are in the context precision.  SFX_F64 contexts with
-   opts->mg_levels = 0 and max(Df, DF) dt/h^2 <= 1 (planar grids: and no
-   velocities) solve the coupled system by Newton defect correction instead (FP64 state and residuals, the
-   correction relaxed by nu1 + nu2 FP32 red-black sweeps with a 2x2 block
-   solve per cell) and fall back to Picard iteration where it does not
-   converge; stats then count its iterations.  SFX_F32 contexts solve the
+   opts->mg_levels = 0, max(Df, DF) dt/h^2 <= 1 and max(Df, DF) <= 65504 eps
+   (planar grids: and no velocities) solve the coupled system by Newton defect
+   correction instead (FP64 state and residuals, norms in float, the correction
+   relaxed by nu1 + nu2 FP32 red-black sweeps with a 2x2 block solve per cell
+   and half-precision drifts).  They fall back to Picard iteration where that
+   does not converge, meets scales outside the FP32 range or leaves the
+   physical branch; stats then count its iterations.  SFX_F32 contexts solve the
    same system by coupled Newton defect correction (SFX_TUNE_F32_SOLVER):
    each iteration evaluates both residuals in pair arithmetic and relaxes
    the correction by nu1 + nu2 FP32 red-black sweeps with a 2x2 block solve

@@ -83,7 +83,7 @@ struct Mg32Coef {
 // Work arrays of SFX_F32 contexts (float drifts, double-float f*, F*).
 struct F32Scratch {
   bool ready = false;
-  float* Bf[3] = {};
+  float* Bf[3] = {};      // (solvers 0 and 2)
   float* BF[3] = {};
   float2* B2[3] = {};     // (B_f, B_F) per face (the Newton residual pass)
   __half2* H2[3] = {};    // (B_f, B_F) per face in half precision (correction sweeps)
@@ -91,7 +91,7 @@ struct F32Scratch {
   float2* Fstar = nullptr;
   float* dsig = nullptr;   // sigma - sigma0
   int predicted = 0;       // Picard iterations to run before the first check
-  float2* falt = nullptr;  // ping-pong partners of f and F for fused sweeps
+  float2* falt = nullptr;  // ping-pong partners of f and F (solvers 0 and 2)
   float2* Falt = nullptr;
   bool fused = true;       // one launch per red-black sweep
   int zchunk = 32;         // planes per block of the 3D fused sweep

@@ -217,7 +217,7 @@ static_assert(sizeof(Ctl64) == kCtlWords * sizeof(int), "control words");
 // radial ones.
 template <int G>
 __device__ __forceinline__ double flux64(const Newton64& q, double Doh, const double* B,
-                                         const double* nb, const bool* has, double a,
+                                         const double* nb, double a,
                                          const double* w) {
   constexpr int NQ = G == SFX_CART3D ? 6 : 4;
   const bool lit = q.p.literal != 0;
@@ -302,8 +302,8 @@ k_resid64(Newton64 q, const double* __restrict__ f, const double* __restrict__ F
       Bf[s] = q.Bf[s / 2][fi[s]];        // zero on walls
       BF[s] = q.BF[s / 2][fi[s]];
     }
-    const double flf = flux64<G>(q, q.Doh[0], Bf, nf, has, fc, w);
-    const double flF = flux64<G>(q, q.Doh[1], BF, nF, has, Fc, w);
+    const double flf = flux64<G>(q, q.Doh[0], Bf, nf, fc, w);
+    const double flF = flux64<G>(q, q.Doh[1], BF, nF, Fc, w);
     const double c1 = q.c1[c], finf = q.finf[c], fst = q.fs[c], Fst = q.Fs[c];
     const double vd = c1 * (finf - fc);
     const double ex = fma(vd, Fc, -(q.kd * fc));     // c1 F (f_inf - f) - r_d f
@@ -591,12 +591,14 @@ sfx_status drift_faces64(sfx_ctx* c, const double* phi, double Df, double DF, do
 // index with 32 bits and its launches put rows in grid y.  The sweeps' drift
 // faces are half precision and at most D/eps: larger ones are left to the
 // Picard solver as well.
-// Planar steps with a flow stay with the Picard solver too: at tol = 1e-10 its
-// states there carry an error of up to 4e-9 in the force (of 30 circles of 50
-// to 512 cells a side, rotating, a third above 1e-9), and programs that
-// compare FP64 runs to 1e-9 would see the change of solver, although Newton's
-// error is 1e-13.  Without a flow, and in the other geometries, the two agree
-// to 3e-10.
+// Planar steps with a flow stay with the Picard solver too.  That is no property
+// of the solvers - the Newton solve is the faster (512^2: 0.87 against 8.0 ms) and
+// the more exact one there as well (1e-13 against up to 4e-9 in the force) - but
+// of what programs that compare FP64 runs would see: on 30 rotating circles of 50
+// to 512 cells a side, at tol = 1e-10, a third of the forces moved by more than
+// 1e-9 between the solvers.  On the steps drawn alike without a flow, and in the
+// other geometries, no force moved by more than 3e-10.  mg_levels = 1 or more
+// names the Picard solver for any step.
 bool newton64_eligible(const sfx_ctx* c, const sfx_params* p, double dt, const sfx_solve_opts* o,
                        bool flow) {
   const Level& L = c->lev[0].lv;
