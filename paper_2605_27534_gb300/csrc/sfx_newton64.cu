@@ -74,22 +74,21 @@ __device__ __forceinline__ void unit_normal(const Level& L, const double* __rest
   const size_t st[3] = {1, (size_t)L.nx, (size_t)L.nx * L.ny};
   const size_t c = cidx(L, x[0], x[1], x[2]);
   const double pc = phi[c];
-  if (((unsigned)__double2hiint(pc) & 0x7ff00000u) == 0x7ff00000u) {
-    // the drift of its faces, a multiple of phi, is not a number
-#pragma unroll
-    for (int d = 0; d < ND; ++d) n[d] = pc - pc;
-    return;
-  }
   double a[ND], b[ND];
-  bool flat = true;
+  bool flat = finite_bits(pc);
 #pragma unroll
   for (int d = 0; d < ND; ++d) {
     a[d] = phi[x[d] + 1 < L.extent(d) ? c + st[d] : c];
     b[d] = phi[x[d] > 0 ? c - st[d] : c];
-    flat = flat && bits_eq(a[d], b[d]);
+    flat &= bits_eq(a[d], b[d]);
     n[d] = 0.0;
   }
   if (flat) return;
+  if (!finite_bits(pc)) {   // the drift of its faces, a multiple of phi, is not a number
+#pragma unroll
+    for (int d = 0; d < ND; ++d) n[d] = pc - pc;
+    return;
+  }
   double m2 = 0.0;
 #pragma unroll
   for (int d = 0; d < ND; ++d) {
@@ -372,7 +371,7 @@ k_resid64(Newton64 q, const double* __restrict__ f, const double* __restrict__ F
 // none that is not finite (the sweeps overflow float where 1/dt is beyond
 // 1e19; no residual follows that would see it).
 __device__ __forceinline__ float2 added(float2 e, const Ctl64* __restrict__ ctl) {
-  if (fabsf(e.x) <= 3.0e38f && fabsf(e.y) <= 3.0e38f) return e;
+  if (finite_bits(e.x) && finite_bits(e.y)) return e;
   return ctl->done ? make_float2(0.0f, 0.0f) : e;
 }
 
