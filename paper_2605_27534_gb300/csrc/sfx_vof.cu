@@ -31,7 +31,7 @@ namespace {
 // widened without the conversion instruction, which issues at the FP64 rate.
 // 256^3 sphere of radius 64 in float: 2.45 ms per step with every face and
 // cell, 0.46 ms now (planes 69, other faces 39, update 24 us per direction,
-// classification 30 us), 0.70 ms after 500 steps of wisps.  The geometry is
+// classification 30 us), 0.72 ms after 500 steps of wisps.  The geometry is
 // inlined once per kernel, for the flow in either direction: twice, its code
 // did not fit the instruction cache (planes 102 us; small grids, where a pass
 // lasts one chain, 28 us instead of 24).
