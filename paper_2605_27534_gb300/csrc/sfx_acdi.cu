@@ -48,6 +48,12 @@ constexpr double kAcdiVeps = 1e-6;
 // falls below 0.1 only where veps dominates psi (phi or 1 - phi below
 // ~0.1 veps).
 constexpr double kAcdiKappa = 0.1;
+// Grids of fewer cells do without marks: two launches less, and in cell blocks a
+// launch of few blocks lasts as long as the fullest of them.  A step of a circle
+// or sphere at rest without and with marks, in FP64 and FP32 contexts: 128^2 29,
+// 51 and 23, 37 us, 32^3 33, 62 and 28, 40, 48^3 72, 80 and 45, 56, 64^3 147, 96
+// and 81, 62.
+constexpr size_t kAcdiMarkCells = (size_t)1 << 17;
 
 // psi/(2h) in float from phi* in [0, 1]: phi* may overshoot by O(veps) where
 // it saturates, and past 1 + veps psi would have no value.  1 - phi is taken
@@ -70,6 +76,21 @@ __device__ __forceinline__ double clip01(double v) {
   return b < 0x3ff0000000000000ULL ? v : 1.0;
 }
 
+// The cell of this thread: with marks (MARK), in cell blocks, of which a block
+// takes a quarter in FP64 contexts (BITS), whose passes are the FP64 pipe's
+// throughout, to even out over the SMs; without, cells in turn.
+template <int ND, bool BITS, bool MARK>
+__device__ __forceinline__ bool acdi_at(const Level& L, int* x) {
+  if (MARK && !BITS) return CellBlock<ND>::at(L, blockIdx.x, x);
+  if (MARK) return CellBlock<ND>::at(L, blockIdx.x / 4, x, (int)(blockIdx.x % 4 * 128 + threadIdx.x));
+  const unsigned c = blockIdx.x * blockDim.x + threadIdx.x;   // (small grids)
+  const unsigned r = c / (unsigned)L.nx;
+  x[0] = (int)(c - r * (unsigned)L.nx);
+  x[1] = (int)(r % (unsigned)L.ny);
+  x[2] = (int)(r / (unsigned)L.ny);
+  return x[2] < L.nz;
+}
+
 template <int ND>
 __device__ __forceinline__ void neighbours(const Level& L, const int* x, size_t c, size_t* o,
                                            bool* has) {
@@ -85,11 +106,11 @@ __device__ __forceinline__ void neighbours(const Level& L, const int* x, size_t 
 
 // mark[c] = 1 where |grad psi| in float is not safely below kAcdiKappa (or
 // not a number: the FP64 passes decide)
-template <int ND>
+template <int ND, bool BITS>
 __global__ void k_acdi_mark(Level L, const float* __restrict__ psi, float thr2,
                             unsigned char* __restrict__ mark) {
   int x[3];
-  if (!CellBlock<ND>::at(L, blockIdx.x, x)) return;
+  if (!acdi_at<ND, BITS, true>(L, x)) return;
   const size_t c = cidx(L, x[0], x[1], x[2]);
   size_t o[2 * ND];
   bool has[2 * ND];
@@ -103,21 +124,27 @@ __global__ void k_acdi_mark(Level L, const float* __restrict__ psi, float thr2,
   mark[c] = m2 < thr2 ? 0 : 1;
 }
 
+// The mark of cell c; without marks every cell counts as marked.
+template <bool MARK>
+__device__ __forceinline__ int marked(const unsigned char* __restrict__ mark, size_t c) {
+  return MARK ? mark[c] : 1;
+}
+
 // r^(1/2) (BITS: r) and psi of the cells that a marked cell's normal or faces
 // read
-template <int ND, bool BITS>
+template <int ND, bool BITS, bool MARK>
 __global__ void k_acdi_cell(Level L, const unsigned char* __restrict__ mark,
                             const double* __restrict__ ps, double eps, double* __restrict__ g,
                             double* __restrict__ psi) {
   int x[3];
-  if (!CellBlock<ND>::at(L, blockIdx.x, x)) return;
+  if (!acdi_at<ND, BITS, MARK>(L, x)) return;
   const size_t c = cidx(L, x[0], x[1], x[2]);
   size_t o[2 * ND];
   bool has[2 * ND];
   neighbours<ND>(L, x, c, o, has);
-  int any = mark[c];
+  int any = marked<MARK>(mark, c);
 #pragma unroll
-  for (int q = 0; q < 2 * ND; ++q) any |= mark[o[q]];
+  for (int q = 0; q < 2 * ND; ++q) any |= marked<MARK>(mark, o[q]);
   if (!any) return;
   const double p = clip01(ps[c]);
   const double rc = (p + kAcdiVeps) / (1.0 - p + kAcdiVeps);
@@ -127,13 +154,13 @@ __global__ void k_acdi_cell(Level L, const unsigned char* __restrict__ mark,
 
 // n = grad psi/|grad psi| of the marked cells (centred differences,
 // zero-gradient ghosts), 0 where psi is flat (above)
-template <int ND, bool BITS>
+template <int ND, bool BITS, bool MARK>
 __global__ void k_acdi_normal(Level L, const unsigned char* __restrict__ mark,
                               const double* __restrict__ psi, double* __restrict__ nv) {
   int x[3];
-  if (!CellBlock<ND>::at(L, blockIdx.x, x)) return;
+  if (!acdi_at<ND, BITS, MARK>(L, x)) return;
   const size_t c = cidx(L, x[0], x[1], x[2]), n = L.ncell();
-  if (!mark[c]) return;
+  if (!marked<MARK>(mark, c)) return;
   // the 1/(2h) of the differences cancels in n; the threshold takes it
   // (kAcdiKappa is far above the guard 1e-30)
   const double thr = kAcdiKappa * (2.0 * L.h);
@@ -163,26 +190,26 @@ __global__ void k_acdi_normal(Level L, const unsigned char* __restrict__ mark,
 
 // The BITS form of the update below: per face the flux
 // zeta [eps (phi*_R - phi*_L)/h - 1/4 w_f nbar_f], w_f = 4 s/(1 + s)^2.
-template <int ND, bool AXI>
+template <int ND, bool AXI, bool MARK>
 __global__ void k_acdi_update_bits(Level L, const unsigned char* __restrict__ mark,
                                    const double* __restrict__ ps, const double* __restrict__ r,
                                    const double* __restrict__ nv, double zeta, double eps,
                                    double dt, int clip, double* __restrict__ phi) {
   int x[3];
-  if (!CellBlock<ND>::at(L, blockIdx.x, x)) return;
+  if (!acdi_at<ND, true, MARK>(L, x)) return;
   const size_t c = cidx(L, x[0], x[1], x[2]), n = L.ncell();
   size_t o[2 * ND];
   bool has[2 * ND];
   neighbours<ND>(L, x, c, o, has);
   const double invh = 1.0 / L.h, pc = ps[c];
-  const int mc = mark[c];
+  const int mc = marked<MARK>(mark, c);
   double div = 0.0;
   for (int q = 0; q < 2 * ND; ++q) {
     if (!has[q]) continue;
     const double s = q & 1 ? 1.0 : -1.0;
     double w = 1.0;
     if (AXI && q < 2) w = 2.0 * (double)(x[0] + q) / (double)(2 * x[0] + 1);
-    const int mo = mark[o[q]];
+    const int mo = marked<MARK>(mark, o[q]);
     double af;
     if (mc | mo) {
       const double* nd = nv + (size_t)(q / 2) * n;
@@ -212,7 +239,7 @@ __global__ void k_acdi_update_bits(Level L, const unsigned char* __restrict__ ma
 // Rows of 40 doubles keep the two rows of a half warp in different banks.
 // 160^3 after 40 steps: 425 -> 304 us; after one 180 -> 145 us (with two instead
 // of three blocks per SM 335 and 165; clipping on the FP64 pipe 319 and 160).
-template <int ND, bool AXI>
+template <int ND, bool AXI, bool MARK>
 __global__ void __launch_bounds__(512, 3)
 k_acdi_update(Level L, const unsigned char* __restrict__ mark, const double* __restrict__ ps,
               const double* __restrict__ g, const double* __restrict__ nv, double k1, double k2,
@@ -238,11 +265,11 @@ k_acdi_update(Level L, const unsigned char* __restrict__ mark, const double* __r
     size_t o[2 * ND];
     bool has[2 * ND];
     neighbours<ND>(L, x, c, o, has);
-    any = mark[c];
+    any = marked<MARK>(mark, c);
     pc = ps[c];
 #pragma unroll
     for (int q = 0; q < 2 * ND; ++q) {
-      any |= mark[o[q]];
+      any |= marked<MARK>(mark, o[q]);
       const double dp = ps[o[q]] - pc;      // 0 at a wall
       lap = AXI && q < 2 ? fma(wr[q], dp, lap) : lap + dp;
     }
@@ -256,7 +283,7 @@ k_acdi_update(Level L, const unsigned char* __restrict__ mark, const double* __r
     const int yd = d == 0 ? yx : (d == 1 ? yy : yz);
     if (yd > 0 && yx < L.nx && yy < L.ny && yz < L.nz) {
       const size_t r = cidx(L, yx, yy, yz), m = r - st[d];
-      const int mr = mark[r], mm = mark[m];
+      const int mr = marked<MARK>(mark, r), mm = marked<MARK>(mark, m);
       if (mr | mm) {
         const double* nd = nv + (size_t)d * n;
         nn = (mr ? nd[r] : 0.0) + (mm ? nd[m] : 0.0);
@@ -301,23 +328,28 @@ k_acdi_update(Level L, const unsigned char* __restrict__ mark, const double* __r
   phi[c] = clip ? clip01(v) : v;
 }
 
-template <int ND, bool AXI>
+template <int ND, bool AXI, bool MARK>
 void acdi_passes(sfx_ctx* c, const double* ps, double* g, double* psi, double* nv,
                  const float* psi32, unsigned char* mark, float thr2, double zeta, double eps,
                  double dt, int clip, double* phi, cudaStream_t s) {
   const Level& L = c->lev[0].lv;
-  const int nb = (int)CellBlock<ND>::count(L), nt = CellBlock<ND>::threads;
-  SFX_KERNEL(c, K_PHASE, k_acdi_mark<ND>, nb, nt, s, L, psi32, thr2, mark);
+  constexpr int threads = CellBlock<ND>::threads;
+  const int blocks = (int)CellBlock<ND>::count(L), turns = (int)((L.ncell() + 255) / 256);
   if (c->prec == SFX_F64) {
-    SFX_KERNEL(c, K_PHASE, (k_acdi_cell<ND, true>), nb, nt, s, L, mark, ps, eps, g, psi);
-    SFX_KERNEL(c, K_PHASE, (k_acdi_normal<ND, true>), nb, nt, s, L, mark, psi, nv);
-    SFX_KERNEL(c, K_PHASE, (k_acdi_update_bits<ND, AXI>), nb, nt, s, L, mark, ps, g, nv, zeta, eps,
-               dt, clip, phi);
+    const int nt = MARK ? threads / 4 : 256, nb = MARK ? 4 * blocks : turns;
+    if (MARK) SFX_KERNEL(c, K_PHASE, (k_acdi_mark<ND, true>), nb, nt, s, L, psi32, thr2, mark);
+    SFX_KERNEL(c, K_PHASE, (k_acdi_cell<ND, true, MARK>), nb, nt, s, L, mark, ps, eps, g, psi);
+    SFX_KERNEL(c, K_PHASE, (k_acdi_normal<ND, true, MARK>), nb, nt, s, L, mark, psi, nv);
+    SFX_KERNEL(c, K_PHASE, (k_acdi_update_bits<ND, AXI, MARK>), nb, nt, s, L, mark, ps, g, nv, zeta,
+               eps, dt, clip, phi);
   } else {
     const double k1 = dt * zeta * eps / (L.h * L.h), k2 = 0.5 * dt * zeta / L.h;
-    SFX_KERNEL(c, K_PHASE, (k_acdi_cell<ND, false>), nb, nt, s, L, mark, ps, eps, g, psi);
-    SFX_KERNEL(c, K_PHASE, (k_acdi_normal<ND, false>), nb, nt, s, L, mark, psi, nv);
-    SFX_KERNEL(c, K_PHASE, (k_acdi_update<ND, AXI>), nb, nt, s, L, mark, ps, g, nv, k1, k2, clip, phi);
+    const int nt = MARK ? threads : 256, nb = MARK ? blocks : turns;
+    if (MARK) SFX_KERNEL(c, K_PHASE, (k_acdi_mark<ND, false>), nb, nt, s, L, psi32, thr2, mark);
+    SFX_KERNEL(c, K_PHASE, (k_acdi_cell<ND, false, MARK>), nb, nt, s, L, mark, ps, eps, g, psi);
+    SFX_KERNEL(c, K_PHASE, (k_acdi_normal<ND, false, MARK>), nb, nt, s, L, mark, psi, nv);
+    SFX_KERNEL(c, K_PHASE, (k_acdi_update<ND, AXI, MARK>), blocks, threads, s, L, mark, ps, g, nv, k1,
+               k2, clip, phi);
   }
 }
 
@@ -336,21 +368,27 @@ sfx_status acdi_step(sfx_ctx* c, const void* ux, const void* uy, const void* uz,
   double* psi = g + n;
   double* nv = psi + n;
   float* psi32 = (float*)nv;              // read before the normals are written
-  unsigned char* mark = (unsigned char*)(nv + (size_t)L.ndim() * n);
+  unsigned char* mark = n >= kAcdiMarkCells ? (unsigned char*)(nv + (size_t)L.ndim() * n) : nullptr;
   if (ux) {
     sfx_status st = advect_phi(c, ux, uy, uz, dt, phi, 1.0, ps, s);
     if (st != SFX_OK) return st;
   } else {
     SFX_CUDA(cudaMemcpyAsync(ps, phi, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
   }
-  SFX_KERNEL(c, K_PHASE, k_acdi_psi32, blocks_for(n, 256), 256, s, n, ps, (float)(0.5 * eps / L.h),
-             psi32);
+  if (mark)
+    SFX_KERNEL(c, K_PHASE, k_acdi_psi32, blocks_for(n, 256), 256, s, n, ps, (float)(0.5 * eps / L.h),
+               psi32);
   // the float psi/(2h) is good to a few 1e-7 of its largest value 7 eps/h
   const double thr = std::max(0.0, 0.9 * kAcdiKappa - 1e-4 * eps / L.h);
   const float thr2 = (float)(thr * thr);
-  if (L.geom == SFX_CART3D) acdi_passes<3, false>(c, ps, g, psi, nv, psi32, mark, thr2, zeta, eps, dt, clip, phi, s);
-  else if (L.geom == SFX_AXISYM) acdi_passes<2, true>(c, ps, g, psi, nv, psi32, mark, thr2, zeta, eps, dt, clip, phi, s);
-  else acdi_passes<2, false>(c, ps, g, psi, nv, psi32, mark, thr2, zeta, eps, dt, clip, phi, s);
+  const auto passes = [&](auto marked, auto every) {
+    (mark ? marked : every)(c, ps, g, psi, nv, psi32, mark, thr2, zeta, eps, dt, clip, phi, s);
+  };
+  switch (L.geom) {
+    case SFX_CART3D: passes(&acdi_passes<3, false, true>, &acdi_passes<3, false, false>); break;
+    case SFX_AXISYM: passes(&acdi_passes<2, true, true>, &acdi_passes<2, true, false>); break;
+    default: passes(&acdi_passes<2, false, true>, &acdi_passes<2, false, false>);
+  }
   SFX_LAUNCH_CHECK();
   return SFX_OK;
 }
