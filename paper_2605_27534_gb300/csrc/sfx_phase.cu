@@ -124,18 +124,20 @@ __device__ __forceinline__ T rd_uniform(double h, double C, T dtau, int iters) {
 
 // chi0 (the first iterate) and aux of every cell; rough[b] = 1 where a cell
 // of block b differs from a face neighbour in C.  The last block also fills
-// uni for the last pass.
-template <typename T, int ND>
+// uni for the last pass.  (LIST false: chi0 and aux alone, in blocks of 128
+// threads that take a quarter of a cell block each.)
+template <typename T, int ND, bool LIST>
 __global__ void __launch_bounds__(512) k_rd_init(Level L, RdGrid R, const double* __restrict__ C,
                                                  T* __restrict__ aux, T* __restrict__ chi,
                                                  unsigned char* __restrict__ rough, T dtau,
                                                  int iters, double eps, RdUniform* uni) {
   using B = RdBlk<ND>;
   const int nb = R.nbx * R.nby * R.nbz;
-  const int3 lc = B::cell(threadIdx.x);
+  constexpr int sub = LIST ? 1 : 4;
+  const int3 lc = B::cell((int)(blockIdx.x % sub * (B::threads / sub) + threadIdx.x));
   const int lx = lc.x, ly = lc.y, lz = lc.z;
   const size_t st[3] = {1, (size_t)L.nx, (size_t)L.nx * L.ny};
-  for (int b = blockIdx.x; b < nb; b += gridDim.x) {
+  for (int b = (int)blockIdx.x / sub; b < nb; b += (int)gridDim.x / sub) {
     const int i = (b % R.nbx) * kBx + lx, j = (b / R.nbx % R.nby) * B::by + ly,
               k = b / R.nbx / R.nby * B::bz + lz;
     bool diff = false;
@@ -173,10 +175,11 @@ __global__ void __launch_bounds__(512) k_rd_init(Level L, RdGrid R, const double
       aux[c] = a;
       chi[c] = s0;
     }
+    if (!LIST) continue;
     diff = __syncthreads_or(diff);
     if (threadIdx.x == 0) rough[b] = diff ? 1 : 0;
   }
-  if (blockIdx.x == gridDim.x - 1 && threadIdx.x < 2) {
+  if (LIST && blockIdx.x == gridDim.x - 1 && threadIdx.x < 2) {
     const double x = (double)rd_uniform<T>(L.h, (double)threadIdx.x, dtau, iters), p = phi_of(x, eps);
     uni->chi[threadIdx.x] = x;
     uni->phi[threadIdx.x] = p;
@@ -265,8 +268,8 @@ __device__ __forceinline__ bool is_inf_bits(float a) {
 __device__ __forceinline__ bool is_neg_bits(double a) { return __double_as_longlong(a) < 0; }
 __device__ __forceinline__ bool is_neg_bits(float a) { return __float_as_int(a) < 0; }
 
-// One Jacobi step of every active block.
-template <typename T, int ND>
+// One Jacobi step of every active block, or (LIST false) of every block.
+template <typename T, int ND, bool LIST>
 __global__ void __launch_bounds__(512) k_rd_step(Level L, RdGrid R, T dtau,
                                                  const int2* __restrict__ list,
                                                  const T* __restrict__ aux,
@@ -279,9 +282,9 @@ __global__ void __launch_bounds__(512) k_rd_step(Level L, RdGrid R, T dtau,
   const int lx = lc.x, ly = lc.y, lz = lc.z;
   const int lo[3] = {lx, ly, lz}, last[3] = {kBx - 1, B::by - 1, B::bz - 1};
   const size_t st[3] = {1, (size_t)L.nx, (size_t)L.nx * L.ny};
-  const int count = list[0].x;
+  const int count = LIST ? list[0].x : R.nbx * R.nby * R.nbz;
   for (int q = (int)blockIdx.x / sub; q < count; q += step) {
-    const int2 e = list[1 + q];
+    const int2 e = LIST ? list[1 + q] : make_int2(q, 63);
     const int b = e.x;
     const int i = (b % R.nbx) * kBx + lx, j = (b / R.nbx % R.nby) * B::by + ly,
               k = b / R.nbx / R.nby * B::bz + lz;
@@ -472,16 +475,17 @@ __global__ void __launch_bounds__(kRdWX* kRdRows)
   }
 }
 
-// phi and delta from chi.  Far from the interface chi holds one value over
-// whole blocks, so a block's first cell is evaluated once and its value
-// shared: only the band pays an FP64 tanh per cell.
+// phi and delta from chi, and (chi_out not null) chi from an iterate.  Far from
+// the interface chi holds one value over whole blocks, so a block's first cell
+// is evaluated once and its value shared: only the band pays an FP64 tanh per
+// cell.
+template <typename T>
 __global__ void __launch_bounds__(256)
-k_phi_delta64(size_t n, double eps, const double* __restrict__ chi, double* __restrict__ phi,
-              double* __restrict__ delta) {
+k_phi_delta64(size_t n, double eps, const T* chi, double* chi_out, double* phi, double* delta) {
   __shared__ double sx, sp;
   for (size_t b = blockIdx.x * (size_t)blockDim.x; b < n; b += (size_t)gridDim.x * blockDim.x) {
     const size_t c = b + threadIdx.x;
-    const double x = c < n ? chi[c] : 0.0;
+    const double x = c < n ? (double)chi[c] : 0.0;
     if (threadIdx.x == 0) {
       sx = x;
       sp = phi_of(x, eps);
@@ -489,6 +493,7 @@ k_phi_delta64(size_t n, double eps, const double* __restrict__ chi, double* __re
     __syncthreads();
     if (c < n) {
       const double p = same_bits(x, sx) ? sp : phi_of(x, eps);
+      if (chi_out) chi_out[c] = x;
       phi[c] = p;
       if (delta) delta[c] = p * (1.0 - p) / eps;
     }
@@ -520,8 +525,24 @@ static sfx_status redistance_blocks(sfx_ctx* c, const double* C, T* aux, T* a, T
   const size_t sub = B::threads / kStepThreads;
   const int grid = (int)std::min(nb * sub, (size_t)c->sm_count * 12 / sub * sub);
   const int sg = (int)std::min((nb + 255) / 256, (size_t)c->sm_count * 8);
+  // where all blocks are resident at once inactive ones cost a step nothing, and
+  // finding the active ones four to five launches: every block iterates (7 steps
+  // of 35 x 86: 75 -> 58 us, 24 of 15 x 31 x 30 186 -> 163, of 48^3 325 -> 298)
+  if (nb * sub <= (size_t)grid) {
+    SFX_KERNEL(c, K_PHASE, (k_rd_init<T, ND, false>), grid, kStepThreads, s, L, R, C, aux, a,
+               nullptr, (T)dtau, iters, eps, nullptr);
+    for (int it = 0; it < iters; ++it) {
+      SFX_KERNEL(c, K_PHASE, (k_rd_step<T, ND, false>), grid, kStepThreads, s, L, R, (T)dtau, nullptr,
+                 aux, a, b);
+      std::swap(a, b);
+    }
+    SFX_KERNEL(c, K_PHASE, k_phi_delta64<T>, blocks_for(L.ncell(), 256), 256, s, L.ncell(), eps, a, chi,
+               phi, delta);
+    SFX_LAUNCH_CHECK();
+    return SFX_OK;
+  }
   SFX_CUDA(cudaMemsetAsync(list, 0, sizeof(int2), s));
-  SFX_KERNEL(c, K_PHASE, (k_rd_init<T, ND>), full, 512, s, L, R, C, aux, a, f0, (T)dtau,
+  SFX_KERNEL(c, K_PHASE, (k_rd_init<T, ND, true>), full, 512, s, L, R, C, aux, a, f0, (T)dtau,
              iters, eps, uni);
   const int ext[3] = {kBx, B::by, B::bz};
   unsigned char *fi = f0, *fo = f1;
@@ -531,7 +552,8 @@ static sfx_status redistance_blocks(sfx_ctx* c, const double* C, T* aux, T* a, T
   }
   SFX_KERNEL(c, K_PHASE, k_rd_list, sg, 256, s, R, fi, list);
   for (int it = 0; it < iters; ++it) {
-    SFX_KERNEL(c, K_PHASE, (k_rd_step<T, ND>), grid, kStepThreads, s, L, R, (T)dtau, list, aux, a, b);
+    SFX_KERNEL(c, K_PHASE, (k_rd_step<T, ND, true>), grid, kStepThreads, s, L, R, (T)dtau, list, aux, a,
+               b);
     std::swap(a, b);
   }
   SFX_KERNEL(c, K_PHASE, (k_rd_finish<T, ND>), full, 512, s, L, R, (T)dtau, iters, eps, fi, uni,
@@ -579,7 +601,7 @@ sfx_status phase_field_build(sfx_ctx* c, const double* C, double* chi, void* phi
       first = false;
       std::swap(a, b);
     } while (it < iters || last_in_scratch);
-    SFX_KERNEL(c, K_PHASE, k_phi_delta64, nb, 256, s, n, eps, chi, ph, de);
+    SFX_KERNEL(c, K_PHASE, k_phi_delta64<double>, nb, 256, s, n, eps, chi, nullptr, ph, de);
     SFX_LAUNCH_CHECK();
     return SFX_OK;
   }
@@ -592,7 +614,8 @@ sfx_status phase_field_build(sfx_ctx* c, const double* C, double* chi, void* phi
 sfx_status phase_field_from_chi(sfx_ctx* c, const double* chi, double* phi, double* delta,
                                 double eps, cudaStream_t s) {
   const size_t n = c->lev[0].lv.ncell();
-  SFX_KERNEL(c, K_PHASE, k_phi_delta64, blocks_for(n, 256), 256, s, n, eps, chi, phi, delta);
+  SFX_KERNEL(c, K_PHASE, k_phi_delta64<double>, blocks_for(n, 256), 256, s, n, eps, chi, nullptr, phi,
+             delta);
   SFX_LAUNCH_CHECK();
   return SFX_OK;
 }
