@@ -19,7 +19,10 @@
 // per plane.  What bounds it is the latency of those chains (seven quotients
 // and a root, the FP64 pipe's in SFX_F64 contexts): 160^3 in float 167 -> 130
 // us, 120 x 110 x 100 in double 670 -> 504, 50 x 64 x 40 in float 119 -> 20 (with
-// chunks of 32 planes throughout 184, 625, 75 us).
+// chunks of 32 planes throughout 184, 625, 75 us).  2D grids, whose one plane
+// waits for nothing, keep a thread per cell, three warps of which take a second
+// normal: in double 512^2 67 -> 49 us, 1024^2 209 -> 152 by the ring and the
+// planes known at compile time alone (72 and 250 with the threads of 3D).
 #include <algorithm>
 
 #include "sfx_f32_dev.cuh"
@@ -31,6 +34,7 @@ namespace {
 constexpr int kCapX = 32, kCapY = 8;
 constexpr int kCapHX = kCapX + 2, kCapHY = kCapY + 2;
 constexpr int kCapThreads = (kCapHX * kCapHY + 31) / 32 * 32;
+constexpr int kCap2D = kCapX * kCapY;
 
 // all components of n at (i,j,k) in FP64
 __device__ __forceinline__ void normal3_f64(const Level& L, const double* __restrict__ phi, int i,
@@ -76,13 +80,13 @@ struct CapNormal<float> {
 
 // T: arithmetic type (double in SFX_F64 contexts, float in SFX_F32);
 // P: storage type of C, sigma, kappa and the force.
-template <typename T, typename P>
-__global__ void __launch_bounds__(kCapThreads, sizeof(T) == 4 ? 4 : 1)
+template <typename T, typename P, bool is3d>
+__global__ void __launch_bounds__(is3d ? kCapThreads : kCap2D, sizeof(T) == 4 ? 4 : 1)
     k_capillary(Level L, const double* __restrict__ phi, const P* __restrict__ C,
                 const P* __restrict__ sigma, double eps, int zc, P* __restrict__ kappa,
                 P* __restrict__ force) {
   // ring of four planes of normals, each with a one-cell halo in x and y
-  __shared__ T sn[4][3][kCapHY][kCapHX];
+  __shared__ T sn[is3d ? 4 : 1][is3d ? 3 : 2][kCapHY][kCapHX];
   const int tx = threadIdx.x % kCapX, ty = threadIdx.x / kCapX;
   const int i0 = blockIdx.x * kCapX, j0 = blockIdx.y * kCapY;
   const int i = i0 + tx, j = j0 + ty;
@@ -90,21 +94,30 @@ __global__ void __launch_bounds__(kCapThreads, sizeof(T) == 4 ? 4 : 1)
   const int px = threadIdx.x % kCapHX, py = threadIdx.x / kCapHX;
   const int a = i0 + px - 1, b = j0 + py - 1;
   const bool halo = py < kCapHY, cell = halo && a >= 0 && a < L.nx && b >= 0 && b < L.ny;
-  const bool is3d = L.geom == SFX_CART3D;
   const int k0 = is3d ? (int)blockIdx.z * zc : 0;
   const int k1 = is3d ? min(k0 + zc, L.nz) : 1;
   const size_t N = L.ncell();
   const T inv_h = (T)(1.0 / L.h);
 
-  // normals of plane k (tile and halo, one per thread) into ring slot k % 4
+  // normals of plane k (tile and halo) into ring slot k % 4: in 3D one per thread
   auto fill = [&](int k) {
     T n[3] = {(T)0, (T)0, (T)0};
-    if (cell) CapNormal<T>::eval(L, phi, a, b, k, eps, n);
-    if (halo) {
-      T(*s)[kCapHY][kCapHX] = sn[k & 3];
-      s[0][py][px] = n[0];
-      s[1][py][px] = n[1];
-      s[2][py][px] = n[2];
+    if (is3d) {
+      if (cell) CapNormal<T>::eval(L, phi, a, b, k, eps, n);
+      if (halo) {
+        T(*s)[kCapHY][kCapHX] = sn[k & 3];
+        s[0][py][px] = n[0];
+        s[1][py][px] = n[1];
+        s[is3d ? 2 : 0][py][px] = n[2];
+      }
+      return;
+    }
+    for (int q = threadIdx.x; q < kCapHX * kCapHY; q += kCap2D) {
+      const int qx = q % kCapHX, qy = q / kCapHX, e = i0 + qx - 1, f = j0 + qy - 1;
+      n[0] = n[1] = (T)0;
+      if (e >= 0 && e < L.nx && f >= 0 && f < L.ny) CapNormal<T>::eval(L, phi, e, f, k, eps, n);
+      sn[0][0][qy][qx] = n[0];
+      sn[0][1][qy][qx] = n[1];
     }
   };
 
@@ -114,7 +127,7 @@ __global__ void __launch_bounds__(kCapThreads, sizeof(T) == 4 ? 4 : 1)
     if (is3d && k + 1 < L.nz) fill(k + 1);
     __syncthreads();
     if (own) {
-      T(*s)[kCapHY][kCapHX] = sn[k & 3];
+      T(*s)[kCapHY][kCapHX] = sn[is3d ? k & 3 : 0];
       const int hx = tx + 1, hy = ty + 1;
       T wm = (T)1, wp = (T)1;
       if (L.geom == SFX_AXISYM) {
@@ -171,8 +184,12 @@ sfx_status capillary_impl(sfx_ctx* c, const double* phi, const P* C, const P* si
   int zc = z > 8 ? 16 : (z > 4 ? 8 : 4);
   while (((long long)L.nz + zc - 1) / zc > 65535) zc *= 2;
   const dim3 grid(gx, gy, L.geom == SFX_CART3D ? (unsigned)((L.nz + zc - 1) / zc) : 1u);
-  SFX_KERNEL(c, K_FORCES, (k_capillary<T, P>), grid, kCapThreads, s, L, phi, C, sigma, eps, zc,
-             kappa, force);
+  if (L.geom == SFX_CART3D)
+    SFX_KERNEL(c, K_FORCES, (k_capillary<T, P, true>), grid, kCapThreads, s, L, phi, C, sigma, eps,
+               zc, kappa, force);
+  else
+    SFX_KERNEL(c, K_FORCES, (k_capillary<T, P, false>), grid, kCap2D, s, L, phi, C, sigma, eps, zc,
+               kappa, force);
   SFX_LAUNCH_CHECK();
   return SFX_OK;
 }
