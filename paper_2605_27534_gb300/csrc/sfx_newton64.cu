@@ -20,7 +20,7 @@
 //
 // Measured against the Picard solver (4 iterations of one V-cycle per field):
 // a 128^2 no-flow step with its force 5.4 -> 0.14 ms, 131 x 257 axisymmetric
-// (odd: one level, 40 coarse sweeps) 5.7 -> 0.17 ms, a 96^3 step 19.2 -> 1.12 ms
+// (odd: one level, 40 coarse sweeps) 5.7 -> 0.17 ms, a 96^3 step 19.2 -> 1.15 ms
 // (residual 71 us for 0.88 M cells: 46 FP64 instructions per cell, the pipe 76 %
 // busy; Picard's was 370 us); the error against a 64-bit solution
 // falls from 1e-11 to 5e-14 at tol = 1e-10.
